@@ -759,7 +759,7 @@ def main():
     sweep_ms = sum(solve_ms) / max(full_equiv, 1e-9)
     bell_achieved = bpsw / (sweep_ms / 1e3) / 1e9
     cs = kernel_counters("bellman_kernel_fused3", env.name) if n_fused == 3 else None
-    roof_build = {"kernel": "build_warp_kernel (+ build_fp32_kernel on wide slices)", "bound": "alu",
+    roof_build = {"kernel": "build_group_kernel (+ build_fp32_kernel on wide slices)", "bound": "alu",
                   "achieved": build_achieved, "peak": issue_peak, "unit": "T warp-inst/s",
                   "frac": build_achieved / issue_peak if cb else None,
                   "traffic": cb["dram_bytes_per_unit"] * n_slices if cb else None,

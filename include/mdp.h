@@ -122,8 +122,9 @@ typedef struct {
                               mdp_autotune) if one was recorded or loaded, else 256 */
   int32_t chunk;           /* realizations staged per pass by that kernel; 0 = the autotuner's
                               choice, else 1024 */
-  int32_t hist_cap;        /* fine-count table cells (32-bit words) per warp of the
-                              warp-per-slice kernel, <= 6144; 0 = the autotuner's choice,
+  int32_t hist_cap;        /* fine-count table cells (32-bit words) per slice of the group
+                              build kernel, <= 6144 (the power of two below is used, a state
+                              of a slice taking its equal share); 0 = the autotuner's choice,
                               else 2048; slices whose tables need more go to the
                               full-window kernel (1 sends every sampled slice there) */
 } mdp_build_opts;
@@ -356,8 +357,8 @@ mdp_status mdp_rollout(const mdp_env *env, const mdp_grid *grid, const mdp_actio
  * authors tuned threads per block by hand for each GPU, Sec. IV-D; here the
  * library does it).  A class is (actions padded to a power of two, modes, N
  * and cells rounded to powers of two, objectives, precision).  The shapes:
- * warps per CTA (4, 8) and fine-table words per warp (1536..4096) of the
- * warp-per-slice build kernel, the CTA size of the full-window kernel when the
+ * warps per CTA (4, 8) and fine-table words per slice (1536..4096) of the
+ * group build kernel, the CTA size of the full-window kernel when the
  * calibration defers slices to it, and the shared memory of the
  * one-state-per-slice Bellman sweep (132, 160, 190 KiB: its slot size).
  * No choice changes a count, entry, R, value or policy -- only the speed.

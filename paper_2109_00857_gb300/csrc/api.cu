@@ -347,6 +347,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
   rw.c_f = actions->c_f; rw.c_r = actions->c_r; rw.r_term = actions->r_term;
   rw.r_out = actions->r_outbound; rw.dt = grid->dt; rw.dx = grid->dx; rw.n_obj = n_obj;
   for (int o = 0; o < n_obj; ++o) rw.objs[o] = objs_h[o];
+  rw.set_floats();
 
   auto fail = [&](mdp_status code) {
     free_model_memory(m, st);
@@ -499,7 +500,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
   // the full-window kernels hold an [L*L][32] histogram in shared memory: the
   // FP32 one halves its realization chunk until it fits (the model does not
   // depend on the chunk); beyond that (sub-grids above 41 x 41 cells) only
-  // the warp kernel's slices can be built
+  // the group kernel's slices can be built
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, m->device);
   const size_t window_limit = (size_t)smem_max - 1024;   // the kernels' static shared memory
@@ -512,8 +513,19 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
   const int build_warps = tun.build_warps;
   if (hist_cap > 6144) return fail(arg_fail("hist_cap must be <= 6144"));
   uint32_t *defer = nullptr;
-  if (prec == MDP_FP32) TRY(dev_alloc((void **)&defer, sizeof(uint32_t) * (size_t)m->n_slices, st));
+  float2 *mom = nullptr;   // a caller's coefficients: their moments per layer (the count windows)
+  if (prec == MDP_FP32) {
+    TRY(dev_alloc((void **)&defer, sizeof(uint32_t) * (size_t)m->n_slices, st));
+    if (env->coeffs && env->K > 0) {
+      TRY(dev_alloc((void **)&mom, sizeof(float2) * (size_t)grid->nt * env->K, st));
+      TRY(launch_coeff_moments(static_cast<const float *>(env->coeffs), grid->nt, N, env->K, mom, st));
+      ++launches;
+    }
+  }
   ba.cap_bins = hist_cap;
+  ba.mom = mom;
+  if (!env->coeffs)
+    for (int k = 0; k < env->K; ++k) ba.coef_var[k] = (float)(env->sigma_h[k] * env->sigma_h[k]);
   ba.defer = defer;
   ba.defer_in = nullptr;
   if (hook) {
@@ -521,6 +533,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
     hook->Yown = Yown;
     hook->sigma_d = sig_d;
     hook->defer = defer;
+    hook->mom = mom;
     hook->pool_cols = cap_cols;
     hook->threads = threads;
     *out = m;
@@ -535,7 +548,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
       TRY(launch_build_fp64(ba, st));
       ++launches;
     } else {
-      // warp-per-slice kernel, then the full-window CTA kernel over what it deferred
+      // group kernel, then the full-window CTA kernel over what it deferred
       TRY(launch_build_warp(ba, build_warps, num_sms(), st));
       BuildArgs bd = ba;
       bd.defer_in = defer;
@@ -565,6 +578,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
       if (Yown) dev_free(Yown, st);
       if (sig_d) dev_free(sig_d, st);
       if (defer) dev_free(defer, st);
+      dev_free(mom, st);
       return fail(MDP_ERR_BUDGET);
     }
     // does not fit the device (or the 32-bit block offsets): reported as MDP_ERR_OOM below
@@ -586,6 +600,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
   if (Yown) dev_free(Yown, st);
   if (sig_d) dev_free(sig_d, st);
   if (defer) dev_free(defer, st);
+  dev_free(mom, st);
   m->deferred = (int64_t)c[CNT_DEFER_N];
 
   float ms = 0.f, kms = 0.f;

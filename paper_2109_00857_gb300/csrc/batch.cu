@@ -4,13 +4,12 @@
 // Create: every item is first built once on its own to calibrate it (the
 // autotuner): the sub-grid side (given or sized from the field extremes), the
 // entry-pool columns it needs, its widest slice, and how many slices overflow
-// the warp kernel's histogram; from these the batch picks the per-lane
-// histogram capacity, sizes each item's pool exactly (plus a margin), and
+// the group kernel's tables; from these the batch picks the table capacity, sizes each item's pool exactly (plus a margin), and
 // sizes the Bellman stages for the widest slice.  Then each item is set up
 // through the same path as mdp_build (allocations, coefficient table, cell
 // classes) without launching its build.
-// Run: one persistent warp-per-slice launch per (states per warp, mode
-// count) group builds its items' slices from one work queue; one CTA launch
+// Run: one persistent launch per (states per slice, mode count) group of items
+// builds their slices from one work queue; one CTA launch
 // finishes the slices any item deferred;
 // the solve runs batched steps -- with tol = 0 the layered pass (step k
 // updates layer nt - k of every item that has it, in place: the exact fixed
@@ -69,10 +68,11 @@ struct mdp_batch_t {
     BatchCta *ctas_d = nullptr;
   };
   SolveClass cls[2];
-  // build launches: items grouped by (states per warp, mode count), each
+  // build launches: items grouped by (states per slice, mode count), each
   // group one persistent launch over its own zero-based prefix segment
   struct Group {
     int start, n, pstart, K, spw;
+    bool dense;
   };
   std::vector<Group> groups;
   size_t cta_smem = 0;
@@ -96,6 +96,7 @@ void batch_release(mdp_batch_t *b) {
     dev_free(it.hook.Yown, b->st);
     dev_free(it.hook.sigma_d, b->st);
     dev_free(it.hook.defer, b->st);
+    dev_free(it.hook.mom, b->st);
     dev_free(it.Vb, b->st);
     dev_free(it.lflags, b->st);
     dev_free(it.res, b->st);
@@ -127,13 +128,15 @@ cudaError_t enqueue(mdp_batch_t *b) {
     if (e == cudaSuccess && it.hook.Yown)
       e = launch_sample_coeffs(g.nt, it.desc.N, env.K, it.hook.sigma_d, env.seed, env.mdp_id, nullptr,
                                (float *)it.hook.Yown, it.m->cnt + CNT_CAPPED, st);
+    if (e == cudaSuccess && it.hook.mom)
+      e = launch_coeff_moments(static_cast<const float *>(env.coeffs), g.nt, it.desc.N, env.K, it.hook.mom, st);
     if (e == cudaSuccess)
       e = launch_prepare(env.obstacle, env.target, it.m->cls, g.nx, g.ny, g.nt, it.m->delta, it.L, st);
   }
   for (size_t g = 0; g < b->groups.size() && e == cudaSuccess; ++g) {
     const auto &G = b->groups[g];
     e = launch_build_warp_batch(b->items_d + G.start, b->prefix_d + G.pstart, G.n, b->work_d + g, b->cap_bins,
-                                G.K, G.spw, st);
+                                G.K, G.spw, G.dense, st);
   }
   if (e == cudaSuccess) e = launch_build_fp32_batch(b->items_d, b->n, b->cta_smem, b->cta_threads, st);
   for (int i = 0; i < b->n && e == cudaSuccess; ++i) {
@@ -258,7 +261,6 @@ extern "C" mdp_status mdp_batch_create(const mdp_batch_item *items_h, int32_t n,
   b->cap_bins = tuned_cap > 0 ? tuned_cap : ((wide * 500 > total_slices) ? 4096 : 2048);
   // ---- set-up of every item through the build path, without launching it
   std::vector<BuildArgs> args(n);
-  std::vector<int64_t> prefix(n + 1, 0);
   std::vector<BatchSolveItem> sitems(n);
 
   // solve classes: the warp-per-slice items first, then the grouped ones
@@ -312,7 +314,6 @@ extern "C" mdp_status mdp_batch_create(const mdp_batch_item *items_h, int32_t n,
     args[i] = it.hook.args;
     args[i].defer_in = it.hook.defer;
     b->cta_smem = std::max(b->cta_smem, fp32_smem_bytes(args[i], b->cta_threads));
-    prefix[i + 1] = prefix[i] + m->n_slices;
     BatchSolveItem &si = sitems[slot[i]];
     memset(&si, 0, sizeof(si));
     si.a.pool = m->pool; si.a.slice_off = m->slice_off; si.a.slice_w = m->slice_w; si.a.nnz = m->nnz;
@@ -332,32 +333,30 @@ extern "C" mdp_status mdp_batch_create(const mdp_batch_item *items_h, int32_t n,
     si.stats = it.stats;
     si.max_sweeps = it.max_sweeps;
   }
-  // group the build items by (states per warp, mode count); prefix segments per group
+  // group the build items by (states per slice, mode count, threshold density); prefix segments per group
   std::vector<int> ord(n);
   for (int i = 0; i < n; ++i) ord[i] = i;
-  auto cls = [&](int i) {
-    const int sc = args[i].spw == 1 ? 0 : (args[i].spw == 2 ? 1 : 2);
-    return sc * 64 + std::min<int>(args[i].K, 63);
-  };
+  auto dense = [&](int i) { return args[i].act.Mx > 2 || args[i].act.My > 2; };
+  auto cls = [&](int i) { return (dense(i) ? 4096 : 0) + args[i].spw * 64 + std::min<int>(args[i].K, 63); };
   std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cls(x) < cls(y); });
   std::vector<BuildArgs> sorted(n);
   std::vector<int64_t> gprefix;
   for (int j = 0; j < n;) {
     int e = j;
     while (e < n && cls(ord[e]) == cls(ord[j])) ++e;
-    mdp_batch_t::Group G{j, e - j, (int)gprefix.size(), args[ord[j]].K, args[ord[j]].spw};
-    if (G.spw != 1 && G.spw != 2) G.spw = 0;
+    mdp_batch_t::Group G{j, e - j, (int)gprefix.size(), args[ord[j]].K, args[ord[j]].spw, dense(ord[j])};
+    const int per = batch_group_slices(G.spw);   // slices per group of the kernel's work queue
     int64_t acc = 0;
     gprefix.push_back(0);
     for (int q = j; q < e; ++q) {
       sorted[q] = args[ord[q]];
-      acc += args[ord[q]].n_slices;
+      acc += (args[ord[q]].n_slices + per - 1) / per;
       gprefix.push_back(acc);
     }
     b->groups.push_back(G);
     j = e;
   }
-  (void)prefix;
+
   ce = dev_alloc((void **)&b->items_d, sizeof(BuildArgs) * n, b->st);
   if (ce == cudaSuccess) ce = dev_alloc((void **)&b->prefix_d, sizeof(int64_t) * gprefix.size(), b->st);
   if (ce == cudaSuccess) ce = dev_alloc((void **)&b->work_d, sizeof(unsigned long long) * b->groups.size(), b->st);

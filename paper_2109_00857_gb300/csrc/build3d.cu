@@ -485,14 +485,14 @@ __global__ void __launch_bounds__(256, sizeof(RT) == 4 ? 4 : 1) build3d_kernel(B
         if (sink) {
           for (int o = 0; o < a.rw.n_obj; ++o) {
             if constexpr (sizeof(RT) == 4)
-              Racc[o] = fmaf((float)sink / (float)a.N, (float)a.rw.r_out, Racc[o]);
+              Racc[o] = fmaf((float)sink / (float)a.N, a.rw.f_r_out, Racc[o]);
             else
               Racc[o] = __dadd_rn(Racc[o], __dmul_rn(__ddiv_rn((double)sink, (double)a.N), a.rw.r_out));
           }
         }
       } else if (kind_l == KIND_SINK) {
         for (int o = 0; o < a.rw.n_obj; ++o)
-          Racc[o] = sizeof(RT) == 4 ? (RT)(float)a.rw.r_out : (RT)__dmul_rn(__ddiv_rn((double)a.N, (double)a.N), a.rw.r_out);
+          Racc[o] = sizeof(RT) == 4 ? (RT)a.rw.f_r_out : (RT)__dmul_rn(__ddiv_rn((double)a.N, (double)a.N), a.rw.r_out);
       }
       if (!write) {
         e = 0;
@@ -820,9 +820,9 @@ __device__ bool warp3_slice(const Build3Args &a, int64_t sl, uint32_t *tab, Warp
             Racc[o] = fmaf((float)n / (float)a.N, step_reward32(a.rw, a.rw.objs[o], F, g_s, g_sp, is_t), Racc[o]);
         }
     if (sink)
-      for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = fmaf((float)sink / (float)a.N, (float)a.rw.r_out, Racc[o]);
+      for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = fmaf((float)sink / (float)a.N, a.rw.f_r_out, Racc[o]);
   } else if (kind_l == KIND_SINK) {
-    for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = (float)a.rw.r_out;
+    for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = a.rw.f_r_out;
   }
   if (!write) {
     e = 0;
@@ -1008,6 +1008,7 @@ extern "C" mdp_status mdp_build3d_ex(const mdp_env3d *env, const mdp_grid3d *gri
   rw.c_f = actions->c_f; rw.c_r = actions->c_r; rw.r_term = actions->r_term;
   rw.r_out = actions->r_outbound; rw.dt = grid->dt; rw.dx = grid->dx; rw.n_obj = n_obj;
   for (int o = 0; o < n_obj; ++o) rw.objs[o] = objs_h[o];
+  rw.set_floats();
   m->rw = rw;
 
   cudaEvent_t ev0, ev1;

@@ -14,12 +14,19 @@ enum : int {
   KIND_NONE = 3       // padding lane (s >= |S| or a >= A)
 };
 
+// s / Nc (the time layer) for 0 <= s < nS: a 32-bit division unless the model
+// has 2^32 states (a 64-bit one is about a hundred instructions).
+__device__ __forceinline__ int64_t layer_of(int64_t s, int64_t Nc, int64_t nS) {
+  if ((nS >> 32) == 0) return (int64_t)((uint32_t)s / (uint32_t)Nc);
+  return s / Nc;
+}
+
 __device__ __forceinline__ int state_kind(const BuildArgs &a, int64_t s) {
   if (s >= a.nS) return KIND_NONE;
   const uint8_t c = a.cls[s];
   if (c & CLS_TARGET) return KIND_TERMINAL;     // terminal is tested first (Alg. 2)
   if (c & CLS_OBSTACLE) return KIND_SINK;
-  if (s / a.Nc == a.nt - 1) return KIND_SINK;   // beyond the finite horizon
+  if (s >= a.nS - a.Nc) return KIND_SINK;       // t = nt - 1: beyond the finite horizon
   return KIND_SAMPLE;
 }
 
@@ -58,19 +65,23 @@ __device__ __forceinline__ double step_reward64(const RewardParams &rw, int obj,
   return r;
 }
 
+// FP32: base(o) + the part that depends on the landing cell.
+// reward_base32: everything known from the row (net energy: before hc g_sp and dt).
+__device__ __forceinline__ float reward_base32(const RewardParams &rw, int obj, float F, float g_s) {
+  if (obj == MDP_OBJ_TIME) return -rw.f_dt;
+  const float eF = __fmul_rn(__fmul_rn(rw.f_c_f, F), F);
+  if (obj == MDP_OBJ_ENERGY) return __fmul_rn(-eF, rw.f_dt);
+  return fmaf(rw.f_hc, g_s, -eF);
+}
+__device__ __forceinline__ float reward_cell32(const RewardParams &rw, int obj, float base, float g_sp,
+                                               bool is_target) {
+  float r = obj == MDP_OBJ_NET_ENERGY ? __fmul_rn(fmaf(rw.f_hc, g_sp, base), rw.f_dt) : base;
+  if (is_target) r = __fadd_rn(r, rw.f_r_term);
+  return r;
+}
 __device__ __forceinline__ float step_reward32(const RewardParams &rw, int obj, float F,
                                                float g_s, float g_sp, bool is_target) {
-  float r;
-  if (obj == MDP_OBJ_TIME) {
-    r = -(float)rw.dt;
-  } else if (obj == MDP_OBJ_ENERGY) {
-    r = -((float)rw.c_f * F * F) * (float)rw.dt;
-  } else {
-    const float hc = 0.5f * (float)rw.c_r;
-    r = ((-((float)rw.c_f * F * F) + hc * g_s) + hc * g_sp) * (float)rw.dt;
-  }
-  if (is_target) r += (float)rw.r_term;
-  return r;
+  return reward_cell32(rw, obj, reward_base32(rw, obj, F, g_s), g_sp, is_target);
 }
 
 template <typename RT>
@@ -160,7 +171,7 @@ __device__ void emit_slice(const BuildArgs &a, uint32_t *hist, int64_t sl,
       if constexpr (sizeof(RT) == 8)
         Racc[o] = __dmul_rn(__ddiv_rn((double)a.N, (double)a.N), a.rw.r_out);
       else
-        Racc[o] = (RT)a.rw.r_out;
+        Racc[o] = (RT)a.rw.f_r_out;
     }
   } else if (kind == KIND_SAMPLE) {
     const int64_t t = s / a.Nc, c = s % a.Nc;
@@ -209,7 +220,7 @@ __device__ void emit_slice(const BuildArgs &a, uint32_t *hist, int64_t sl,
           const double p = __ddiv_rn((double)sink, (double)a.N);
           Racc[o] = __dadd_rn(Racc[o], __dmul_rn(p, a.rw.r_out));
         } else {
-          Racc[o] = fmaf((float)sink * invN, (float)a.rw.r_out, Racc[o]);
+          Racc[o] = fmaf((float)sink * invN, a.rw.f_r_out, Racc[o]);
         }
       }
     }

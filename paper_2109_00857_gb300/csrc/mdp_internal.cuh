@@ -96,6 +96,16 @@ struct RewardParams {
   double c_f, c_r, r_term, r_out, dt, dx;
   int32_t n_obj;
   int32_t objs[3];
+  // the FP32 kernels' values, rounded once on the host (a conversion from FP64
+  // inside an emit loop is an FP64-rate instruction per use); hc = c_r / 2
+  float f_c_f, f_hc, f_r_term, f_r_out, f_dt;
+  void set_floats() {
+    f_c_f = (float)c_f;
+    f_hc = 0.5f * (float)c_r;
+    f_r_term = (float)r_term;
+    f_r_out = (float)r_out;
+    f_dt = (float)dt;
+  }
 };
 
 // Everything the build kernels need, passed by value.
@@ -117,16 +127,18 @@ struct BuildArgs {
   unsigned long long *cnt;
   int32_t chunk;             // realizations per staged pass (FP32 CTA kernel)
   int64_t slice_begin, slice_end;  // work range [begin, end)
-  int32_t cap_bins;          // fine-table words per warp of the warp kernel
-  uint32_t *defer;           // slices deferred by the warp kernel ([n_slices])
+  int32_t cap_bins;          // fine-table words per slice of the group kernel (used: the power of two below)
+  const float2 *mom;         // [nt][K] mean and variance of a caller's coefficients (nullptr: drawn, mean 0)
+  float coef_var[kMaxModes]; // variances of drawn coefficients
+  uint32_t *defer;           // slices deferred by the group kernel ([n_slices])
   const uint32_t *defer_in;  // non-NULL: the CTA kernel works on this list (count CNT_DEFER_N)
   // HYB spill area (nullptr: none; rows beyond row_cap then only count their
   // need in CNT_SPILL_WORDS / CNT_SPILL_FULL)
   uint32_t *spill;
   uint32_t *spill_off;       // [n_slices] word offset of the slice's block, or kNoSlice
   uint64_t spill_cap_words;
-  // single-model warp kernel: 0 = persistent warps (one CTA wave pulls every
-  // slice); q > 0 = each warp builds at most q slices and the grid covers the
+  // single-model group kernel: 0 = persistent CTAs (one CTA wave pulls every
+  // group); q > 0 = each CTA builds at most q groups and the grid covers the
   // model, so CTAs retire all along the build and the block scheduler can
   // place higher-priority work (another request's launches) between them
   int32_t slices_per_warp;
@@ -206,11 +218,13 @@ cudaError_t launch_sample_coeffs(int nt, int N, int K, const double *sigma_d, ui
                                  uint64_t mdp_id, double *Y64, float *Y32,
                                  unsigned long long *capped, cudaStream_t st);
 // build
-// warp-per-slice kernel (fast path) followed by the CTA kernel over the
-// slices it deferred (fine tables larger than cap_bins)
+// group kernel (fast path) followed by the CTA kernel over the slices it
+// deferred (fine tables larger than cap_bins)
 cudaError_t launch_build_fp32(const BuildArgs &a, int threads, int sms, cudaStream_t st);
 cudaError_t launch_build_warp(const BuildArgs &a, int warps_per_cta, int sms, cudaStream_t st);
 cudaError_t launch_build_fp64(const BuildArgs &a, cudaStream_t st);
+// mom[t][k] = (mean, variance) of Y[t][.][k]
+cudaError_t launch_coeff_moments(const float *Y, int nt, int N, int K, float2 *mom, cudaStream_t st);
 // cell classes + sub-grid delta table
 cudaError_t launch_prepare(const uint8_t *obstacle, const uint8_t *target, uint8_t *cls,
                            int nx, int ny, int nt, int32_t *delta, int L, cudaStream_t st);
@@ -250,8 +264,8 @@ struct SolveArgs {
 // Launch shapes chosen by the autotuner (mdp_autotune) per workload class;
 // every choice gives the same model and values bit for bit.
 struct Tuning {
-  int32_t build_warps = 8;       // warps per CTA of the warp-per-slice build kernel
-  int32_t hist_cap = 2048;       // fine-table words per warp of that kernel
+  int32_t build_warps = 8;       // warps (slices of a group) per CTA of the group build kernel
+  int32_t hist_cap = 2048;       // fine-table words per slice of that kernel
   int32_t threads = 256;         // CTA size of the full-window build kernel
   int32_t chunk = 1024;          // realizations staged per pass by that kernel
   int32_t sweep_smem_kb = 160;   // shared memory of the one-state-per-slice Bellman sweep
@@ -291,12 +305,14 @@ cudaError_t prepare_bellman_batch(int wcap, int grouped, int *stage_bytes, int *
 cudaError_t launch_bellman_batch(const BatchSolveItem *items_d, int n, BatchCta *ctas_d, int G, int k,
                                  int stage_bytes, int grouped, int layered, cudaStream_t st);
 cudaError_t launch_finalize_batch(const BatchSolveItem *items_d, int n, int layered, cudaStream_t st);
-// batched build (FP32): one persistent warp launch over the slices of n
-// models that share the mode count K and the states per warp spw (prefix[m]
-// = first slice of model m in the launch, prefix[n] = total); then the
-// full-window CTA kernel over every model's deferred slices
+// batched build (FP32): one persistent launch over the groups of slices of n
+// models that share the mode count K, the states per slice spw and the
+// density of their thresholds (prefix[m] = first group of model m in the
+// launch, prefix[n] = total; a group is batch_group_slices(spw) slices); then
+// the full-window CTA kernel over every model's deferred slices
+int batch_group_slices(int spw);
 cudaError_t launch_build_warp_batch(const BuildArgs *items_d, const int64_t *prefix_d, int n,
-                                    unsigned long long *work_d, int cap_bins, int K, int spw,
+                                    unsigned long long *work_d, int cap_bins, int K, int spw, bool dense,
                                     cudaStream_t st);
 cudaError_t launch_build_fp32_batch(const BuildArgs *items_d, int n, size_t smem, int threads,
                                     cudaStream_t st);
@@ -343,6 +359,7 @@ struct BuildHook {
   void *Yown = nullptr;       // out: coefficient table owned by the caller now
   double *sigma_d = nullptr;  // out: device sigma (owned by the caller now)
   uint32_t *defer = nullptr;  // out: deferred-slice list (owned by the caller now)
+  float2 *mom = nullptr;      // out: moments of the caller's coefficients (owned by the caller now)
   int threads = 256;          // out: CTA size of the full-window kernel
 };
 // A caller that accounts device memory (the server) fixes the entry pool's
@@ -353,7 +370,7 @@ struct BuildLimits {
   uint64_t pool_cols_needed = 0;   // out (MDP_ERR_BUDGET): the columns the slices need
   uint64_t spill_words = 0;        // in (with pool_cols): spill words to allocate (0: none)
   uint64_t spill_words_needed = 0; // out (MDP_ERR_BUDGET): the spill words the rows need
-  int32_t slices_per_warp = 0;     // in: BuildArgs::slices_per_warp of the warp kernel
+  int32_t slices_per_warp = 0;     // in: BuildArgs::slices_per_warp of the group kernel
 };
 mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_actions *actions, int32_t N,
                       int32_t subgrid_L, const int32_t *objs_h, int32_t n_obj, const mdp_build_opts *opts,

@@ -193,6 +193,7 @@ extern "C" mdp_status mdp_rollout(const mdp_env *env, const mdp_grid *grid, cons
   a.rw.c_f = actions->c_f; a.rw.c_r = actions->c_r; a.rw.r_term = actions->r_term;
   a.rw.r_out = actions->r_outbound; a.rw.dt = grid->dt; a.rw.dx = grid->dx; a.rw.n_obj = n_obj;
   for (int o = 0; o < n_obj; ++o) a.rw.objs[o] = objs_h[o];
+  a.rw.set_floats();
   // scratch: starts, own coefficient table (when drawn here), outputs the
   // caller did not ask for but the summary needs
   const bool own_ret = !ret, own_steps = !steps, own_status = !status;
