@@ -83,15 +83,29 @@ def kernel_counters(kernel, workload_name):
         return None
 
 
-def bellman_bytes_per_sweep(info, nS, n_obj=1):
-    """Algorithmic bytes of one Jacobi sweep solving n_obj objectives on one
-    P: 4 B per in-domain successor (offset, count), read once for all
-    objectives; per objective 4 B of R per row and, per state, the old V
-    read, the V and policy writes and one read of V(s') of the next layer
-    (the gathers are served from L1/L2); the cell class once per state.
-    Sink entries need no bytes (V = 0); the sliced-ELL padding the layout
-    carries is not counted."""
-    return 4 * info.nnz_domain + n_obj * (4 * info.rows + nS * (4 + 4 + 2 + 4)) + nS * 1
+def bellman_bytes_per_sweep(info, nS, n_obj=1, chains=0):
+    """Algorithmic bytes of one pass over P solving n_obj objectives: 4 B per
+    in-domain successor (offset, count), read once for all objectives; per
+    objective 4 B of R per row and, per state, the old V read, the V and
+    policy writes and one read of V(s') of the next layer (the gathers are
+    served from L1/L2); the cell class once per state.  chains > 0: a backward
+    pass carrying that many chains of values (no old V; V written and V(s')
+    read once per chain).  Sink entries need no bytes (V = 0); the sliced-ELL
+    padding the layout carries is not counted."""
+    per_state = 4 + 4 + 2 + 4 if chains == 0 else 8 * chains + 2
+    return 4 * info.nnz_domain + n_obj * (4 * info.rows + nS * per_state) + nS * 1
+
+
+def solve_passes(st, env, jacobi=True):
+    """(passes over P in full-sweep units, chains per pass, launches) of one
+    solve: a Jacobi run that ends in sweep nt + 1 comes from one backward pass
+    of two chains (two backups per state and action; one launch per layer and
+    a finalize); others from sweeps over the layers that changed (nt + 1
+    launches, those after convergence exiting at once, and a finalize)."""
+    full = st.backups / (env.nS * env.A)
+    if jacobi and st.sweeps == env.nt + 1 and st.backups == 2 * env.nS * env.A:
+        return 1.0, 2, env.nt + 1
+    return full, 0 if jacobi else 1, env.nt + 2 if jacobi else env.nt
 
 
 class ClockSampler:
@@ -396,15 +410,16 @@ def run_cube(args):
         solve_ms.append(sts[0].solve_ms)
         samples += info.samples
         backups += sum(s.backups for s in sts)
-        full_equiv += max(s.backups / (env.nS * env.A) for s in sts)
-        launches += info.launches + (env.nt + 1) + len(sts)
+        passes = [solve_passes(s, env) for s in sts]
+        full_equiv += max(p[0] for p in passes)
+        launches += info.launches + max(p[2] for p in passes)
     e1.record(stream)
     torch.cuda.synchronize()
     clocks = clk.stop()
     t_ms = e0.elapsed_time(e1)
     info = rec["info"]
     hbm, sm_mhz, peak_kind = peaks()
-    bpsw = bellman_bytes_per_sweep(info, env.nS, len(objs))
+    bpsw = bellman_bytes_per_sweep(info, env.nS, len(objs), max(p[1] for p in passes))
     sweep_ms = sum(solve_ms) / max(full_equiv, 1e-9)
     bell = bpsw / (sweep_ms / 1e3) / 1e9
     # 3-D build kernel against the issue-slot roofline (as the 2-D build)
@@ -723,14 +738,11 @@ def main():
         samples += info.samples
         backups += sum(s.backups for s in sts)
         sweeps.append([s.sweeps for s in sts])
-        per_obj = [s.backups / (env.nS * env.A) for s in sts]
-        full_equiv += sum(per_obj) if args.separate else max(per_obj)
-        # Jacobi: nt + 1 sweep launches (those after convergence exit at once) + one
-        # finalize per objective; layered: one launch per time layer
-        n_solves = len(sts) if args.separate else 1
         jac = method != mdp.MDP_SOLVE_LAYERED
-        launches += info.launches + n_solves * ((env.nt + 1) if jac else env.nt)
-        launches += len(sts) if jac else (0 if args.separate or len(sts) == 1 else 1)
+        passes = [solve_passes(s, env, jac) for s in sts]
+        full_equiv += sum(p[0] for p in passes) if args.separate else max(p[0] for p in passes)
+        launches += info.launches + (sum(p[2] for p in passes) if args.separate else max(p[2] for p in passes))
+        launches += 0 if jac or args.separate or len(sts) == 1 else 1
     e1.record(stream)
     torch.cuda.synchronize()
     if world > 1:
@@ -753,9 +765,9 @@ def main():
     build_achieved = cb["warp_inst_per_unit"] * n_slices / (kmean / 1e3) / 1e12 if cb else None
     # Bellman sweep against HBM
     n_fused = 1 if args.separate else len(objs)
-    bpsw = bellman_bytes_per_sweep(info, env.nS, n_fused)
-    # device time per full-sweep equivalent of work (Jacobi: the layers the
-    # sweeps recomputed; layered: one pass = one sweep's work)
+    bpsw = bellman_bytes_per_sweep(info, env.nS, n_fused, max(p[1] for p in passes))
+    # device time per pass over P (two-chain Jacobi and layered: one pass;
+    # Jacobi sweeps: full-sweep equivalents of the layers they recomputed)
     sweep_ms = sum(solve_ms) / max(full_equiv, 1e-9)
     bell_achieved = bpsw / (sweep_ms / 1e3) / 1e9
     cs = kernel_counters("bellman_kernel_fused3", env.name) if n_fused == 3 else None
@@ -780,6 +792,7 @@ def main():
                  "traffic": cs["dram_bytes_per_unit"] * n_slices if cs else None,
                  "bytes_per_sweep": bpsw, "ms_per_sweep": sweep_ms,
                  "full_sweep_equivalents_per_solve": full_equiv / args.steps,
+                 "chains_per_pass": max(p[1] for p in passes),
                  "counters": cs["summary"] if cs else "stale or absent",
                  "peak_basis": f"hbm_gbs ({peak_kind})"}
     build_share = sum(kern_ms) / t_ms

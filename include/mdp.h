@@ -187,7 +187,11 @@ typedef enum {
                                 * A sweep recomputes only the time layers t whose own values or
                                 * whose successor layer t+1 changed in the previous sweep; every
                                 * other state has V_{k+1}(s) = V_k(s) exactly, so iterates, policy,
-                                * residuals and sweep count equal MDP_SOLVE_JACOBI_FULL bit for bit */
+                                * residuals and sweep count equal MDP_SOLVE_JACOBI_FULL bit for bit.
+                                * A cold-started FP32 run that is certain to end in sweep nt + 1 (two
+                                * backward chains over the layers bound every earlier residual from
+                                * below) is returned from those chains, without sweeping: the same V,
+                                * policy, sweeps and residual bit for bit */
   MDP_SOLVE_LAYERED = 1,      /* one backward pass over time layers t = nt-1..0 (same fixed point) */
   MDP_SOLVE_JACOBI_FULL = 2,  /* Jacobi sweeps over every state in every sweep */
   MDP_SOLVE_WARM = 16         /* flag, OR-ed into MDP_SOLVE_JACOBI or _JACOBI_FULL of mdp_solve
@@ -202,7 +206,8 @@ typedef struct {
   int32_t sweeps;          /* sweeps executed (layered: 1) */
   double residual;         /* max |V_k - V_{k-1}| of the last sweep (layered: 0) */
   double solve_ms;         /* device time of the solve kernels (CUDA events) */
-  int64_t backups;         /* (s,a) Bellman backups computed (MDP_SOLVE_JACOBI: the
+  int64_t backups;         /* (s,a) Bellman backups computed (MDP_SOLVE_JACOBI: two per
+                            * (s,a) when the two chains gave the result, else of the
                             * recomputed layers only; fused solves: for all objectives) */
 } mdp_solve_stats;
 

@@ -708,37 +708,46 @@ extern "C" mdp_status mdp_export_csr(mdp_model m, int32_t obj, int64_t *rowptr, 
   return MDP_OK;
 }
 
-// Value iteration for n objectives on one model: the Bellman kernels stream
-// P once per sweep for all of them (mdp_solve is the n = 1 case).
-static mdp_status solve_impl(mdp_model m, int32_t n, const int32_t *objs, int32_t method, double tol,
-                             int32_t max_sweeps, void *const *V, int16_t *const *policy, void *stream,
-                             mdp_solve_stats *stats) {
-  if (!m) return arg_fail("NULL model");
-  if (n < 1 || n > 3) return arg_fail("n must be 1, 2 or 3");
-  if (!objs || !V || !policy) return arg_fail("NULL objs, V or policy");
-  for (int o = 0; o < n; ++o) {
-    if (!V[o] || !policy[o]) return arg_fail("NULL V or policy");
-    if (objs[o] < 0 || objs[o] >= m->n_obj) return arg_fail("objective slot out of range");
-  }
-  const bool warm = (method & MDP_SOLVE_WARM) != 0;
-  method &= ~MDP_SOLVE_WARM;
-  if (method != MDP_SOLVE_JACOBI && method != MDP_SOLVE_LAYERED && method != MDP_SOLVE_JACOBI_FULL)
-    return arg_fail("method");
-  if (warm && (n != 1 || method == MDP_SOLVE_LAYERED))
-    return arg_fail("MDP_SOLVE_WARM applies to single-objective Jacobi solves");
-  if (!(tol >= 0) && !(tol < 0)) return arg_fail("tol is NaN");
-  if (max_sweeps < 0) return arg_fail("max_sweeps must be >= 0");
-  if (max_sweeps == 0) max_sweeps = m->nt + 1;
+// Kernel arguments of a solve on m (the error word is the caller's).
+static SolveArgs solve_args(mdp_model m, const SolveIO &io, double tol) {
+  SolveArgs a;
+  a.pool = m->pool; a.slice_off = m->slice_off; a.slice_w = m->slice_w; a.nnz = m->nnz;
+  a.wcap = std::max(1, m->max_row_nnz);
+  a.spill = m->spill;
+  a.spill_off = m->spill_off;
+  a.small_ctas = m->sweep_small_ctas;
+  a.R = io.R[0];
+  a.cls = m->cls; a.delta = m->delta;
+  a.nS = m->nS; a.Nc = m->Nc; a.n_slices = m->n_slices;
+  a.A = m->A; a.A_pad = m->A_pad; a.spw = m->spw; a.N = m->N; a.nbins = m->nbins; a.tol = tol;
+  a.err = nullptr;
+  a.nt = m->nt;
+  a.pool_ordered = m->pool_ordered;
+  a.sweep_smem_kb = m->sweep_smem_kb;
+  return a;
+}
+
+// Device buffer freed on every return path, events likewise.
+struct Scratch {
+  void *p = nullptr;
+  cudaStream_t st;
+  explicit Scratch(cudaStream_t s) : st(s) {}
+  ~Scratch() { dev_free(p, st); }
+};
+struct EventPair {
+  cudaEvent_t e[2] = {nullptr, nullptr};
+  EventPair() { for (auto &x : e) cudaEventCreate(&x); }
+  ~EventPair() { for (auto &x : e) if (x) cudaEventDestroy(x); }
+};
+
+// The sweeps (or layered pass) of a solve whose arguments are checked: the
+// Bellman kernels stream P once per sweep for all n objectives.
+static mdp_status solve_sweeps(mdp_model m, int32_t n, const int32_t *objs, int32_t method, bool warm, double tol,
+                               int32_t max_sweeps, void *const *V, int16_t *const *policy, void *stream,
+                               mdp_solve_stats *stats) {
   cudaStream_t st = (cudaStream_t)stream;
   const size_t fsz = m->precision == MDP_FP64_CHECK ? 8 : 4;
   const size_t vbytes = fsz * (size_t)(m->nS + 1);
-  // the solver streams slices with 16-byte-aligned bulk copies and indexes
-  // successors with 32-bit offsets
-  if ((((uintptr_t)m->pool) | ((uintptr_t)m->R) | ((uintptr_t)m->nnz)) & 15) {
-    set_error("model arrays are not 16-byte aligned");
-    return MDP_ERR_CUDA;
-  }
-  if (m->nS + m->Nc >= ((int64_t)1 << 31)) return arg_fail("more than 2^31 states is not supported by the solver");
   const bool jac = method != MDP_SOLVE_LAYERED;
   const bool active = method == MDP_SOLVE_JACOBI;   // active-layer sweeps
   // n = 1 iterates in V and the model's cached partner buffer; n > 1 in
@@ -776,20 +785,8 @@ static mdp_status solve_impl(mdp_model m, int32_t n, const int32_t *objs, int32_
   }
   if (ce == cudaSuccess && io.Vtmp[0]) ce = cudaMemsetAsync(io.Vtmp[0], 0, vbytes, st);
   if (ce == cudaSuccess && tables) ce = cudaMemsetAsync(tables, 0, tbytes * n_tables, st);
-  SolveArgs a;
-  a.pool = m->pool; a.slice_off = m->slice_off; a.slice_w = m->slice_w; a.nnz = m->nnz;
-  a.wcap = std::max(1, m->max_row_nnz);
-  a.spill = m->spill;
-  a.spill_off = m->spill_off;
-  a.small_ctas = m->sweep_small_ctas;
-  a.R = io.R[0];
-  a.cls = m->cls; a.delta = m->delta;
-  a.nS = m->nS; a.Nc = m->Nc; a.n_slices = m->n_slices;
-  a.A = m->A; a.A_pad = m->A_pad; a.spw = m->spw; a.N = m->N; a.nbins = m->nbins; a.tol = tol;
+  SolveArgs a = solve_args(m, io, tol);
   a.err = reinterpret_cast<int *>(sd + 2);
-  a.nt = m->nt;
-  a.pool_ordered = m->pool_ordered;
-  a.sweep_smem_kb = m->sweep_smem_kb;
   take_test_injection(a);
   if (active) {
     a.work = reinterpret_cast<unsigned long long *>(sd + blk * n);
@@ -839,6 +836,119 @@ static mdp_status solve_impl(mdp_model m, int32_t n, const int32_t *objs, int32_
     }
   }
   return MDP_OK;
+}
+
+// A cold-started FP32 Jacobi run by two backward chains (bellman.cu): fills V,
+// policy and stats of every objective whose run is certain to end in sweep
+// nt + 1, sets done[o] for those and leaves the others to the sweeps.
+static mdp_status solve_two_chains(mdp_model m, int32_t n, const int32_t *objs, double tol, void *const *V,
+                                   int16_t *const *policy, void *stream, mdp_solve_stats *stats, bool *done,
+                                   float *ms) {
+  cudaStream_t st = (cudaStream_t)stream;
+  const int nc = n == 1 ? 2 : (n == 2 ? 4 : 8);   // packed components per state
+  const size_t tbytes = sizeof(float) * (size_t)nc * (size_t)(m->nS + 1);
+  const size_t nd = (size_t)n * m->nt;   // residual bounds, then the error word
+  Scratch tab(st), dd(st);
+  EventPair ev;
+  MDP_CUDA_TRY(dev_alloc(&tab.p, tbytes, st));
+  MDP_CUDA_TRY(dev_alloc(&dd.p, sizeof(unsigned int) * (nd + 1), st));
+  SolveIO io{};
+  io.n = n;
+  for (int o = 0; o < n; ++o) {
+    io.R[o] = static_cast<const char *>(m->R) + sizeof(float) * (size_t)objs[o] * m->rows_pad;
+    io.V[o] = V[o];
+    io.policy[o] = policy[o];
+  }
+  io.table[0] = tab.p;
+  MDP_CUDA_TRY(cudaMemsetAsync(tab.p, 0, tbytes, st));
+  MDP_CUDA_TRY(cudaMemsetAsync(dd.p, 0, sizeof(unsigned int) * (nd + 1), st));
+  SolveArgs a = solve_args(m, io, tol);
+  unsigned int *d = static_cast<unsigned int *>(dd.p);
+  a.err = reinterpret_cast<int *>(d + nd);
+  take_test_injection(a);
+  cudaEventRecord(ev.e[0], st);
+  MDP_CUDA_TRY(launch_two_chains(a, m->nt, io, d, st));
+  cudaEventRecord(ev.e[1], st);
+  std::vector<unsigned int> hd(nd + 1);
+  MDP_CUDA_TRY(cudaMemcpyAsync(hd.data(), d, sizeof(unsigned int) * (nd + 1), cudaMemcpyDeviceToHost, st));
+  MDP_CUDA_TRY(cudaStreamSynchronize(st));
+  if (hd[nd]) {
+    set_error("a bounded device wait expired in the Bellman pipeline");
+    return MDP_ERR_TIMEOUT;
+  }
+  cudaEventElapsedTime(ms, ev.e[0], ev.e[1]);
+  for (int o = 0; o < n; ++o) {
+    done[o] = true;
+    for (int t = 0; t < m->nt && done[o]; ++t) {
+      float x;
+      memcpy(&x, &hd[(size_t)o * m->nt + t], sizeof(x));
+      done[o] = (double)x > tol;   // sweep nt - t does not stop the run
+    }
+    if (done[o] && stats) {
+      stats[o].sweeps = m->nt + 1;
+      stats[o].residual = 0.0;
+      stats[o].solve_ms = *ms;
+      stats[o].backups = 2 * m->nS * m->A;   // one per chain
+    }
+  }
+  return MDP_OK;
+}
+
+// Value iteration for n objectives on one model (mdp_solve is the n = 1 case).
+static mdp_status solve_impl(mdp_model m, int32_t n, const int32_t *objs, int32_t method, double tol,
+                             int32_t max_sweeps, void *const *V, int16_t *const *policy, void *stream,
+                             mdp_solve_stats *stats) {
+  if (!m) return arg_fail("NULL model");
+  if (n < 1 || n > 3) return arg_fail("n must be 1, 2 or 3");
+  if (!objs || !V || !policy) return arg_fail("NULL objs, V or policy");
+  for (int o = 0; o < n; ++o) {
+    if (!V[o] || !policy[o]) return arg_fail("NULL V or policy");
+    if (objs[o] < 0 || objs[o] >= m->n_obj) return arg_fail("objective slot out of range");
+  }
+  const bool warm = (method & MDP_SOLVE_WARM) != 0;
+  method &= ~MDP_SOLVE_WARM;
+  if (method != MDP_SOLVE_JACOBI && method != MDP_SOLVE_LAYERED && method != MDP_SOLVE_JACOBI_FULL)
+    return arg_fail("method");
+  if (warm && (n != 1 || method == MDP_SOLVE_LAYERED))
+    return arg_fail("MDP_SOLVE_WARM applies to single-objective Jacobi solves");
+  if (!(tol >= 0) && !(tol < 0)) return arg_fail("tol is NaN");
+  if (max_sweeps < 0) return arg_fail("max_sweeps must be >= 0");
+  if (max_sweeps == 0) max_sweeps = m->nt + 1;
+  // the solver streams slices with 16-byte-aligned bulk copies and indexes
+  // successors with 32-bit offsets
+  if ((((uintptr_t)m->pool) | ((uintptr_t)m->R) | ((uintptr_t)m->nnz)) & 15) {
+    set_error("model arrays are not 16-byte aligned");
+    return MDP_ERR_CUDA;
+  }
+  if (m->nS + m->Nc >= ((int64_t)1 << 31)) return arg_fail("more than 2^31 states is not supported by the solver");
+  // A cold-started run that may reach sweep nt + 1 almost always does (the
+  // horizon's penalty reaches one more layer in every sweep up to there): try
+  // the two chains, and sweep only for the objectives they leave open.  FP64
+  // check mode keeps the literal sweeps.
+  if (method == MDP_SOLVE_JACOBI && !warm && m->precision == MDP_FP32 && tol >= 0 && max_sweeps >= m->nt + 1) {
+    bool done[3] = {false, false, false};
+    float chains_ms = 0.f;
+    mdp_status s = solve_two_chains(m, n, objs, tol, V, policy, stream, stats, done, &chains_ms);
+    if (s != MDP_OK) return s;
+    int32_t left[3], left_obj[3], n_left = 0;
+    void *Vl[3];
+    int16_t *pl[3];
+    for (int o = 0; o < n; ++o) {
+      if (done[o]) continue;
+      left[n_left] = o;
+      left_obj[n_left] = objs[o];
+      Vl[n_left] = V[o];
+      pl[n_left++] = policy[o];
+    }
+    if (n_left == 0) return MDP_OK;
+    mdp_solve_stats sl[3] = {};
+    s = solve_sweeps(m, n_left, left_obj, method, warm, tol, max_sweeps, Vl, pl, stream, sl);
+    if (s != MDP_OK || !stats) return s;
+    for (int i = 0; i < n_left; ++i) stats[left[i]] = sl[i];
+    for (int o = 0; o < n; ++o) stats[o].solve_ms = chains_ms + sl[0].solve_ms;   // the whole solve
+    return MDP_OK;
+  }
+  return solve_sweeps(m, n, objs, method, warm, tol, max_sweeps, V, policy, stream, stats);
 }
 
 extern "C" mdp_status mdp_solve(mdp_model m, int32_t obj, int32_t method, double tol,

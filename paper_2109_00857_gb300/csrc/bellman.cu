@@ -177,7 +177,7 @@ struct PipeRange {
   int64_t sl_lo, sl_hi;   // slices of this launch
   int64_t s_lo, s_hi;     // states whose V this launch writes
   int stage_bytes;        // bytes per stage
-  int dtab_smem;          // 1: delta table staged in shared memory
+  int zero_second;        // two-chain pass: the second chain's values of this layer are 0
   int grouped;            // 1: bellman_body_g (kGS states per warp step, batched sweeps); 2: bellman_kernel_ws
                           // (stage_bytes = entry bytes per slot)
 };
@@ -197,12 +197,13 @@ static int stage_bytes_for(int wcap) { return wcap * 128; }
 // res != nullptr: Jacobi sweep k (exits at once if sweep k-1 met the
 // tolerance) with the residual reduced into res[k-1].
 // One CTA, slices [b_lo, b_hi) of one model (all threads call it).
-// Values of NO objectives of one state, stored side by side (objective o
-// in v[o]; NO = 3 is padded to four) so that one vector load gathers V(s')
-// of every objective of a fused solve.
-template <typename RT, int NO>
-struct alignas(sizeof(RT) * (NO == 3 ? 4 : NO)) VPack {
-  static constexpr int W = (NO == 3) ? 4 : NO;
+// Values of NC components of one state (the objectives of a fused solve; of a
+// two-chain pass, the objectives' values and then their second chain's),
+// stored side by side and padded to a power of two so that vector loads gather
+// V(s') of every component.
+template <typename RT, int NC>
+struct alignas(sizeof(RT) * (NC <= 2 ? NC : (NC <= 4 ? 4 : 8))) VPack {
+  static constexpr int W = NC <= 2 ? NC : (NC <= 4 ? 4 : 8);
   RT v[W];
 };
 
@@ -212,11 +213,14 @@ struct alignas(sizeof(RT) * (NO == 3 ? 4 : NO)) VPack {
 // packed table (in = V_k, out = V_{k+1}; equal for the in-place layered
 // pass).  res[o] == nullptr marks a layered pass (no residual, no early
 // exit).
-template <typename RT, int NO>
+// TWO: a two-chain layered pass (launch_two_chains): components NO..2 NO - 1
+// are a second chain of values with the same R, whose policy is not kept.
+template <typename RT, int NO, bool TWO = false>
 struct VSet {
+  static constexpr int NC = TWO ? 2 * NO : NO;
   const RT *R[NO];
-  const VPack<RT, NO> *in;
-  VPack<RT, NO> *out;
+  const VPack<RT, NC> *in;
+  VPack<RT, NC> *out;
   int16_t *pol[NO];
   unsigned long long *res[NO];
 };
@@ -225,25 +229,37 @@ struct VSet {
 // block (HYB), added to the row's sums in its stored (ascending) order after
 // the ELL columns: the same sum as over one plain row.  Called only for
 // models with a spill area (a.spill_off != nullptr).
-template <typename RT, int NO>
-__device__ __forceinline__ void add_spill(const SolveArgs &a, int64_t sl, int lane, const VPack<RT, NO> *Vn,
-                                          Acc<RT> (&acc)[NO]) {
+template <typename RT, int NC>
+__device__ __forceinline__ void add_spill(const SolveArgs &a, int64_t sl, int lane, const VPack<RT, NC> *Vn,
+                                          Acc<RT> (&acc)[NC]) {
   const uint32_t off = __ldg(a.spill_off + sl);
   if (off == kNoSlice) return;
   const uint32_t *blk = a.spill + off;
   const uint32_t b = __ldg(blk + lane), e = __ldg(blk + lane + 1);
   for (uint32_t i = b; i < e; ++i) {
     const uint32_t w = __ldg(blk + kSpillHdr + i);
-    const VPack<RT, NO> g = Vn[(int)(int16_t)(w & 0xFFFFu)];
+    const VPack<RT, NC> g = Vn[(int)(int16_t)(w & 0xFFFFu)];
 #pragma unroll
-    for (int o = 0; o < NO; ++o) acc[o].add(w >> 16, g.v[o], a.N);
+    for (int o = 0; o < NC; ++o) acc[o].add(w >> 16, g.v[o], a.N);
   }
 }
 
-template <typename RT, int NO>
-__device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, NO> &v, int k, int64_t b_lo,
+// Programmatic dependent launch (the layered passes): a layer's kernel may
+// start while the previous layer's finishes -- its prologue and first entry
+// copies touch nothing that kernel writes -- and waits here before it reads V.
+// Both return at once in kernels launched without the attribute.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename RT, int NO, bool TWO = false>
+__device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, int64_t b_lo,
                                              int64_t b_hi, const PipeRange &pr, unsigned char *sm,
                                              double *wmax, int *wst_s) {
+  using Pk = VPack<RT, VSet<RT, NO, TWO>::NC>;
+  constexpr int NC = VSet<RT, NO, TWO>::NC;
+  const bool layered = v.res[0] == nullptr;
+  pdl_trigger();
+  if (!layered) pdl_wait();
   // objectives whose previous sweep met the tolerance are finished
   unsigned live = (1u << NO) - 1u;
   if (k > 1) {
@@ -318,6 +334,7 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
 #pragma unroll
   for (int o = 0; o < NO; ++o) Rn[o] = (RT)0;
   if (n_mine > 0) load_r(0, Rn);
+  if (layered) pdl_wait();   // from here on V of the next layer is read
   int st = 0;
   uint32_t phase = 0;
   int s = sl0 * a.spw + q;                      // state of this lane's row in my j-th slice
@@ -343,19 +360,19 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     for (int o = 0; o < NO; ++o) Rv[o] = Rn[o];
     if (j + 1 < n_mine) load_r(j + 1, Rn);
     const int W = wst_s[warp * kDepth + st];
-    Acc<RT> acc[NO];
+    Acc<RT> acc[NC];
     // successor layer base of this state; rows without successors (last
     // layer, padding lanes) hold only padding words and read V[|S|] = 0
     const int sn = (s + Nc <= nS) ? s + Nc : nS;
-    const VPack<RT, NO> *Vn = v.in + sn;
+    const Pk *Vn = v.in + sn;
 #pragma unroll 4
     for (int kk = 0; kk < W; ++kk) {   // every column of the slice, ascending
       const uint32_t w = ent[kk * 32];
-      const VPack<RT, NO> g = Vn[(int)(int16_t)(w & 0xFFFFu)];
+      const Pk g = Vn[(int)(int16_t)(w & 0xFFFFu)];
 #pragma unroll
-      for (int o = 0; o < NO; ++o) acc[o].add(w >> 16, g.v[o], a.N);
+      for (int o = 0; o < NC; ++o) acc[o].add(w >> 16, g.v[o], a.N);
     }
-    if (a.spill_off) add_spill<RT, NO>(a, sl0 + (int64_t)j * kWarps, lane, Vn, acc);
+    if (a.spill_off) add_spill<RT, NC>(a, sl0 + (int64_t)j * kWarps, lane, Vn, acc);
     __syncwarp();
     if (j + kDepth < n_mine) issue(j + kDepth, st);   // refill the stage just read
     if (++st == kDepth) {
@@ -364,11 +381,11 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     }
     const bool head = act == 0 && s >= s_lo && s < s_hi;   // the lane that writes state s
     const bool term = head && __ldg(a.cls + s) != CLS_FREE;
-    VPack<RT, NO> old{}, nv;
-    if (head) old = v.in[s];
+    Pk old{}, nv;
+    if (head && !layered) old = v.in[s];
 #pragma unroll
-    for (int o = 0; o < NO; ++o) {
-      RT qv = valid ? acc[o].q(Rv[o], invN) : -(RT)INFINITY;
+    for (int o = 0; o < NC; ++o) {
+      RT qv = valid ? acc[o].q(Rv[o % NO], invN) : -(RT)INFINITY;
       int qa = act;
       if (sizeof(RT) == 4 && a.A_pad == 32) {
         // one state per warp: order-preserving integer key, warp max in one
@@ -388,17 +405,21 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
           }
         }
       }
+      if (o >= NO) {   // second chain: the value alone
+        nv.v[o] = pr.zero_second ? (RT)0 : qv;
+        continue;
+      }
       // a finished objective carries its value forward unchanged
       const bool upd = (live >> o) & 1u;
       nv.v[o] = upd ? qv : old.v[o];
       if (head && upd) {
-        v.pol[o][s] = term ? (int16_t)-1 : (int16_t)qa;
-        if constexpr (sizeof(RT) == 4) rf[o] = fmaxf(rf[o], fabsf(qv - old.v[o]));
-        else r[o] = fmax(r[o], fabs(qv - old.v[o]));
+        v.pol[o % NO][s] = term ? (int16_t)-1 : (int16_t)qa;
+        if constexpr (sizeof(RT) == 4) rf[o % NO] = fmaxf(rf[o % NO], fabsf(qv - old.v[o]));
+        else r[o % NO] = fmax(r[o % NO], fabs(qv - old.v[o]));
       }
     }
 #pragma unroll
-    for (int o = NO; o < VPack<RT, NO>::W; ++o) nv.v[o] = (RT)0;
+    for (int o = NC; o < Pk::W; ++o) nv.v[o] = (RT)0;
     if (head) {
       v.out[s] = nv;
       if (chg_out) {
@@ -470,9 +491,9 @@ __device__ __forceinline__ bool active_range(const SolveArgs &a, int k, PipeRang
   return true;
 }
 
-template <typename RT, int NO>
-__global__ void __launch_bounds__(32 * kWarps, 4) bellman_kernel(SolveArgs a, VSet<RT, NO> v, int k,
-                                                              PipeRange pr) {
+template <typename RT, int NO, bool TWO>
+__global__ void __launch_bounds__(32 * kWarps, TWO && NO == 3 ? 3 : 4) bellman_kernel(SolveArgs a, VSet<RT, NO, TWO> v,
+                                                                                   int k, PipeRange pr) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWarps * NO];
   __shared__ int wst_s[kWarps * kDepth];   // columns of the slice in each stage
@@ -481,7 +502,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) bellman_kernel(SolveArgs a, VS
   const int64_t per_cta = (total + gridDim.x - 1) / gridDim.x;
   const int64_t b_lo = pr.sl_lo + (int64_t)blockIdx.x * per_cta;
   const int64_t b_hi = min(pr.sl_hi, b_lo + per_cta);
-  bellman_body<RT, NO>(a, v, k, b_lo, b_hi, pr, sm, wmax, wst_s);
+  bellman_body<RT, NO, TWO>(a, v, k, b_lo, b_hi, pr, sm, wmax, wst_s);
 }
 
 // ---- grouped sweep: kGS states per warp step (models with A_pad = 32) ----
@@ -813,11 +834,15 @@ __device__ int64_t ws_cut(const SolveArgs &a, int64_t lo, int64_t hi, int64_t b,
   return h;
 }
 
-template <typename RT, int NO>
-__device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<RT, NO> &v, int k,
+template <typename RT, int NO, bool TWO>
+__device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k,
                                                 const PipeRange &pr, unsigned char *sm, double *wmax, int *s_flag,
                                                 int64_t *s_cut) {
-  using Pk = VPack<RT, NO>;
+  constexpr int NC = VSet<RT, NO, TWO>::NC;
+  using Pk = VPack<RT, NC>;
+  const bool layered = v.res[0] == nullptr;
+  pdl_trigger();
+  if (!layered) pdl_wait();
   unsigned live = (1u << NO) - 1u;
   if (k > 1) {
 #pragma unroll
@@ -851,7 +876,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   constexpr int kRBytes = ws_r_bytes<RT>(NO);
   const int ecap = pr.stage_bytes;                         // entry bytes per slot
   const int slot_bytes = kRBytes + ecap;
-  unsigned char *slots = sm + ws_hdr_bytes() + ws_old_bytes<RT, NO>();
+  unsigned char *slots = sm + ws_hdr_bytes() + ws_old_bytes<RT, NC>();
   if (tid < kWsSlots) {
     mbar_init(smem_u32(&hdr->full[tid]), 1);
     mbar_init(smem_u32(&hdr->empty[tid]), kWsCons);
@@ -887,7 +912,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
           off[i] = __ldg(a.slice_off + x);
           W[i] = __ldg(a.slice_w + x);
           cls[i] = __ldg(a.cls + x);   // spw = 1: state = slice
-          old[i] = v.in[x];
+          if (!layered) old[i] = v.in[x];
         }
       }
     };
@@ -922,7 +947,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
           e[i] = cum - W[i] * 128;
           if (lane < ni) {
             hdr->slice[slot][32 * i + lane] = make_int2(e[i], W[i] | (cls[i] << 8));
-            olds[slot * kWsTab + 32 * i + lane] = old[i];
+            if (!layered) olds[slot * kWsTab + 32 * i + lane] = old[i];
           }
           n += ni;
           if (ni < 32) open = false;
@@ -989,6 +1014,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
     }
   } else {
     // ---------------------------------------------------------- consumers
+    if (layered) pdl_wait();   // from here on V of the next layer is read
     const int nS = (int)a.nS, Nc = (int)a.Nc;
     const int s_lo = (int)pr.s_lo, s_hi = (int)pr.s_hi;
     const RT invN = (RT)1 / (RT)a.N;
@@ -1017,7 +1043,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
       }
       const int2 rdesc = hdr->round[slot];
       if (rdesc.y == 0) break;
-      Acc<RT> accs[kWsPer][NO];
+      Acc<RT> accs[kWsPer][NC];
       RT Rvs[kWsPer][NO];
       Pk olds_i[kWsPer];
       int wcs[kWsPer], Ws[kWsPer];
@@ -1042,7 +1068,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
           const RT *Rs = reinterpret_cast<const RT *>(sb) + j * 32 + lane;
 #pragma unroll
           for (int o = 0; o < NO; ++o) Rvs[i][o] = Rs[o * kWsTab * 32];
-          olds_i[i] = olds[slot * kWsTab + j];
+          if (!layered) olds_i[i] = olds[slot * kWsTab + j];
         }
         Wm = max(Wm, Ws[i]);
       }
@@ -1054,7 +1080,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
             const uint32_t w = ents[i][kk * 32];
             const Pk g = Vns[i][(int)(int16_t)(w & 0xFFFFu)];
 #pragma unroll
-            for (int o = 0; o < NO; ++o) accs[i][o].add(w >> 16, g.v[o], a.N);
+            for (int o = 0; o < NC; ++o) accs[i][o].add(w >> 16, g.v[o], a.N);
           }
         }
       }
@@ -1068,16 +1094,16 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
       for (int i = 0; i < kWsPer; ++i) {
         if (warp + kWsCons * i >= rdesc.y) continue;
         const int s = rdesc.x + warp + kWsCons * i;
-        Acc<RT> (&acc)[NO] = accs[i];
+        Acc<RT> (&acc)[NC] = accs[i];
         RT (&Rv)[NO] = Rvs[i];
         const Pk old = olds_i[i];
         const int wc = wcs[i];
-        if (a.spill_off) add_spill<RT, NO>(a, s, lane, v.in + ((s + Nc <= nS) ? s + Nc : nS), acc);
-        RT qv[NO];
+        if (a.spill_off) add_spill<RT, NC>(a, s, lane, v.in + ((s + Nc <= nS) ? s + Nc : nS), acc);
+        RT qv[NC];
         int qa[NO];
 #pragma unroll
-        for (int o = 0; o < NO; ++o) {
-          RT q = act_ok ? acc[o].q(Rv[o], invN) : -(RT)INFINITY;
+        for (int o = 0; o < NC; ++o) {
+          RT q = act_ok ? acc[o].q(Rv[o % NO], invN) : -(RT)INFINITY;
           int ia = lane;
           if constexpr (sizeof(RT) == 4) {
             // order-preserving key (-0 keys like +0): the max in one redux,
@@ -1085,6 +1111,10 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
             const uint32_t bits = __float_as_uint((float)q + 0.0f);
             const uint32_t key = bits ^ ((uint32_t)((int32_t)bits >> 31) | 0x80000000u);
             const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+            if (o >= NO) {   // second chain: the value alone, from its key
+              qv[o] = __uint_as_float(kmax ^ ((uint32_t)((int32_t)~kmax >> 31) | 0x80000000u));
+              continue;
+            }
             ia = __ffs(__ballot_sync(0xffffffffu, key == kmax)) - 1;
             q = __shfl_sync(0xffffffffu, q, ia);
           } else {
@@ -1099,7 +1129,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
             }
           }
           qv[o] = q;
-          qa[o] = ia;
+          if (o < NO) qa[o % NO] = ia;
         }
         if (s < s_lo || s >= s_hi) continue;
         const bool term = (wc >> 8) != CLS_FREE;
@@ -1114,7 +1144,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
           }
         }
 #pragma unroll
-        for (int o = NO; o < Pk::W; ++o) nv.v[o] = (RT)0;
+        for (int o = NO; o < Pk::W; ++o) nv.v[o] = (o < NC && !pr.zero_second) ? qv[o < NC ? o : 0] : (RT)0;
         int myqa = qa[0];
 #pragma unroll
         for (int o = 1; o < NO; ++o)
@@ -1155,15 +1185,15 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   }
 }
 
-template <typename RT, int NO>
-__global__ void __launch_bounds__(32 * (kWsCons + 1), 1) bellman_kernel_ws(SolveArgs a, VSet<RT, NO> v, int k,
+template <typename RT, int NO, bool TWO>
+__global__ void __launch_bounds__(32 * (kWsCons + 1), 1) bellman_kernel_ws(SolveArgs a, VSet<RT, NO, TWO> v, int k,
                                                                          PipeRange pr) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWsCons * NO];
   __shared__ int s_flag;
   __shared__ int64_t s_cut[2];
   if (a.lflags && k >= 1 && !active_range(a, k, pr, blockIdx.x == 0)) return;
-  bellman_body_ws<RT, NO>(a, v, k, pr, sm, wmax, &s_flag, s_cut);
+  bellman_body_ws<RT, NO, TWO>(a, v, k, pr, sm, wmax, &s_flag, s_cut);
 }
 
 // Plan of batched Jacobi sweep k (one block): per model, the slices of the
@@ -1261,7 +1291,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) bellman_batch_kernel(const Bat
   pr.s_lo = c.s_lo;
   pr.s_hi = c.s_hi;
   pr.stage_bytes = stage_bytes;
-  pr.dtab_smem = 0;
+  pr.zero_second = 0;
   pr.grouped = 0;
   VSet<float, 1> v;
   v.R[0] = static_cast<const float *>(it.a.R);
@@ -1289,7 +1319,7 @@ __global__ void __launch_bounds__(32 * kWarpsG, 1) bellman_batch_kernel_g(const 
   pr.s_lo = c.s_lo;
   pr.s_hi = c.s_hi;
   pr.stage_bytes = stage_bytes;
-  pr.dtab_smem = 0;
+  pr.zero_second = 0;
   pr.grouped = 1;
   VSet<float, 1> v;
   v.R[0] = static_cast<const float *>(it.a.R);
@@ -1396,25 +1426,25 @@ __global__ void finalize_kernel(const unsigned long long *res, int max_sweeps, d
 // same memory make shorter rounds and are slower.)
 constexpr size_t kWsSmem = 160 * 1024;
 
-template <typename RT, int NO>
+template <typename RT, int NO, bool TWO>
 static int ws_entry_bytes(int wcap, int smem_kb) {
   const size_t budget = smem_kb > 0 ? (size_t)smem_kb * 1024 : kWsSmem;
-  const long per_slot = (long)((budget - ws_hdr_bytes() - ws_old_bytes<RT, NO>()) / kWsSlots) - ws_r_bytes<RT>(NO);
+  const long per_slot = (long)((budget - ws_hdr_bytes() - ws_old_bytes<RT, VSet<RT, NO, TWO>::NC>()) / kWsSlots) - ws_r_bytes<RT>(NO);
   long e = std::max<long>(per_slot, (long)wcap * 128);
   return (int)(e & ~127L);
 }
 
-template <typename RT, int NO>
+template <typename RT, int NO, bool TWO = false>
 static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, PipeRange *pr, size_t *smem, int *blocks) {
-  pr->dtab_smem = 0;
+  pr->zero_second = 0;
   if (a.spw == 1 && !a.small_ctas) {   // one state per slice: the warp-specialized sweep, any width
     pr->grouped = 2;
-    pr->stage_bytes = ws_entry_bytes<RT, NO>(a.wcap, a.sweep_smem_kb);
-    *smem = ws_hdr_bytes() + ws_old_bytes<RT, NO>() + (size_t)kWsSlots * (ws_r_bytes<RT>(NO) + pr->stage_bytes);
-    cudaError_t e = allow_max_smem((const void *)bellman_kernel_ws<RT, NO>);
+    pr->stage_bytes = ws_entry_bytes<RT, NO, TWO>(a.wcap, a.sweep_smem_kb);
+    *smem = ws_hdr_bytes() + ws_old_bytes<RT, VSet<RT, NO, TWO>::NC>() + (size_t)kWsSlots * (ws_r_bytes<RT>(NO) + pr->stage_bytes);
+    cudaError_t e = allow_max_smem((const void *)bellman_kernel_ws<RT, NO, TWO>);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel_ws<RT, NO>, 32 * (kWsCons + 1), *smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel_ws<RT, NO, TWO>, 32 * (kWsCons + 1), *smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t b = (int64_t)num_sms() * per_sm;
@@ -1428,10 +1458,10 @@ static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, PipeRange *pr
   pr->stage_bytes = stage_bytes_for(a.wcap);
   *smem = 256 + (size_t)kWarps * kDepth * pr->stage_bytes;
   if (*smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO>);
+  cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO, TWO>);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO>, 32 * kWarps, *smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO, TWO>, 32 * kWarps, *smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int64_t b = (int64_t)num_sms() * per_sm;
@@ -1482,13 +1512,23 @@ __global__ void finalize_multi_kernel(const double *stats_base, size_t blk, int 
   }
 }
 
-template <typename RT, int NO>
-static void launch_sweep(const SolveArgs &a, const VSet<RT, NO> &v, int k, const PipeRange &pr, int blocks,
-                         size_t smem, cudaStream_t st) {
-  if (pr.grouped == 2)
-    bellman_kernel_ws<RT, NO><<<blocks, 32 * (kWsCons + 1), smem, st>>>(a, v, k, pr);
-  else
-    bellman_kernel<RT, NO><<<blocks, 32 * kWarps, smem, st>>>(a, v, k, pr);
+// pdl: the launch may start while the previous kernel of the stream finishes
+// (the layers of a layered pass).
+template <typename RT, int NO, bool TWO>
+static void launch_sweep(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, const PipeRange &pr, int blocks,
+                         size_t smem, cudaStream_t st, bool pdl = false) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(pr.grouped == 2 ? 32 * (kWsCons + 1) : 32 * kWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  if (pr.grouped == 2) cudaLaunchKernelEx(&cfg, bellman_kernel_ws<RT, NO, TWO>, a, v, k, pr);
+  else cudaLaunchKernelEx(&cfg, bellman_kernel<RT, NO, TWO>, a, v, k, pr);
 }
 
 // Objective o's status block: stats_d + o*(4 + max_sweeps) holds sweeps,
@@ -1531,7 +1571,7 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
   pr.s_lo = 0;
   pr.s_hi = a.nS;
   for (int k = 1; k <= max_sweeps; ++k)
-    launch_sweep<RT, NO>(a, (k & 1) ? odd : even, k, pr, blocks, smem, st);
+    launch_sweep(a, (k & 1) ? odd : even, k, pr, blocks, smem, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int64_t fb = (a.nS + 1 + 255) / 256;
@@ -1596,13 +1636,15 @@ static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, doub
     v.pol[o] = io.policy[o];
     v.res[o] = nullptr;
   }
+  SolveArgs rest = a;   // a test's injected failure is for the first launch alone
+  rest.test_extra_tx = 0;
   for (int t_ = nt - 1; t_ >= 0; --t_) {
     PipeRange pr = pr0;
     pr.s_lo = (int64_t)t_ * a.Nc;
     pr.s_hi = pr.s_lo + a.Nc;
     pr.sl_lo = pr.s_lo / a.spw;
     pr.sl_hi = (pr.s_hi + a.spw - 1) / a.spw;
-    launch_sweep<RT, NO>(a, v, 0, pr, blocks, smem, st);
+    launch_sweep(t_ < nt - 1 ? rest : a, v, 0, pr, blocks, smem, st, t_ < nt - 1);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess || NO == 1) return e;
@@ -1613,6 +1655,94 @@ static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, doub
   finalize_multi_kernel<RT, NO><<<(unsigned)fb, 256, 0, st>>>(stats_d, 0, 0, a.tol, t, t, out, a.nS + 1,
                                                                stats_d, 1);
   return cudaGetLastError();
+}
+
+// ---- the Jacobi result by two chains ----
+// What a cold-started Jacobi run (V_0 = 0) to tolerance tol >= 0 returns, from
+// one pass over P instead of nt + 1 sweeps, when that is certain.  In this
+// time-layered MDP V_k = V* on the layers t >= nt - k, bit for bit (layer nt-1
+// has no successors, and layer t's values are computed from layer t+1's by the
+// same operations in every sweep).  Let W(t) = V_{nt-t-1}(t) be layer t's last
+// iterate before that: W(nt-1) = 0 and W(t) = T W(t+1), a second backward
+// chain.  Sweep k = nt - t changes layer t from W(t) to V*(t), so its residual
+// is at least d_t = max |V*(t) - W(t)|.  If every d_t exceeds tol, no sweep
+// 1..nt stops the run, and sweep nt + 1 changes nothing: the run ends there
+// with V*, its greedy policy, nt + 1 sweeps and residual 0.  (Otherwise the
+// caller runs the sweeps.)  Both chains share the entry stream, so the pass
+// costs little more than a layered one.
+//
+// Copies the first chain to V[o] and reduces d[o * nt + t] (float bits,
+// zeroed by the caller; NaN terms drop out as they do in the sweeps' residual).
+template <int NO>
+__global__ void finalize_two_kernel(const VPack<float, 2 * NO> *tab, VOut<float, NO> out, int64_t nS, int64_t Nc,
+                                    int nt, unsigned int *d) {
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t n = nS + 1, n_pad = (n + 31) & ~(int64_t)31;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_pad; i += stride) {
+    const bool in = i < n;
+    VPack<float, 2 * NO> p{};
+    if (in) p = tab[i];
+    const int64_t i0 = i - lane, t0 = i0 / Nc;
+    const bool one = (i0 + 31) < (t0 + 1) * Nc && i0 + 31 < nS;   // the warp's states share a layer
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      if (in) out.V[o][i] = p.v[o];
+      const float diff = i < nS ? fmaxf(0.f, fabsf(p.v[o] - p.v[NO + o])) : 0.f;
+      if (one) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(diff));
+        if (lane == 0 && m > d[o * nt + t0]) atomicMax(&d[o * nt + t0], m);
+      } else if (i < nS) {
+        atomicMax(&d[o * nt + i / Nc], __float_as_uint(diff));
+      }
+    }
+  }
+}
+
+// io.table[0]: the packed table of 2 n components per state, zeroed by the caller.
+template <int NO>
+static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st) {
+  PipeRange pr0;
+  size_t smem = 0;
+  int blocks = 1;
+  cudaError_t e = pipe_config<float, NO, true>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
+  if (e != cudaSuccess) return e;
+  VSet<float, NO, true> v;
+  auto *t = static_cast<VPack<float, 2 * NO> *>(io.table[0]);
+  v.in = t;
+  v.out = t;
+  VOut<float, NO> out;
+  for (int o = 0; o < NO; ++o) {
+    v.R[o] = static_cast<const float *>(io.R[o]);
+    v.pol[o] = io.policy[o];
+    v.res[o] = nullptr;
+    out.V[o] = static_cast<float *>(io.V[o]);
+  }
+  SolveArgs rest = a;   // a test's injected failure is for the first launch alone
+  rest.test_extra_tx = 0;
+  for (int t_ = nt - 1; t_ >= 0; --t_) {
+    PipeRange pr = pr0;
+    pr.s_lo = (int64_t)t_ * a.Nc;
+    pr.s_hi = pr.s_lo + a.Nc;
+    pr.sl_lo = pr.s_lo / a.spw;
+    pr.sl_hi = (pr.s_hi + a.spw - 1) / a.spw;
+    pr.zero_second = t_ == nt - 1;
+    launch_sweep(t_ < nt - 1 ? rest : a, v, 0, pr, blocks, smem, st, t_ < nt - 1);
+  }
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const int64_t fb = std::min<int64_t>((a.nS + 256) / 256, (int64_t)num_sms() * 8);
+  finalize_two_kernel<NO><<<(unsigned)fb, 256, 0, st>>>(t, out, a.nS, a.Nc, nt, d);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st) {
+  switch (io.n) {
+    case 1: return two_chains_t<1>(a, nt, io, d, st);
+    case 2: return two_chains_t<2>(a, nt, io, d, st);
+    case 3: return two_chains_t<3>(a, nt, io, d, st);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 template <typename RT>

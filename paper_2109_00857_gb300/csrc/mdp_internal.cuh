@@ -333,6 +333,10 @@ cudaError_t launch_jacobi_multi(const SolveArgs &a, int precision, int max_sweep
                                 double *stats_d, cudaStream_t st);
 cudaError_t launch_layered_multi(const SolveArgs &a, int precision, int nt, const SolveIO &io,
                                  double *stats_d, cudaStream_t st);
+// FP32 Jacobi result by two backward chains (see bellman.cu): V[o], policies
+// and d[o * nt + t], the lower bound of the residual of sweep nt - t (float
+// bits); io.table[0] holds 2 n values per state, zeroed by the caller like d
+cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st);
 cudaError_t launch_jacobi(const SolveArgs &a, int precision, int max_sweeps, void *Va, void *Vb,
                           int16_t *policy, double *stats_d, cudaStream_t st);
 // Copies the slices' entry columns from `pool` (any order) into `out` in
