@@ -110,8 +110,7 @@ mdp_status check_device() {
 // the exact FP64 value of 1 - frac(d) (frac(d) of a float has at most 24
 // significant bits; when 1 - frac(d) is not exact in FP64 it lies within
 // 2^-29 of 1 and rounds up to 1 all the same); 2 when frac(d) = 0.
-static void offset_thresholds(const float *d, int A, int32_t *c, float *th, float *T, int32_t *le, int32_t *D,
-                              uint8_t *L, int32_t *M) {
+static void offset_thresholds(const float *d, int A, int32_t *c, float *th, float *T, int32_t *le, int32_t *D) {
   std::vector<float> u;
   for (int a = 0; a < A; ++a) {
     const double dd = (double)d[a];
@@ -141,15 +140,36 @@ static void offset_thresholds(const float *d, int A, int32_t *c, float *th, floa
     le[a] = (a < A && th[a] < 2.0f) ? n : (int32_t)u.size() + 1;
   }
   for (int a = A; a < kMaxActions; ++a) { c[a] = 0; th[a] = 2.0f; }
-  // rank lookup: thresholds bucketed by floor(128 T) (clamped to the last bucket)
-  std::vector<int> inb(kRankBuckets, 0);
-  for (float v : u) inb[std::min((int)std::floor((double)v * kRankBuckets), kRankBuckets - 1)]++;
-  int below = 0;
-  *M = 0;
-  for (int b = 0; b < kRankBuckets; ++b) {
-    L[b] = (uint8_t)below;
-    below += inb[b];
-    *M = std::max(*M, inb[b]);
+}
+
+// The group kernel's rank lookup for the two axes' thresholds (ActionTable).
+static void rank_plan(ActionTable *t) {
+  const float *T[2] = {t->Tx, t->Ty};
+  const int D[2] = {t->Dx, t->Dy};
+  for (int B = 128; B <= kMaxBuckets; B *= 2) {
+    bool ok = true;
+    float trap = 0.f;
+    for (int x = 0; x < 2 && ok; ++x) {
+      std::vector<int> in(B + 1, 0);
+      for (int i = 0; i < D[x]; ++i) in[(int)std::floor((double)T[x][i] * B)]++;
+      for (int b = 1; b <= B; ++b) ok = ok && in[b] <= 1;
+      if (in[0] >= 2) trap = std::max(trap, T[x][in[0] - 2]);
+    }
+    // (a trap that realizations do meet would count their states twice)
+    if (ok && trap <= 0x1p-24f) {
+      t->rank_mode = 1;
+      t->rank_buckets = B;
+      t->rank_trap = trap;
+      return;
+    }
+  }
+  t->rank_buckets = 128;
+  t->rank_trap = 0.f;
+  t->rank_mode = 2;
+  for (int x = 0; x < 2; ++x) {
+    std::vector<int> in(129, 0);
+    for (int i = 0; i < D[x]; ++i)
+      if (++in[(int)std::floor((double)T[x][i] * 128)] > 2) t->rank_mode = 3;
   }
 }
 
@@ -181,8 +201,9 @@ mdp_status make_actions(const mdp_actions *ac, double lam, ActionTable *t, int *
     t->dyl[a] = (float)(dy * lam);
     t->F[a] = (float)F;
   }
-  offset_thresholds(t->dxl, A, t->cx, t->thx, t->Tx, t->lex, &t->Dx, t->Lx, &t->Mx);
-  offset_thresholds(t->dyl, A, t->cy, t->thy, t->Ty, t->ley, &t->Dy, t->Ly, &t->My);
+  offset_thresholds(t->dxl, A, t->cx, t->thx, t->Tx, t->lex, &t->Dx);
+  offset_thresholds(t->dyl, A, t->cy, t->thy, t->Ty, t->ley, &t->Dy);
+  rank_plan(t);
   *A_out = A;
   return MDP_OK;
 }

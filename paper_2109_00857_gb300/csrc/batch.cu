@@ -72,7 +72,7 @@ struct mdp_batch_t {
   // group one persistent launch over its own zero-based prefix segment
   struct Group {
     int start, n, pstart, K, spw;
-    bool dense;
+    int rank_mode;
   };
   std::vector<Group> groups;
   size_t cta_smem = 0;
@@ -136,7 +136,7 @@ cudaError_t enqueue(mdp_batch_t *b) {
   for (size_t g = 0; g < b->groups.size() && e == cudaSuccess; ++g) {
     const auto &G = b->groups[g];
     e = launch_build_warp_batch(b->items_d + G.start, b->prefix_d + G.pstart, G.n, b->work_d + g, b->cap_bins,
-                                G.K, G.spw, G.dense, st);
+                                G.K, G.spw, G.rank_mode, st);
   }
   if (e == cudaSuccess) e = launch_build_fp32_batch(b->items_d, b->n, b->cta_smem, b->cta_threads, st);
   for (int i = 0; i < b->n && e == cudaSuccess; ++i) {
@@ -333,18 +333,18 @@ extern "C" mdp_status mdp_batch_create(const mdp_batch_item *items_h, int32_t n,
     si.stats = it.stats;
     si.max_sweeps = it.max_sweeps;
   }
-  // group the build items by (states per slice, mode count, threshold density); prefix segments per group
+  // group the build items by (states per slice, mode count, rank lookup); prefix segments per group
   std::vector<int> ord(n);
   for (int i = 0; i < n; ++i) ord[i] = i;
-  auto dense = [&](int i) { return args[i].act.Mx > 2 || args[i].act.My > 2; };
-  auto cls = [&](int i) { return (dense(i) ? 4096 : 0) + args[i].spw * 64 + std::min<int>(args[i].K, 63); };
+  auto cls = [&](int i) { return args[i].act.rank_mode * 4096 + args[i].spw * 64 + std::min<int>(args[i].K, 63); };
   std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cls(x) < cls(y); });
   std::vector<BuildArgs> sorted(n);
   std::vector<int64_t> gprefix;
   for (int j = 0; j < n;) {
     int e = j;
     while (e < n && cls(ord[e]) == cls(ord[j])) ++e;
-    mdp_batch_t::Group G{j, e - j, (int)gprefix.size(), args[ord[j]].K, args[ord[j]].spw, dense(ord[j])};
+    mdp_batch_t::Group G{j, e - j, (int)gprefix.size(), args[ord[j]].K, args[ord[j]].spw,
+                         args[ord[j]].act.rank_mode};
     const int per = batch_group_slices(G.spw);   // slices per group of the kernel's work queue
     int64_t acc = 0;
     gprefix.push_back(0);

@@ -15,34 +15,38 @@
 // per axis, in the state's fine table.
 //
 // A CTA of NW warps builds a group of NW consecutive slices (NW spw states):
-//   count    every warp covers all the group's states -- lane (q, i) state q,
-//            realizations i, i + 32/spw, ... -- so a warp's loads touch only
-//            32 / (NW spw) coefficient rows (one 128-byte wavefront per 16
-//            bytes a lane; a warp on a state of its own needs eight), and
-//            each row is read once per group, not once per state.  One pass:
-//            the state's table is a window predicted from the coefficients'
-//            spread, the exact extremes of u are tracked beside the counts
-//            (three-input minima, one instruction per two realizations), and
-//            the window is checked afterwards.  Table addresses are masked to
-//            the state's power-of-two table, so a realization outside the
-//            window corrupts only its own state's table, which is then
-//            counted again with the exact window (recount_state; never on the
-//            workloads measured: the windows hold 5 to 7 standard deviations,
-//            N = 5000 draws reach 4).
+//   count    every warp covers all the group's states: lane (i, p) the states 2 p
+//            and 2 p + 1, realizations i, i + 64/spw, ...  The LSU returns 128
+//            bytes a cycle to the lanes whatever the addresses, so what a
+//            realization's row costs is set by how many states a lane applies
+//            it to: two (a third would not fit the registers).  One pass: the
+//            state's table is a window predicted from the coefficients' spread,
+//            the exact extremes of u are tracked beside the counts (three-input
+//            minima, one instruction per two realizations), and the window is
+//            checked afterwards.  Table addresses are taken modulo the state's
+//            power-of-two table, so a realization outside the window corrupts
+//            only its own state's table, which is then counted again with the
+//            exact window (recount_state; rare: the windows hold 5 to 7 standard
+//            deviations, N = 5000 draws reach 4).
+//            Bound by issue and the LSU: 46 warp instructions and 11 LSU
+//            wavefronts per 32 (state, realization) items -- 17 FMAs, 4 lookups,
+//            3 wavefronts of shared counts, 4 of coefficients (the earlier
+//            kernel, one state per lane and warp, 128 and 45 over its two passes).
 //   prefix   warp v owns slice v: in-place 2-D inclusive prefix sums of its
 //            states' tables over their exact extents.
 //   emit     lane l = row (state q, action a): an offset bin (dx, dy) collects
 //            exactly the fine cells X in [(dx - c_a - 1) S + le_a, + S) (and
-//            likewise in y) -- a box whose count is four prefix lookups; two
-//            scans of the row's bounding box count the entries (sink folded),
-//            allocate the slice's columns and write the entry words in
-//            ascending order with R(s,a) from the counts.
+//            likewise in y) -- a box of the prefix table.  One scan of the row's
+//            bins stages its entry words in ascending order (sink folded), the
+//            group allocates its columns, and the rows are copied out with
+//            R(s,a) from the counts.
 // Slices whose exact fine tables do not fit are appended to a list that the
 // CTA kernel of build_fp32.cu finishes with a full-window histogram and the
 // same landing offsets, so a slice's output does not depend on which kernel
 // built it.
 #pragma once
 #include <climits>
+#include <cstddef>
 
 #include "build_common.cuh"
 
@@ -68,121 +72,158 @@ __device__ __forceinline__ float max_nan(float a, float b, float c) {
   return r;
 }
 
+// Two floats in one 64-bit register pair and their packed operations: one
+// instruction works on both (each half rounds like the scalar operation, so a
+// realization's u does not depend on the pairing).
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack2(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 fma2_down(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 add2_down(f2 a, f2 b) {
+  f2 r;
+  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Mode-count variants: KT > 0 exactly KT modes; KT == 0 up to kMaxModes (runtime).
 template <int KT>
 constexpr int kPhi = KT > 0 ? KT : kMaxModes;
 
-// A realization's coefficient row in registers, with the widest loads its
-// alignment allows (coeffs are 16-byte aligned).
+// A realization's coefficient row, with the widest loads its alignment allows
+// (coeffs are 16-byte aligned).
 template <int KT>
-struct Row {
-  float y[kPhi<KT>];
-};
-template <int KT>
-__device__ __forceinline__ void load_row(const float *__restrict__ yw, int K, Row<KT> &r) {
+__device__ __forceinline__ void load_row(const float *__restrict__ yw, int K, float (&y)[kPhi<KT>]) {
   if constexpr (KT > 0 && KT % 4 == 0) {
 #pragma unroll
     for (int k = 0; k < KT; k += 4) {
       const float4 v = __ldg(reinterpret_cast<const float4 *>(yw + k));
-      r.y[k] = v.x; r.y[k + 1] = v.y; r.y[k + 2] = v.z; r.y[k + 3] = v.w;
+      y[k] = v.x; y[k + 1] = v.y; y[k + 2] = v.z; y[k + 3] = v.w;
     }
   } else if constexpr (KT > 0 && KT % 2 == 0) {
 #pragma unroll
     for (int k = 0; k < KT; k += 2) {
       const float2 v = __ldg(reinterpret_cast<const float2 *>(yw + k));
-      r.y[k] = v.x; r.y[k + 1] = v.y;
+      y[k] = v.x; y[k + 1] = v.y;
     }
-  } else if constexpr (KT > 0) {
-#pragma unroll
-    for (int k = 0; k < KT; ++k) r.y[k] = __ldg(yw + k);
   } else {
 #pragma unroll
-    for (int k = 0; k < kMaxModes; ++k)
-      if (k < K) r.y[k] = __ldg(yw + k);
+    for (int k = 0; k < kPhi<KT>; ++k)
+      if (KT > 0 || k < K) y[k] = __ldg(yw + k);
   }
 }
-
-// u of one realization: the CTA kernel's FP32 operations (FMA chain over
-// ascending k, then u = fma(w, lam, 1/2)).
+// Warps (slices of a group) per CTA, and the CTAs per SM that the registers have
+// to allow: five CTAs of four warps at 96 registers, two realizations of two
+// states in flight per lane.  Measured (build kernel of the large, energy and
+// 16-action CSR workloads): 62.8 / 2.81 / 1.04 ms; four CTAs at 128 registers
+// 61.2 / 2.95 / 1.08; two CTAs of eight warps 66.4 / 3.08 / 1.17; one realization
+// in flight 70.6 / 3.08 / 1.12.
+constexpr int kGroupWarps = 4;
 template <int KT>
-__device__ __forceinline__ float2 velocity_u(const Row<KT> &r, const float (&phx)[kPhi<KT>],
-                                             const float (&phy)[kPhi<KT>], float vbx, float vby, int K, float lam) {
-  float wx = vbx, wy = vby;
-#pragma unroll
-  for (int k = 0; k < kPhi<KT>; ++k) {
-    if (KT > 0 || k < K) {
-      wx = fmaf(r.y[k], phx[k], wx);
-      wy = fmaf(r.y[k], phy[k], wy);
-    }
-  }
-  return make_float2(fmaf(wx, lam, 0.5f), fmaf(wy, lam, 0.5f));
-}
+constexpr int kMinCtas = KT == 0 ? 4 : 5;
 
 // ---- fractional ranks ----
-// Per CTA, in shared memory: per axis the thresholds T[i] (2 for i >= D) and
-// the lookup L[b] = 4 #{T in buckets < b} over kRankBuckets buckets of [0, 1]
-// (entry kRankBuckets: f = 1 exactly, which counts like the last bucket).
+// Per CTA, in shared memory: per axis T[1 + i] the thresholds (T[0] = -1, 2
+// after the last) and the lookup L[b] = 4 * (thresholds up to and including
+// bucket b; MODE 2 and 3: below bucket b) over act.rank_buckets buckets of
+// [0, 1]; f = 1 has its own.  The displacements' per-action constants.
 struct RankTables {
   float T[2][kMaxActions + 4];
-  uint8_t L[2][kRankBuckets + 4];
+  uint8_t L[2][kMaxBuckets + 4];
+  int c[2][kMaxActions], le[2][kMaxActions];
+  float th[2][kMaxActions], F[kMaxActions];
 };
-struct RankTab {
-  const float *T;
-  const uint8_t *L;
-};
-__device__ __forceinline__ RankTab rank_tab(const RankTables &rt, int axis) { return RankTab{rt.T[axis], rt.L[axis]}; }
 
-// Copies a model's rank tables (whole CTA; the caller synchronises).
+// Fills a model's tables (whole CTA; the caller synchronises).  (The action
+// constants are read per lane: from the constant bank that would be one
+// access per distinct action.)
 __device__ __forceinline__ void load_rank_tables(const BuildArgs &a, RankTables &rt) {
-  for (int i = threadIdx.x; i < kMaxActions + 2; i += blockDim.x) {
-    rt.T[0][i] = a.act.Tx[i];
-    rt.T[1][i] = a.act.Ty[i];
+  const int B = a.act.rank_buckets;
+  for (int i = threadIdx.x; i < kMaxActions + 3; i += blockDim.x) {
+    rt.T[0][i] = i == 0 ? -1.f : (i <= a.act.Dx ? a.act.Tx[i - 1] : 2.f);
+    rt.T[1][i] = i == 0 ? -1.f : (i <= a.act.Dy ? a.act.Ty[i - 1] : 2.f);
   }
-  for (int b = threadIdx.x; b <= kRankBuckets; b += blockDim.x) {
-    rt.L[0][b] = (uint8_t)(4 * a.act.Lx[min(b, kRankBuckets - 1)]);
-    rt.L[1][b] = (uint8_t)(4 * a.act.Ly[min(b, kRankBuckets - 1)]);
+  for (int i = threadIdx.x; i < kMaxActions; i += blockDim.x) {
+    rt.c[0][i] = a.act.cx[i]; rt.c[1][i] = a.act.cy[i];
+    rt.le[0][i] = a.act.lex[i]; rt.le[1][i] = a.act.ley[i];
+    rt.th[0][i] = a.act.thx[i]; rt.th[1][i] = a.act.thy[i];
+    rt.F[i] = a.act.F[i];
+  }
+  const bool upto = a.act.rank_mode == 1;
+  for (int b = threadIdx.x; b <= B; b += blockDim.x) {
+    int nx = 0, ny = 0;
+    for (int i = 0; i < a.act.Dx; ++i) nx += (int)(a.act.Tx[i] * (float)B) < b + (upto ? 1 : 0) ? 1 : 0;
+    for (int i = 0; i < a.act.Dy; ++i) ny += (int)(a.act.Ty[i] * (float)B) < b + (upto ? 1 : 0) ? 1 : 0;
+    rt.L[0][b] = (uint8_t)(4 * nx);
+    rt.L[1][b] = (uint8_t)(4 * ny);
   }
 }
 
-// floor(u) and the rank of its fraction for |u| < kTame: the floor by adding
-// 1.5 2^23 rounded down (its low mantissa bits are floor(u)), the bucket
-// floor(128 f) by a product rounded down to a multiple of the smallest float
-// (whose bits are the integer): no conversion instruction.  Any other u gives
-// some fraction in [0, 1] (saturation; NaN gives 0), so the lookups stay in
-// their tables.
+// floor(u) for |u| < kTame by adding 1.5 2^23 rounded down: the low mantissa
+// bits of the sum are floor(u).
 constexpr float kTame = 16384.f;
 constexpr float kFloorMagic = 12582912.f;          // 1.5 2^23
 constexpr uint32_t kFloorBits = 0x4B400000u;       // its bits
-struct FloorRank {
-  uint32_t n;    // floor(u) + kFloorBits
-  uint32_t r4;   // 4 rank
-};
-// DENSE: more than two thresholds in some bucket (the tail is scanned).
-template <bool DENSE>
-__device__ __forceinline__ FloorRank floor_rank(float u, const RankTab &rt) {
+// An integer i < 2^23 as the float whose bits it is (i times the smallest
+// float): a product or sum of such floats rounded down is integer arithmetic.
+__device__ __forceinline__ float int_float(uint32_t i) { return __uint_as_float(i); }
+
+// Fine coordinate of u (|u| < kTame) along an axis: floor(u) S + rank, rank =
+// #{T <= u - floor(u)}; exact for any table.
+template <int MODE>
+__device__ __forceinline__ int fine_coord(float u, int S, const RankTables &rt, int axis, int buckets) {
   const float t = __fadd_rd(u, kFloorMagic);
   const float f = __saturatef(u - (t - kFloorMagic));
-  const uint32_t b = __float_as_uint(__fmul_rd(f, __uint_as_float((uint32_t)kRankBuckets)));
-  uint32_t r4 = rt.L[b];
-  const float *T = reinterpret_cast<const float *>(reinterpret_cast<const char *>(rt.T) + r4);
-  // the thresholds below f's bucket come from the lookup; those in the bucket
-  // follow them in T and every later one exceeds f, so with at most two per
-  // bucket two comparisons finish it
-  if constexpr (!DENSE) {
-    r4 += (T[0] <= f ? 4u : 0u) + (T[1] <= f ? 4u : 0u);
+  int r = rt.L[axis][__float_as_uint(__fmul_rd(f, int_float((uint32_t)buckets)))] >> 2;
+  const float *T = rt.T[axis] + 1;
+  if constexpr (MODE == 1) {
+    while (r > 0 && T[r - 1] > f) --r;
   } else {
-    while (*T <= f) {   // T[D] = 2 > f ends it
-      ++T;
-      r4 += 4u;
-    }
+    while (T[r] <= f) ++r;   // T[D] = 2 > f ends it
   }
-  return FloorRank{__float_as_uint(t), r4};
+  return (int)(__float_as_uint(t) - kFloorBits) * S + r;
 }
-// Fine coordinate of u (|u| < kTame): floor(u) S + rank.
-template <bool DENSE>
-__device__ __forceinline__ int fine_coord(float u, int S, const RankTab &rt) {
-  const FloorRank fr = floor_rank<DENSE>(u, rt);
-  return (int)(fr.n - kFloorBits) * S + (int)(fr.r4 >> 2);
+
+// 4 rank of f, its lookup entry at shared address `l`; AXIS selects the
+// tables, which follow one another.  MODE 1 is one comparison with the last
+// threshold up to f's bucket, MODE 2 two with those in it.
+template <int MODE, int AXIS>
+__device__ __forceinline__ uint32_t rank4(uint32_t l, float f, uint32_t t_base) {
+  uint32_t r;
+  if constexpr (MODE == 1) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .f32 t;\n\t.reg .u32 a;\n\t"
+        "ld.shared.u8 %0, [%1 + %4];\n\tadd.u32 a, %0, %3;\n\tld.shared.f32 t, [a + %5];\n\t"
+        "setp.lt.f32 p, %2, t;\n\t@p sub.u32 %0, %0, 4;\n\t}"
+        : "=&r"(r)
+        : "r"(l), "f"(f), "r"(t_base), "n"(AXIS * (int)sizeof(RankTables::L[0])), "n"(AXIS * (int)sizeof(RankTables::T[0])));
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .f32 t, v;\n\t.reg .u32 a;\n\t"
+        "ld.shared.u8 %0, [%1 + %4];\n\tadd.u32 a, %0, %3;\n\tld.shared.f32 t, [a + %5];\n\t"
+        "ld.shared.f32 v, [a + %6];\n\tsetp.le.f32 p, t, %2;\n\tsetp.le.f32 q, v, %2;\n\t"
+        "@p add.u32 %0, %0, 4;\n\t@q add.u32 %0, %0, 4;\n\t}"
+        : "=&r"(r)
+        : "r"(l), "f"(f), "r"(t_base), "n"(AXIS * (int)sizeof(RankTables::L[0])),
+          "n"(AXIS * (int)sizeof(RankTables::T[0]) + 4), "n"(AXIS * (int)sizeof(RankTables::T[0]) + 8));
+  }
+  return r;
 }
 
 // A state's fine table over X in [xmin, xmin + gx), Y in [ymin, ymin + gy):
@@ -195,67 +236,57 @@ struct FineGeo {
 
 // ---- shared memory of a CTA ----
 // GroupSmem (the batched kernel: with the model's arguments), the extremes
-// [NW][NW spw] float4, then, aligned to a state's table, NW slices of `words`
-// table words each; a state has words / spw of them, a power of two.
-constexpr int kGroupWarps = 8;     // most warps (slices) per CTA
+// [NW][NW spw] float4, then NW slices of `words` table words each; a state has
+// words / spw of them, a power of two.
 // Per-warp totals, added to the model's counters by warp_flush().
 struct WarpAcc {
   unsigned long long samples, nnz, dom, maxrow;
 };
+// A state's count set-up.  Its table address of fine cell (X, Y), X = n S + rank
+// with n = floor(u) as the bits n + kFloorBits and r4 = 4 rank: the cell index
+// modulo the table by 32-bit overflow, lin = n_x aN + r4_x aR + n_y bN + r4_y bR +
+// c0 in units of 2^32 / words, its byte offset the high half of lin * bytes.
+struct StateSetup {
+  int4 win;              // the window's (xmin, ymin, gx, pitch << 8 | rotation); gy = pitch - 1
+  uint32_t base, bytes, aN, aR, c0;
+  int32_t layer;         // time layer; -1: not sampled, -2: sampled, but tables have no words
+  int32_t kind;          // state_kind
+  float vbx, vby;
+};
 struct GroupSmem {
   RankTables rt;
-  int4 win[32];                    // [state]: the count window's (xmin, ymin, gx, pitch); gy = pitch - 1
   WarpAcc acc[kGroupWarps];        // per warp (in shared memory: the registers are the count loop's)
   long long next[2];               // next group of the work queue, alternating
   unsigned long long base[kGroupWarps];   // the slices' places in the pool
   int cols[kGroupWarps];           // and their columns
+  uint32_t dummy[32];              // where lanes without a state to count put their counts
+  unsigned int trap;               // states to count again (a fraction below act.rank_trap)
+  StateSetup st[32];               // the group's states (last: only NW spw are laid out)
 };
-// Table words of a slice: the largest power of two <= cap_bins (at least one
-// word per state, else 0: no slice fits and all go to the CTA kernel).
+// Table words of a slice: the largest power of two <= cap_bins, if a state's
+// share of it is at least 16 words (else 0: no slice fits and all go to the
+// CTA kernel).
 __host__ __device__ constexpr int table_words(int cap_bins, int spw) {
   int w = 1;
   while (2 * w <= cap_bins) w *= 2;
-  return w >= 32 && w >= spw ? w : 0;
-}
-// A slice's table memory starts at a multiple of this: a state's table, for
-// the address mask, and 16 bytes, for the vector stores that clear it.
-__host__ __device__ constexpr uint32_t table_align(int words, int spw) {
-  return 4u * (uint32_t)(words / spw) > 16u ? 4u * (uint32_t)(words / spw) : 16u;
+  return w >= 32 && w >= 16 * spw ? w : 0;
 }
 __host__ __device__ constexpr int group_warps(int warps, int spw) {
   const int most = 32 / spw < kGroupWarps ? 32 / spw : kGroupWarps;   // at most one state per lane
   return warps < most ? warps : most;
 }
-// Bytes before the table memory is aligned: the head struct and the extremes.
-__host__ __device__ constexpr uint32_t group_head_bytes(size_t head, int spw, int nw) {
-  return (uint32_t)((head + 15) & ~(size_t)15) + 16u * (uint32_t)(nw * nw * spw);
+constexpr int kStage = 12;   // entries per row the emit stages (longest row measured: 12); 1.5 KB per warp
+// Bytes before the table memory (the head, the extremes, the entry stages), and
+// of a CTA's dynamic shared memory.
+// `before`: bytes the kernel puts in front of GroupSmem (a multiple of 16).
+__host__ __device__ constexpr uint32_t group_ext_offset(uint32_t before, int spw, int nw) {
+  return (before + (uint32_t)offsetof(GroupSmem, st) + (uint32_t)(nw * spw) * (uint32_t)sizeof(StateSetup) + 15u) & ~15u;
 }
-// Dynamic shared memory of a CTA.  `reserved` bytes precede it in the shared
-// window (the system's; the kernels have no static shared memory), so the
-// head fills the gap below the first aligned table: 72 KB and three CTAs per
-// SM at 2048 words, where reserving a worst-case gap allowed two.
-inline size_t group_smem_bytes(size_t head, int reserved, int cap_bins, int spw, int nw) {
-  const int words = table_words(cap_bins, spw);
-  const uint32_t al = table_align(words, spw), hd = (uint32_t)reserved + group_head_bytes(head, spw, nw);
-  return (size_t)((hd + al - 1) / al * al - (uint32_t)reserved) + (size_t)nw * 4u * (size_t)words;
+__host__ __device__ constexpr uint32_t group_head_bytes(uint32_t before, int spw, int nw) {
+  return group_ext_offset(before, spw, nw) + 16u * (uint32_t)(nw * nw * spw) + 128u * (uint32_t)(nw * kStage);
 }
-inline cudaError_t reserved_smem(int *bytes) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(bytes, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-  return e;
-}
-// The CTA's table memory in its dynamic shared memory.  Should the tables not
-// fit behind the alignment (another layout of the shared window), *words
-// becomes 0: every sampled slice then goes to the CTA kernel.
-__device__ __forceinline__ uint32_t *table_memory(unsigned char *smem, size_t head, int *words, int spw) {
-  const int nw = blockDim.x >> 5;
-  const uint32_t used = group_head_bytes(head, spw, nw), al = table_align(*words, spw);
-  const uint32_t b = smem_u32(smem) + used, off = used + (((b + al - 1) & ~(al - 1)) - b);
-  uint32_t size;
-  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(size));
-  if (off + (uint32_t)nw * 4u * (uint32_t)*words > size) *words = 0;
-  return reinterpret_cast<uint32_t *>(smem + off);
+inline size_t group_smem_bytes(uint32_t before, int cap_bins, int spw, int nw) {
+  return group_head_bytes(before, spw, nw) + (size_t)nw * 4u * (size_t)table_words(cap_bins, spw);
 }
 // (lane 0 of each warp owns its totals)
 __device__ __forceinline__ void warp_clear(GroupSmem &sm) {
@@ -279,64 +310,131 @@ __device__ __forceinline__ void clear_tables(uint32_t *tabs, int words) {   // w
 // standard deviations (the coefficients' means and variances per layer through
 // the state's modes), the half widths shrunk together until the table fits,
 // spare rows split between both ends.  Measured need on the large workload:
-// 921 cells on average, 1739 at most, of 2048.
+// 921 cells on average, 1739 at most, of 2048.  The table is rotated by up to
+// 31 words (base) so that the group's states have their centres in different
+// banks: the counts of a warp then meet 3.4-fold conflicts, not 4.7.
 constexpr float kSpread = 7.f;
-template <int KT, bool DENSE>
-__device__ __forceinline__ FineGeo predict_window(const BuildArgs &a, int64_t t, const float (&phx)[kPhi<KT>],
-                                                  const float (&phy)[kPhi<KT>], float vbx, float vby, int K, int Sx,
-                                                  int Sy, const RankTables &rt, int words) {
-  float cx = vbx, cy = vby, vx = 0.f, vy = 0.f;
-#pragma unroll
-  for (int k = 0; k < kPhi<KT>; ++k) {
-    if (KT > 0 || k < K) {
-      float m = 0.f, v = a.coef_var[k];
+__host__ __device__ constexpr int window_words(int words) { return words >= 256 ? words - 32 : words; }
+// Warp v's part for the group whose first slice is sl0: the set-up of its
+// slice's states, 32 / spw lanes per state over the modes (so that the count
+// loop's warps, which all work on all states, find it in shared memory).  In
+// two halves: the loads are issued before the previous group's write and used
+// after it.
+struct SetupLoads {
+  int kind;
+  int64_t t;
+  float2 vb, ph;   // the state's mean flow; mode lane % per
+};
+template <int SPW>
+__device__ __forceinline__ SetupLoads setup_load(const BuildArgs &a, int64_t sl0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, spw = SPW > 0 ? SPW : a.spw, per = 32 / spw;
+  const int64_t sl = sl0 + warp, s = sl * spw + lane / per, Nc = a.Nc;
+  SetupLoads l{KIND_NONE, 0, make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  if (sl < a.slice_end && s < a.nS) {
+    l.kind = state_kind(a, s);
+    l.t = layer_of(s, Nc, a.nS);
+    l.vb = __ldg(reinterpret_cast<const float2 *>(a.vbar) + s);
+    const int k = lane % per;
+    if (k < a.K) l.ph = __ldg(reinterpret_cast<const float2 *>(a.modes) + l.t * (a.K - 1) * Nc + s + k * Nc);
+  }
+  return l;
+}
+__device__ __forceinline__ float sqrt_fast(float x) {   // (where a window lies, not a result)
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+template <int SPW, int MODE>
+__device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, int64_t sl0, const SetupLoads &ld,
+                                            uint32_t *tabs, int words) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
+  const int spw = SPW > 0 ? SPW : a.spw, per = 32 / spw, K = a.K, G = NW * spw, table = words / spw;
+  const int q = warp * spw + lane / per;   // state of the group
+  const int64_t t = ld.t;
+  const bool sampled = ld.kind == KIND_SAMPLE, sample = sampled && table > 0;
+  float mx = 0.f, my = 0.f, vx = 0.f, vy = 0.f;
+  if (sample) {
+    for (int k = lane % per; k < K; k += per) {
+      const float2 ph = k < per ? ld.ph
+                                : reinterpret_cast<const float2 *>(a.modes)[t * (K - 1) * a.Nc + sl0 * spw + q + k * a.Nc];
+      float v = a.coef_var[k];
       if (a.mom) {
         const float2 mv = __ldg(a.mom + (size_t)t * K + k);
-        m = mv.x;
         v = mv.y;
+        mx = fmaf(mv.x, ph.x, mx);
+        my = fmaf(mv.x, ph.y, my);
       }
-      cx = fmaf(m, phx[k], cx);
-      cy = fmaf(m, phy[k], cy);
-      vx = fmaf(v * phx[k], phx[k], vx);
-      vy = fmaf(v * phy[k], phy[k], vy);
+      vx = fmaf(v * ph.x, ph.x, vx);
+      vy = fmaf(v * ph.y, ph.y, vy);
     }
   }
-  const float lim = 0.5f * kTame;
-  cx = fmaf(cx, a.lam, 0.5f);
-  cy = fmaf(cy, a.lam, 0.5f);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    if (off >= per) continue;
+    vx += __shfl_xor_sync(0xffffffffu, vx, off);
+    vy += __shfl_xor_sync(0xffffffffu, vy, off);
+    if (a.mom) {
+      mx += __shfl_xor_sync(0xffffffffu, mx, off);
+      my += __shfl_xor_sync(0xffffffffu, my, off);
+    }
+  }
+  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1, room = window_words(table);
+  const float lam = a.lam, lim = 0.5f * kTame;
+  float cx = fmaf(ld.vb.x + mx, lam, 0.5f), cy = fmaf(ld.vb.y + my, lam, 0.5f);
   if (!(fabsf(cx) < lim)) cx = 0.f;
   if (!(fabsf(cy) < lim)) cy = 0.f;
-  // standard deviations in cells, at least one fine cell and at most 64 cells
-  const float sx = fminf(fmaxf(a.lam * sqrtf(vx), 1.f / (float)Sx), 64.f);
-  const float sy = fminf(fmaxf(a.lam * sqrtf(vy), 1.f / (float)Sy), 64.f);
-  // (2 h sx Sx + 2)(2 h sy Sy + 2) <= words for the half width h (in standard deviations)
-  const float p = 2.f * sx * (float)Sx, q = 2.f * sy * (float)Sy, s = p + q;
-  const float h = fminf(kSpread, (sqrtf(s * s + p * q * ((float)words - 4.f)) - s) / (p * q));
-  FineGeo g;
-  g.ymin = fine_coord<DENSE>(cy - h * sy, Sy, rank_tab(rt, 1));
-  g.gy = min(fine_coord<DENSE>(cy + h * sy, Sy, rank_tab(rt, 1)) - g.ymin + 1, words / 2 - 2);
-  g.gy = max(g.gy, 1);
-  g.pitch = (g.gy + 1) | 1;
-  g.gy = g.pitch - 1;
-  g.gx = words / g.pitch - 1;
-  const int x0 = fine_coord<DENSE>(cx - h * sx, Sx, rank_tab(rt, 0));
-  const int x1 = fine_coord<DENSE>(cx + h * sx, Sx, rank_tab(rt, 0));
-  g.xmin = x0 - (g.gx - (x1 - x0 + 1)) / 2;
-  g.base = 0;
-  return g;
+  // the window's size in fine cells: h standard deviations (at least half a
+  // fine cell each, at most 64 cells) to either side, the fine cells taken as even,
+  //   (2 h sx Sx + 2)(2 h sy Sy + 2) <= room
+  const float p = 2.f * fminf(fmaxf(lam * sqrt_fast(vx) * (float)Sx, 1.f), 64.f * (float)Sx);
+  const float r = 2.f * fminf(fmaxf(lam * sqrt_fast(vy) * (float)Sy, 1.f), 64.f * (float)Sy);
+  const float d = p + r, h = fminf(kSpread, __fdividef(sqrt_fast(d * d + p * r * ((float)room - 4.f)) - d, p * r));
+  const int gy0 = max(min((int)(h * r) + 2, room / 2 - 2), 1), pitch = (gy0 + 1) | 1, gy = pitch - 1;
+  int gx = (int)__fdividef((float)room, (float)pitch);   // rows: room / pitch, one of them the border
+  gx -= gx * pitch > room ? 2 : 1;
+  // the centre's fine coordinates (x on even lanes, y on odd ones of the state;
+  // one lane per state does both)
+  int Xc, Yc;
+  if (SPW > 0 && SPW <= 16) {
+    const bool odd = lane & 1;
+    const int c = fine_coord<MODE>(odd ? cy : cx, odd ? Sy : Sx, sm.rt, odd, a.act.rank_buckets);
+    const int o = __shfl_xor_sync(0xffffffffu, c, 1);
+    Xc = odd ? o : c;
+    Yc = odd ? c : o;
+  } else {
+    Xc = fine_coord<MODE>(cx, Sx, sm.rt, 0, a.act.rank_buckets);
+    Yc = fine_coord<MODE>(cy, Sy, sm.rt, 1, a.act.rank_buckets);
+  }
+  const int xmin = Xc - gx / 2, ymin = Yc - gy / 2;
+  const int centre = (Xc - xmin + 1) * pitch + Yc - ymin + 1;
+  const int rot = room < table ? (q * 32 / G - centre) & 31 : 0;
+  if (lane % per != 0) return;
+  StateSetup st;
+  st.win = make_int4(xmin, ymin, gx, pitch << 8 | rot);
+  st.layer = sample ? (int32_t)t : (sampled ? -2 : -1);
+  st.kind = ld.kind;
+  st.vbx = ld.vb.x;
+  st.vby = ld.vb.y;
+  const uint32_t sc = table > 0 ? 0x80000000u / (uint32_t)(table / 2) : 0u;   // 2^32 / table
+  st.base = smem_u32(tabs + (size_t)q * table);
+  st.bytes = 4u * (uint32_t)table;
+  st.aN = (uint32_t)(Sx * pitch) * sc;
+  st.aR = (uint32_t)pitch * (sc / 4);
+  st.c0 = ((uint32_t)(1 - xmin) * (uint32_t)pitch + (uint32_t)(1 - ymin + rot)) * sc - kFloorBits * (st.aN + (uint32_t)Sy * sc);
+  sm.st[q] = st;
 }
 
 // Counts state s again with the exact table g (the warp owning its slice;
 // tab: the state's table memory).  Rare: see the file comment.
-template <int KT, bool DENSE>
+template <int KT, int MODE>
 __device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables &rt, int64_t s, const FineGeo g,
                                            uint32_t *tab, int words) {
-  const int lane = threadIdx.x & 31, K = KT > 0 ? KT : a.K;
-  const RankTab rx = rank_tab(rt, 0), ry = rank_tab(rt, 1);
+  const int lane = threadIdx.x & 31, K = KT > 0 ? KT : a.K, B = a.act.rank_buckets;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
   const int64_t t = s / a.Nc, c = s % a.Nc;
   const float *vbar = static_cast<const float *>(a.vbar), *modes = static_cast<const float *>(a.modes);
   const float *Yt = static_cast<const float *>(a.Y) + (size_t)t * a.N * K;
+  const float vbx = vbar[2 * s], vby = vbar[2 * s + 1];
   float phx[kPhi<KT>], phy[kPhi<KT>];
 #pragma unroll
   for (int k = 0; k < kPhi<KT>; ++k) {
@@ -347,14 +445,20 @@ __device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables 
       phy[k] = ph.y;
     }
   }
-  const float vbx = vbar[2 * s], vby = vbar[2 * s + 1];
   for (int i = lane; i < words; i += 32) tab[i] = 0u;
   __syncwarp();
   for (int w = lane; w < a.N; w += 32) {
-    Row<KT> y;
+    float y[kPhi<KT>], wx = vbx, wy = vby;
     load_row<KT>(Yt + (size_t)w * K, K, y);
-    const float2 u = velocity_u<KT>(y, phx, phy, vbx, vby, K, a.lam);
-    const int X = fine_coord<DENSE>(u.x, Sx, rx) - g.xmin, Y = fine_coord<DENSE>(u.y, Sy, ry) - g.ymin;
+#pragma unroll
+    for (int k = 0; k < kPhi<KT>; ++k) {
+      if (KT > 0 || k < K) {
+        wx = fmaf(y[k], phx[k], wx);
+        wy = fmaf(y[k], phy[k], wy);
+      }
+    }
+    const int X = fine_coord<MODE>(fmaf(wx, a.lam, 0.5f), Sx, rt, 0, B) - g.xmin;
+    const int Y = fine_coord<MODE>(fmaf(wy, a.lam, 0.5f), Sy, rt, 1, B) - g.ymin;
     red_add_shared(smem_u32(tab) + 4u * (uint32_t)((X + 1) * g.pitch + Y + 1), 1u);
   }
   __syncwarp();
@@ -362,42 +466,47 @@ __device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables 
 
 // In-place 2-D inclusive prefix sums of a counted table (whole warp): P[i][j] =
 // sum of the counts X' < i, Y' < j.  Lanes take rows, then columns, four
-// cells loaded before they are stored (a lane's loads overlap).
-__device__ __forceinline__ void prefix_table(uint32_t *P, const FineGeo &g) {
+// cells loaded before they are stored (a lane's loads overlap).  A few lines
+// beyond a multiple of 32 (kScanLines) are scanned across the lanes instead:
+// another trip would have them on a few lanes (large workload: 33 x 31 cells
+// on average).
+constexpr int kScanLines = 8;
+__device__ __forceinline__ void prefix_lines(uint32_t *P, int lines, int line_step, int cells, int step) {
   const int lane = threadIdx.x & 31;
-  __syncwarp();
-  for (int i = 1 + lane; i <= g.gx; i += 32) {
-    uint32_t *p = P + i * g.pitch + 1;
+  const int tail = (lines & 31) <= kScanLines && cells <= 64 ? lines & 31 : 0, by_lane = lines - tail;
+  for (int i = 1 + lane; i <= by_lane; i += 32) {
+    uint32_t *p = P + i * line_step + step;
     uint32_t v = 0;
     int j = 0;
-    for (; j + 4 <= g.gy; j += 4, p += 4) {
-      uint32_t x0 = p[0], x1 = p[1], x2 = p[2], x3 = p[3];
+    for (; j + 4 <= cells; j += 4, p += 4 * step) {
+      uint32_t x0 = p[0], x1 = p[step], x2 = p[2 * step], x3 = p[3 * step];
       x0 += v; x1 += x0; x2 += x1; x3 += x2;
-      p[0] = x0; p[1] = x1; p[2] = x2; p[3] = x3;
+      p[0] = x0; p[step] = x1; p[2 * step] = x2; p[3 * step] = x3;
       v = x3;
     }
-    for (; j < g.gy; ++j, ++p) {
+    for (; j < cells; ++j, p += step) {
       v += *p;
       *p = v;
     }
   }
-  __syncwarp();
-  for (int j = 1 + lane; j <= g.gy; j += 32) {
-    uint32_t *p = P + g.pitch + j;
-    uint32_t v = 0;
-    int i = 0;
-    for (; i + 4 <= g.gx; i += 4, p += 4 * g.pitch) {
-      uint32_t x0 = p[0], x1 = p[g.pitch], x2 = p[2 * g.pitch], x3 = p[3 * g.pitch];
-      x0 += v; x1 += x0; x2 += x1; x3 += x2;
-      p[0] = x0; p[g.pitch] = x1; p[2 * g.pitch] = x2; p[3 * g.pitch] = x3;
-      v = x3;
+  for (int i = by_lane + 1; i <= lines; ++i) {   // lane l: cells 2 l and 2 l + 1 of the line
+    uint32_t *p = P + i * line_step + (2 * lane + 1) * step;
+    const uint32_t x0 = 2 * lane < cells ? p[0] : 0u, x1 = 2 * lane + 1 < cells ? p[step] : 0u;
+    uint32_t incl = x0 + x1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += x;
     }
-    for (; i < g.gx; ++i, p += g.pitch) {
-      v += *p;
-      *p = v;
-    }
+    if (2 * lane < cells) p[0] = incl - x1;
+    if (2 * lane + 1 < cells) p[step] = incl;
   }
   __syncwarp();
+}
+__device__ __forceinline__ void prefix_table(uint32_t *P, const FineGeo &g) {
+  __syncwarp();
+  prefix_lines(P, g.gx, g.pitch, g.gy, 1);
+  prefix_lines(P, g.gy, 1, g.gx, g.pitch);
 }
 
 // One row of a slice (lane l = row (q, a)) and its state's prefix table.
@@ -530,163 +639,211 @@ __device__ __noinline__ SliceTotals write_general(const BuildArgs &a, int64_t sl
 }
 
 // ---- the usual slice: every state's landings in a box of at most 8 x 8
-// cells, at most 32 offset bins per row, no row beyond row_cap ----
+// cells, at most 32 offset bins and kStage entries per row ----
 // The classes of a state's box come as bit masks (one coalesced read per state
-// instead of one byte per entry and scan); one scan finds the row's nonzero
-// in-domain bins as a mask, with two prefix lookups per bin (a bin's upper edge
-// is the next one's lower edge); the write then walks the set bits in step:
-// column k of all 32 rows, padding included, is one 128-byte store.
+// instead of one byte per entry and scan); one branch-free scan over the
+// row's bins, two prefix lookups per bin (a bin's upper edge is the next one's
+// lower edge; bins past the row's end come out empty), stages the entry words in
+// shared memory; once the columns are allocated, the rows are copied out in
+// step -- column k of all 32 rows, padding included, is one 128-byte store --
+// and R is formed from the staged counts.
 constexpr int kBox = 8;
 struct SmallRow {
-  uint32_t mask;      // nonzero in-domain bins, bit dj mbx + di
-  int mbx;            // bins per mask row; 0: the slice takes the general emit
-  int xoff, yoff;     // table coordinates of the first bin's lower edges
-  uint32_t tg0, tg1;  // targets in the state's box (bit cy 8 + cx)
-  int bit0;           // box bit of the row's first bin
+  bool small;         // else the slice takes the general emit
+  bool any_target;    // some state of the slice may land on a target
+};
+// The box's part: classes loaded (and turned into masks by ballots later).
+struct BoxCells {
+  int bx0, by0, mbx, mby;   // the state's box, most bins of a row per axis
+  uint8_t cc[2];            // SPW == 1: the lane's two cells
 };
 template <int SPW>
-__device__ __forceinline__ RowCount count_small(const BuildArgs &a, int64_t sl, const uint32_t *grid, const RowGeo &r,
-                                                SmallRow &sr) {
+__device__ __forceinline__ BoxCells box_cells(const BuildArgs &a, int64_t sl, const RowGeo &r, SmallRow &sr,
+                                              uint64_t &blk) {
   const int lane = threadIdx.x & 31;
-  const int spw = SPW > 0 ? SPW : a.spw, A_pad = 32 / spw, q_l = lane / A_pad, a_l = lane % A_pad;
+  const int spw = SPW > 0 ? SPW : a.spw, A_pad = 32 / spw, q_l = lane / A_pad;
   const int nx = a.nx, ny = a.ny;
   const int64_t Nc = a.Nc;
-  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
-  sr = SmallRow{};
+  sr = SmallRow{false, false};
+  blk = 0;
   // bounding box of the state's rows
   int bx0 = r.rows ? r.lox : INT_MAX, bx1 = r.rows ? r.hix : INT_MIN;
   int by0 = r.rows ? r.loy : INT_MAX, by1 = r.rows ? r.hiy : INT_MIN;
+  if (SPW == 1) {
+    bx0 = __reduce_min_sync(0xffffffffu, bx0);
+    bx1 = __reduce_max_sync(0xffffffffu, bx1);
+    by0 = __reduce_min_sync(0xffffffffu, by0);
+    by1 = __reduce_max_sync(0xffffffffu, by1);
+  } else {
 #pragma unroll
-  for (int off = A_pad >> 1; off >= 1; off >>= 1) {
-    bx0 = min(bx0, __shfl_xor_sync(0xffffffffu, bx0, off));
-    bx1 = max(bx1, __shfl_xor_sync(0xffffffffu, bx1, off));
-    by0 = min(by0, __shfl_xor_sync(0xffffffffu, by0, off));
-    by1 = max(by1, __shfl_xor_sync(0xffffffffu, by1, off));
+    for (int off = A_pad >> 1; off >= 1; off >>= 1) {
+      bx0 = min(bx0, __shfl_xor_sync(0xffffffffu, bx0, off));
+      bx1 = max(bx1, __shfl_xor_sync(0xffffffffu, bx1, off));
+      by0 = min(by0, __shfl_xor_sync(0xffffffffu, by0, off));
+      by1 = max(by1, __shfl_xor_sync(0xffffffffu, by1, off));
+    }
   }
   const int nbx = r.rows ? r.hix - r.lox + 1 : 0, nby = r.rows ? r.hiy - r.loy + 1 : 0;
-  const int mbx = __reduce_max_sync(0xffffffffu, nbx), mby = __reduce_max_sync(0xffffffffu, nby);
+  BoxCells bc{bx0, by0, (int)__reduce_max_sync(0xffffffffu, nbx), (int)__reduce_max_sync(0xffffffffu, nby), {0, 0}};
   const bool small = bx1 < bx0 || (bx1 - bx0 < kBox && by1 - by0 < kBox);
-  RowCount rc{0, r.kind == KIND_SINK ? (uint32_t)a.N : 0u};
-  if (!__all_sync(0xffffffffu, small) || mbx * mby > 32) return rc;
-  sr.mbx = max(mbx, 1);
-  // blocked (outside or obstacle) and target cells of the boxes
-  uint32_t blk0 = 0, blk1 = 0;
+  sr.small = __all_sync(0xffffffffu, small) && bc.mbx * bc.mby <= 32;
+  if (!sr.small) return bc;
   for (int q = 0; q < spw; ++q) {
     const int src = q * A_pad;
-    const int x0 = __shfl_sync(0xffffffffu, bx0, src), y0 = __shfl_sync(0xffffffffu, by0, src);
-    const int x1 = __shfl_sync(0xffffffffu, bx1, src), y1 = __shfl_sync(0xffffffffu, by1, src);
+    const int x0 = SPW == 1 ? bx0 : __shfl_sync(0xffffffffu, bx0, src), y0 = SPW == 1 ? by0 : __shfl_sync(0xffffffffu, by0, src);
+    const int x1 = SPW == 1 ? bx1 : __shfl_sync(0xffffffffu, bx1, src), y1 = SPW == 1 ? by1 : __shfl_sync(0xffffffffu, by1, src);
     if (x1 < x0) continue;
     const int64_t s = sl * spw + q, t = layer_of(s, Nc, a.nS), c = s - t * Nc;
     const int cj = (int)layer_of(c, nx, a.nS), ci = (int)(c - (int64_t)cj * nx);
     const uint8_t *cn = a.cls + (t + 1) * Nc;
+    uint8_t cc[2];
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       const int cx = lane % kBox, cy = lane / kBox + 4 * half;
       const int ip = ci + x0 + cx, jp = cj + y0 + cy;
-      uint8_t cc = CLS_OBSTACLE;
-      if (x0 + cx <= x1 && y0 + cy <= y1 && ip >= 0 && ip < nx && jp >= 0 && jp < ny) cc = cn[(int64_t)jp * nx + ip];
-      const uint32_t b = __ballot_sync(0xffffffffu, (cc & CLS_OBSTACLE) != 0);
-      const uint32_t g = __ballot_sync(0xffffffffu, (cc & CLS_TARGET) != 0);
-      if (q == q_l) {
-        if (half) { blk1 = b; sr.tg1 = g; }
-        else { blk0 = b; sr.tg0 = g; }
-      }
+      cc[half] = CLS_OBSTACLE;
+      if (x0 + cx <= x1 && y0 + cy <= y1 && ip >= 0 && ip < nx && jp >= 0 && jp < ny) cc[half] = cn[(int64_t)jp * nx + ip];
+    }
+    if (SPW == 1) {
+      bc.cc[0] = cc[0];
+      bc.cc[1] = cc[1];
+    } else {
+      const uint32_t b0 = __ballot_sync(0xffffffffu, (cc[0] & CLS_OBSTACLE) != 0);
+      const uint32_t b1 = __ballot_sync(0xffffffffu, (cc[1] & CLS_OBSTACLE) != 0);
+      sr.any_target |= __any_sync(0xffffffffu, ((cc[0] | cc[1]) & CLS_TARGET) != 0) != 0;
+      if (q == q_l) blk = (uint64_t)b1 << 32 | b0;
     }
   }
-  const FineGeo &gl = r.g;
+  return bc;
+}
+template <int SPW>
+__device__ __forceinline__ RowCount count_small(const BuildArgs &a, const RankTables &rt, const uint32_t *grid,
+                                                const RowGeo &r, const BoxCells &bc, uint64_t blk, uint32_t *stage,
+                                                SmallRow &sr) {
+  const int lane = threadIdx.x & 31;
+  const int A_pad = SPW > 0 ? 32 / SPW : 32 / a.spw, a_l = lane % A_pad;
+  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1, nx = a.nx, mbx = bc.mbx, mby = bc.mby;
+  RowCount rc{0, r.kind == KIND_SINK ? (uint32_t)a.N : 0u};
+  if (SPW == 1) {
+    const uint32_t b0 = __ballot_sync(0xffffffffu, (bc.cc[0] & CLS_OBSTACLE) != 0);
+    const uint32_t b1 = __ballot_sync(0xffffffffu, (bc.cc[1] & CLS_OBSTACLE) != 0);
+    sr.any_target = __any_sync(0xffffffffu, ((bc.cc[0] | bc.cc[1]) & CLS_TARGET) != 0) != 0;
+    blk = (uint64_t)b1 << 32 | b0;
+  }
+  const FineGeo &gl = r.g;   // (all zero in rows without a table: every bin comes out empty)
   const uint32_t *P = grid + gl.base;
+  int xoff = 0, y = 0, off = 0;
   if (r.rows) {
-    sr.xoff = (r.lox - a.act.cx[a_l] - 1) * Sx + a.act.lex[a_l] - gl.xmin;
-    sr.yoff = (r.loy - a.act.cy[a_l] - 1) * Sy + a.act.ley[a_l] - gl.ymin;
-    sr.bit0 = (r.loy - by0) * kBox + (r.lox - bx0);
+    xoff = (r.lox - rt.c[0][a_l] - 1) * Sx + rt.le[0][a_l] - gl.xmin;
+    y = (r.loy - rt.c[1][a_l] - 1) * Sy + rt.le[1][a_l] - gl.ymin;
+    blk >>= (r.loy - bc.by0) * kBox + (r.lox - bc.bx0);
+    off = r.loy * nx + r.lox;
   }
-  int j0 = 0, y = sr.yoff, bin = 0, row0 = sr.bit0;   // the first bins start at or below the table's edge
-  for (int dj = 0; dj < mby; ++dj, row0 += kBox) {
+  const int gx = r.rows ? gl.gx : 0, gy = r.rows ? gl.gy : 0;
+  const uint32_t *p0 = P;   // the first bins start at or below the table's edge
+  uint32_t *st = stage + lane;
+  for (int dj = 0; dj < mby; ++dj) {
     y += Sy;
-    const int j1 = min(y, gl.gy);
-    const bool vj = dj < nby;
-    uint32_t prev = 0;
-    int x = sr.xoff;
-    for (int di = 0; di < mbx; ++di, ++bin) {
-      x += Sx;
-      if (vj && di < nbx) {
-        const int row = min(x, gl.gx) * gl.pitch;   // x > 0: the first bin holds the state's extreme
-        const uint32_t v = P[row + j1] - P[row + j0], n = v - prev;
-        prev = v;
-        const int bit = row0 + di;
-        if (((bit & 32 ? blk1 : blk0) >> (bit & 31)) & 1u) rc.sink += n;
-        else if (n) sr.mask |= 1u << bin;
+    const uint32_t *p1 = P + min(y, gy);
+    uint32_t prev = 0, bits = (uint32_t)blk;
+    int x = xoff;
+    for (int d0 = 0; d0 < mbx; d0 += 4) {   // four bins' lookups in flight
+      uint32_t v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        x += Sx;
+        const int row = min(x, gx) * gl.pitch;   // x > 0: the first bin holds the state's extreme
+        v[i] = p1[row] - p0[row];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t n = v[i] - prev;
+        prev = v[i];
+        if (n) {
+          if (bits & 1u) {
+            rc.sink += n;
+          } else {
+            if (rc.e < kStage) *st = entry_word(off + d0 + i, n);
+            st += 32;
+            ++rc.e;
+          }
+        }
+        bits >>= 1;
       }
     }
-    j0 = j1;
+    p0 = p1;
+    blk >>= kBox;
+    off += nx;
   }
-  rc.e = __popc(sr.mask);
-  if (!__all_sync(0xffffffffu, rc.e <= a.row_cap)) sr.mbx = 0;
+  sr.small = __all_sync(0xffffffffu, rc.e <= min(a.row_cap, kStage));
   return rc;
 }
 template <int SPW, bool HYB>
-__device__ __forceinline__ SliceTotals write_small(const BuildArgs &a, int64_t sl, const uint32_t *grid,
-                                                   const RowGeo &r, const RowCount &rc, const SmallRow &sr,
-                                                   const SlicePlace &pl) {
+__device__ __forceinline__ SliceTotals write_small(const BuildArgs &a, const RankTables &rt, int64_t sl,
+                                                   const RowGeo &r, const RowCount &rc, const uint32_t *stage,
+                                                   const SmallRow &sr, const SlicePlace &pl) {
   const int lane = threadIdx.x & 31;
   const int spw = SPW > 0 ? SPW : a.spw, A_pad = 32 / spw, q_l = lane / A_pad, a_l = lane % A_pad;
-  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1, nx = a.nx;
   if constexpr (HYB) {
     if (lane == 0 && a.spill_off) a.spill_off[sl] = kNoSlice;
   }
-  const FineGeo &gl = r.g;
-  const uint32_t *P = grid + gl.base;
   const float *__restrict__ gbar = static_cast<const float *>(a.gbar);
-  const float *gn = gbar + sl * spw + q_l + a.Nc;   // the state's cell, one layer on
+  const int64_t next = sl * spw + q_l + a.Nc;   // the state's cell, one layer on
   const float invN = 1.0f / (float)a.N;
   const int n_obj = a.rw.n_obj;
-  float rb[3] = {0.f, 0.f, 0.f};   // the rewards' parts known from the row
+  // the rewards' parts known from the row; net energy's (the same for every
+  // objective slot that asks for it) is finished per cell
+  float rb[3] = {0.f, 0.f, 0.f}, rb_net = 0.f;
+  bool is_net[3] = {false, false, false};
   bool net = false;
   {
-    const float F = r.rows ? a.act.F[a_l] : 0.f;
-    const float g_s = r.rows && gbar ? gbar[sl * spw + q_l] : 0.f;
+    const float F = rt.F[a_l];
+    const float g_s = r.rows && gbar ? gbar[next - a.Nc] : 0.f;
 #pragma unroll
     for (int o = 0; o < 3; ++o) {
       if (o < n_obj) {
         rb[o] = reward_base32(a.rw, a.rw.objs[o], F, g_s);
-        net |= a.rw.objs[o] == MDP_OBJ_NET_ENERGY;
+        is_net[o] = a.rw.objs[o] == MDP_OBJ_NET_ENERGY;
+        if (is_net[o]) rb_net = rb[o];
+        net |= is_net[o];
       }
     }
   }
-  const int div = (65536 + sr.mbx - 1) / sr.mbx;   // bin / mbx for bin < 32
-  const bool any_target = __any_sync(0xffffffffu, (sr.tg0 | sr.tg1) != 0);
   uint32_t *dst = a.pool + pl.base * 32 + lane;
-  uint32_t mask = sr.mask;
+  const uint32_t *st = stage + lane;
   float R[3] = {0.f, 0.f, 0.f};
-  for (int k = 0; k < pl.W; ++k, dst += 32) {
-    uint32_t wd = 0u;
-    if (mask) {
-      const int bin = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const int dj = (bin * div) >> 16, di = bin - dj * sr.mbx;
-      const int x0 = sr.xoff + di * Sx, y0 = sr.yoff + dj * Sy;
-      const int r0 = max(x0, 0) * gl.pitch, r1 = min(x0 + Sx, gl.gx) * gl.pitch;
-      const int j0 = max(y0, 0), j1 = min(y0 + Sy, gl.gy);
-      const uint32_t n = P[r1 + j1] - P[r0 + j1] - P[r1 + j0] + P[r0 + j0];
-      const int off = (r.loy + dj) * nx + r.lox + di;
-      wd = entry_word(off, n);
-      const float p = (float)n * invN;
-      const float g_sp = net ? gn[off] : 0.f;
-      bool is_t = false;
-      if (any_target) {
-        const int bit = sr.bit0 + dj * kBox + di;
-        is_t = (((bit & 32 ? sr.tg1 : sr.tg0) >> (bit & 31)) & 1u) != 0;
-      }
+  for (int k0 = 0; k0 < pl.W; k0 += 4, dst += 128, st += 128) {   // four columns' loads in flight
+    uint32_t wd[4];
+    float g[4];
+    uint8_t cc[4];
 #pragma unroll
-      for (int o = 0; o < 3; ++o)
-        if (o < n_obj) R[o] = fmaf(p, reward_cell32(a.rw, a.rw.objs[o], rb[o], g_sp, is_t), R[o]);
+    for (int i = 0; i < 4; ++i) {
+      const bool in = k0 + i < rc.e;
+      wd[i] = in ? st[32 * i] : 0u;
+      const int off = (int)(int16_t)(wd[i] & 0xFFFFu);
+      g[i] = net && in ? gbar[next + off] : 0.f;
+      cc[i] = sr.any_target && in ? a.cls[next + off] : (uint8_t)0;
     }
-    if (pl.fits) *dst = wd;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (pl.fits && k0 + i < pl.W) dst[32 * i] = wd[i];
+      if (k0 + i < rc.e) {
+        const float p = (float)(wd[i] >> 16) * invN;
+        const float rn = reward_cell32(a.rw, MDP_OBJ_NET_ENERGY, rb_net, g[i], false);
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+          float x = is_net[o] ? rn : rb[o];
+          if (sr.any_target && (cc[i] & CLS_TARGET)) x = __fadd_rn(x, a.rw.f_r_term);
+          R[o] = fmaf(p, x, R[o]);
+        }
+      }
+    }
   }
   const int e = pl.fits ? rc.e : 0;
   return emit_tail(a, sl, r, e, e, rc.sink, pl, R);
 }
 
+// (set up by setup_slice, synchronised)
 // The CTA builds the slices [sl0, sl0 + NW) of model a (those below
 // a.slice_end), NW = blockDim.x / 32 with NW SPW <= 32 states; every thread
 // calls it, and the caller synchronises before sm is used again.  ext: the
@@ -698,9 +855,11 @@ __device__ __forceinline__ SliceTotals write_small(const BuildArgs &a, int64_t s
 // a row is counted in CNT_ROW_CAP and left empty.
 // next_group: thread 0's next work-queue index, published in sm.next[par]
 // (taken before the count, so its latency is hidden).
-template <int KT, int SPW, bool HYB, bool DENSE>
+// next_first(g): the first slice of queue index g if it belongs to the same
+// model and is to be set up here, else -1.
+template <int KT, int SPW, bool HYB, int MODE, class F>
 __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, GroupSmem &sm, float4 *ext,
-                                             uint32_t *tabs, int words, long long next_group, int par) {
+                                             uint32_t *tabs, int words, long long next_group, int par, F &&next_first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int spw = SPW > 0 ? SPW : a.spw;
   const int K = KT > 0 ? KT : a.K;
@@ -709,86 +868,180 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   const int N = a.N;
   const int64_t Nc = a.Nc;
   const float lam = a.lam;
-  const RankTab rx = rank_tab(sm.rt, 0), ry = rank_tab(sm.rt, 1);
+  const int B = a.act.rank_buckets;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
   const int swords = words / spw;   // a state's table (power of two)
-  const int G = NW * spw, lps = 32 / G;
+  const int G = NW * spw;           // states of the group (even, <= 32)
 
-  // ---- count: lane (q_t, i) state q_t of the group
+  // ---- count: lane (i, p) states 2 p and 2 p + 1 of the group, realizations
+  // i, i + step, ...; the two states are the halves of every packed operation
   {
-    const int q_t = lane / lps, w0 = warp * lps + lane % lps;
-    const int64_t s_t = sl0 * spw + q_t;
-    const bool sample = q_t < G && s_t < a.slice_end * spw && state_kind(a, s_t) == KIND_SAMPLE;
-    float mnx = INFINITY, mny = INFINITY, mxx = -INFINITY, mxy = -INFINITY;
-    if (sample && swords > 0) {
-      const int64_t t = layer_of(s_t, Nc, a.nS), c = s_t - t * Nc;
-      const float vbx = static_cast<const float *>(a.vbar)[2 * s_t], vby = static_cast<const float *>(a.vbar)[2 * s_t + 1];
-      const float *modes = static_cast<const float *>(a.modes);
-      float phx[kPhi<KT>], phy[kPhi<KT>];
+    const int np = G / 2, p_t = lane % np, sub = lane / np, subs = 32 / np;
+    const int w0 = warp * subs + sub, step = 64 / spw;   // step = NW subs
+    const float *modes = static_cast<const float *>(a.modes);
+    const int layer0 = sm.st[2 * p_t].layer, layer1 = sm.st[2 * p_t + 1].layer;
+    const bool split = layer0 >= 0 && layer1 >= 0 && layer0 != layer1;
+    float phx[2][kPhi<KT>], phy[2][kPhi<KT>];
+    {
+      // neighbouring cells of a layer, unless the pair is split
+      const int64_t s0 = sl0 * spw + 2 * p_t;
+      const int la = layer0 >= 0 ? layer0 : max(layer1, 0);
+      const float *m0 = modes + 2 * ((int64_t)la * (K - 1) * Nc + s0);   // (la K + k) Nc + (s0 - la Nc) at k = 0
+      const float *m1 = split ? modes + 2 * ((int64_t)layer1 * (K - 1) * Nc + s0 + 1) : m0 + 2;
 #pragma unroll
       for (int k = 0; k < kPhi<KT>; ++k) {
-        phx[k] = phy[k] = 0.f;
+        float2 p0 = make_float2(0.f, 0.f), p1 = p0;
         if (KT > 0 || k < K) {
-          const float2 ph = *reinterpret_cast<const float2 *>(modes + 2 * ((t * K + k) * Nc + c));
-          phx[k] = ph.x;
-          phy[k] = ph.y;
+          if (layer0 >= 0) p0 = __ldg(reinterpret_cast<const float2 *>(m0));
+          if (layer1 >= 0) p1 = __ldg(reinterpret_cast<const float2 *>(m1));
+          m0 += 2 * Nc;
+          m1 += 2 * Nc;
         }
+        phx[0][k] = p0.x;
+        phy[0][k] = p0.y;
+        phx[1][k] = p1.x;
+        phy[1][k] = p1.y;
       }
-      const FineGeo win = predict_window<KT, DENSE>(a, t, phx, phy, vbx, vby, K, Sx, Sy, sm.rt, swords);
-      if (threadIdx.x < 32 && lane % lps == 0) sm.win[q_t] = make_int4(win.xmin, win.ymin, win.gx, win.pitch);
-      // byte address of fine cell (X, Y): base | (4 ((X - xmin + 1) pitch + Y - ymin + 1) mod the table),
-      // X = (n - kFloorBits) S + r4 / 4, the constants folded modulo 2^32
-      const uint32_t base = smem_u32(tabs + (size_t)q_t * swords), mask = 4u * (uint32_t)(swords - 1);
-      const uint32_t cX = 4u * (uint32_t)(Sx * win.pitch), cY = 4u * (uint32_t)Sy, pitch = (uint32_t)win.pitch;
-      const uint32_t c0 = 4u * ((uint32_t)(1 - win.xmin) * pitch + (uint32_t)(1 - win.ymin)) - kFloorBits * (cX + cY);
-      auto count = [&](float2 u) {
-        const FloorRank fx = floor_rank<DENSE>(u.x, rx), fy = floor_rank<DENSE>(u.y, ry);
-        const uint32_t lin = fx.n * cX + fx.r4 * pitch + fy.n * cY + (fy.r4 + c0);
-        red_add_shared((lin & mask) | base, 1u);
+    }
+    const uint32_t sc = swords > 0 ? 0x80000000u / (uint32_t)(swords / 2) : 0u;
+    const uint32_t bN = (uint32_t)Sy * sc, bR = sc / 4;
+    const uint32_t t_base = smem_u32(&sm.rt.T[0][0]);
+    const float lut = int_float(smem_u32(&sm.rt.L[0][0])), bk = int_float((uint32_t)B);
+    const f2 lut2 = pack2(lut, lut), bk2 = pack2(bk, bk);
+    const f2 magic2 = pack2(kFloorMagic, kFloorMagic), nmagic2 = pack2(-kFloorMagic, -kFloorMagic);
+    // a pair of states on both sides of a layer boundary: the second on its own
+    // layer's coefficients, in a second round
+    const int rounds = __any_sync(0xffffffffu, split) ? 2 : 1;
+#pragma unroll 1
+    for (int round = 0; round < rounds; ++round) {
+      const int t = round == 0 && layer0 >= 0 ? layer0 : layer1;
+      const bool on0 = layer0 >= 0 && round == 0, on1 = layer1 >= 0 && (split ? round == 1 : round == 0);
+      const StateSetup *st = &sm.st[2 * p_t];
+      const uint32_t dummy = smem_u32(&sm.dummy[lane]);
+      const uint32_t base0 = on0 ? st[0].base : dummy, base1 = on1 ? st[1].base : dummy;
+      const uint32_t bytes0 = on0 ? st[0].bytes : 0u, bytes1 = on1 ? st[1].bytes : 0u;
+      const uint32_t aN0 = st[0].aN, aN1 = st[1].aN, aR0 = st[0].aR, aR1 = st[1].aR, c00 = st[0].c0, c01 = st[1].c0;
+      const float vbx0 = st[0].vbx, vby0 = st[0].vby, vbx1 = st[1].vbx, vby1 = st[1].vby;
+      float mnx0 = INFINITY, mny0 = INFINITY, mnx1 = INFINITY, mny1 = INFINITY;
+      float mxx0 = -INFINITY, mxy0 = -INFINITY, mxx1 = -INFINITY, mxy1 = -INFINITY;
+      float fmn = 2.f;
+      auto red = [&](uint32_t lin, uint32_t bytes, uint32_t base) {
+        uint32_t addr;
+        asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(addr) : "r"(lin), "r"(bytes), "r"(base));
+        red_add_shared(addr, 1u);
       };
-      const int step = 32 / spw;
+      // u of a realization for both states (FMA chain over ascending k, then u =
+      // fma(w, lam, 1/2): the CTA kernel's operations)
+      // (scalar: packed FMAs of the two states would need every coefficient
+      // twice in a register pair, two moves each)
+      auto velocity = [&](const float (&y)[kPhi<KT>], f2 &ux, f2 &uy) {
+        float wx[2] = {vbx0, vbx1}, wy[2] = {vby0, vby1};
+#pragma unroll
+        for (int k = 0; k < kPhi<KT>; ++k) {
+          if (KT > 0 || k < K) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              wx[h] = fmaf(y[k], phx[h][k], wx[h]);
+              wy[h] = fmaf(y[k], phy[h][k], wy[h]);
+            }
+          }
+        }
+        ux = pack2(fmaf(wx[0], lam, 0.5f), fmaf(wx[1], lam, 0.5f));
+        uy = pack2(fmaf(wy[0], lam, 0.5f), fmaf(wy[1], lam, 0.5f));
+      };
+      auto count = [&](f2 wx, f2 wy) {
+        const float2 ux = unpack2(wx), uy = unpack2(wy);
+        // floor by the magic sum; the fraction saturated to [0, 1] (NaN: 0), so
+        // that the lookups stay in their tables whatever u is
+        const f2 tx = add2_down(wx, magic2), ty = add2_down(wy, magic2);
+        const float2 nx = unpack2(add2(tx, nmagic2)), ny = unpack2(add2(ty, nmagic2));
+        const float fx0 = __saturatef(ux.x - nx.x), fx1 = __saturatef(ux.y - nx.y);
+        const float fy0 = __saturatef(uy.x - ny.x), fy1 = __saturatef(uy.y - ny.y);
+        if constexpr (MODE == 1) {
+          fmn = fminf(fmn, fminf(fx0, fy0));
+          fmn = fminf(fmn, fminf(fx1, fy1));
+        }
+        uint32_t rx0, rx1, ry0, ry1;
+        if constexpr (MODE <= 2) {
+          // lookup addresses L + floor(B f): integer arithmetic on float bits
+          const float2 lx = unpack2(fma2_down(pack2(fx0, fx1), bk2, lut2));
+          const float2 ly = unpack2(fma2_down(pack2(fy0, fy1), bk2, lut2));
+          rx0 = rank4<MODE, 0>(__float_as_uint(lx.x), fx0, t_base);
+          ry0 = rank4<MODE, 1>(__float_as_uint(ly.x), fy0, t_base);
+          rx1 = rank4<MODE, 0>(__float_as_uint(lx.y), fx1, t_base);
+          ry1 = rank4<MODE, 1>(__float_as_uint(ly.y), fy1, t_base);
+        } else {
+          auto r4 = [&](float f, int axis) {
+            int r = sm.rt.L[axis][__float_as_uint(__fmul_rd(f, bk))] >> 2;
+            while (sm.rt.T[axis][r + 1] <= f) ++r;
+            return 4u * (uint32_t)r;
+          };
+          rx0 = r4(fx0, 0); ry0 = r4(fy0, 1);
+          rx1 = r4(fx1, 0); ry1 = r4(fy1, 1);
+        }
+        const float2 bx = unpack2(tx), by = unpack2(ty);
+        red(__float_as_uint(bx.x) * aN0 + rx0 * aR0 + __float_as_uint(by.x) * bN + ry0 * bR + c00, bytes0, base0);
+        red(__float_as_uint(bx.y) * aN1 + rx1 * aR1 + __float_as_uint(by.y) * bN + ry1 * bR + c01, bytes1, base1);
+      };
+      auto extremes = [&](f2 ax, f2 ay, f2 bx, f2 by) {   // of two realizations
+        const float2 ux = unpack2(ax), uy = unpack2(ay), vx = unpack2(bx), vy = unpack2(by);
+        mnx0 = min_nan(mnx0, ux.x, vx.x); mxx0 = max_nan(mxx0, ux.x, vx.x);
+        mny0 = min_nan(mny0, uy.x, vy.x); mxy0 = max_nan(mxy0, uy.x, vy.x);
+        mnx1 = min_nan(mnx1, ux.y, vx.y); mxx1 = max_nan(mxx1, ux.y, vx.y);
+        mny1 = min_nan(mny1, uy.y, vy.y); mxy1 = max_nan(mxy1, uy.y, vy.y);
+      };
       const float *yp = static_cast<const float *>(a.Y) + ((size_t)t * N + w0) * K;
-      // two realizations per trip; their rows are loaded one trip ahead
-      int w = w0;
-      Row<KT> y0, y1;
-      if (w + step < N) {
+      int w = on0 || on1 ? w0 : N;
+#pragma unroll 1
+      for (; w + step < N; w += 2 * step, yp += (size_t)(2 * step) * K) {   // two realizations per trip
+        float y0[kPhi<KT>], y1[kPhi<KT>];
         load_row<KT>(yp, K, y0);
         load_row<KT>(yp + (size_t)step * K, K, y1);
+        f2 ax, ay, bx, by;
+        velocity(y0, ax, ay);
+        velocity(y1, bx, by);
+        extremes(ax, ay, bx, by);
+        count(ax, ay);
+        count(bx, by);
       }
-#pragma unroll 1
-      for (; w + step < N; w += 2 * step) {
-        yp += (size_t)(2 * step) * K;
-        const float2 u0 = velocity_u<KT>(y0, phx, phy, vbx, vby, K, lam);
-        const float2 u1 = velocity_u<KT>(y1, phx, phy, vbx, vby, K, lam);
-        if (w + 3 * step < N) {
-          load_row<KT>(yp, K, y0);
-          load_row<KT>(yp + (size_t)step * K, K, y1);
-        }
-        mnx = min_nan(mnx, u0.x, u1.x);
-        mny = min_nan(mny, u0.y, u1.y);
-        mxx = max_nan(mxx, u0.x, u1.x);
-        mxy = max_nan(mxy, u0.y, u1.y);
-        count(u0);
-        count(u1);
-      }
-      if (w < N) {   // the last realization of an odd number
+      if (w < N) {   // the last of an odd number
+        float y0[kPhi<KT>];
         load_row<KT>(yp, K, y0);
-        const float2 u0 = velocity_u<KT>(y0, phx, phy, vbx, vby, K, lam);
-        mnx = min_nan(mnx, u0.x);
-        mny = min_nan(mny, u0.y);
-        mxx = max_nan(mxx, u0.x, u0.x);
-        mxy = max_nan(mxy, u0.y, u0.y);
-        count(u0);
+        f2 ax, ay;
+        velocity(y0, ax, ay);
+        extremes(ax, ay, ax, ay);
+        count(ax, ay);
+      }
+      // (a trapped fraction of either state: both are counted again)
+      if (MODE == 1 && fmn < a.act.rank_trap) atomicOr(&sm.trap, ((on0 ? 1u : 0u) | (on1 ? 2u : 0u)) << (2 * p_t));
+      // extremes (min x, min y, -max x, -max y of both states) over the lanes of
+      // the pair: halved in number with every exchange while there are several
+      float v[8] = {mnx0, mny0, -mxx0, -mxy0, mnx1, mny1, -mxx1, -mxy1};
+      int first = 0, left = 8;
+#pragma unroll
+      for (int off = 16; off >= 4; off >>= 1) {
+        if (off < np) break;
+        const bool up = (lane & off) != 0;
+        constexpr int kHalf[3] = {4, 2, 1};
+        const int half = kHalf[off == 16 ? 0 : (off == 8 ? 1 : 2)];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (i < half) {
+            const float send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+            v[i] = min_nan(keep, __shfl_xor_sync(0xffffffffu, send, off));
+          }
+        }
+        first += up ? half : 0;
+        left = half;
+      }
+      if (np <= 2) v[0] = min_nan(v[0], __shfl_xor_sync(0xffffffffu, v[0], 2));
+      if (np > 2 || (lane & 2) == 0) {
+        float *ef = reinterpret_cast<float *>(ext + warp * G + 2 * p_t);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < left && (first + i < 4 ? on0 : on1)) ef[first + i] = v[i];
       }
     }
-    float nxx = -mxx, nxy = -mxy;
-    for (int off = lps >> 1; off >= 1; off >>= 1) {
-      mnx = min_nan(mnx, __shfl_xor_sync(0xffffffffu, mnx, off));
-      mny = min_nan(mny, __shfl_xor_sync(0xffffffffu, mny, off));
-      nxx = min_nan(nxx, __shfl_xor_sync(0xffffffffu, nxx, off));
-      nxy = min_nan(nxy, __shfl_xor_sync(0xffffffffu, nxy, off));
-    }
-    if (q_t < G && lane % lps == 0) ext[warp * G + q_t] = make_float4(mnx, mny, nxx, nxy);
     if (threadIdx.x == 0) sm.next[par] = next_group;
   }
   __syncthreads();
@@ -796,34 +1049,37 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   // ---- warp v: slice v, lane l = row (q_l, a_l)
   const int64_t sl = sl0 + warp;
   uint32_t *grid = tabs + (size_t)warp * words;
+  uint32_t *stage = tabs - (size_t)(NW - warp) * (32 * kStage);   // the stages precede the tables
   RowGeo r{};
   r.hix = r.hiy = -1;
   bool build = sl < a.slice_end, defer = false;
   if (build) {
     const int q_l = lane / (32 / spw), a_l = lane % (32 / spw);
-    r.kind = a_l < a.A ? state_kind(a, sl * spw + q_l) : (int)KIND_NONE;
+    r.kind = a_l < a.A ? sm.st[warp * spw + q_l].kind : (int)KIND_NONE;
     r.rows = r.kind == KIND_SAMPLE;
     for (int q = 0; q < spw; ++q) {
       const int qg = warp * spw + q;
       const int64_t s = sl * spw + q;
-      if (state_kind(a, s) != KIND_SAMPLE) continue;
+      const int layer = sm.st[qg].layer;
+      if (layer == -1) continue;   // not sampled
       // the state's extremes over all warps: lane (i, v) warp i's component v
       const int i = lane >> 2;
       float m = i < NW ? reinterpret_cast<const float *>(&ext[i * G + qg])[lane & 3] : INFINITY;
       m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
       m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 8));
       m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 16));
-      const float mnx = __shfl_sync(0xffffffffu, m, 0), mny = __shfl_sync(0xffffffffu, m, 1);
-      const float mxx = -__shfl_sync(0xffffffffu, m, 2), mxy = -__shfl_sync(0xffffffffu, m, 3);
-      // non-finite or far velocities: the CTA kernel's path
-      const bool tame = mnx > -kTame && mxx < kTame && mny > -kTame && mxy < kTame;
-      if (!tame || swords == 0) {
+      if (lane & 2) m = -m;
+      // no table, or non-finite or far velocities: the CTA kernel's path
+      if (layer < 0 || !__all_sync(0xffffffffu, m > -kTame && m < kTame)) {
         defer = true;
         continue;
       }
+      const int X = fine_coord<MODE>(m, lane & 1 ? Sy : Sx, sm.rt, lane & 1, B);
+      const float mnx = __shfl_sync(0xffffffffu, m, 0), mny = __shfl_sync(0xffffffffu, m, 1);
+      const float mxx = __shfl_sync(0xffffffffu, m, 2), mxy = __shfl_sync(0xffffffffu, m, 3);
       if (q == q_l && r.rows) {
-        const int cxa = a.act.cx[a_l], cya = a.act.cy[a_l];
-        const float thxa = a.act.thx[a_l], thya = a.act.thy[a_l];
+        const int cxa = sm.rt.c[0][a_l], cya = sm.rt.c[1][a_l];
+        const float thxa = sm.rt.th[0][a_l], thya = sm.rt.th[1][a_l];
         r.lox = land_offset(mnx, cxa, thxa); r.hix = land_offset(mxx, cxa, thxa);
         r.loy = land_offset(mny, cya, thya); r.hiy = land_offset(mxy, cya, thya);
         if (r.lox < -a.h || r.hix > a.h || r.loy < -a.h || r.hiy > a.h) {   // sub-grid overflow
@@ -833,15 +1089,15 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
       }
       // the exact table inside the window (its pitch, its own origin)
       FineGeo g;
-      g.xmin = fine_coord<DENSE>(mnx, Sx, rx);
-      g.ymin = fine_coord<DENSE>(mny, Sy, ry);
-      g.gx = fine_coord<DENSE>(mxx, Sx, rx) - g.xmin + 1;
-      g.gy = fine_coord<DENSE>(mxy, Sy, ry) - g.ymin + 1;
-      const int4 win = sm.win[qg];
-      g.pitch = win.w;
-      g.base = q * swords + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
-      if (g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + win.w) {
-        // outside the predicted window: the exact table, if it fits
+      g.xmin = __shfl_sync(0xffffffffu, X, 0);
+      g.ymin = __shfl_sync(0xffffffffu, X, 1);
+      g.gx = __shfl_sync(0xffffffffu, X, 2) - g.xmin + 1;
+      g.gy = __shfl_sync(0xffffffffu, X, 3) - g.ymin + 1;
+      const int4 win = sm.st[qg].win;
+      g.pitch = win.w >> 8;
+      g.base = q * swords + (win.w & 255) + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
+      if ((MODE == 1 && ((sm.trap >> qg) & 1u)) || g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + g.pitch) {
+        // outside the predicted window (or a trapped fraction): the exact table, if it fits
         const long long pitch = ((long long)g.gy + 1) | 1;
         if (((long long)g.gx + 1) * pitch > (long long)swords) {
           defer = true;
@@ -849,10 +1105,10 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         }
         g.pitch = (int)pitch;
         g.base = q * swords;
-        if (!defer) recount_state<KT, DENSE>(a, sm.rt, s, g, grid + g.base, swords);
+        if (!defer) recount_state<KT, MODE>(a, sm.rt, s, g, grid + g.base, swords);
       }
       if (q == q_l) r.g = g;
-      if (!defer) prefix_table(grid + g.base, g);
+      if (SPW != 1 && !defer) prefix_table(grid + g.base, g);
     }
     if (defer) {   // too wide (or not finite): the CTA kernel builds the slice
       build = false;
@@ -866,8 +1122,12 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   SmallRow sr{};
   SlicePlace pl{};
   if (build) {
-    rc = count_small<SPW>(a, sl, grid, r, sr);
-    if (!sr.mbx) {
+    // (the box's classes are on their way while the table is summed)
+    uint64_t blk;
+    const BoxCells bc = box_cells<SPW>(a, sl, r, sr, blk);
+    if (SPW == 1 && sm.st[warp].layer >= 0) prefix_table(grid + r.g.base, r.g);
+    if (sr.small) rc = count_small<SPW>(a, sm.rt, grid, r, bc, blk, stage, sr);
+    if (!sr.small) {
       const uint32_t sink = r.kind == KIND_SINK ? (uint32_t)N : 0u;
       rc = count_general<HYB>(a, sl, grid, r);
       rc.sink += sink;
@@ -883,23 +1143,26 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
     const int w = lane < NW ? sm.cols[lane] : 0;
     int incl = w;
 #pragma unroll
-    for (int d = 1; d < kGroupWarps; d <<= 1) {
+    for (int d = 1; d < 8; d <<= 1) {
       const int x = __shfl_up_sync(0xffffffffu, incl, d);
       if (lane >= d) incl += x;
     }
-    const int total = __shfl_sync(0xffffffffu, incl, kGroupWarps - 1);
+    const int total = __shfl_sync(0xffffffffu, incl, 7);
     unsigned long long base = 0;
     if (lane == 0 && total > 0) base = atomicAdd(&a.cnt[CNT_POOL_COLS], (unsigned long long)total);
     base = __shfl_sync(0xffffffffu, base, 0);
     if (lane < NW) sm.base[lane] = base + (unsigned long long)(incl - w);
+    if (lane == 0) sm.trap = 0u;   // read above, set again by the next group
   }
   __syncthreads();
+  const long long g1 = sm.next[par];
+  const SetupLoads ld = next_first(g1) >= 0 ? setup_load<SPW>(a, next_first(g1)) : SetupLoads{};
   if (build) {
     pl.base = sm.base[warp];
     pl.fits = pl.W == 0 || pl.base + (unsigned long long)pl.W <= a.pool_cap_cols;
     if (!pl.fits && lane == 0) atomicAdd(&a.cnt[CNT_POOL_FULL], 1ULL);
-    const SliceTotals tot = sr.mbx ? write_small<SPW, HYB>(a, sl, grid, r, rc, sr, pl)
-                                   : write_general<HYB>(a, sl, grid, r, rc, pl);
+    const SliceTotals tot = sr.small ? write_small<SPW, HYB>(a, sm.rt, sl, r, rc, stage, sr, pl)
+                                     : write_general<HYB>(a, sl, grid, r, rc, pl);
     const int sampled = __popc(__ballot_sync(0xffffffffu, r.rows));
     if (lane == 0) {
       WarpAcc &acc = sm.acc[warp];
@@ -913,6 +1176,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   __syncwarp();
   uint4 *p = reinterpret_cast<uint4 *>(grid);
   for (int i = lane; i < words / 4; i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (next_first(g1) >= 0) setup_slice<SPW, MODE>(a, sm, next_first(g1), ld, tabs, words);
 }
 
 }  // namespace mdpgb

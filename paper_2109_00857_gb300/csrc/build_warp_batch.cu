@@ -4,101 +4,134 @@
 
 namespace mdpgb {
 
-// Many models: persistent CTAs pull global group indices; g -> (model m,
-// group g - prefix[m]) by binary search over the prefix sums.  The models of
-// one launch share the mode count (KT > 0; KT == 0: runtime, up to
-// kMaxModes), the states per slice (SPW; 0: runtime, but one value per launch)
-// and the density of their thresholds.
-struct BatchSmem {
-  GroupSmem g;
-  BuildArgs a;   // the current model's arguments
-};
+// The current model's arguments in shared memory: BuildArgs up to the action
+// constants that the group build reads.  The whole of it would leave four CTAs
+// an SM instead of five (16 uneven models: 38.3 ms of kernels; 42 ms so).
+static_assert(sizeof(BuildArgs) % 16 == 0, "an array of them is copied as 16-byte vectors");
+constexpr uint32_t kArgsBytes = (uint32_t)((offsetof(BuildArgs, act) + offsetof(ActionTable, dxl) + 15) & ~(size_t)15);
 
-template <int KT, int SPW, bool DENSE>
-__global__ void __launch_bounds__(32 * kGroupWarps, KT == 0 ? 2 : 3)
+// Many models: persistent CTAs pull global group indices, a few consecutive
+// ones at a time; g -> (model m, group g - prefix[m]), by binary search over
+// the prefix sums when g leaves the current model.  The models of one launch
+// share the mode count (KT > 0; KT == 0: runtime, up to kMaxModes), the states
+// per slice (SPW; 0: runtime, but one value per launch) and the rank lookup's
+// mode.
+template <int KT, int SPW, int MODE>
+__global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>)
     build_group_batch_kernel(const BuildArgs *__restrict__ items, const int64_t *__restrict__ prefix, int n,
                              unsigned long long *work, int words, int spw) {
   extern __shared__ __align__(16) unsigned char gsm[];
-  BatchSmem &sm = *reinterpret_cast<BatchSmem *>(gsm);
-  float4 *ext = reinterpret_cast<float4 *>(gsm + ((sizeof(BatchSmem) + 15) & ~(size_t)15));
-  uint32_t *tabs = table_memory(gsm, sizeof(BatchSmem), &words, SPW > 0 ? SPW : spw);
-  const int NW = blockDim.x >> 5;
+  const BuildArgs &a = *reinterpret_cast<const BuildArgs *>(gsm);
+  GroupSmem &sm = *reinterpret_cast<GroupSmem *>(gsm + kArgsBytes);
+  const int NW = blockDim.x >> 5, states = SPW > 0 ? SPW : spw;
+  float4 *ext = reinterpret_cast<float4 *>(gsm + group_ext_offset(kArgsBytes, states, NW));
+  uint32_t *tabs = reinterpret_cast<uint32_t *>(gsm + group_head_bytes(kArgsBytes, states, NW));
   const int64_t total = prefix[n];
+  // groups per queue grab (see launch_g)
+  const unsigned long long chunk = (unsigned long long)max((int64_t)1, min((int64_t)8, total / (16 * (int64_t)gridDim.x)));
   clear_tables(tabs, words);
-  warp_clear(sm.g);
-  if (threadIdx.x == 0) sm.g.next[0] = (long long)atomicAdd(work, 1ULL);
+  warp_clear(sm);
+  if (threadIdx.x == 0) {
+    sm.next[0] = (long long)atomicAdd(work, chunk);
+    sm.trap = 0u;
+  }
   __syncthreads();
-  int cur = -1;
-  for (int par = 0;; par ^= 1) {
-    const long long g = sm.g.next[par];
-    if (g >= total) break;
-    long long next = total;
-    if (threadIdx.x == 0) next = (long long)atomicAdd(work, 1ULL);
-    int lo = 0, hi = n - 1;   // last m with prefix[m] <= g
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (prefix[mid] <= g) lo = mid; else hi = mid - 1;
+  // the model of group g: last m with prefix[m] <= g; [lo, hi) the current one's groups
+  auto model_of = [&](long long g) {
+    int x = 0, y = n - 1;
+    while (x < y) {
+      const int mid = (x + y + 1) >> 1;
+      if (prefix[mid] <= g) x = mid; else y = mid - 1;
     }
-    if (lo != cur) {
-      if (cur >= 0) warp_flush(items[cur], sm.g);
-      cur = lo;
-      static_assert(sizeof(BuildArgs) % 8 == 0, "copied as 64-bit words");
-      const uint64_t *src = reinterpret_cast<const uint64_t *>(items + lo);
-      uint64_t *dst = reinterpret_cast<uint64_t *>(&sm.a);
-      for (int i = threadIdx.x; i < (int)(sizeof(BuildArgs) / 8); i += blockDim.x) dst[i] = src[i];
-      load_rank_tables(items[lo], sm.g.rt);
+    return x;
+  };
+  int cur = -1, left = (int)chunk - 1;   // left: groups of the last grab still to do (thread 0)
+  int64_t lo = 0, hi = 0;
+  for (int par = 0;; par ^= 1) {
+    const long long g = sm.next[par];
+    if (g >= total) break;
+    if (g < lo || g >= hi) {
+      if (cur >= 0) warp_flush(items[cur], sm);
+      cur = model_of(g);
+      lo = prefix[cur];
+      hi = prefix[cur + 1];
+      const uint4 *src = reinterpret_cast<const uint4 *>(items + cur);
+      uint4 *dst = reinterpret_cast<uint4 *>(gsm);
+      for (int i = threadIdx.x; i < (int)(kArgsBytes / 16); i += blockDim.x) dst[i] = src[i];
+      load_rank_tables(items[cur], sm.rt);
+      __syncthreads();
+      setup_slice<SPW, MODE>(a, sm, (g - lo) * NW, setup_load<SPW>(a, (g - lo) * NW), tabs, words);
       __syncthreads();
     }
-    group_slices<KT, SPW, false, DENSE>(sm.a, (g - prefix[lo]) * NW, sm.g, ext, tabs, words, next, par ^ 1);
+    long long next = total;
+    if (threadIdx.x == 0) {
+      if (left > 0) {
+        next = g + 1;
+        --left;
+      } else {
+        next = (long long)atomicAdd(work, chunk);
+        left = (int)chunk - 1;
+      }
+    }
+    group_slices<KT, SPW, false, MODE>(a, (g - lo) * NW, sm, ext, tabs, words, next, par ^ 1,
+                                       [&](long long g1) {   // (another model's group is set up after the switch)
+                                         return g1 >= lo && g1 < hi ? (int64_t)(g1 - lo) * NW : (int64_t)-1;
+                                       });
     __syncthreads();
   }
-  if (cur >= 0) warp_flush(items[cur], sm.g);
+  if (cur >= 0) warp_flush(items[cur], sm);
 }
 
-template <int KT, int SPW, bool DENSE = false>
+template <int KT, int SPW, int MODE>
 static cudaError_t launch_gb(const BuildArgs *items_d, const int64_t *prefix_d, int n, unsigned long long *work_d,
                              int cap, int spw, cudaStream_t st) {
   const int nw = batch_group_slices(spw), words = table_words(cap, spw);
-  int reserved = 0;
-  cudaError_t e = reserved_smem(&reserved);
-  if (e != cudaSuccess) return e;
-  const size_t smem = group_smem_bytes(sizeof(BatchSmem), reserved, cap, spw, nw);
-  e = allow_max_smem((const void *)build_group_batch_kernel<KT, SPW, DENSE>);
+  const size_t smem = group_smem_bytes(kArgsBytes, cap, spw, nw);
+  cudaError_t e = allow_max_smem((const void *)build_group_batch_kernel<KT, SPW, MODE>);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_group_batch_kernel<KT, SPW, DENSE>, nw * 32, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_group_batch_kernel<KT, SPW, MODE>, nw * 32, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  build_group_batch_kernel<KT, SPW, DENSE>
+  build_group_batch_kernel<KT, SPW, MODE>
       <<<num_sms() * per_sm, nw * 32, smem, st>>>(items_d, prefix_d, n, work_d, words, spw);
   return cudaGetLastError();
 }
 
-template <int SPW>
+template <int SPW, int MODE>
 static cudaError_t launch_gb_k(const BuildArgs *items_d, const int64_t *prefix_d, int n, unsigned long long *work_d,
                                int cap_bins, int K, int spw, cudaStream_t st) {
   switch (K) {
-    case 1: return launch_gb<1, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 2: return launch_gb<2, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 3: return launch_gb<3, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 4: return launch_gb<4, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 5: return launch_gb<5, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 6: return launch_gb<6, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 7: return launch_gb<7, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    case 8: return launch_gb<8, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-    default: return launch_gb<0, SPW>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 1: return launch_gb<1, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 2: return launch_gb<2, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 3: return launch_gb<3, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 4: return launch_gb<4, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 5: return launch_gb<5, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 6: return launch_gb<6, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 7: return launch_gb<7, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    case 8: return launch_gb<8, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    default: return MODE == 1 ? launch_gb<0, 0, 1>(items_d, prefix_d, n, work_d, cap_bins, spw, st)
+                              : launch_gb<0, 0, 2>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
   }
 }
 
 int batch_group_slices(int spw) { return group_warps(kGroupWarps, spw); }
 
+// (the single-model kernel's instantiations)
 cudaError_t launch_build_warp_batch(const BuildArgs *items_d, const int64_t *prefix_d, int n,
-                                    unsigned long long *work_d, int cap_bins, int K, int spw, bool dense,
+                                    unsigned long long *work_d, int cap_bins, int K, int spw, int rank_mode,
                                     cudaStream_t st) {
-  if (dense) return launch_gb<0, 0, true>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
-  if (spw == 1) return launch_gb_k<1>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
-  if (spw == 2) return launch_gb_k<2>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
-  return launch_gb_k<0>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+  if (rank_mode == 1) {
+    if (spw == 1) return launch_gb_k<1, 1>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+    if (spw == 2) return launch_gb_k<2, 1>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+    return launch_gb_k<0, 1>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+  }
+  if (rank_mode == 2) {
+    if (spw == 1) return launch_gb_k<1, 2>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+    if (spw == 2) return launch_gb_k<2, 2>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
+    return launch_gb<0, 0, 2>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+  }
+  return launch_gb<0, 0, 3>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
 }
 
 }  // namespace mdpgb

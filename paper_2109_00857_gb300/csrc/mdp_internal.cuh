@@ -64,32 +64,38 @@ enum {
 // row.  Slices without a spill block hold kNoSlice in spill_off.
 constexpr int kSpillHdr = 33;
 
-constexpr int kRankBuckets = 128;
+constexpr int kMaxBuckets = 512;   // of the rank lookup (128 suffice for evenly spread headings)
 
+// The members before dxl are what the group build reads per slice (the batched
+// kernel keeps them in shared memory).
 struct ActionTable {
-  float dxl[kMaxActions];   // F cos(theta) * dt/dx   (FP32 kinematics, grid units)
-  float dyl[kMaxActions];
-  float F[kMaxActions];
-  double dx64[kMaxActions];  // F cos(theta), F sin(theta), F in FP64 (check mode)
-  double dy64[kMaxActions];
-  double F64[kMaxActions];
   // FP32 landing offsets: floor(u + d) of the exact sum of the floats u and
   // d = floor(u) + c + [u - floor(u) >= th] with c = floor(d) and th the
   // smallest float >= 1 - (d - c) (2 when d is an integer: never reached).
-  int32_t cx[kMaxActions], cy[kMaxActions];
-  float thx[kMaxActions], thy[kMaxActions];
-  // The distinct thresholds below 2, ascending, padded with 2 (Dx, Dy of
-  // them), and each action's rank le = #{T <= th}: a sample's fractional
-  // rank rho = #{T <= u - floor(u)} decides [u - floor(u) >= th] = [rho >= le]
-  // for every action at once.
-  float Tx[kMaxActions + 2], Ty[kMaxActions + 2];
-  int32_t lex[kMaxActions], ley[kMaxActions];
+  // The distinct thresholds below 2, ascending, are T (Dx, Dy of them), and
+  // each action's rank le = #{T <= th}: a sample's fractional rank
+  // rho = #{T <= u - floor(u)} decides [u - floor(u) >= th] = [rho >= le] for
+  // every action at once.
   int32_t Dx, Dy;
-  // Rank lookup over kRankBuckets equal buckets of [0, 1]: entry b =
-  // #{T in buckets < b}, bucket(v) = min(floor(128 v), 127) (exact: 128 is a
-  // power of two); Mx, My = most thresholds in one bucket.
-  uint8_t Lx[kRankBuckets], Ly[kRankBuckets];
-  int32_t Mx, My;
+  // Rank lookup of the group kernel over rank_buckets equal buckets of [0, 1]
+  // (bucket floor(B f); f = 1 has its own).  Mode 1: every bucket but the first
+  // holds at most one threshold, so rank = (thresholds up to and including
+  // f's bucket) - [f < the last of them], right for every f >= rank_trap (the
+  // first bucket may hold several thresholds below 2^-24, the displacements
+  // that are zero up to rounding).  Mode 2: at most two per bucket, two
+  // comparisons after the thresholds below it.  Mode 3: a scan.
+  int32_t rank_mode, rank_buckets;
+  float rank_trap;
+  int32_t cx[kMaxActions], cy[kMaxActions];
+  int32_t lex[kMaxActions], ley[kMaxActions];
+  float F[kMaxActions];
+  // displacements F cos(theta) dt/dx, F sin(theta) dt/dx (FP32 kinematics, grid units)
+  float dxl[kMaxActions], dyl[kMaxActions];
+  float thx[kMaxActions], thy[kMaxActions];
+  float Tx[kMaxActions + 2], Ty[kMaxActions + 2];   // padded with 2
+  double dx64[kMaxActions];  // F cos(theta), F sin(theta), F in FP64 (check mode)
+  double dy64[kMaxActions];
+  double F64[kMaxActions];
 };
 
 struct RewardParams {
@@ -109,13 +115,12 @@ struct RewardParams {
 };
 
 // Everything the build kernels need, passed by value.
-struct BuildArgs {
+struct alignas(16) BuildArgs {
   int32_t nx, ny, nt, K, N, A, A_pad, spw, L, h, nbins, row_cap;
   int64_t Nc, nS, n_slices, rows_pad;
   float lam;                 // dt / dx
   const void *vbar, *modes, *Y, *gbar;
   const uint8_t *cls;
-  ActionTable act;
   RewardParams rw;
   uint32_t *pool;
   uint64_t pool_cap_cols;
@@ -142,6 +147,7 @@ struct BuildArgs {
   // model, so CTAs retire all along the build and the block scheduler can
   // place higher-priority work (another request's launches) between them
   int32_t slices_per_warp;
+  ActionTable act;           // last: see ActionTable
 };
 
 struct mdp_model_impl;
@@ -307,12 +313,12 @@ cudaError_t launch_bellman_batch(const BatchSolveItem *items_d, int n, BatchCta 
 cudaError_t launch_finalize_batch(const BatchSolveItem *items_d, int n, int layered, cudaStream_t st);
 // batched build (FP32): one persistent launch over the groups of slices of n
 // models that share the mode count K, the states per slice spw and the
-// density of their thresholds (prefix[m] = first group of model m in the
+// rank lookup's mode (prefix[m] = first group of model m in the
 // launch, prefix[n] = total; a group is batch_group_slices(spw) slices); then
 // the full-window CTA kernel over every model's deferred slices
 int batch_group_slices(int spw);
 cudaError_t launch_build_warp_batch(const BuildArgs *items_d, const int64_t *prefix_d, int n,
-                                    unsigned long long *work_d, int cap_bins, int K, int spw, bool dense,
+                                    unsigned long long *work_d, int cap_bins, int K, int spw, int rank_mode,
                                     cudaStream_t st);
 cudaError_t launch_build_fp32_batch(const BuildArgs *items_d, int n, size_t smem, int threads,
                                     cudaStream_t st);
