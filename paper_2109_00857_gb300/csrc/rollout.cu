@@ -16,6 +16,8 @@
 
 namespace mdpgb {
 
+constexpr int kRollThreads = 128;
+
 struct RolloutArgs {
   int32_t nx, ny, nt, K, N, n_obj, n_starts;
   int64_t Nc, nS;
@@ -32,85 +34,176 @@ struct RolloutArgs {
   int8_t *status;          // [n_starts][N]
 };
 
-template <typename RT>
-__global__ void __launch_bounds__(256) rollout_kernel(RolloutArgs a) {
+// Loads of read-only data that stay where they are written: as plain loads, the
+// compiler moves each behind the branches before its first use.
+__device__ __forceinline__ float load_now(const float *p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double load_now(const double *p) {
+  double v;
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int load_now(const uint8_t *p) {
+  int v;
+  asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int load_now(const int16_t *p) {
+  int v;
+  asm volatile("ld.global.nc.s16 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+// Two fields of a vector cell: one 8-byte load where the caller's array allows it.
+template <typename RT, bool VEC>
+__device__ __forceinline__ void load_pair(const RT *p, RT &x, RT &y) {
+  if constexpr (VEC && sizeof(RT) == 4) {
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "l"(p));
+  } else {
+    x = load_now(p);
+    y = load_now(p + 1);
+  }
+}
+// One realization's coefficients (VEC: rows of whole 8- or 16-byte pieces are
+// aligned to them).
+template <int KT, bool VEC>
+__device__ __forceinline__ void load_coeffs(const float *p, float (&y)[KT]) {
+  if constexpr (VEC && KT % 4 == 0) {
+#pragma unroll
+    for (int k = 0; k < KT; k += 4)
+      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(y[k]), "=f"(y[k + 1]), "=f"(y[k + 2]), "=f"(y[k + 3]) : "l"(p + k));
+  } else if constexpr (VEC && KT % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < KT; k += 2) load_pair<float, true>(p + k, y[k], y[k + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < KT; ++k) y[k] = load_now(p + k);
+  }
+}
+
+// A step waits for memory, so everything that the state (t, cell) decides --
+// its kind, its action, its velocity, the reward of the move that led to it --
+// is loaded together at the top of the step, before any of it is looked at: one
+// latency a step.  (Branch by branch it was five, and two loads per vector: 64
+// starts, 5000 realizations of eight modes, 120 layers: 841 us, 440 us
+// so, two thirds of the LSU rate that the gathers allow.)
+// KT > 0: FP32, exactly KT modes, held in registers; KT == 0: any.
+template <typename RT, int KT, bool VEC>
+__global__ void __launch_bounds__(kRollThreads) rollout_kernel(const __grid_constant__ RolloutArgs a) {
+  // the actions' landing constants (FP32): a warp's lanes take several at once
+  __shared__ int4 land[sizeof(RT) == 4 ? kMaxActions : 1];   // cx, cy, thx, thy
+  __shared__ float thrust[sizeof(RT) == 4 ? kMaxActions : 1];
+  if constexpr (sizeof(RT) == 4) {
+    for (int k = threadIdx.x; k < kMaxActions; k += blockDim.x) {
+      land[k] = make_int4(a.act.cx[k], a.act.cy[k], __float_as_int(a.act.thx[k]), __float_as_int(a.act.thy[k]));
+      thrust[k] = a.act.F[k];
+    }
+    __syncthreads();
+  }
   const int64_t path = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (path >= (int64_t)a.n_starts * a.N) return;
   const int q = (int)(path / a.N), w = (int)(path % a.N);
+  const int K = KT > 0 ? KT : a.K, nx = a.nx, ny = a.ny, nt = a.nt, n_obj = a.n_obj;
   const int64_t Nc = a.Nc;
   const RT *vbar = static_cast<const RT *>(a.vbar);
   const RT *modes = static_cast<const RT *>(a.modes);
-  const RT *Y = static_cast<const RT *>(a.Y);
   const RT *gbar = static_cast<const RT *>(a.gbar);
+  const RT *yw = static_cast<const RT *>(a.Y) + (int64_t)w * K;   // row of (t, w)
   RT ret[3] = {0, 0, 0};
   int i = a.starts[2 * q], j = a.starts[2 * q + 1];
-  int n = 0, st = 1;
-  for (int t = 0; t < a.nt; ++t) {
-    const int64_t c = (int64_t)j * a.nx + i, s = (int64_t)t * Nc + c;
-    if (a.target[c]) {   // arrived: terminal states are absorbing
+  int n = 0, st = 1, act = -1;   // act: the move that led here
+  RT g_s = 0;
+  for (int t = 0;; ++t, yw += (int64_t)a.N * K) {
+    const int64_t c = (int64_t)j * nx + i, s = t * Nc + c;
+    const int obst = load_now(a.obstacle + s);
+    const bool is_t = load_now(a.target + c) != 0;
+    const int next_act = load_now(a.policy + s);
+    const RT g_here = gbar ? load_now(gbar + s) : (RT)0;
+    RT vx, vy;
+    load_pair<RT, VEC>(vbar + 2 * s, vx, vy);
+    const RT *ph = modes + 2 * ((int64_t)t * K * Nc + c);
+    if constexpr (KT > 0) {
+      // the FP32 build's velocity: FMA chain over ascending k
+      float y[KT], px[KT], py[KT];
+      load_coeffs<KT, VEC>(yw, y);
+#pragma unroll
+      for (int k = 0; k < KT; ++k) load_pair<float, VEC>(ph + 2 * k * Nc, px[k], py[k]);
+#pragma unroll
+      for (int k = 0; k < KT; ++k) {
+        vx = fmaf(y[k], px[k], vx);
+        vy = fmaf(y[k], py[k], vy);
+      }
+    }
+    if (t > 0) {   // the move that led here: into the sink, or its reward
+      if (obst) {
+#pragma unroll
+        for (int o = 0; o < 3; ++o) ret[o] += (RT)a.rw.r_out;
+        break;
+      }
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        if (o >= n_obj) break;
+        if constexpr (sizeof(RT) == 4)
+          ret[o] += step_reward32(a.rw, a.rw.objs[o], thrust[act], g_s, g_here, is_t);
+        else
+          ret[o] = __dadd_rn(ret[o], step_reward64(a.rw, a.rw.objs[o], a.act.F64[act], g_s, g_here, is_t));
+      }
+    }
+    if (is_t) {   // arrived: terminal states are absorbing
       st = 0;
       break;
     }
-    const int act = a.policy[s];
+    act = next_act;
+    g_s = g_here;
     ++n;
-    if (a.obstacle[s] || t == a.nt - 1 || act < 0) {   // every move ends in the sink
-      for (int o = 0; o < a.n_obj; ++o) ret[o] += (RT)a.rw.r_out;
-      break;
-    }
-    const RT *yw = Y + ((int64_t)t * a.N + w) * a.K;
-    int ip, jp;
-    if constexpr (sizeof(RT) == 4) {
-      // the FP32 build's velocity and landing offsets (FMA chain over
-      // ascending k, u = w dt/dx + 1/2, exact floor of u + d_a)
-      float wx = vbar[2 * s], wy = vbar[2 * s + 1];
-      for (int k = 0; k < a.K; ++k) {
-        const float y = yw[k];
-        const float *ph = reinterpret_cast<const float *>(modes) + 2 * (((int64_t)t * a.K + k) * Nc + c);
-        wx = fmaf(y, ph[0], wx);
-        wy = fmaf(y, ph[1], wy);
+    int ip = -1, jp = -1;   // the sink: from an obstacle, the last layer or without an action
+    if (!obst && t < nt - 1 && act >= 0) {
+      if constexpr (sizeof(RT) == 4) {
+        // the FP32 build's landing offsets (u = w dt/dx + 1/2, exact floor of u + d_a)
+        if constexpr (KT == 0) {
+          for (int k = 0; k < K; ++k) {
+            float px, py;
+            const float y = __ldg(yw + k);
+            load_pair<float, VEC>(ph + 2 * k * Nc, px, py);
+            vx = fmaf(y, px, vx);
+            vy = fmaf(y, py, vy);
+          }
+        }
+        float ux = fmaf(vx, a.lam, 0.5f), uy = fmaf(vy, a.lam, 0.5f);
+        if (!(fabsf(ux) < 1e30f)) ux = 1e30f;
+        if (!(fabsf(uy) < 1e30f)) uy = 1e30f;
+        const int4 l = land[act];
+        ip = i + land_offset(ux, l.x, __int_as_float(l.z));
+        jp = j + land_offset(uy, l.y, __int_as_float(l.w));
+      } else {
+        // the oracle's literal FP64 kinematics, round-to-nearest, no contraction
+        for (int k = 0; k < K; ++k) {
+          vx = __dadd_rn(vx, __dmul_rn(yw[k], ph[2 * k * Nc]));
+          vy = __dadd_rn(vy, __dmul_rn(yw[k], ph[2 * k * Nc + 1]));
+        }
+        const double x = __dmul_rn((double)i + 0.5, a.dx), y = __dmul_rn((double)j + 0.5, a.dx);
+        const double xp = __dadd_rn(x, __dmul_rn(__dadd_rn(vx, a.act.dx64[act]), a.dt));
+        const double yp = __dadd_rn(y, __dmul_rn(__dadd_rn(vy, a.act.dy64[act]), a.dt));
+        const double fx = floor(__ddiv_rn(xp, a.dx)), fy = floor(__ddiv_rn(yp, a.dx));
+        // far outside the grid the cell index does not fit an int: the sink
+        ip = (fx >= 0.0 && fx < (double)nx) ? (int)fx : -1;
+        jp = (fy >= 0.0 && fy < (double)ny) ? (int)fy : -1;
       }
-      float ux = fmaf(wx, a.lam, 0.5f), uy = fmaf(wy, a.lam, 0.5f);
-      if (!(fabsf(ux) < 1e30f)) ux = 1e30f;
-      if (!(fabsf(uy) < 1e30f)) uy = 1e30f;
-      const int di = land_offset(ux, a.act.cx[act], a.act.thx[act]);
-      const int dj = land_offset(uy, a.act.cy[act], a.act.thy[act]);
-      ip = i + di;
-      jp = j + dj;
-    } else {
-      // the oracle's literal FP64 kinematics, round-to-nearest, no contraction
-      double vx = vbar[2 * s], vy = vbar[2 * s + 1];
-      for (int k = 0; k < a.K; ++k) {
-        const double *ph = reinterpret_cast<const double *>(modes) + 2 * (((int64_t)t * a.K + k) * Nc + c);
-        vx = __dadd_rn(vx, __dmul_rn(yw[k], ph[0]));
-        vy = __dadd_rn(vy, __dmul_rn(yw[k], ph[1]));
-      }
-      const double x = __dmul_rn((double)i + 0.5, a.dx), y = __dmul_rn((double)j + 0.5, a.dx);
-      const double xp = __dadd_rn(x, __dmul_rn(__dadd_rn(vx, a.act.dx64[act]), a.dt));
-      const double yp = __dadd_rn(y, __dmul_rn(__dadd_rn(vy, a.act.dy64[act]), a.dt));
-      const double fx = floor(__ddiv_rn(xp, a.dx)), fy = floor(__ddiv_rn(yp, a.dx));
-      // far outside the grid the cell index does not fit an int: the sink
-      ip = (fx >= 0.0 && fx < (double)a.nx) ? (int)fx : -1;
-      jp = (fy >= 0.0 && fy < (double)a.ny) ? (int)fy : -1;
     }
-    if (ip < 0 || ip >= a.nx || jp < 0 || jp >= a.ny ||
-        a.obstacle[(int64_t)(t + 1) * Nc + (int64_t)jp * a.nx + ip]) {
-      for (int o = 0; o < a.n_obj; ++o) ret[o] += (RT)a.rw.r_out;
+    if (ip < 0 || ip >= nx || jp < 0 || jp >= ny) {
+#pragma unroll
+      for (int o = 0; o < 3; ++o) ret[o] += (RT)a.rw.r_out;
       break;
-    }
-    const int64_t cp = (int64_t)jp * a.nx + ip;
-    const bool is_t = a.target[cp] != 0;
-    const RT g_s = gbar ? gbar[s] : (RT)0, g_sp = gbar ? gbar[(int64_t)(t + 1) * Nc + cp] : (RT)0;
-    for (int o = 0; o < a.n_obj; ++o) {
-      if constexpr (sizeof(RT) == 4)
-        ret[o] += step_reward32(a.rw, a.rw.objs[o], a.act.F[act], g_s, g_sp, is_t);
-      else
-        ret[o] = __dadd_rn(ret[o], step_reward64(a.rw, a.rw.objs[o], a.act.F64[act], g_s, g_sp, is_t));
     }
     i = ip;
     j = jp;
   }
   if (a.ret)
-    for (int o = 0; o < a.n_obj; ++o) static_cast<RT *>(a.ret)[path * a.n_obj + o] = ret[o];
+    for (int o = 0; o < 3; ++o)
+      if (o < n_obj) static_cast<RT *>(a.ret)[path * n_obj + o] = ret[o];
   if (a.steps) a.steps[path] = n;
   if (a.status) a.status[path] = (int8_t)st;
 }
@@ -123,13 +216,15 @@ __global__ void rollout_summary_kernel(const RT *ret, const int32_t *steps, cons
   __shared__ double sh[256][5];
   const int q = blockIdx.x, tid = threadIdx.x;
   double acc[5] = {0, 0, 0, 0, 0};   // returns x3, arrivals, steps of arrivals
+#pragma unroll 4   // (every load unconditional: four paths' in flight)
   for (int w = tid; w < N; w += blockDim.x) {
     const int64_t p = (int64_t)q * N + w;
-    for (int o = 0; o < n_obj; ++o) acc[o] += (double)ret[p * n_obj + o];
-    if (status[p] == 0) {
-      acc[3] += 1.0;
-      acc[4] += (double)steps[p];
-    }
+    const int n = steps[p];
+    const bool there = status[p] == 0;
+#pragma unroll
+    for (int o = 0; o < 3; ++o) acc[o] += o < n_obj ? (double)ret[p * n_obj + o] : 0.0;
+    acc[3] += there ? 1.0 : 0.0;
+    acc[4] += there ? (double)n : 0.0;
   }
   for (int v = 0; v < 5; ++v) sh[tid][v] = acc[v];
   __syncthreads();
@@ -139,6 +234,31 @@ __global__ void rollout_summary_kernel(const RT *ret, const int32_t *steps, cons
     __syncthreads();
   }
   if (tid < 5) out[q * 5 + tid] = sh[0][tid];
+}
+
+template <typename RT, int KT, bool VEC>
+static void launch_roll(const RolloutArgs &a, cudaStream_t st) {
+  const int64_t paths = (int64_t)a.n_starts * a.N;
+  rollout_kernel<RT, KT, VEC><<<(unsigned)((paths + kRollThreads - 1) / kRollThreads), kRollThreads, 0, st>>>(a);
+}
+// Vector loads where the caller's arrays are aligned for them (torch's are;
+// a view at an odd element is not), the mode count fixed up to eight.
+static void launch_rollout(const RolloutArgs &a, int prec, cudaStream_t st) {
+  if (prec == MDP_FP64_CHECK) return launch_roll<double, 0, false>(a, st);
+  auto aligned = [](const void *p, size_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; };
+  const size_t row = a.K % 4 == 0 ? 16 : (a.K % 2 == 0 ? 8 : 4);
+  if (!aligned(a.vbar, 8) || !aligned(a.modes, 8) || !aligned(a.Y, row)) return launch_roll<float, 0, false>(a, st);
+  switch (a.K) {
+    case 1: return launch_roll<float, 1, true>(a, st);
+    case 2: return launch_roll<float, 2, true>(a, st);
+    case 3: return launch_roll<float, 3, true>(a, st);
+    case 4: return launch_roll<float, 4, true>(a, st);
+    case 5: return launch_roll<float, 5, true>(a, st);
+    case 6: return launch_roll<float, 6, true>(a, st);
+    case 7: return launch_roll<float, 7, true>(a, st);
+    case 8: return launch_roll<float, 8, true>(a, st);
+    default: return launch_roll<float, 0, true>(a, st);
+  }
 }
 
 }  // namespace mdpgb
@@ -233,9 +353,7 @@ extern "C" mdp_status mdp_rollout(const mdp_env *env, const mdp_grid *grid, cons
   a.ret = ret ? ret : buf[2];
   a.steps = steps ? steps : static_cast<int32_t *>(buf[3]);
   a.status = status ? status : static_cast<int8_t *>(buf[4]);
-  const unsigned blocks = (unsigned)((paths + 255) / 256);
-  if (prec == MDP_FP64_CHECK) rollout_kernel<double><<<blocks, 256, 0, st>>>(a);
-  else rollout_kernel<float><<<blocks, 256, 0, st>>>(a);
+  launch_rollout(a, prec, st);
   ce = cudaGetLastError();
   std::vector<double> sums;
   if (ce == cudaSuccess && need_all) {
