@@ -29,7 +29,7 @@
 #include <cstring>
 #include <vector>
 
-#include "build_common.cuh"
+#include "build_warp.cuh"
 
 namespace mdpgb {
 
@@ -70,9 +70,8 @@ struct Build3Args {
   uint16_t *sinkc;
   void *R;
   unsigned long long *cnt;
-  // warp-per-slice kernel (FP32 rank counting): table words per warp, the
-  // list of slices it leaves to the CTA kernel, and (CTA kernel) that list
-  int32_t cap3;
+  // warp-per-slice kernel (FP32 rank counting): the list of slices it leaves to
+  // the CTA kernel, and (CTA kernel) that list
   uint32_t *defer;
   const uint32_t *defer_in;
 };
@@ -532,25 +531,46 @@ __global__ void __launch_bounds__(256, sizeof(RT) == 4 ? 4 : 1) build3d_kernel(B
 }
 
 // ---- warp per slice (FP32 rank counting) ----
-// A warp builds one slice alone, in private shared memory and without block
-// barriers -- the 2-D warp kernel's scheme in three dimensions: pass 1 forms
-// u for the warp's (state, realization) items and reduces each state's exact
-// extremes per axis; the states' fine tables are laid out in the warp's table
-// memory; pass 2 forms u again and counts each realization at its fine
-// coordinate; an in-place 3-D prefix sum; then lane l emits row l exactly as
-// the CTA kernel's rank path does (the same offsets, eight-corner box sums,
-// entry order and R accumulation), so a slice's output does not depend on
+// A CTA takes groups of kWarps3 consecutive slices; each warp builds its slice in
+// private shared memory -- the 2-D group kernel's scheme in three dimensions:
+// pass 1 forms u for the warp's (state, realization) items and reduces each
+// state's exact extremes per axis; the states' fine tables are laid out in the
+// warp's table memory; pass 2 forms u again and counts each realization at
+// its fine coordinate; an in-place 3-D prefix sum; then lane l scans row l's
+// box (four prefix lookups per offset bin: a bin's upper face is the next one's
+// lower face) and stages the entry words; the group allocates its columns with
+// one atomic and the warps copy the rows out.  Offsets, counts, entry order
+// and R are the CTA kernel's rank path's, so a slice's output does not depend on
 // the kernel that built it.  Slices whose tables do not fit the warp's memory
 // (or whose velocity extremes are not finite or widely spread) go to a list
 // that the CTA kernel builds afterwards.
-constexpr int kWarps3 = 8;   // warps per CTA of the warp kernel
+//
+// Bound by instruction issue.  The modes, coefficients (one vector load per
+// realization) and vbar stay in registers with the mode count fixed (KT),
+// floors are magic sums, the table address is six multiply-adds of the floors'
+// bits and the ranks, and thresholds are compared two at a time, as many as the
+// axis has; the actions' constants come from shared memory (indexed by
+// lane, a constant-bank read would be repeated per action).  64 x 64 x 16 cells, 40
+// layers, four modes, 1000 realizations, 24 actions: 42.9 ms with a warp's own
+// pool and queue atomics, run-time mode counts, two scans of eight lookups per
+// bin and 10,100 warp instructions a slice; 20.3 ms and 6,307 so.
+constexpr int kWarps3 = 4;   // warps per CTA of the warp kernel
 constexpr int kCap3 = 2048;  // table words per warp (8 KB)
+constexpr int kStage3 = 16;  // entries of a row that are staged (2 KB per warp)
 
 struct Warp3Acc {
   unsigned long long tot = 0, dom = 0, samp = 0, maxw = 0;
 };
+struct Warp3Smem {
+  int4 act[3][kMaxActions];   // c, le, bits of th, bits of F
+  long long next[2];          // queue: the group after this one (double-buffered, as the next two)
+  unsigned long long base[2];
+  int cols[2][kWarps3];
+};
+constexpr uint32_t kWarp3Stage = (uint32_t)((sizeof(Warp3Smem) + 127) & ~(size_t)127);
+constexpr uint32_t kWarp3Tabs = kWarp3Stage + kWarps3 * kStage3 * 128;
 
-// u of realization w of state s (layer t, cell c): the CTA kernel's phase A
+// u of realization w of state s (layer t, cell c), any mode count
 __device__ __forceinline__ void velocity3(const Build3Args &a, int64_t s, int64_t t, int64_t c, int w, float (&u)[3]) {
   const float *vbar = static_cast<const float *>(a.vbar);
   const float *modes = static_cast<const float *>(a.modes);
@@ -565,32 +585,6 @@ __device__ __forceinline__ void velocity3(const Build3Args &a, int64_t s, int64_
   u[0] = fmaf(vx, a.lam, 0.5f);
   u[1] = fmaf(vy, a.lam, 0.5f);
   u[2] = fmaf(vz, a.lam, 0.5f);
-#pragma unroll
-  for (int x = 0; x < 3; ++x)
-    if (!(fabsf(u[x]) < 1e30f)) u[x] = 1e30f;
-}
-
-// the same with the state's mode vectors in registers (K <= 4)
-__device__ __forceinline__ void velocity3r(const Build3Args &a, int64_t s, int64_t t, int w, const float (&ph)[4][3],
-                                           float (&u)[3]) {
-  const float *vbar = static_cast<const float *>(a.vbar);
-  const float *yw = static_cast<const float *>(a.Y) + ((size_t)t * a.N + w) * a.K;
-  float vx = vbar[3 * s], vy = vbar[3 * s + 1], vz = vbar[3 * s + 2];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    if (k < a.K) {
-      const float y = yw[k];
-      vx = fmaf(y, ph[k][0], vx);
-      vy = fmaf(y, ph[k][1], vy);
-      vz = fmaf(y, ph[k][2], vz);
-    }
-  }
-  u[0] = fmaf(vx, a.lam, 0.5f);
-  u[1] = fmaf(vy, a.lam, 0.5f);
-  u[2] = fmaf(vz, a.lam, 0.5f);
-#pragma unroll
-  for (int x = 0; x < 3; ++x)
-    if (!(fabsf(u[x]) < 1e30f)) u[x] = 1e30f;
 }
 
 __device__ __forceinline__ Geo3 shfl_geo3(const Geo3 &g, int src) {
@@ -605,275 +599,498 @@ __device__ __forceinline__ Geo3 shfl_geo3(const Geo3 &g, int src) {
   return o;
 }
 
-// Slice sl by one warp; tab: the warp's cap words of table memory (zero).
-// Returns false when the slice was put on the CTA kernel's list.
-__device__ bool warp3_slice(const Build3Args &a, int64_t sl, uint32_t *tab, Warp3Acc &acc) {
-  const int lane = threadIdx.x & 31;
-  const int spw = a.spw, h = a.h, L = a.L;
-  const int64_t Nc = a.Nc, nxy = (int64_t)a.nx * a.ny;
-  const int q_l = lane / a.A_pad, a_l = lane % a.A_pad;
-  const bool act_ok = a_l < a.A;
-  const int q_t = lane % spw, wi = lane / spw, wstep = 32 / spw;
-  auto kind = [&](int64_t s) {
-    if (s >= a.nS) return (int)KIND_NONE;
-    if (a.target[s % Nc]) return (int)KIND_TERMINAL;
-    if (a.obstacle[s] || s / Nc == a.nt - 1) return (int)KIND_SINK;
-    return (int)KIND_SAMPLE;
-  };
-  const int64_t s_l = sl * spw + q_l, s_t = sl * spw + q_t;
-  const int kind_l = act_ok ? kind(s_l) : KIND_NONE;
-  const int kind_t = kind(s_t);
-  const int64_t t_t = s_t / Nc, c_t = s_t % Nc;
-  // up to four modes: the state's mode vectors in registers for both passes
-  // (else each realization reloads them, 3K floats, from L1)
-  const bool preph = a.K <= 4;
-  float ph[4][3];
+// ln / G for 0 <= ln < 2^16 with m = div_magic(G): ceil(2^32 / G) ln errs below ln / 2^32
+__device__ __forceinline__ uint32_t div_magic(int G) { return 0xFFFFFFFFu / (uint32_t)G + 1u; }
+__device__ __forceinline__ int div_by(int ln, uint32_t m) { return m ? (int)__umulhi((uint32_t)ln, m) : ln; }
+
+// In-place inclusive prefix sum of n cells p[step], p[2 step], ... (four loads in flight)
+__device__ __forceinline__ void prefix_line(uint32_t *p, int n, int step) {
+  uint32_t v = 0;
+  int i = 0;
+  for (; i + 4 <= n; i += 4) {
+    uint32_t x0 = p[step], x1 = p[2 * step], x2 = p[3 * step], x3 = p[4 * step];
+    x0 += v; x1 += x0; x2 += x1; x3 += x2;
+    p[step] = x0; p[2 * step] = x1; p[3 * step] = x2; p[4 * step] = x3;
+    v = x3;
+    p += 4 * step;
+  }
+  for (; i < n; ++i) {
+    p += step;
+    v += *p;
+    *p = v;
+  }
+}
+
+// A row of the slice: its box of offset bins and its state's table.
+struct Row3 {
+  int n[3];         // most bins per axis over the slice's rows
+  int f[3];         // fine coordinate of the first bin's lower face (<= 0 within the sub-grid)
+  int G[3];         // the table's cells (0: every bin comes out empty)
+  int li, lj, lk;   // the cell of the first bin
+  int off;          // its successor offset
+  int base;
+};
+
+// Calls f(offset, count, class, cell) for the row's non-empty bins in ascending
+// order; a landing outside the domain has class CLS_OBSTACLE.  Whole warp.
+template <class F>
+__device__ __forceinline__ void scan3(const Build3Args &a, const Row3 &r, const uint32_t *tab, const uint8_t *cls_next,
+                                      F &&f) {
+  const int Sx = a.act.D[0] + 1, Sy = a.act.D[1] + 1, Sz = a.act.D[2] + 1, nx = a.nx;
+  const int Pz = r.G[2] + 1, PyPz = (r.G[1] + 1) * Pz;
+  const uint32_t *P = tab + r.base;
+  int z0 = 0, zf = r.f[2];
+  for (int dk = 0; dk < r.n[2]; ++dk) {
+    zf += Sz;
+    const int z1 = min(zf, r.G[2]);
+    int y0 = 0, yf = r.f[1];
+    for (int dj = 0; dj < r.n[1]; ++dj) {
+      yf += Sy;
+      const int y1 = min(yf, r.G[1]) * Pz;
+      const uint32_t *p11 = P + y1 + z1, *p01 = P + y0 + z1, *p10 = P + y1 + z0, *p00 = P + y0 + z0;
+      const int jp = r.lj + dj, kp = r.lk + dk;
+      const bool row_in = jp >= 0 && jp < a.ny && kp >= 0 && kp < a.nz;
+      const int cell0 = (kp * a.ny + jp) * nx, off0 = r.off + dk * nx * a.ny + dj * nx;
+      uint32_t prev = 0;
+      int xf = r.f[0];
+      for (int d0 = 0; d0 < r.n[0]; d0 += 4) {   // four bins' lookups in flight
+        uint32_t v[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
+        for (int i = 0; i < 4; ++i) {
+          xf += Sx;
+          const int x = min(xf, r.G[0]) * PyPz;
+          v[i] = p11[x] - p01[x] - p10[x] + p00[x];
+        }
+        int cc[4];
 #pragma unroll
-    for (int x = 0; x < 3; ++x)
-      ph[k][x] = (preph && k < a.K && kind_t == KIND_SAMPLE)
-                     ? static_cast<const float *>(a.modes)[3 * ((t_t * a.K + k) * Nc + c_t) + x] : 0.f;
-  // ---- pass 1: exact extremes of u per state and axis
-  float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
-  if (kind_t == KIND_SAMPLE) {
-    for (int w = wi; w < a.N; w += wstep) {
-      float u[3];
-      if (preph) velocity3r(a, s_t, t_t, w, ph, u);
-      else velocity3(a, s_t, t_t, c_t, w, u);
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t n = v[i] - prev;
+          prev = v[i];
+          v[i] = n;
+          const int ip = r.li + d0 + i;
+          cc[i] = CLS_OBSTACLE;
+          if (n && row_in && ip >= 0 && ip < nx) cc[i] = cls_next[cell0 + ip];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (v[i]) f(off0 + d0 + i, v[i], cc[i], cell0 + r.li + d0 + i);
+      }
+      y0 = y1;
+    }
+    z0 = z1;
+  }
+}
+
+// Rows with more entries than are staged: a second scan writes them.
+__device__ __noinline__ void write_scan3(const Build3Args &a, const Row3 r, const uint32_t *tab, const uint8_t *cls_next,
+                                         const float *g_next, float F, float g_s, bool write, uint32_t *dst, float *R) {
+  float acc[3] = {0.f, 0.f, 0.f};
+  int k = 0;
+  scan3(a, r, tab, cls_next, [&](int off, uint32_t n, int cc, int cell) {
+    if (cc & CLS_OBSTACLE) return;
+    if (write) dst[(size_t)k * 32] = entry_word(off, n);
+    ++k;
+    const float g_sp = g_next ? g_next[cell] : 0.f;
+    for (int o = 0; o < a.rw.n_obj; ++o)
+      acc[o] = fmaf((float)n / (float)a.N,
+                    step_reward32(a.rw, a.rw.objs[o], F, g_s, g_sp, (cc & CLS_TARGET) != 0), acc[o]);
+  });
+  for (int o = 0; o < 3; ++o) R[o] = acc[o];
+}
+
+// The group of slices [sl0, sl0 + kWarps3), one per warp.  tab: the warp's kCap3
+// words of table memory (zero on entry and return); stage: its entry words.
+// next: thread 0's next queue index.
+template <int KT>
+__device__ __forceinline__ void warp3_group(const Build3Args &a, int64_t sl0, Warp3Smem &sm, uint32_t *tab,
+                                            uint32_t *stage, long long next, int par, Warp3Acc &acc) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t sl = sl0 + warp;
+  const int spw = a.spw, h = a.h, N = a.N;
+  const int64_t Nc = a.Nc;
+  const int q_l = lane / a.A_pad, a_l = lane % a.A_pad, q_t = lane % spw, wi = lane / spw, wstep = 32 / spw;
+  // the state that the lane counts for
+  const int64_t s_t = sl * spw + q_t;
+  int kind_t = KIND_NONE;
+  if (sl < a.n_slices && s_t < a.nS) {
+    const uint8_t c = a.cls[s_t];
+    kind_t = c & CLS_TARGET ? KIND_TERMINAL : ((c & CLS_OBSTACLE) || s_t >= a.nS - Nc ? KIND_SINK : KIND_SAMPLE);
+  }
+  const bool on = kind_t == KIND_SAMPLE;
+  const int64_t t = layer_of(s_t, Nc, a.nS), c = s_t - t * Nc;
+  const float *vbar = static_cast<const float *>(a.vbar);
+  float vb[3] = {0.f, 0.f, 0.f}, ph[kPhi<KT>][3];
+  if constexpr (KT > 0) {
+#pragma unroll
+    for (int k = 0; k < KT; ++k)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) ph[k][x] = on ? static_cast<const float *>(a.modes)[3 * ((t * KT + k) * Nc + c) + x] : 0.f;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) vb[x] = on ? vbar[3 * s_t + x] : 0.f;
+  }
+  const float *Yt = static_cast<const float *>(a.Y) + (size_t)t * N * a.K;
+  const float lam = a.lam;
+  // u of a realization: FMA chain over ascending k, then u = fma(w, lam, 1/2)
+  auto velocity = [&](int w, float (&u)[3]) {
+    if constexpr (KT > 0) {
+      float y[kPhi<KT>];
+      load_row<KT>(Yt + (size_t)w * KT, KT, y);
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
-        mn[x] = fminf(mn[x], u[x]);
-        mx[x] = fmaxf(mx[x], u[x]);
+        float v = vb[x];
+#pragma unroll
+        for (int k = 0; k < KT; ++k) v = fmaf(y[k], ph[k][x], v);
+        u[x] = fmaf(v, lam, 0.5f);
       }
+    } else {
+      velocity3(a, s_t, t, c, w, u);
+    }
+  };
+  // ---- pass 1: exact extremes of u per state and axis (a NaN stays in them)
+  float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
+  const int N_on = on ? N : 0;
+#pragma unroll 1
+  for (int w = wi; w < N_on; w += 2 * wstep) {   // two realizations per trip (the last one twice)
+    float u[3], v[3];
+    velocity(w, u);
+    velocity(min(w + wstep, N - 1), v);
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      mn[x] = min_nan(mn[x], u[x], v[x]);
+      mx[x] = max_nan(mx[x], u[x], v[x]);
     }
   }
   for (int off = 16; off >= spw; off >>= 1) {
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-      mn[x] = fminf(mn[x], __shfl_xor_sync(0xffffffffu, mn[x], off));
-      mx[x] = fmaxf(mx[x], __shfl_xor_sync(0xffffffffu, mx[x], off));
+      mn[x] = min_nan(mn[x], __shfl_xor_sync(kAll, mn[x], off));
+      const float o = __shfl_xor_sync(kAll, mx[x], off);
+      mx[x] = max_nan(mx[x], o, o);
     }
   }
-  // lane q < spw: the fine table of state q (the CTA kernel's rules)
+  // the state's fine table (the CTA kernel's rules), on all its lanes
   Geo3 g{};
-  long long cells = 0;
-  if (lane < spw && kind(sl * spw + lane) == KIND_SAMPLE) {
-    cells = 1;
-    for (int x = 0; x < 3 && cells > 0; ++x) {
-      if (!(mn[x] > -1e6f) || !(mx[x] < 1e6f) || mx[x] - mn[x] > 1024.f) {
-        cells = -1;
+  int cells = 0;
+  if (on) {
+    long long n = 1;
+    for (int x = 0; x < 3 && n > 0; ++x) {
+      if (!(mn[x] > -1e6f) || !(mx[x] < 1e6f) || !(mx[x] - mn[x] <= 1024.f)) {
+        n = -1;
         break;
       }
       const int S = a.act.D[x] + 1;
       g.n0[x] = (int)floorf(mn[x]);
       g.fmin[x] = fine3(mn[x], g.n0[x], S, a.act.T[x], a.act.D[x]);
       g.G[x] = fine3(mx[x], g.n0[x], S, a.act.T[x], a.act.D[x]) - g.fmin[x] + 1;
-      cells *= (long long)(g.G[x] + 1);
+      n *= (long long)(g.G[x] + 1);
     }
+    cells = (int)min(n, (long long)kCap3 + 1);
   }
-  long long total = 0;
+  int total = 0;
   bool fit = true;
   for (int q = 0; q < spw; ++q) {
-    const long long cq = __shfl_sync(0xffffffffu, cells, q);
-    if (lane == q) g.base = (int)min(total, (long long)a.cap3);
-    if (cq < 0) fit = false;
-    total += max(cq, 0LL);
+    const int cq = __shfl_sync(kAll, cells, q);
+    if (q_t == q) g.base = min(total, kCap3);
+    fit = fit && cq >= 0;
+    total += max(cq, 0);
   }
-  if (!fit || total > (long long)a.cap3) {   // the CTA kernel builds it
-    if (lane == 0) {
-      const unsigned long long i = atomicAdd(&a.cnt[CNT_DEFER_N], 1ULL);
-      a.defer[i] = (uint32_t)sl;
-    }
-    return false;
+  fit = fit && total <= kCap3;
+  const int kind_l = __shfl_sync(kAll, kind_t, q_l);
+  const bool rows = kind_l == KIND_SAMPLE && a_l < a.A;
+  if (!fit && lane == 0) {   // the CTA kernel builds it
+    const unsigned long long i = atomicAdd(&a.cnt[CNT_DEFER_N], 1ULL);
+    a.defer[i] = (uint32_t)sl;
   }
-  // ---- pass 2: one count per realization at its fine coordinate
-  const Geo3 gt = shfl_geo3(g, q_t);
-  if (kind_t == KIND_SAMPLE) {
-    const int Py = gt.G[1] + 1, Pz = gt.G[2] + 1;
-    const uint32_t hb = smem_u32(tab);
-#pragma unroll 1
-    for (int w = wi; w < a.N; w += wstep) {
-      float u[3];
-      if (preph) velocity3r(a, s_t, t_t, w, ph, u);
-      else velocity3(a, s_t, t_t, c_t, w, u);
-      int X = fine3(u[0], gt.n0[0], a.act.D[0] + 1, a.act.T[0], a.act.D[0]) - gt.fmin[0];
-      int Y = fine3(u[1], gt.n0[1], a.act.D[1] + 1, a.act.T[1], a.act.D[1]) - gt.fmin[1];
-      int Z = fine3(u[2], gt.n0[2], a.act.D[2] + 1, a.act.T[2], a.act.D[2]) - gt.fmin[2];
-      X = min(max(X, 0), gt.G[0] - 1);
-      Y = min(max(Y, 0), gt.G[1] - 1);
-      Z = min(max(Z, 0), gt.G[2] - 1);
-      const uint32_t idx = (uint32_t)(gt.base + ((X + 1) * Py + (Y + 1)) * Pz + (Z + 1));
-      asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(hb + 4u * idx), "r"(1u));
-    }
-  }
-  __syncwarp();
-  // ---- in-place inclusive prefix sums along z, y and x (border planes stay zero)
-  for (int q = 0; q < spw; ++q) {
-    if (__shfl_sync(0xffffffffu, cells, q) <= 0) continue;
-    const Geo3 gq = shfl_geo3(g, q);
-    const int Gx = gq.G[0], Gy = gq.G[1], Gz = gq.G[2], Py = Gy + 1, Pz = Gz + 1;
-    uint32_t *P = tab + gq.base;
-    for (int ln = lane; ln < Gx * Gy; ln += 32) {
-      uint32_t *r = P + ((ln / Gy + 1) * Py + (ln % Gy + 1)) * Pz;
-      for (int z = 1; z <= Gz; ++z) r[z] += r[z - 1];
-    }
-    __syncwarp();
-    for (int ln = lane; ln < Gx * Gz; ln += 32) {
-      uint32_t *r = P + (ln / Gz + 1) * Py * Pz + (ln % Gz + 1);
-      for (int y = 1; y <= Gy; ++y) r[y * Pz] += r[(y - 1) * Pz];
-    }
-    __syncwarp();
-    for (int ln = lane; ln < Gy * Gz; ln += 32) {
-      uint32_t *r = P + (ln / Gz + 1) * Pz + (ln % Gz + 1);
-      for (int x = 1; x <= Gx; ++x) r[x * Py * Pz] += r[(x - 1) * Py * Pz];
-    }
-    __syncwarp();
-  }
-  // ---- emit: lane l = row (q_l, a_l), the CTA kernel's rank path
-  const Geo3 gl = shfl_geo3(g, q_l);
-  float umn[3], umx[3];
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    umn[x] = __shfl_sync(0xffffffffu, mn[x], q_l);
-    umx[x] = __shfl_sync(0xffffffffu, mx[x], q_l);
-  }
-  auto rank_count = [&](int di, int dj, int dk) -> uint32_t {
-    const int off[3] = {di, dj, dk};
-    int c0[3], c1[3];
-    for (int x = 0; x < 3; ++x) {
-      const int S = a.act.D[x] + 1;
-      const int f0 = (off[x] - a.act.c[x][a_l] - gl.n0[x] - 1) * S + a.act.le[x][a_l] - gl.fmin[x];
-      c0[x] = max(f0, 0);
-      c1[x] = min(f0 + S - 1, gl.G[x] - 1);
-      if (c0[x] > c1[x]) return 0u;
-    }
-    const int Py = gl.G[1] + 1, Pz = gl.G[2] + 1;
-    const uint32_t *P = tab + gl.base;
-    auto at = [&](int x, int y, int z) { return P[(x * Py + y) * Pz + z]; };
-    const int x0 = c0[0], y0 = c0[1], z0 = c0[2], x1 = c1[0] + 1, y1 = c1[1] + 1, z1 = c1[2] + 1;
-    return at(x1, y1, z1) - at(x0, y1, z1) - at(x1, y0, z1) - at(x1, y1, z0) + at(x0, y0, z1) +
-           at(x0, y1, z0) + at(x1, y0, z0) - at(x0, y0, z0);
-  };
-  const int64_t ir = sl * 32 + lane;
-  const int64_t t = s_l / Nc, c = s_l % Nc;
-  const int64_t li = c % a.nx, lj = (c / a.nx) % a.ny, lk = c / nxy;
-  const int64_t nxt = (t + 1) * Nc;
-  int e = 0;
+  int e = 0, W = 0;
   uint32_t sink = 0;
-  int lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
-  if (kind_l == KIND_SAMPLE) {
-    for (int x = 0; x < 3; ++x) {
-      lo[x] = box_offset(umn[x], a.act.c[x][a_l], a.act.th[x][a_l], h);
-      hi[x] = box_offset(umx[x], a.act.c[x][a_l], a.act.th[x][a_l], h);
-      if (lo[x] < -h || hi[x] > h) atomicAdd(&a.cnt[CNT_OVERFLOW], 1ULL);
-      lo[x] = max(lo[x], -h);
-      hi[x] = min(hi[x], h);
+  bool cap_hit = false, any_target = false;
+  Row3 r{};
+  const int64_t s_l = sl * spw + q_l, t_l = layer_of(s_l, Nc, a.nS);
+  const uint8_t *cls_next = a.cls + (t_l + 1) * Nc;
+  const int4 ax = sm.act[0][a_l], ay = sm.act[1][a_l], az = sm.act[2][a_l];
+  if (fit && total > 0) {
+    // ---- pass 2: one count per realization at its fine coordinate
+    // index = base + ((X + 1) Py + Y + 1) Pz + Z + 1, X = (floor - n0) S + rank - fmin, as
+    // multiply-adds of the floors' bits (floor_bits = kMagicBits + floor)
+    {
+      const int Sx = a.act.D[0] + 1, Sy = a.act.D[1] + 1, Sz = a.act.D[2] + 1;
+      const uint32_t pz = (uint32_t)(g.G[2] + 1), pyz = (uint32_t)(g.G[1] + 1) * pz;
+      const uint32_t bx = (uint32_t)Sx * pyz, by = (uint32_t)Sy * pz, bz = (uint32_t)Sz;
+      const uint32_t magic = __float_as_uint(kFloorMagic);
+      const uint32_t c0 = (uint32_t)g.base + (uint32_t)(1 - g.fmin[0]) * pyz + (uint32_t)(1 - g.fmin[1]) * pz +
+                          (uint32_t)(1 - g.fmin[2]) - (magic + (uint32_t)g.n0[0]) * bx - (magic + (uint32_t)g.n0[1]) * by -
+                          (magic + (uint32_t)g.n0[2]) * bz;
+      const uint32_t hb = smem_u32(tab), last = (uint32_t)total - 1u;
+      auto rank = [&](float f, int x) {   // #{T <= f}, two at a time: the thresholds beyond D are 2
+        uint32_t k = (a.act.T[x][0] <= f ? 1u : 0u) + (a.act.T[x][1] <= f ? 1u : 0u);
+#pragma unroll
+        for (int i = 2; i < kRank3; i += 2)
+          if (a.act.D[x] > i) k += (a.act.T[x][i] <= f ? 1u : 0u) + (a.act.T[x][i + 1] <= f ? 1u : 0u);
+        return k;
+      };
+      auto count = [&](const float (&u)[3]) {
+        const float tx = __fadd_rd(u[0], kFloorMagic), ty = __fadd_rd(u[1], kFloorMagic), tz = __fadd_rd(u[2], kFloorMagic);
+        const uint32_t rx = rank(u[0] - (tx - kFloorMagic), 0), ry = rank(u[1] - (ty - kFloorMagic), 1),
+                       rz = rank(u[2] - (tz - kFloorMagic), 2);
+        const uint32_t idx = __float_as_uint(tx) * bx + rx * pyz + __float_as_uint(ty) * by + ry * pz +
+                             __float_as_uint(tz) * bz + rz + c0;
+        red_add_shared(hb + 4u * min(idx, last), 1u);
+      };
+      int w = wi;
+#pragma unroll 1
+      for (; w + wstep < N_on; w += 2 * wstep) {
+        float u[3], v[3];
+        velocity(w, u);
+        velocity(w + wstep, v);
+        count(u);
+        count(v);
+      }
+      if (w < N_on) {
+        float u[3];
+        velocity(w, u);
+        count(u);
+      }
     }
-    for (int dk = lo[2]; dk <= hi[2]; ++dk)
-      for (int dj = lo[1]; dj <= hi[1]; ++dj)
-        for (int di = lo[0]; di <= hi[0]; ++di) {
-          const uint32_t n = rank_count(di, dj, dk);
-          if (!n) continue;
-          const int64_t ip = li + di, jp = lj + dj, kp = lk + dk;
-          const bool inside = ip >= 0 && ip < a.nx && jp >= 0 && jp < a.ny && kp >= 0 && kp < a.nz;
-          if (!inside || a.obstacle[nxt + (kp * a.ny + jp) * a.nx + ip]) sink += n;
-          else ++e;
+    __syncwarp();
+    // ---- in-place inclusive prefix sums along z, y and x (border planes stay zero)
+    for (int q = 0; q < spw; ++q) {
+      if (__shfl_sync(kAll, cells, q) <= 0) continue;
+      const Geo3 gq = shfl_geo3(g, q);
+      const int Gx = gq.G[0], Gy = gq.G[1], Gz = gq.G[2], Pz = Gz + 1, PyPz = (Gy + 1) * Pz;
+      uint32_t *P = tab + gq.base;
+      const uint32_t my = div_magic(Gy), mz = div_magic(Gz);
+      for (int ln = lane; ln < Gx * Gy; ln += 32) {
+        const int i = div_by(ln, my);
+        prefix_line(P + (i + 1) * PyPz + (ln - i * Gy + 1) * Pz, Gz, 1);
+      }
+      __syncwarp();
+      for (int ln = lane; ln < Gx * Gz; ln += 32) {
+        const int i = div_by(ln, mz);
+        prefix_line(P + (i + 1) * PyPz + (ln - i * Gz + 1), Gy, Pz);
+      }
+      __syncwarp();
+      for (int ln = lane; ln < Gy * Gz; ln += 32) {
+        const int i = div_by(ln, mz);
+        prefix_line(P + (i + 1) * Pz + (ln - i * Gz + 1), Gx, PyPz);
+      }
+      __syncwarp();
+    }
+    // ---- scan: lane l = row (q_l, a_l)
+    const Geo3 gl = shfl_geo3(g, q_l);
+    int nb[3] = {0, 0, 0};
+    {
+      const int4 k[3] = {ax, ay, az};
+      int lo[3] = {0, 0, 0};
+      bool scanned = rows;   // (a row that leaves the sub-grid comes out empty: the build fails)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const float umn = __shfl_sync(kAll, mn[x], q_l), umx = __shfl_sync(kAll, mx[x], q_l);
+        if (rows) {
+          const int S = a.act.D[x] + 1;
+          lo[x] = box_offset(umn, k[x].x, __int_as_float(k[x].z), h);
+          const int hi = box_offset(umx, k[x].x, __int_as_float(k[x].z), h);
+          if (lo[x] < -h || hi > h) {
+            atomicAdd(&a.cnt[CNT_OVERFLOW], 1ULL);
+            scanned = false;
+          }
+          nb[x] = hi - lo[x] + 1;
+          r.f[x] = (lo[x] - k[x].x - gl.n0[x] - 1) * S + k[x].y - gl.fmin[x];
+          r.G[x] = gl.G[x];
         }
-  } else if (kind_l == KIND_SINK) {
-    sink = (uint32_t)a.N;
+      }
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        if (!scanned) nb[x] = r.f[x] = r.G[x] = 0;
+        r.n[x] = (int)__reduce_max_sync(kAll, (unsigned)nb[x]);
+      }
+      if (scanned) {
+        const int cell = (int)(s_l - t_l * Nc), plane = a.nx * a.ny;
+        const int kk = cell / plane, jj = (cell - kk * plane) / a.nx, ii = cell - kk * plane - jj * a.nx;
+        r.li = ii + lo[0];
+        r.lj = jj + lo[1];
+        r.lk = kk + lo[2];
+        r.off = lo[2] * plane + lo[1] * a.nx + lo[0];
+        r.base = gl.base;
+      }
+    }
+    uint32_t *st = stage + lane;
+    scan3(a, r, tab, cls_next, [&](int off, uint32_t n, int cc, int) {
+      if (cc & CLS_OBSTACLE) {
+        sink += n;
+        return;
+      }
+      if (e < kStage3) *st = entry_word(off, n);
+      st += 32;
+      ++e;
+      any_target |= (cc & CLS_TARGET) != 0;
+    });
   }
-  (void)L;
-  const bool cap_hit = e + (sink > 0 ? 1 : 0) > a.row_cap;
-  if (cap_hit) {
-    atomicAdd(&a.cnt[CNT_ROW_CAP], 1ULL);
-    e = 0;
+  if (kind_l == KIND_SINK && a_l < a.A) sink = (uint32_t)N;
+  const int found = e;
+  if (fit && sl < a.n_slices) {
+    cap_hit = e + (sink > 0 ? 1 : 0) > a.row_cap;
+    if (cap_hit) {
+      atomicAdd(&a.cnt[CNT_ROW_CAP], 1ULL);
+      e = 0;
+    }
+    W = (int)__reduce_max_sync(kAll, (unsigned)e);
   }
-  int W = e;
-  for (int off = 16; off > 0; off >>= 1) W = max(W, __shfl_xor_sync(0xffffffffu, W, off));
-  unsigned long long base = 0;
-  if (lane == 0 && W > 0) base = atomicAdd(&a.cnt[CNT_POOL_COLS], (unsigned long long)W);
-  base = __shfl_sync(0xffffffffu, base, 0);
-  const bool fits = (W == 0) || (base + (unsigned long long)W <= a.pool_cap_cols);
-  if (!fits && lane == 0) atomicAdd(&a.cnt[CNT_POOL_FULL], 1ULL);
-  const bool write = fits && !cap_hit;
-  float Racc[3] = {0.f, 0.f, 0.f};
-  uint32_t *dst = a.pool + base * 32 + lane;
-  int k = 0;
-  if (kind_l == KIND_SAMPLE) {
-    const float F = a.act.F[a_l];
-    const float g_s = a.gbar ? static_cast<const float *>(a.gbar)[s_l] : 0.f;
-    for (int dk = lo[2]; dk <= hi[2]; ++dk)
-      for (int dj = lo[1]; dj <= hi[1]; ++dj)
-        for (int di = lo[0]; di <= hi[0]; ++di) {
-          const uint32_t n = rank_count(di, dj, dk);
-          if (!n) continue;
-          const int64_t ip = li + di, jp = lj + dj, kp = lk + dk;
-          const bool inside = ip >= 0 && ip < a.nx && jp >= 0 && jp < a.ny && kp >= 0 && kp < a.nz;
-          const int64_t cp = (kp * a.ny + jp) * a.nx + ip;
-          if (!inside || a.obstacle[nxt + cp]) continue;
-          if (write) dst[(size_t)k * 32] = entry_word((int)(dk * nxy + dj * a.nx + di), n);
-          ++k;
-          const bool is_t = a.target[cp] != 0;
-          const float g_sp = a.gbar ? static_cast<const float *>(a.gbar)[nxt + cp] : 0.f;
-          for (int o = 0; o < a.rw.n_obj; ++o)
-            Racc[o] = fmaf((float)n / (float)a.N, step_reward32(a.rw, a.rw.objs[o], F, g_s, g_sp, is_t), Racc[o]);
+  // ---- the group's columns
+  if (lane == 0) sm.cols[par][warp] = W;
+  if (threadIdx.x == 0) sm.next[par] = next;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int v = 0; v < kWarps3; ++v) n += sm.cols[par][v];
+    sm.base[par] = n ? atomicAdd(&a.cnt[CNT_POOL_COLS], (unsigned long long)n) : 0ULL;
+  }
+  __syncthreads();
+  if (fit && sl < a.n_slices) {
+    unsigned long long base = sm.base[par];
+    for (int v = 0; v < warp; ++v) base += (unsigned long long)sm.cols[par][v];
+    const bool fits = W == 0 || base + (unsigned long long)W <= a.pool_cap_cols;
+    if (!fits && lane == 0) atomicAdd(&a.cnt[CNT_POOL_FULL], 1ULL);
+    const bool write = fits && !cap_hit;
+    const float F = __int_as_float(ax.w);
+    const float *gbar = static_cast<const float *>(a.gbar);
+    const float g_s = rows && gbar ? gbar[s_l] : 0.f;
+    uint32_t *dst = a.pool + base * 32 + lane;
+    float R[3] = {0.f, 0.f, 0.f};
+    any_target = __any_sync(kAll, any_target);
+    if (__all_sync(kAll, found <= kStage3)) {
+      float rb[3] = {0.f, 0.f, 0.f}, rb_net = 0.f;
+      bool is_net[3] = {false, false, false}, net = false;
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        if (o < a.rw.n_obj) {
+          rb[o] = reward_base32(a.rw, a.rw.objs[o], F, g_s);
+          is_net[o] = a.rw.objs[o] == MDP_OBJ_NET_ENERGY;
+          if (is_net[o]) rb_net = rb[o];
+          net |= is_net[o];
         }
-    if (sink)
-      for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = fmaf((float)sink / (float)a.N, a.rw.f_r_out, Racc[o]);
-  } else if (kind_l == KIND_SINK) {
-    for (int o = 0; o < a.rw.n_obj; ++o) Racc[o] = a.rw.f_r_out;
+      }
+      const uint32_t *st = stage + lane;
+      const int64_t to = s_l + Nc;
+      const int cols = max(W, (int)__reduce_max_sync(kAll, (unsigned)found));   // (a row over the cap keeps its R)
+      for (int k0 = 0; k0 < cols; k0 += 4, st += 128) {   // four columns' loads in flight
+        uint32_t wd[4];
+        float gn[4];
+        uint8_t cc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const bool in = k0 + i < found;
+          wd[i] = in ? st[32 * i] : 0u;
+          const int off = (int)(int16_t)(wd[i] & 0xFFFFu);
+          gn[i] = net && in ? gbar[to + off] : 0.f;
+          cc[i] = any_target && in ? a.cls[to + off] : (uint8_t)0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (write && k0 + i < W) dst[(size_t)(k0 + i) * 32] = wd[i];
+          if (k0 + i < found) {
+            const float p = (float)(wd[i] >> 16) / (float)N;
+            const float rn = reward_cell32(a.rw, MDP_OBJ_NET_ENERGY, rb_net, gn[i], false);
+#pragma unroll
+            for (int o = 0; o < 3; ++o) {
+              float x = is_net[o] ? rn : rb[o];
+              if (cc[i] & CLS_TARGET) x = __fadd_rn(x, a.rw.f_r_term);
+              R[o] = fmaf(p, x, R[o]);
+            }
+          }
+        }
+      }
+    } else {
+      write_scan3(a, r, tab, cls_next, gbar ? gbar + (t_l + 1) * Nc : nullptr, F, g_s, write, dst, R);
+      if (write)
+        for (int kk = e; kk < W; ++kk) dst[(size_t)kk * 32] = 0u;
+    }
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      if (rows && sink) R[o] = fmaf((float)sink / (float)N, a.rw.f_r_out, R[o]);
+      if (kind_l == KIND_SINK && a_l < a.A) R[o] = a.rw.f_r_out;
+    }
+    if (!write) e = 0;
+    if (!fits) sink = 0;
+    if (lane == 0) {
+      a.slice_off[sl] = (fits && W > 0) ? (uint32_t)base : kNoSlice;
+      a.slice_w[sl] = (fits && W > 0) ? (uint8_t)W : (uint8_t)0;
+    }
+    const int64_t ir = sl * 32 + lane;
+    a.nnz[ir] = (uint8_t)e;
+    a.sinkc[ir] = (uint16_t)sink;
+#pragma unroll
+    for (int o = 0; o < 3; ++o)
+      if (o < a.rw.n_obj) static_cast<float *>(a.R)[(int64_t)o * a.rows_pad + ir] = R[o];
+    const int dom = __reduce_add_sync(kAll, e);
+    acc.dom += (unsigned long long)dom;
+    acc.tot += (unsigned long long)(dom + __popc(__ballot_sync(kAll, sink > 0)));
+    acc.samp += (unsigned long long)__popc(__ballot_sync(kAll, rows)) * (unsigned long long)N;
+    acc.maxw = max(acc.maxw, (unsigned long long)W);
+    __syncwarp();
+    for (int i = lane; 4 * i < total; i += 32)   // zero for the next slice
+      reinterpret_cast<uint4 *>(tab)[i] = make_uint4(0u, 0u, 0u, 0u);
   }
-  if (!write) {
-    e = 0;
-    k = 0;
-  }
-  if (write)
-    for (int kk = k; kk < W; ++kk) dst[(size_t)kk * 32] = 0u;
-  if (!fits) sink = 0;
-  if (lane == 0) {
-    a.slice_off[sl] = (fits && W > 0) ? (uint32_t)base : kNoSlice;
-    a.slice_w[sl] = (fits && W > 0) ? (uint8_t)W : (uint8_t)0;
-  }
-  a.nnz[ir] = (uint8_t)e;
-  a.sinkc[ir] = (uint16_t)sink;
-  for (int o = 0; o < a.rw.n_obj; ++o) static_cast<float *>(a.R)[(int64_t)o * a.rows_pad + ir] = Racc[o];
-  int dom = e, tot = e + (sink > 0 ? 1 : 0);
-  for (int off = 16; off > 0; off >>= 1) {
-    tot += __shfl_xor_sync(0xffffffffu, tot, off);
-    dom += __shfl_xor_sync(0xffffffffu, dom, off);
-  }
-  const int sampled = __popc(__ballot_sync(0xffffffffu, kind_l == KIND_SAMPLE));
-  acc.tot += (unsigned long long)tot;
-  acc.dom += (unsigned long long)dom;
-  acc.samp += (unsigned long long)sampled * (unsigned long long)a.N;
-  acc.maxw = max(acc.maxw, (unsigned long long)W);
   __syncwarp();
-  for (int i = lane; i < (int)total; i += 32) tab[i] = 0u;   // zero for the next slice
-  __syncwarp();
-  return true;
 }
 
-__global__ void __launch_bounds__(32 * kWarps3, 2) build3d_warp_kernel(Build3Args a) {
-  extern __shared__ __align__(16) uint32_t smem3w[];
+// groups per queue grab: chunk consecutive ones (as in the 2-D group kernel)
+template <int KT>
+__global__ void __launch_bounds__(32 * kWarps3, 5) build3d_warp_kernel(const __grid_constant__ Build3Args a, int chunk) {
+  extern __shared__ __align__(128) unsigned char smem3w[];
+  Warp3Smem &sm = *reinterpret_cast<Warp3Smem *>(smem3w);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t *tab = smem3w + (size_t)warp * a.cap3;
-  for (int i = lane; i < a.cap3; i += 32) tab[i] = 0u;
-  __syncwarp();
+  uint32_t *stage = reinterpret_cast<uint32_t *>(smem3w + kWarp3Stage) + warp * (kStage3 * 32);
+  uint32_t *tab = reinterpret_cast<uint32_t *>(smem3w + kWarp3Tabs) + warp * kCap3;
+  for (int i = lane; i < kCap3; i += 32) tab[i] = 0u;
+  for (int i = threadIdx.x; i < 3 * kMaxActions; i += blockDim.x) {
+    const int x = i / kMaxActions, k = i % kMaxActions;
+    sm.act[x][k] = make_int4(a.act.c[x][k], a.act.le[x][k], __float_as_int(a.act.th[x][k]), __float_as_int(a.act.F[k]));
+  }
+  long long next = 0;
+  int left = chunk - 1;   // thread 0: groups of its last grab still to do
+  if (threadIdx.x == 0) sm.next[1] = (long long)atomicAdd(&a.cnt[CNT_WORK], (unsigned long long)chunk);
+  __syncthreads();
   Warp3Acc acc;
-  unsigned long long next = 0;
-  if (lane == 0) next = atomicAdd(&a.cnt[CNT_WORK], 1ULL);
-  for (;;) {
-    const int64_t sl = (int64_t)__shfl_sync(0xffffffffu, next, 0);
-    if (sl >= a.n_slices) break;
-    if (lane == 0) next = atomicAdd(&a.cnt[CNT_WORK], 1ULL);
-    warp3_slice(a, sl, tab, acc);
+  const int64_t n_groups = (a.n_slices + kWarps3 - 1) / kWarps3;
+  for (int par = 0;; par ^= 1) {
+    const long long g = sm.next[par ^ 1];
+    if (g >= n_groups) break;
+    if (threadIdx.x == 0) {
+      if (left > 0) {
+        next = g + 1;
+        --left;
+      } else {
+        next = (long long)atomicAdd(&a.cnt[CNT_WORK], (unsigned long long)chunk);
+        left = chunk - 1;
+      }
+    }
+    warp3_group<KT>(a, g * kWarps3, sm, tab, stage, next, par, acc);
   }
   if (lane == 0) {
     if (acc.tot) atomicAdd(&a.cnt[CNT_NNZ], acc.tot);
     if (acc.dom) atomicAdd(&a.cnt[CNT_DOMAIN], acc.dom);
     if (acc.samp) atomicAdd(&a.cnt[CNT_SAMPLES], acc.samp);
     if (acc.maxw) atomicMax(&a.cnt[CNT_MAXROW], acc.maxw);
+  }
+}
+
+using Warp3Kernel = void (*)(Build3Args, int);
+// The mode count fixed where rows of coefficients can be loaded as vectors (16
+// or 8 bytes for multiples of four or two modes).
+static Warp3Kernel warp3_kernel(int K, const void *Y) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(Y);
+  if (at % (K % 4 == 0 ? 16 : (K % 2 == 0 ? 8 : 4)) != 0) return build3d_warp_kernel<0>;
+  switch (K) {
+    case 1: return build3d_warp_kernel<1>;
+    case 2: return build3d_warp_kernel<2>;
+    case 3: return build3d_warp_kernel<3>;
+    case 4: return build3d_warp_kernel<4>;
+    case 5: return build3d_warp_kernel<5>;
+    case 6: return build3d_warp_kernel<6>;
+    case 7: return build3d_warp_kernel<7>;
+    case 8: return build3d_warp_kernel<8>;
+    default: return build3d_warp_kernel<0>;
   }
 }
 
@@ -1092,21 +1309,25 @@ extern "C" mdp_status mdp_build3d_ex(const mdp_env3d *env, const mdp_grid3d *gri
   uint32_t *defer = nullptr;
   int64_t wblocks = 0;
   size_t wsmem = 0;
+  Warp3Kernel warp_fn = nullptr;
+  int wchunk = 1;
   if (use_warp) {
-    ba.cap3 = kCap3;
-    wsmem = (size_t)kWarps3 * kCap3 * 4;
+    warp_fn = warp3_kernel(env->K, Y);
+    wsmem = kWarp3Tabs + (size_t)kWarps3 * kCap3 * 4;
     TRY3(dev_alloc((void **)&defer, sizeof(uint32_t) * (size_t)m->n_slices, st));
     ba.defer = defer;
-    TRY3(allow_max_smem((const void *)build3d_warp_kernel));
+    TRY3(allow_max_smem((const void *)warp_fn));
     int wper = 0;
-    TRY3(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper, build3d_warp_kernel, 32 * kWarps3, wsmem));
+    TRY3(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper, warp_fn, 32 * kWarps3, wsmem));
     if (wper < 1) {
       release();
       dev_free(defer, st);
       set_error("the 3-D warp kernel's tables do not fit shared memory");
       return fail(MDP_ERR_CUDA);
     }
-    wblocks = std::min<int64_t>((int64_t)num_sms() * wper, (m->n_slices + kWarps3 - 1) / kWarps3);
+    const int64_t groups = (m->n_slices + kWarps3 - 1) / kWarps3;
+    wblocks = std::min<int64_t>((int64_t)num_sms() * wper, groups);
+    wchunk = (int)std::min<int64_t>(8, std::max<int64_t>(1, groups / (32 * wblocks)));
   }
   unsigned long long c[CNT_N];
   for (int attempt = 0;; ++attempt) {
@@ -1115,7 +1336,7 @@ extern "C" mdp_status mdp_build3d_ex(const mdp_env3d *env, const mdp_grid3d *gri
     if (prec == MDP_FP64_CHECK) {
       build3d_kernel<double><<<(unsigned)blocks, 256, smem, st>>>(ba);
     } else if (use_warp) {
-      build3d_warp_kernel<<<(unsigned)wblocks, 32 * kWarps3, wsmem, st>>>(ba);
+      warp_fn<<<(unsigned)wblocks, 32 * kWarps3, wsmem, st>>>(ba, wchunk);
       TRY3(cudaGetLastError());
       Build3Args bd = ba;
       bd.defer_in = defer;
