@@ -27,6 +27,7 @@ UNITS = {
     "build_warp.cu": [],
     "build_warp_batch.cu": [],
     "bellman.cu": [],
+    "export.cu": [],
     "serve.cu": [],
     "noalloc.cu": [],
     "batch.cu": [],

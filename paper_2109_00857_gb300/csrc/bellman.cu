@@ -1,6 +1,5 @@
 // bellman.cu -- sparse value iteration (steps a7-a8) and the small helper
-// kernels of the build (cell classes, sub-grid offset table, field extremes)
-// and of the paper-layout export.
+// kernels of the build (cell classes, sub-grid offset table, field extremes).
 //
 // Bellman backup (Sec. II-B): Q(s,a) = R(s,a) + sum_j P_j V(s'_j),
 // V_{k+1}(s) = max_a Q(s,a), pi(s) = argmax_a Q(s,a) (lowest index wins ties).
@@ -1793,199 +1792,6 @@ cudaError_t launch_layered_multi(const SolveArgs &a, int precision, int nt, cons
                                  double *stats_d, cudaStream_t st) {
   if (precision == MDP_FP64_CHECK) return layered_n<double>(a, nt, io, stats_d, st);
   return layered_n<float>(a, nt, io, stats_d, st);
-}
-
-// -------------------------------------------------------------- export ----
-// Paper layout row r = a*|S| + s.
-// entries of internal row ir = 32 sl + lane held in its slice's spill block
-__device__ __forceinline__ int spill_len(const uint32_t *spill, const uint32_t *spill_off, int64_t sl, int lane) {
-  if (!spill_off) return 0;
-  const uint32_t off = spill_off[sl];
-  return off == kNoSlice ? 0 : (int)(spill[off + lane + 1] - spill[off + lane]);
-}
-
-__global__ void export_count_kernel(const uint8_t *__restrict__ nnz, const uint16_t *__restrict__ sinkc,
-                                    const uint32_t *__restrict__ spill, const uint32_t *__restrict__ spill_off,
-                                    int64_t nS, int A, int A_pad, int64_t *__restrict__ rowlen) {
-  const int64_t rows = nS * A;
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t act = r / nS, s = r % nS;
-    const int64_t ir = s * A_pad + act;
-    rowlen[r] = nnz[ir] + spill_len(spill, spill_off, ir / 32, (int)(ir % 32)) + (sinkc[ir] ? 1 : 0);
-  }
-}
-
-// in-place exclusive scan of x[0..n) (int64), tile = 1024 per block
-__global__ void scan_tiles_kernel(int64_t *x, int64_t n, int64_t *tile_sums) {
-  __shared__ int64_t sh[1024];
-  const int64_t base = (int64_t)blockIdx.x * 1024;
-  for (int i = threadIdx.x; i < 1024; i += blockDim.x) sh[i] = (base + i < n) ? x[base + i] : 0;
-  __syncthreads();
-  // Hillis-Steele inclusive scan over 1024 entries with 256 threads x 4
-  for (int off = 1; off < 1024; off <<= 1) {
-    int64_t v[4];
-    for (int u = 0; u < 4; ++u) {
-      const int i = threadIdx.x * 4 + u;
-      v[u] = (i >= off) ? sh[i - off] : 0;
-    }
-    __syncthreads();
-    for (int u = 0; u < 4; ++u) sh[threadIdx.x * 4 + u] += v[u];
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < 1024; i += blockDim.x) {
-    if (base + i < n) x[base + i] = (i == 0) ? 0 : sh[i - 1];
-  }
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = sh[1023];
-}
-
-__global__ void scan_add_kernel(int64_t *x, int64_t n, const int64_t *tile_offs) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] += tile_offs[i / 1024];
-}
-
-// exclusive scan in place; scratch must hold ceil(n/1024) + ceil(n/1024^2) + ... entries
-static cudaError_t exclusive_scan(int64_t *x, int64_t n, int64_t *scratch, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  const int64_t tiles = (n + 1023) / 1024;
-  scan_tiles_kernel<<<(unsigned)tiles, 256, 0, st>>>(x, n, scratch);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || tiles == 1) return e;
-  e = exclusive_scan(scratch, tiles, scratch + tiles, st);
-  if (e != cudaSuccess) return e;
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > 65535) blocks = 65535;
-  scan_add_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, n, scratch);
-  return cudaGetLastError();
-}
-
-// One warp per slice: the slice's W columns are W*128 contiguous bytes in
-// both pools, copied as 16-byte vectors; then the new offset is recorded.
-__global__ void pool_reorder_kernel(const uint32_t *__restrict__ pool, uint32_t *__restrict__ out,
-                                    uint32_t *slice_off, const uint8_t *__restrict__ slice_w,
-                                    const int64_t *__restrict__ new_off, int64_t n_slices) {
-  const int lane = threadIdx.x & 31;
-  const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t sl = wid; sl < n_slices; sl += nwarps) {
-    const int W = slice_w[sl];
-    const int64_t no = new_off[sl];
-    if (W) {
-      const uint4 *src = reinterpret_cast<const uint4 *>(pool + (size_t)slice_off[sl] * 32);
-      uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)no * 32);
-      for (int i = lane; i < W * 8; i += 32) dst[i] = src[i];
-    }
-    __syncwarp();
-    if (lane == 0) slice_off[sl] = (uint32_t)no;
-  }
-}
-
-__global__ void slice_width_kernel(const uint8_t *__restrict__ slice_w, int64_t *x, int64_t n_slices) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n_slices; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] = i < n_slices ? (int64_t)slice_w[i] : 0;
-}
-
-cudaError_t launch_pool_reorder(const uint32_t *pool, uint32_t *out, uint32_t *slice_off, const uint8_t *slice_w,
-                                int64_t n_slices, cudaStream_t st) {
-  const int64_t n = n_slices + 1;
-  int64_t need = n, nn = n;   // offsets, then the scan's tile sums
-  while (nn > 1) { nn = (nn + 1023) / 1024; need += nn; }
-  int64_t *x = nullptr;
-  cudaError_t e = dev_alloc((void **)&x, sizeof(int64_t) * (size_t)(need + 1), st);
-  if (e != cudaSuccess) return e;
-  int64_t blocks = std::min<int64_t>(8192, (n + 255) / 256);
-  slice_width_kernel<<<(unsigned)blocks, 256, 0, st>>>(slice_w, x, n_slices);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = exclusive_scan(x, n, x + n, st);
-  if (e == cudaSuccess) {
-    blocks = std::min<int64_t>(num_sms() * 16, (n_slices + 7) / 8);
-    if (blocks < 1) blocks = 1;
-    pool_reorder_kernel<<<(unsigned)blocks, 256, 0, st>>>(pool, out, slice_off, slice_w, x, n_slices);
-    e = cudaGetLastError();
-  }
-  dev_free(x, st);
-  return e;
-}
-
-template <typename RT>
-__global__ void export_fill_kernel(const uint32_t *__restrict__ pool, const uint32_t *__restrict__ slice_off,
-                                   const uint8_t *__restrict__ nnz, const uint16_t *__restrict__ sinkc,
-                                   const uint32_t *__restrict__ spill, const uint32_t *__restrict__ spill_off,
-                                   const RT *__restrict__ Rsrc, int64_t nS, int64_t Nc, int A, int A_pad,
-                                   int spw, int64_t n_slices, const int64_t *__restrict__ rowptr,
-                                   int64_t *col, int32_t *count, RT *Rdst) {
-  const int64_t nrow = n_slices * 32;
-  for (int64_t ir = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ir < nrow; ir += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t sl = ir / 32;
-    const int lane = (int)(ir % 32);
-    const int q = lane / A_pad, act = lane % A_pad;
-    const int64_t s = sl * spw + q;
-    if (s >= nS || act >= A) continue;
-    const int64_t r = (int64_t)act * nS + s;
-    if (Rdst) Rdst[r] = Rsrc[ir];
-    if (!col && !count) continue;
-    int e = nnz[ir];
-    const int64_t o = rowptr[r];
-    if (e > 0) {
-      const uint32_t off = slice_off[sl];
-      for (int k = 0; k < e; ++k) {
-        const uint32_t w = pool[((size_t)off + k) * 32 + lane];
-        if (col) col[o + k] = s + Nc + (int64_t)(int16_t)(w & 0xFFFFu);
-        if (count) count[o + k] = (int32_t)(w >> 16);
-      }
-    }
-    const int ns = spill_len(spill, spill_off, sl, lane);
-    if (ns > 0) {   // the row's tail, after its ELL entries (ascending order continues)
-      const uint32_t *ent = spill + spill_off[sl] + kSpillHdr + spill[spill_off[sl] + lane];
-      for (int k = 0; k < ns; ++k) {
-        const uint32_t w = ent[k];
-        if (col) col[o + e + k] = s + Nc + (int64_t)(int16_t)(w & 0xFFFFu);
-        if (count) count[o + e + k] = (int32_t)(w >> 16);
-      }
-      e += ns;
-    }
-    if (sinkc[ir]) {
-      if (col) col[o + e] = nS;
-      if (count) count[o + e] = (int32_t)sinkc[ir];
-    }
-  }
-}
-
-cudaError_t launch_export(const mdp_model_t *m, int obj, int64_t *rowptr, int64_t *col,
-                          int32_t *count, void *R, cudaStream_t st) {
-  const int64_t rows = m->nS * m->A;
-  int64_t blocks = (rows + 255) / 256;
-  if (blocks > 8192) blocks = 8192;
-  if (blocks < 1) blocks = 1;
-  export_count_kernel<<<(unsigned)blocks, 256, 0, st>>>(m->nnz, m->sinkc, m->spill, m->spill_off, m->nS, m->A,
-                                                         m->A_pad, rowptr);
-  cudaError_t e = cudaMemsetAsync(rowptr + rows, 0, sizeof(int64_t), st);
-  if (e != cudaSuccess) return e;
-  // scan scratch: geometric series of tile counts
-  int64_t need = 0, nn = rows + 1;
-  while (nn > 1) { nn = (nn + 1023) / 1024; need += nn; }
-  int64_t *scratch = nullptr;
-  e = dev_alloc((void **)&scratch, sizeof(int64_t) * (size_t)(need + 1), st);
-  if (e != cudaSuccess) return e;
-  e = exclusive_scan(rowptr, rows + 1, scratch, st);
-  if (e != cudaSuccess) { dev_free(scratch, st); return e; }
-  int64_t nrow = m->n_slices * 32;
-  int64_t fb = (nrow + 255) / 256;
-  if (fb > 8192) fb = 8192;
-  const size_t esz = (m->precision == MDP_FP64_CHECK) ? 8 : 4;
-  if (m->precision == MDP_FP64_CHECK)
-    export_fill_kernel<double><<<(unsigned)fb, 256, 0, st>>>(
-        m->pool, m->slice_off, m->nnz, m->sinkc, m->spill, m->spill_off,
-        static_cast<const double *>(m->R) + (size_t)obj * m->rows_pad,
-        m->nS, m->Nc, m->A, m->A_pad, m->spw, m->n_slices, rowptr, col, count, (double *)R);
-  else
-    export_fill_kernel<float><<<(unsigned)fb, 256, 0, st>>>(
-        m->pool, m->slice_off, m->nnz, m->sinkc, m->spill, m->spill_off,
-        static_cast<const float *>(m->R) + (size_t)obj * m->rows_pad,
-        m->nS, m->Nc, m->A, m->A_pad, m->spw, m->n_slices, rowptr, col, count, (float *)R);
-  (void)esz;
-  e = cudaGetLastError();
-  dev_free(scratch, st);
-  return e;
 }
 
 }  // namespace mdpgb
