@@ -152,11 +152,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait: gives up after ~2 s of clock cycles so a lost arrival can
 // never hang the GPU; the caller reports the timeout through the error word.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit = 4000000000LL) {
   if (mbar_try_wait(bar, parity)) return true;   // usual case: the data is there
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > 4000000000LL) return false;
+    if (clock64() - t0 > limit) return false;
   }
   return true;
 }
@@ -319,6 +319,7 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
   const uint32_t ring0 = smem_u32(myring), bar0 = smem_u32(full + warp * kDepth);
   uint32_t m_off = 0, m_w = 0;   // lane l: metadata of my slice 32*(j/32) + l
   const uint64_t stream_policy = l2_evict_first();
+  const long long wait_limit = a.wait_cycles > 0 ? a.wait_cycles : 4000000000LL;   // ~2 s
 
   // issue(j, st): copy my j-th slice into stage st = j % kDepth (whole warp calls it)
   auto issue = [&](int j, int st) {
@@ -337,7 +338,9 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
       const uint32_t sbase = ring0 + (uint32_t)(st * pr.stage_bytes);
       const uint32_t fb = bar0 + 8u * (uint32_t)st;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier reads of the stage
-      mbar_expect_tx(fb, W * 128u);
+      // (a.test_extra_tx: bytes that never arrive, on CTA 0's first slice -- failure
+      // injection for tests)
+      mbar_expect_tx(fb, W * 128u + (j == 0 && warp == 0 && blockIdx.x == 0 ? a.test_extra_tx : 0u));
       if (W) bulk_g2s_stream(sbase, a.pool + (size_t)off * 32, W * 128u, fb, stream_policy);
     }
     __syncwarp();
@@ -377,11 +380,11 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
   int t_cur = s / Nc, t_end = (t_cur + 1) * Nc;
   bool chg = false;
   for (int j = 0; j < n_mine; ++j, s += s_step) {
-    if (!mbar_wait(bar0 + 8u * (uint32_t)st, phase)) {
+    if (!mbar_wait(bar0 + 8u * (uint32_t)st, phase, wait_limit)) {
       if (lane == 0) atomicOr(a.err, 1);
       // drain: wait (bounded) for the copies still in flight into my stages
       for (int jj = j + 1; jj < j + kDepth && jj < n_mine; ++jj)
-        mbar_wait(bar0 + 8u * (uint32_t)(jj % kDepth), (uint32_t)(jj / kDepth) & 1);
+        mbar_wait(bar0 + 8u * (uint32_t)(jj % kDepth), (uint32_t)(jj / kDepth) & 1, wait_limit);
       break;
     }
     const unsigned char *sb = myring + st * pr.stage_bytes;
@@ -1466,16 +1469,40 @@ static int ws_entry_bytes(int wcap, int smem_kb) {
   return (int)(e & ~127L);
 }
 
+// Launch shape of a sweep over `slices` slices (layer: of a layer of a backward
+// pass, a launch per layer).
+// A layer is as long as its longest warp, so the warp-per-slice kernel spreads
+// one over all the warps it can (a sweep gives a warp at least four slices, which
+// keeps its copies ahead of its sums).  Measured per layer, two chains: 200 slices
+// 6.3 us with four slices a warp, 3.3 with one; 1733 slices 7.6 and 3.4;
+// 12,800 slices 10.4 and 7.5.
+// For one state per slice that kernel also takes the layers up to kLayerSlices
+// slices per resident warp from the warp-specialized one, whose rounds of 31 slices
+// pay off above (us a layer of 10,000 / 40,000 slices, 32 actions: one objective, two
+// chains 6.1 / 14.9 against 7.6 / 14.5; three objectives, one chain 7.1 / 18.6
+// against 8.3 / 16.5, two chains 9.4 / 28.9 against 10.4 / 22.2).
+template <int NC>
+constexpr int kLayerSlices = NC <= 2 ? 7 : 3;
 template <typename RT, int NO, bool TWO = false>
-static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, PipeRange *pr, size_t *smem, int *blocks) {
+static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, bool layer, PipeRange *pr, size_t *smem, int *blocks) {
   pr->zero_second = 0;
-  if (a.spw == 1 && !a.small_ctas) {   // one state per slice: the warp-specialized sweep, any width
+  // the warp-per-slice kernel's stages
+  const int stage = stage_bytes_for(a.wcap);
+  const size_t warp_smem = 256 + (size_t)kWarps * kDepth * stage;
+  const bool ws = a.spw == 1 && !a.small_ctas;   // one state per slice: the warp-specialized sweep, any width
+  int per_sm = 0;
+  if (warp_smem <= 227 * 1024 && (!ws || (layer && sizeof(RT) == 4))) {
+    cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO, TWO>);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO, TWO>, 32 * kWarps, warp_smem);
+    if (e != cudaSuccess) return e;
+  }
+  if (ws && slices > (int64_t)num_sms() * per_sm * kWarps * kLayerSlices<VSet<RT, NO, TWO>::NC>) {
     pr->grouped = 2;
     pr->stage_bytes = ws_entry_bytes<RT, NO, TWO>(a.wcap, a.sweep_smem_kb);
     *smem = ws_hdr_bytes() + ws_old_bytes<RT, VSet<RT, NO, TWO>::NC>() + (size_t)kWsSlots * (ws_r_bytes<RT>(NO) + pr->stage_bytes);
     cudaError_t e = allow_max_smem((const void *)bellman_kernel_ws<RT, NO, TWO>);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel_ws<RT, NO, TWO>, 32 * (kWsCons + 1), *smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -1486,18 +1513,13 @@ static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, PipeRange *pr
     *blocks = (int)b;
     return cudaSuccess;
   }
-  pr->grouped = 0;   // several states per slice: the warp-per-slice kernel
-  pr->stage_bytes = stage_bytes_for(a.wcap);
-  *smem = 256 + (size_t)kWarps * kDepth * pr->stage_bytes;
-  if (*smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO, TWO>);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO, TWO>, 32 * kWarps, *smem);
-  if (e != cudaSuccess) return e;
+  pr->grouped = 0;   // the warp-per-slice kernel
+  pr->stage_bytes = stage;
+  *smem = warp_smem;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int64_t b = (int64_t)num_sms() * per_sm;
-  const int64_t want = (slices + 4 * kWarps - 1) / (4 * kWarps);   // >= 4 slices per warp
+  const int per_warp = layer ? 1 : 4;
+  const int64_t want = (slices + per_warp * kWarps - 1) / (per_warp * kWarps);
   if (b > want) b = want;
   if (b < 1) b = 1;
   *blocks = (int)b;
@@ -1596,7 +1618,7 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
   PipeRange pr;
   size_t smem = 0;
   int blocks = 1;
-  cudaError_t e = pipe_config<RT, NO>(a, a.n_slices, &pr, &smem, &blocks);
+  cudaError_t e = pipe_config<RT, NO>(a, a.n_slices, false, &pr, &smem, &blocks);
   if (e != cudaSuccess) return e;
   pr.sl_lo = 0;
   pr.sl_hi = a.n_slices;
@@ -1657,7 +1679,7 @@ static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, doub
   size_t smem = 0;
   int blocks = 1;
   // every layer has the same number of slices (up to one straddling slice)
-  cudaError_t e = pipe_config<RT, NO>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
+  cudaError_t e = pipe_config<RT, NO>(a, (a.Nc + a.spw - 1) / a.spw + 1, true, &pr0, &smem, &blocks);
   if (e != cudaSuccess) return e;
   VSet<RT, NO> v;
   Pk *t = static_cast<Pk *>(NO == 1 ? io.V[0] : io.table[0]);
@@ -1737,7 +1759,7 @@ static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, u
   PipeRange pr0;
   size_t smem = 0;
   int blocks = 1;
-  cudaError_t e = pipe_config<float, NO, true>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
+  cudaError_t e = pipe_config<float, NO, true>(a, (a.Nc + a.spw - 1) / a.spw + 1, true, &pr0, &smem, &blocks);
   if (e != cudaSuccess) return e;
   VSet<float, NO, true> v;
   auto *t = static_cast<VPack<float, 2 * NO> *>(io.table[0]);
