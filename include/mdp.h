@@ -362,8 +362,8 @@ mdp_status mdp_rollout(const mdp_env *env, const mdp_grid *grid, const mdp_actio
  * authors tuned threads per block by hand for each GPU, Sec. IV-D; here the
  * library does it).  A class is (actions padded to a power of two, modes, N
  * and cells rounded to powers of two, objectives, precision).  The shapes:
- * warps per CTA (4, 8) and fine-table words per slice (1536..4096) of the
- * group build kernel, the CTA size of the full-window kernel when the
+ * warps per CTA (4, 8: the kernel takes at most 4) and fine-table words per
+ * slice (1536..4096, the power of two below) of the group build kernel, the CTA size of the full-window kernel when the
  * calibration defers slices to it, and the shared memory of the
  * one-state-per-slice Bellman sweep (132, 160, 190 KiB: its slot size).
  * No choice changes a count, entry, R, value or policy -- only the speed.

@@ -168,9 +168,13 @@ static void rank_plan(ActionTable *t) {
   t->rank_mode = 2;
   for (int x = 0; x < 2; ++x) {
     std::vector<int> in(129, 0);
-    for (int i = 0; i < D[x]; ++i)
-      if (++in[(int)std::floor((double)T[x][i] * 128)] > 2) t->rank_mode = 3;
+    for (int i = 0; i < D[x]; ++i) in[(int)std::floor((double)T[x][i] * 128)]++;
+    for (int b = 1; b <= 128; ++b)
+      if (in[b] > 2) t->rank_mode = 3;
+    if (in[0] > 2) t->rank_trap = std::max(t->rank_trap, T[x][in[0] - 3]);
   }
+  if (t->rank_trap > 0x1p-24f) t->rank_mode = 3;
+  if (t->rank_mode == 3) t->rank_trap = 0.f;
 }
 
 mdp_status make_actions(const mdp_actions *ac, double lam, ActionTable *t, int *A_out) {

@@ -10,9 +10,10 @@
 // slots, 31 consumer warps each sum one slice, lane l row l, and take the max
 // and argmax with one redux.sync key per objective); warp per slice for
 // several states per slice (a segmented butterfly over the A_pad lanes of a
-// state); and the grouped sweep, kept for the batch's one-state-per-slice
-// class (four states per warp step, each lane summing four rows and keeping
-// a running max, a 3-step shuffle per state).  Residual max|V_{k+1} - V_k|
+// state) and for the smaller layers of backward passes; and the grouped sweep,
+// kept for the batch's one-state-per-slice class (four states per warp step,
+// each lane summing four rows and keeping a running max, a 3-step shuffle per
+// state).  Residual max|V_{k+1} - V_k|
 // is reduced on the device; a sweep whose predecessor met the tolerance
 // exits at once, so a fixed launch sequence needs no host round trip between
 // sweeps.

@@ -170,6 +170,13 @@ __device__ __forceinline__ void load_rank_tables(const BuildArgs &a, RankTables 
     int nx = 0, ny = 0;
     for (int i = 0; i < a.act.Dx; ++i) nx += (int)(a.act.Tx[i] * (float)B) < b + (upto ? 1 : 0) ? 1 : 0;
     for (int i = 0; i < a.act.Dy; ++i) ny += (int)(a.act.Ty[i] * (float)B) < b + (upto ? 1 : 0) ? 1 : 0;
+    if (a.act.rank_mode == 2 && b == 0) {   // all but the first bucket's last two (see ActionTable)
+      int mx = 0, my = 0;
+      for (int i = 0; i < a.act.Dx; ++i) mx += (int)(a.act.Tx[i] * (float)B) == 0 ? 1 : 0;
+      for (int i = 0; i < a.act.Dy; ++i) my += (int)(a.act.Ty[i] * (float)B) == 0 ? 1 : 0;
+      nx = max(mx - 2, 0);
+      ny = max(my - 2, 0);
+    }
     rt.L[0][b] = (uint8_t)(4 * nx);
     rt.L[1][b] = (uint8_t)(4 * ny);
   }
@@ -192,9 +199,10 @@ __device__ __forceinline__ int fine_coord(float u, int S, const RankTables &rt, 
   const float f = __saturatef(u - (t - kFloorMagic));
   int r = rt.L[axis][__float_as_uint(__fmul_rd(f, int_float((uint32_t)buckets)))] >> 2;
   const float *T = rt.T[axis] + 1;
-  if constexpr (MODE == 1) {
+  if constexpr (MODE <= 2) {
     while (r > 0 && T[r - 1] > f) --r;
-  } else {
+  }
+  if constexpr (MODE >= 2) {
     while (T[r] <= f) ++r;   // T[D] = 2 > f ends it
   }
   return (int)(__float_as_uint(t) - kFloorBits) * S + r;
@@ -957,7 +965,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         const float2 nx = unpack2(add2(tx, nmagic2)), ny = unpack2(add2(ty, nmagic2));
         const float fx0 = __saturatef(ux.x - nx.x), fx1 = __saturatef(ux.y - nx.y);
         const float fy0 = __saturatef(uy.x - ny.x), fy1 = __saturatef(uy.y - ny.y);
-        if constexpr (MODE == 1) {
+        if constexpr (MODE <= 2) {
           fmn = fminf(fmn, fminf(fx0, fy0));
           fmn = fminf(fmn, fminf(fx1, fy1));
         }
@@ -1013,7 +1021,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         count(ax, ay);
       }
       // (a trapped fraction of either state: both are counted again)
-      if (MODE == 1 && fmn < a.act.rank_trap) atomicOr(&sm.trap, ((on0 ? 1u : 0u) | (on1 ? 2u : 0u)) << (2 * p_t));
+      if (MODE <= 2 && fmn < a.act.rank_trap) atomicOr(&sm.trap, ((on0 ? 1u : 0u) | (on1 ? 2u : 0u)) << (2 * p_t));
       // extremes (min x, min y, -max x, -max y of both states) over the lanes of
       // the pair: halved in number with every exchange while there are several
       float v[8] = {mnx0, mny0, -mxx0, -mxy0, mnx1, mny1, -mxx1, -mxy1};
@@ -1096,7 +1104,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
       const int4 win = sm.st[qg].win;
       g.pitch = win.w >> 8;
       g.base = q * swords + (win.w & 255) + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
-      if ((MODE == 1 && ((sm.trap >> qg) & 1u)) || g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + g.pitch) {
+      if ((MODE <= 2 && ((sm.trap >> qg) & 1u)) || g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + g.pitch) {
         // outside the predicted window (or a trapped fraction): the exact table, if it fits
         const long long pitch = ((long long)g.gy + 1) | 1;
         if (((long long)g.gx + 1) * pitch > (long long)swords) {

@@ -83,7 +83,8 @@ struct ActionTable {
   // f's bucket) - [f < the last of them], right for every f >= rank_trap (the
   // first bucket may hold several thresholds below 2^-24, the displacements
   // that are zero up to rounding).  Mode 2: at most two per bucket, two
-  // comparisons after the thresholds below it.  Mode 3: a scan.
+  // comparisons after the thresholds below it; the first bucket's beyond two are
+  // taken as passed, right for every f >= rank_trap.  Mode 3: a scan.
   int32_t rank_mode, rank_buckets;
   float rank_trap;
   int32_t cx[kMaxActions], cy[kMaxActions];
@@ -270,7 +271,7 @@ struct SolveArgs {
 // Launch shapes chosen by the autotuner (mdp_autotune) per workload class;
 // every choice gives the same model and values bit for bit.
 struct Tuning {
-  int32_t build_warps = 8;       // warps (slices of a group) per CTA of the group build kernel
+  int32_t build_warps = 8;       // warps (slices of a group) per CTA of the group build kernel (8 is taken as 4)
   int32_t hist_cap = 2048;       // fine-table words per slice of that kernel
   int32_t threads = 256;         // CTA size of the full-window build kernel
   int32_t chunk = 1024;          // realizations staged per pass by that kernel

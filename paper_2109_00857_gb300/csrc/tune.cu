@@ -4,8 +4,8 @@
 //
 // A workload class is (actions padded to a power of two, modes, N and cells
 // rounded to powers of two, objectives, precision).  The shapes tuned are the
-// warps per CTA and the fine-table capacity of the warp-per-slice build
-// kernel, the CTA size of the full-window build kernel (when the calibration
+// warps per CTA (a group has at most four) and the fine-table capacity of the
+// group build kernel, the CTA size of the full-window build kernel (when the calibration
 // defers slices to it), and the shared memory of the one-state-per-slice
 // Bellman sweep (which sets its slot size).  None of them changes a count, an
 // entry, an R value, a value or a policy: the table only picks the fastest
