@@ -284,6 +284,20 @@ __device__ __forceinline__ void add_spill(const SolveArgs &a, int64_t sl, int la
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A CTA whose solve has timed out (its error word is set) gives up before it
+// waits on anything.  The word may be set while the CTA starts -- by the layer
+// that a dependent launch overlaps, or by another CTA of the same launch -- so
+// one thread reads it for all: threads that disagreed would leave the others
+// with barriers nobody initialized.  A dependent launch still waits for the
+// kernel before it, so that the stream's next work (a copy, a free) starts after
+// every layer has ended.  (CTAs without slices may leave without that wait: the
+// launch has one with slices, which does not.)  Synchronises the CTA.
+__device__ __forceinline__ bool cta_gives_up(const SolveArgs &a) {
+  if (!__syncthreads_or(threadIdx.x == 0 && *(volatile int *)a.err != 0)) return false;
+  pdl_wait();
+  return true;
+}
+
 template <typename RT, int NO, bool TWO = false>
 __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, int64_t b_lo,
                                              int64_t b_hi, const PipeRange &pr, unsigned char *sm,
@@ -301,8 +315,6 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
       if (v.res[o] && __longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
   if (!live) return;
-  if (*(volatile int *)a.err) return;   // an earlier launch of this solve timed out
-  if (a.work && k >= 1 && blockIdx.x == 0 && threadIdx.x == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
   uint64_t *full = reinterpret_cast<uint64_t *>(sm);   // [kWarps][kDepth]
   unsigned char *ring = sm + 256;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -311,7 +323,8 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
 
   if (tid < kWarps * kDepth) mbar_init(smem_u32(full + tid), 1);
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  __syncthreads();
+  if (cta_gives_up(a)) return;
+  if (a.work && k >= 1 && blockIdx.x == 0 && tid == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
   unsigned char *myring = ring + (size_t)warp * kDepth * pr.stage_bytes;
 
   // 32-bit slice/state indices (the host guarantees |S| + Nc < 2^31)
@@ -575,8 +588,6 @@ __device__ __forceinline__ void bellman_body_g(const SolveArgs &a, const VSet<RT
       if (v.res[o] && __longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
   if (!live) return;
-  if (*(volatile int *)a.err) return;   // an earlier launch of this solve timed out
-  if (a.work && k >= 1 && blockIdx.x == 0 && threadIdx.x == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
   uint64_t *full = reinterpret_cast<uint64_t *>(sm);   // [kWarpsG][kDepth]
   unsigned char *ring = sm + 256;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -585,7 +596,8 @@ __device__ __forceinline__ void bellman_body_g(const SolveArgs &a, const VSet<RT
 
   if (tid < kWarpsG * kDepth) mbar_init(smem_u32(full + tid), 1);
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  __syncthreads();
+  if (cta_gives_up(a)) return;
+  if (a.work && k >= 1 && blockIdx.x == 0 && tid == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
   const int slot = pr.stage_bytes / kGS;
   unsigned char *myring = ring + (size_t)warp * kDepth * pr.stage_bytes;
   const int n_groups = (int)((n_local + kGS - 1) / kGS);
@@ -901,7 +913,10 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
     if (lane == 0) s_cut[warp] = x;
   }
   __syncthreads();
-  if (*s_flag) return;
+  if (*s_flag) {   // (see cta_gives_up)
+    pdl_wait();
+    return;
+  }
   if (a.work && k >= 1 && blockIdx.x == 0 && tid == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
   const int64_t b_lo = s_cut[0], b_hi = s_cut[1];
   if (b_hi <= b_lo) return;
