@@ -123,9 +123,8 @@ typedef struct {
   int32_t chunk;           /* realizations staged per pass by that kernel; 0 = the autotuner's
                               choice, else 1024 */
   int32_t hist_cap;        /* fine-count table cells (32-bit words) per slice of the group
-                              build kernel, <= 6144 (the power of two below is used, a state
-                              of a slice taking its equal share); 0 = the autotuner's choice,
-                              else 2048; slices whose tables need more go to the
+                              build kernel, <= 6144; 0 = the autotuner's choice, else 2048;
+                              slices whose states' tables need more together go to the
                               full-window kernel (1 sends every sampled slice there) */
 } mdp_build_opts;
 

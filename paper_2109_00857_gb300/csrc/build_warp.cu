@@ -52,7 +52,7 @@ cudaError_t launch_coeff_moments(const float *Y, int nt, int N, int K, float2 *m
 // covers the model, so every group is taken).
 template <int KT, int SPW, int MODE>
 __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_kernel(const __grid_constant__ BuildArgs a, int words,
-                                                                                int chunk) {
+                                                                                int share, int chunk) {
   extern __shared__ __align__(16) unsigned char gsm[];
   GroupSmem &sm = *reinterpret_cast<GroupSmem *>(gsm);
   const int NW = blockDim.x >> 5, spw = SPW > 0 ? SPW : a.spw;
@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_ke
   // queue index g: chunk consecutive groups; the first slice of a group, or -1
   auto first_slice = [&](long long g) { return g < n_groups ? a.slice_begin + g * NW : (int64_t)-1; };
   if (first_slice(sm.next[0]) >= 0)
-    setup_slice<SPW, MODE>(a, sm, first_slice(sm.next[0]), setup_load<SPW>(a, first_slice(sm.next[0])), tabs, words);
+    setup_slice<SPW, MODE>(a, sm, first_slice(sm.next[0]), setup_load<SPW>(a, first_slice(sm.next[0])), tabs, words,
+                           share);
   __syncthreads();
   int left = chunk - 1;   // thread 0: groups of its last queue grab still to do
   for (int n = 1, par = 0;; ++n, par ^= 1) {
@@ -86,7 +87,8 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_ke
         left = chunk - 1;
       }
     }
-    group_slices<KT, SPW, true, MODE>(a, a.slice_begin + g * NW, sm, ext, tabs, words, next, par ^ 1, first_slice);
+    group_slices<KT, SPW, true, MODE>(a, a.slice_begin + g * NW, sm, ext, tabs, words, share, next, par ^ 1,
+                                        first_slice);
     __syncthreads();
   }
   warp_flush(a, sm);
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_ke
 
 template <int KT, int SPW, int MODE>
 static cudaError_t launch_g(const BuildArgs &a, int warps, int sms, cudaStream_t st) {
-  const int nw = group_warps(warps, a.spw), words = table_words(a.cap_bins, a.spw);
+  const int nw = group_warps(warps, a.spw), words = slice_words(a.cap_bins);
   const size_t smem = group_smem_bytes(0, a.cap_bins, a.spw, nw);
   cudaError_t e = allow_max_smem((const void *)build_group_kernel<KT, SPW, MODE>);
   if (e != cudaSuccess) return e;
@@ -110,7 +112,8 @@ static cudaError_t launch_g(const BuildArgs &a, int warps, int sms, cudaStream_t
   if (a.slices_per_warp > 0) chunk = 1;
   if (a.slices_per_warp > 0)   // bounded CTAs: a grid that covers every group
     blocks = (groups + a.slices_per_warp - 1) / a.slices_per_warp;
-  build_group_kernel<KT, SPW, MODE><<<(unsigned)std::max<int64_t>(blocks, 1), nw * 32, smem, st>>>(a, words, chunk);
+  build_group_kernel<KT, SPW, MODE><<<(unsigned)std::max<int64_t>(blocks, 1), nw * 32, smem, st>>>(
+      a, words, share_words(a.cap_bins, a.spw), chunk);
   return cudaGetLastError();
 }
 

@@ -27,7 +27,9 @@
 //            power-of-two table, so a realization outside the window corrupts
 //            only its own state's table, which is then counted again with the
 //            exact window (recount_state; rare: the windows hold 5 to 7 standard
-//            deviations, N = 5000 draws reach 4).
+//            deviations, N = 5000 draws reach 4).  A state's table is an equal
+//            share of the slice's words; a slice with a state that needs more has
+//            all its states' exact tables packed and counted again (pack_slice).
 //            Bound by issue and the LSU: 46 warp instructions and 11 LSU
 //            wavefronts per 32 (state, realization) items -- 17 FMAs, 4 lookups,
 //            3 wavefronts of shared counts, 4 of coefficients (the earlier
@@ -40,7 +42,7 @@
 //            bins stages its entry words in ascending order (sink folded), the
 //            group allocates its columns, and the rows are copied out with
 //            R(s,a) from the counts.
-// Slices whose exact fine tables do not fit are appended to a list that the
+// Slices whose exact fine tables do not fit together are appended to a list that the
 // CTA kernel of build_fp32.cu finishes with a full-window histogram and the
 // same landing offsets, so a slice's output does not depend on which kernel
 // built it.
@@ -184,7 +186,7 @@ __device__ __forceinline__ void load_rank_tables(const BuildArgs &a, RankTables 
 
 // floor(u) for |u| < kTame by adding 1.5 2^23 rounded down: the low mantissa
 // bits of the sum are floor(u).
-constexpr float kTame = 16384.f;
+constexpr float kTame = 1e6f;
 constexpr float kFloorMagic = 12582912.f;          // 1.5 2^23
 constexpr uint32_t kFloorBits = 0x4B400000u;       // its bits
 // An integer i < 2^23 as the float whose bits it is (i times the smallest
@@ -244,8 +246,10 @@ struct FineGeo {
 
 // ---- shared memory of a CTA ----
 // GroupSmem (the batched kernel: with the model's arguments), the extremes
-// [NW][NW spw] float4, then NW slices of `words` table words each; a state has
-// words / spw of them, a power of two.
+// [NW][NW spw] float4, then NW slices of `words` table words each.  A state
+// counts into its share of them, a power of two; a slice with a state that needs
+// more than its share has its states' exact tables packed into the whole
+// (pack_slice).
 // Per-warp totals, added to the model's counters by warp_flush().
 struct WarpAcc {
   unsigned long long samples, nnz, dom, maxrow;
@@ -257,7 +261,7 @@ struct WarpAcc {
 struct StateSetup {
   int4 win;              // the window's (xmin, ymin, gx, pitch << 8 | rotation); gy = pitch - 1
   uint32_t base, bytes, aN, aR, c0;
-  int32_t layer;         // time layer; -1: not sampled, -2: sampled, but tables have no words
+  int32_t layer;         // time layer; -1: not sampled
   int32_t kind;          // state_kind
   float vbx, vby;
 };
@@ -271,13 +275,14 @@ struct GroupSmem {
   unsigned int trap;               // states to count again (a fraction below act.rank_trap)
   StateSetup st[32];               // the group's states (last: only NW spw are laid out)
 };
-// Table words of a slice: the largest power of two <= cap_bins, if a state's
-// share of it is at least 16 words (else 0: no slice fits and all go to the
-// CTA kernel).
-__host__ __device__ constexpr int table_words(int cap_bins, int spw) {
-  int w = 1;
-  while (2 * w <= cap_bins) w *= 2;
-  return w >= 32 && w >= 16 * spw ? w : 0;
+// Table words of a slice (whole 16-byte vectors), and a state's share: the largest
+// power of two that leaves every state one, if that is at least 16 words (else
+// 0: nothing is counted at first, and every slice is packed).
+__host__ __device__ constexpr int slice_words(int cap_bins) { return (cap_bins + 3) & ~3; }
+__host__ __device__ constexpr int share_words(int cap_bins, int spw) {
+  int w = 16;
+  while (2 * w * spw <= cap_bins) w *= 2;
+  return w * spw <= cap_bins ? w : 0;
 }
 __host__ __device__ constexpr int group_warps(int warps, int spw) {
   const int most = 32 / spw < kGroupWarps ? 32 / spw : kGroupWarps;   // at most one state per lane
@@ -294,7 +299,7 @@ __host__ __device__ constexpr uint32_t group_head_bytes(uint32_t before, int spw
   return group_ext_offset(before, spw, nw) + 16u * (uint32_t)(nw * nw * spw) + 128u * (uint32_t)(nw * kStage);
 }
 inline size_t group_smem_bytes(uint32_t before, int cap_bins, int spw, int nw) {
-  return group_head_bytes(before, spw, nw) + (size_t)nw * 4u * (size_t)table_words(cap_bins, spw);
+  return group_head_bytes(before, spw, nw) + (size_t)nw * 4u * (size_t)slice_words(cap_bins);
 }
 // (lane 0 of each warp owns its totals)
 __device__ __forceinline__ void warp_clear(GroupSmem &sm) {
@@ -354,12 +359,12 @@ __device__ __forceinline__ float sqrt_fast(float x) {   // (where a window lies,
 }
 template <int SPW, int MODE>
 __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, int64_t sl0, const SetupLoads &ld,
-                                            uint32_t *tabs, int words) {
+                                            uint32_t *tabs, int words, int table) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
-  const int spw = SPW > 0 ? SPW : a.spw, per = 32 / spw, K = a.K, G = NW * spw, table = words / spw;
+  const int spw = SPW > 0 ? SPW : a.spw, per = 32 / spw, K = a.K, G = NW * spw;
   const int q = warp * spw + lane / per;   // state of the group
   const int64_t t = ld.t;
-  const bool sampled = ld.kind == KIND_SAMPLE, sample = sampled && table > 0;
+  const bool sample = ld.kind == KIND_SAMPLE;
   float mx = 0.f, my = 0.f, vx = 0.f, vy = 0.f;
   if (sample) {
     for (int k = lane % per; k < K; k += per) {
@@ -419,12 +424,12 @@ __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, i
   if (lane % per != 0) return;
   StateSetup st;
   st.win = make_int4(xmin, ymin, gx, pitch << 8 | rot);
-  st.layer = sample ? (int32_t)t : (sampled ? -2 : -1);
+  st.layer = sample ? (int32_t)t : -1;
   st.kind = ld.kind;
   st.vbx = ld.vb.x;
   st.vby = ld.vb.y;
   const uint32_t sc = table > 0 ? 0x80000000u / (uint32_t)(table / 2) : 0u;   // 2^32 / table
-  st.base = smem_u32(tabs + (size_t)q * table);
+  st.base = table > 0 ? smem_u32(tabs + warp * words + lane / per * table) : smem_u32(&sm.dummy[q]);
   st.bytes = 4u * (uint32_t)table;
   st.aN = (uint32_t)(Sx * pitch) * sc;
   st.aR = (uint32_t)pitch * (sc / 4);
@@ -515,6 +520,65 @@ __device__ __forceinline__ void prefix_table(uint32_t *P, const FineGeo &g) {
   __syncwarp();
   prefix_lines(P, g.gx, g.pitch, g.gy, 1);
   prefix_lines(P, g.gy, 1, g.gx, g.pitch);
+}
+
+// A state's extreme over all warps, component lane & 3 of (min x, min y, max x, max y)
+// (whole warp: lane (i, v) reads warp i's component v).
+__device__ __forceinline__ float state_extreme(const float4 *ext, int qg, int NW, int G) {
+  const int lane = threadIdx.x & 31, i = lane >> 2;
+  float m = i < NW ? reinterpret_cast<const float *>(&ext[i * G + qg])[lane & 3] : INFINITY;
+  m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
+  m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 8));
+  m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  return lane & 2 ? -m : m;
+}
+// The table of exactly a state's extremes (m of state_extreme), base unset.
+template <int MODE>
+__device__ __forceinline__ FineGeo exact_table(float m, int Sx, int Sy, const RankTables &rt, int buckets) {
+  const int lane = threadIdx.x & 31;
+  const int X = fine_coord<MODE>(m, lane & 1 ? Sy : Sx, rt, lane & 1, buckets);
+  FineGeo g;
+  g.xmin = __shfl_sync(0xffffffffu, X, 0);
+  g.ymin = __shfl_sync(0xffffffffu, X, 1);
+  g.gx = __shfl_sync(0xffffffffu, X, 2) - g.xmin + 1;
+  g.gy = __shfl_sync(0xffffffffu, X, 3) - g.ymin + 1;
+  g.pitch = (g.gy + 1) | 1;
+  g.base = 0;
+  return g;
+}
+__device__ __forceinline__ long long table_cells(const FineGeo &g) { return (long long)(g.gx + 1) * g.pitch; }
+
+// A slice with a state that needs more than its share of the table memory: the
+// states' exact tables back to back in all `words` words, each counted again (and
+// summed, if SUM) -- what a state leaves is another's.  Returns the table of the
+// lane's row (base -1 in every lane: they do not fit together).  Whole warp; rare.
+template <int KT, int MODE, bool SUM>
+__device__ __noinline__ FineGeo pack_slice(const BuildArgs &a, const GroupSmem &sm, const float4 *ext, int64_t sl,
+                                           uint32_t *grid, int words, int spw) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5, G = NW * spw;
+  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1, B = a.act.rank_buckets, q_l = lane / (32 / spw);
+  FineGeo mine{};
+  long long total = 0;
+  for (int q = 0; q < spw; ++q) {
+    if (sm.st[warp * spw + q].layer < 0) continue;
+    total += table_cells(exact_table<MODE>(state_extreme(ext, warp * spw + q, NW, G), Sx, Sy, sm.rt, B));
+  }
+  if (total > (long long)words) {
+    mine.base = -1;
+    return mine;
+  }
+  int base = 0;
+  for (int q = 0; q < spw; ++q) {
+    if (sm.st[warp * spw + q].layer < 0) continue;
+    FineGeo g = exact_table<MODE>(state_extreme(ext, warp * spw + q, NW, G), Sx, Sy, sm.rt, B);
+    const int cells = (int)table_cells(g);
+    g.base = base;
+    recount_state<KT, MODE>(a, sm.rt, sl * spw + q, g, grid + base, cells);
+    if (SUM) prefix_table(grid + base, g);
+    if (q == q_l) mine = g;
+    base += cells;
+  }
+  return mine;
 }
 
 // One row of a slice (lane l = row (q, a)) and its state's prefix table.
@@ -856,7 +920,8 @@ __device__ __forceinline__ SliceTotals write_small(const BuildArgs &a, const Ran
 // a.slice_end), NW = blockDim.x / 32 with NW SPW <= 32 states; every thread
 // calls it, and the caller synchronises before sm is used again.  ext: the
 // extremes' exchange, (min x, min y, -max x, -max y) of u.  tabs: the
-// slices' table memory (all zero on entry and on return), `words` words each.
+// slices' table memory (all zero on entry and on return), `words` words each,
+// `share` of them a state's.
 // SPW > 0: states per slice fixed at compile time; SPW == 0: runtime spw.
 // KT: see kPhi.  HYB: rows beyond row_cap keep their tail in the slice's spill
 // block; without it (the batched build, whose models keep no spill area) such
@@ -867,7 +932,8 @@ __device__ __forceinline__ SliceTotals write_small(const BuildArgs &a, const Ran
 // model and is to be set up here, else -1.
 template <int KT, int SPW, bool HYB, int MODE, class F>
 __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, GroupSmem &sm, float4 *ext,
-                                             uint32_t *tabs, int words, long long next_group, int par, F &&next_first) {
+                                             uint32_t *tabs, int words, int share, long long next_group, int par,
+                                             F &&next_first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int spw = SPW > 0 ? SPW : a.spw;
   const int K = KT > 0 ? KT : a.K;
@@ -878,7 +944,6 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   const float lam = a.lam;
   const int B = a.act.rank_buckets;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
-  const int swords = words / spw;   // a state's table (power of two)
   const int G = NW * spw;           // states of the group (even, <= 32)
 
   // ---- count: lane (i, p) states 2 p and 2 p + 1 of the group, realizations
@@ -911,7 +976,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         phy[1][k] = p1.y;
       }
     }
-    const uint32_t sc = swords > 0 ? 0x80000000u / (uint32_t)(swords / 2) : 0u;
+    const uint32_t sc = share > 0 ? 0x80000000u / (uint32_t)(share / 2) : 0u;
     const uint32_t bN = (uint32_t)Sy * sc, bR = sc / 4;
     const uint32_t t_base = smem_u32(&sm.rt.T[0][0]);
     const float lut = int_float(smem_u32(&sm.rt.L[0][0])), bk = int_float((uint32_t)B);
@@ -1060,7 +1125,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   uint32_t *stage = tabs - (size_t)(NW - warp) * (32 * kStage);   // the stages precede the tables
   RowGeo r{};
   r.hix = r.hiy = -1;
-  bool build = sl < a.slice_end, defer = false;
+  bool build = sl < a.slice_end, defer = false, pack = false;
   if (build) {
     const int q_l = lane / (32 / spw), a_l = lane % (32 / spw);
     r.kind = a_l < a.A ? sm.st[warp * spw + q_l].kind : (int)KIND_NONE;
@@ -1070,19 +1135,11 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
       const int64_t s = sl * spw + q;
       const int layer = sm.st[qg].layer;
       if (layer == -1) continue;   // not sampled
-      // the state's extremes over all warps: lane (i, v) warp i's component v
-      const int i = lane >> 2;
-      float m = i < NW ? reinterpret_cast<const float *>(&ext[i * G + qg])[lane & 3] : INFINITY;
-      m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
-      m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 8));
-      m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 16));
-      if (lane & 2) m = -m;
-      // no table, or non-finite or far velocities: the CTA kernel's path
-      if (layer < 0 || !__all_sync(0xffffffffu, m > -kTame && m < kTame)) {
+      const float m = state_extreme(ext, qg, NW, G);
+      if (!__all_sync(0xffffffffu, m > -kTame && m < kTame)) {   // non-finite or far velocities: the CTA kernel's path
         defer = true;
         continue;
       }
-      const int X = fine_coord<MODE>(m, lane & 1 ? Sy : Sx, sm.rt, lane & 1, B);
       const float mnx = __shfl_sync(0xffffffffu, m, 0), mny = __shfl_sync(0xffffffffu, m, 1);
       const float mxx = __shfl_sync(0xffffffffu, m, 2), mxy = __shfl_sync(0xffffffffu, m, 3);
       if (q == q_l && r.rows) {
@@ -1096,27 +1153,27 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         }
       }
       // the exact table inside the window (its pitch, its own origin)
-      FineGeo g;
-      g.xmin = __shfl_sync(0xffffffffu, X, 0);
-      g.ymin = __shfl_sync(0xffffffffu, X, 1);
-      g.gx = __shfl_sync(0xffffffffu, X, 2) - g.xmin + 1;
-      g.gy = __shfl_sync(0xffffffffu, X, 3) - g.ymin + 1;
+      FineGeo g = exact_table<MODE>(m, Sx, Sy, sm.rt, B);
       const int4 win = sm.st[qg].win;
+      const int exact_pitch = g.pitch;
       g.pitch = win.w >> 8;
-      g.base = q * swords + (win.w & 255) + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
+      g.base = q * share + (win.w & 255) + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
       if ((MODE <= 2 && ((sm.trap >> qg) & 1u)) || g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + g.pitch) {
         // outside the predicted window (or a trapped fraction): the exact table, if it fits
-        const long long pitch = ((long long)g.gy + 1) | 1;
-        if (((long long)g.gx + 1) * pitch > (long long)swords) {
-          defer = true;
+        g.pitch = exact_pitch;
+        g.base = q * share;
+        if (table_cells(g) > (long long)share) {
+          pack = true;
           continue;
         }
-        g.pitch = (int)pitch;
-        g.base = q * swords;
-        if (!defer) recount_state<KT, MODE>(a, sm.rt, s, g, grid + g.base, swords);
+        if (!defer && !pack) recount_state<KT, MODE>(a, sm.rt, s, g, grid + g.base, share);
       }
       if (q == q_l) r.g = g;
-      if (SPW != 1 && !defer) prefix_table(grid + g.base, g);
+      if (SPW != 1 && !defer && !pack) prefix_table(grid + g.base, g);
+    }
+    if (pack && !defer) {   // a state needs more than its share
+      r.g = pack_slice<KT, MODE, SPW != 1>(a, sm, ext, sl, grid, words, spw);
+      defer = r.g.base < 0;
     }
     if (defer) {   // too wide (or not finite): the CTA kernel builds the slice
       build = false;
@@ -1183,8 +1240,9 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   // the slice's tables are zero again
   __syncwarp();
   uint4 *p = reinterpret_cast<uint4 *>(grid);
-  for (int i = lane; i < words / 4; i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (next_first(g1) >= 0) setup_slice<SPW, MODE>(a, sm, next_first(g1), ld, tabs, words);
+  const int used = (pack ? words : share * spw) / 4;
+  for (int i = lane; i < used; i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (next_first(g1) >= 0) setup_slice<SPW, MODE>(a, sm, next_first(g1), ld, tabs, words, share);
 }
 
 }  // namespace mdpgb

@@ -19,7 +19,7 @@ constexpr uint32_t kArgsBytes = (uint32_t)((offsetof(BuildArgs, act) + offsetof(
 template <int KT, int SPW, int MODE>
 __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>)
     build_group_batch_kernel(const BuildArgs *__restrict__ items, const int64_t *__restrict__ prefix, int n,
-                             unsigned long long *work, int words, int spw) {
+                             unsigned long long *work, int words, int share, int spw) {
   extern __shared__ __align__(16) unsigned char gsm[];
   const BuildArgs &a = *reinterpret_cast<const BuildArgs *>(gsm);
   GroupSmem &sm = *reinterpret_cast<GroupSmem *>(gsm + kArgsBytes);
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>)
       for (int i = threadIdx.x; i < (int)(kArgsBytes / 16); i += blockDim.x) dst[i] = src[i];
       load_rank_tables(items[cur], sm.rt);
       __syncthreads();
-      setup_slice<SPW, MODE>(a, sm, (g - lo) * NW, setup_load<SPW>(a, (g - lo) * NW), tabs, words);
+      setup_slice<SPW, MODE>(a, sm, (g - lo) * NW, setup_load<SPW>(a, (g - lo) * NW), tabs, words, share);
       __syncthreads();
     }
     long long next = total;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>)
         left = (int)chunk - 1;
       }
     }
-    group_slices<KT, SPW, false, MODE>(a, (g - lo) * NW, sm, ext, tabs, words, next, par ^ 1,
+    group_slices<KT, SPW, false, MODE>(a, (g - lo) * NW, sm, ext, tabs, words, share, next, par ^ 1,
                                        [&](long long g1) {   // (another model's group is set up after the switch)
                                          return g1 >= lo && g1 < hi ? (int64_t)(g1 - lo) * NW : (int64_t)-1;
                                        });
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>)
 template <int KT, int SPW, int MODE>
 static cudaError_t launch_gb(const BuildArgs *items_d, const int64_t *prefix_d, int n, unsigned long long *work_d,
                              int cap, int spw, cudaStream_t st) {
-  const int nw = batch_group_slices(spw), words = table_words(cap, spw);
+  const int nw = batch_group_slices(spw), words = slice_words(cap);
   const size_t smem = group_smem_bytes(kArgsBytes, cap, spw, nw);
   cudaError_t e = allow_max_smem((const void *)build_group_batch_kernel<KT, SPW, MODE>);
   if (e != cudaSuccess) return e;
@@ -94,7 +94,7 @@ static cudaError_t launch_gb(const BuildArgs *items_d, const int64_t *prefix_d, 
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   build_group_batch_kernel<KT, SPW, MODE>
-      <<<num_sms() * per_sm, nw * 32, smem, st>>>(items_d, prefix_d, n, work_d, words, spw);
+      <<<num_sms() * per_sm, nw * 32, smem, st>>>(items_d, prefix_d, n, work_d, words, share_words(cap, spw), spw);
   return cudaGetLastError();
 }
 

@@ -133,7 +133,7 @@ struct alignas(16) BuildArgs {
   unsigned long long *cnt;
   int32_t chunk;             // realizations per staged pass (FP32 CTA kernel)
   int64_t slice_begin, slice_end;  // work range [begin, end)
-  int32_t cap_bins;          // fine-table words per slice of the group kernel (used: the power of two below)
+  int32_t cap_bins;          // fine-table words per slice of the group kernel
   const float2 *mom;         // [nt][K] mean and variance of a caller's coefficients (nullptr: drawn, mean 0)
   float coef_var[kMaxModes]; // variances of drawn coefficients
   uint32_t *defer;           // slices deferred by the group kernel ([n_slices])
