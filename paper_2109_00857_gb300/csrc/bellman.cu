@@ -971,6 +971,9 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
     int slot = 0;
     uint32_t ph = 0;   // phase parity of the slot's current round
     for (int r = 0;; ++r) {
+      // (a layer's consumers free no slot before the layer it overlaps has ended: the
+      // wait's limit starts then)
+      if (layered && r == kWsSlots) pdl_wait();
       if (r >= kWsSlots && !mbar_wait_suspend(empty0 + 8u * (uint32_t)slot, ph ^ 1u, wait_limit)) {
         if (lane == 0) atomicOr(a.err, 1);
         failed = true;
