@@ -281,7 +281,7 @@ extern "C" mdp_status mdp_batch_create(const mdp_batch_item *items_h, int32_t n,
     auto &C = b->cls[c];
     if (C.n == 0) continue;
     int per_sm = 1;
-    ce = prepare_bellman_batch(C.wcap, c, &C.stage_bytes, &per_sm);
+    ce = prepare_bellman_batch(C.wcap, c, b->layered, &C.stage_bytes, &per_sm);
     if (ce != cudaSuccess) return fail(cuda_fail(ce, "prepare_bellman_batch"));
     // two waves of CTAs share each sweep's recomputed slices (plus one entry
     // per model for the chunk remainders)

@@ -244,13 +244,17 @@ struct alignas(sizeof(RT) * (NC <= 2 ? NC : (NC <= 4 ? 4 : 8))) VPack {
 // streamed transition slices (each slice is copied once per sweep), each
 // with its own R, policy and residual slots; their values live in one
 // packed table (in = V_k, out = V_{k+1}; equal for the in-place layered
-// pass).  res[o] == nullptr marks a layered pass (no residual, no early
+// pass).  A layered pass has no res (no residual, no early
 // exit).
-// TWO: a two-chain layered pass (launch_two_chains): components NO..2 NO - 1
+// P == kChains: a two-chain layered pass (launch_two_chains): components NO..2 NO - 1
 // are a second chain of values with the same R, whose policy is not kept.
-template <typename RT, int NO, bool TWO = false>
+// (What a launch is for is fixed at compile time: chosen at run time, the full
+// sweeps took 2 to 3 % longer -- 100 x 100 cells, 60 layers, 32 actions 8.66 ms
+// against 8.47.)
+enum Pass : int { kSweep = 0, kLayer = 1, kChains = 2 };
+template <typename RT, int NO, Pass P = kSweep>
 struct VSet {
-  static constexpr int NC = TWO ? 2 * NO : NO;
+  static constexpr int NC = P == kChains ? 2 * NO : NO;
   const RT *R[NO];
   const VPack<RT, NC> *in;
   VPack<RT, NC> *out;
@@ -298,21 +302,20 @@ __device__ __forceinline__ bool cta_gives_up(const SolveArgs &a) {
   return true;
 }
 
-template <typename RT, int NO, bool TWO = false>
-__device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, int64_t b_lo,
+template <typename RT, int NO, Pass P = kSweep>
+__device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, NO, P> &v, int k, int64_t b_lo,
                                              int64_t b_hi, const PipeRange &pr, unsigned char *sm,
                                              double *wmax, int *wst_s) {
-  using Pk = VPack<RT, VSet<RT, NO, TWO>::NC>;
-  constexpr int NC = VSet<RT, NO, TWO>::NC;
-  const bool layered = v.res[0] == nullptr;
-  pdl_trigger();
-  if (!layered) pdl_wait();
+  using Pk = VPack<RT, VSet<RT, NO, P>::NC>;
+  constexpr int NC = VSet<RT, NO, P>::NC;
+  constexpr bool layered = P != kSweep;
+  if (layered) pdl_trigger();
   // objectives whose previous sweep met the tolerance are finished
   unsigned live = (1u << NO) - 1u;
-  if (k > 1) {
+  if (!layered && k > 1) {
 #pragma unroll
     for (int o = 0; o < NO; ++o)
-      if (v.res[o] && __longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
+      if (__longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
   if (!live) return;
   uint64_t *full = reinterpret_cast<uint64_t *>(sm);   // [kWarps][kDepth]
@@ -486,7 +489,7 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     }
   }
   if (chg_out && chg) chg_out[t_cur] = 1;
-  if (v.res[0]) {
+  if (!layered) {
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
       double ro = (sizeof(RT) == 4) ? (double)rf[o] : r[o];
@@ -540,8 +543,8 @@ __device__ __forceinline__ bool active_range(const SolveArgs &a, int k, PipeRang
   return true;
 }
 
-template <typename RT, int NO, bool TWO>
-__global__ void __launch_bounds__(32 * kWarps, TWO && NO == 3 ? 3 : 4) bellman_kernel(SolveArgs a, VSet<RT, NO, TWO> v,
+template <typename RT, int NO, Pass P>
+__global__ void __launch_bounds__(32 * kWarps, P == kChains && NO == 3 ? 3 : 4) bellman_kernel(SolveArgs a, VSet<RT, NO, P> v,
                                                                                    int k, PipeRange pr) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWarps * NO];
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(32 * kWarps, TWO && NO == 3 ? 3 : 4) bellman_k
   const int64_t per_cta = (total + gridDim.x - 1) / gridDim.x;
   const int64_t b_lo = pr.sl_lo + (int64_t)blockIdx.x * per_cta;
   const int64_t b_hi = min(pr.sl_hi, b_lo + per_cta);
-  bellman_body<RT, NO, TWO>(a, v, k, b_lo, b_hi, pr, sm, wmax, wst_s);
+  bellman_body<RT, NO, P>(a, v, k, b_lo, b_hi, pr, sm, wmax, wst_s);
 }
 
 // ---- grouped sweep: kGS states per warp step (models with A_pad = 32) ----
@@ -882,20 +885,19 @@ __device__ int64_t ws_cut(const SolveArgs &a, int64_t lo, int64_t hi, int64_t b,
   return h;
 }
 
-template <typename RT, int NO, bool TWO>
-__device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k,
+template <typename RT, int NO, Pass P>
+__device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<RT, NO, P> &v, int k,
                                                 const PipeRange &pr, unsigned char *sm, double *wmax, int *s_flag,
                                                 int64_t *s_cut) {
-  constexpr int NC = VSet<RT, NO, TWO>::NC;
+  constexpr int NC = VSet<RT, NO, P>::NC;
   using Pk = VPack<RT, NC>;
-  const bool layered = v.res[0] == nullptr;
-  pdl_trigger();
-  if (!layered) pdl_wait();
+  constexpr bool layered = P != kSweep;
+  if (layered) pdl_trigger();
   unsigned live = (1u << NO) - 1u;
-  if (k > 1) {
+  if (!layered && k > 1) {
 #pragma unroll
     for (int o = 0; o < NO; ++o)
-      if (v.res[o] && __longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
+      if (__longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
   if (!live) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -914,7 +916,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   }
   __syncthreads();
   if (*s_flag) {   // (see cta_gives_up)
-    pdl_wait();
+    if (layered) pdl_wait();
     return;
   }
   if (a.work && k >= 1 && blockIdx.x == 0 && tid == 0) a.work[k - 1] = (unsigned long long)(pr.sl_hi - pr.sl_lo);
@@ -1221,12 +1223,12 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
       }
     }
     if (chg_out && chg && lane == 0) chg_out[t_cur] = 1;
-    if (v.res[0] && lane == 0) {
+    if (!layered && lane == 0) {
 #pragma unroll
       for (int o = 0; o < NO; ++o) wmax[warp * NO + o] = (sizeof(RT) == 4) ? (double)rf[o] : rd[o];
     }
   }
-  if (v.res[0]) {
+  if (!layered) {
     __syncthreads();
 #pragma unroll
     for (int o = 0; o < NO; ++o) {   // thread o publishes objective o
@@ -1239,15 +1241,15 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   }
 }
 
-template <typename RT, int NO, bool TWO>
-__global__ void __launch_bounds__(32 * (kWsCons + 1), 1) bellman_kernel_ws(SolveArgs a, VSet<RT, NO, TWO> v, int k,
+template <typename RT, int NO, Pass P>
+__global__ void __launch_bounds__(32 * (kWsCons + 1), 1) bellman_kernel_ws(SolveArgs a, VSet<RT, NO, P> v, int k,
                                                                          PipeRange pr) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWsCons * NO];
   __shared__ int s_flag;
   __shared__ int64_t s_cut[2];
   if (a.lflags && k >= 1 && !active_range(a, k, pr, blockIdx.x == 0)) return;
-  bellman_body_ws<RT, NO, TWO>(a, v, k, pr, sm, wmax, &s_flag, s_cut);
+  bellman_body_ws<RT, NO, P>(a, v, k, pr, sm, wmax, &s_flag, s_cut);
 }
 
 // Plan of batched Jacobi sweep k (one block): per model, the slices of the
@@ -1370,9 +1372,10 @@ __device__ BatchCta layer_share(const BatchSolveItem *items, int n, int k, int G
 // Batched Jacobi sweep k over many models: CTA b works on ctas[b] (one
 // model's contiguous slice range, from the plan); each model stops on its
 // own residual.
+template <bool layered>
 __global__ void __launch_bounds__(32 * kWarps, 4) bellman_batch_kernel(const BatchSolveItem *items,
                                                                     const BatchCta *ctas, int k,
-                                                                    int stage_bytes, int layered, int n, int G) {
+                                                                    int stage_bytes, int n, int G) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWarps];
   __shared__ int wst_s[kWarps * kDepth];
@@ -1388,20 +1391,21 @@ __global__ void __launch_bounds__(32 * kWarps, 4) bellman_batch_kernel(const Bat
   pr.stage_bytes = stage_bytes;
   pr.zero_second = 0;
   pr.grouped = 0;
-  VSet<float, 1> v;
+  VSet<float, 1, layered ? kLayer : kSweep> v;
   v.R[0] = static_cast<const float *>(it.a.R);
   // Jacobi: ping-pong (sweep k reads Va when k is odd); layered: in place in Va
   v.in = reinterpret_cast<const VPack<float, 1> *>((layered || (k & 1)) ? it.Va : it.Vb);
   v.out = reinterpret_cast<VPack<float, 1> *>((layered || !(k & 1)) ? it.Va : it.Vb);
   v.pol[0] = it.policy;
   v.res[0] = layered ? nullptr : it.res;
-  bellman_body<float, 1>(it.a, v, layered ? 0 : k, pr.sl_lo, pr.sl_hi, pr, sm, wmax, wst_s);
+  bellman_body(it.a, v, layered ? 0 : k, pr.sl_lo, pr.sl_hi, pr, sm, wmax, wst_s);
 }
 
 // The same over models with one state per slice, by the grouped sweep.
+template <bool layered>
 __global__ void __launch_bounds__(32 * kWarpsG, 1) bellman_batch_kernel_g(const BatchSolveItem *items,
                                                                        const BatchCta *ctas, int k,
-                                                                       int stage_bytes, int layered, int n, int G) {
+                                                                       int stage_bytes, int n, int G) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWarpsG];
   __shared__ int wst_s[kWarpsG * kDepth * kGS];
@@ -1461,10 +1465,12 @@ cudaError_t launch_bellman_batch(const BatchSolveItem *items_d, int n, BatchCta 
   }
   if (grouped) {
     const size_t smem = 256 + (size_t)kWarpsG * kDepth * stage_bytes;
-    bellman_batch_kernel_g<<<G + n, 32 * kWarpsG, smem, st>>>(items_d, ctas_d, k, stage_bytes, layered, n, G);
+    auto *fn = layered ? bellman_batch_kernel_g<true> : bellman_batch_kernel_g<false>;
+    fn<<<G + n, 32 * kWarpsG, smem, st>>>(items_d, ctas_d, k, stage_bytes, n, G);
   } else {
     const size_t smem = 256 + (size_t)kWarps * kDepth * stage_bytes;
-    bellman_batch_kernel<<<G + n, 32 * kWarps, smem, st>>>(items_d, ctas_d, k, stage_bytes, layered, n, G);
+    auto *fn = layered ? bellman_batch_kernel<true> : bellman_batch_kernel<false>;
+    fn<<<G + n, 32 * kWarps, smem, st>>>(items_d, ctas_d, k, stage_bytes, n, G);
   }
   return cudaGetLastError();
 }
@@ -1476,21 +1482,23 @@ cudaError_t launch_finalize_batch(const BatchSolveItem *items_d, int n, int laye
 
 bool bellman_grouped_fits(int spw, int wcap) { return spw == 1 && grouped_smem(wcap) <= kGroupedSmemMax; }
 
-cudaError_t prepare_bellman_batch(int wcap, int grouped, int *stage_bytes, int *per_sm) {
+cudaError_t prepare_bellman_batch(int wcap, int grouped, int layered, int *stage_bytes, int *per_sm) {
   if (grouped) {
     *stage_bytes = kGS * slot_bytes_g(wcap);
     const size_t smem = grouped_smem(wcap);
     if (smem > kGroupedSmemMax) return cudaErrorInvalidConfiguration;
-    cudaError_t e = allow_max_smem((const void *)bellman_batch_kernel_g);
+    auto *fn = layered ? bellman_batch_kernel_g<true> : bellman_batch_kernel_g<false>;
+    cudaError_t e = allow_max_smem((const void *)fn);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, bellman_batch_kernel_g, 32 * kWarpsG, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, 32 * kWarpsG, smem);
   }
   *stage_bytes = stage_bytes_for(wcap);
   const size_t smem = 256 + (size_t)kWarps * kDepth * (*stage_bytes);
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = allow_max_smem((const void *)bellman_batch_kernel);
+  auto *fn = layered ? bellman_batch_kernel<true> : bellman_batch_kernel<false>;
+  cudaError_t e = allow_max_smem((const void *)fn);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, bellman_batch_kernel, 32 * kWarps, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, 32 * kWarps, smem);
 }
 
 // stats_d[0] = sweeps, [1] = residual of the last sweep.  Copies the final
@@ -1524,16 +1532,16 @@ __global__ void finalize_kernel(const unsigned long long *res, int max_sweeps, d
 // same memory make shorter rounds and are slower.)
 constexpr size_t kWsSmem = 160 * 1024;
 
-template <typename RT, int NO, bool TWO>
+template <typename RT, int NO, Pass P>
 static int ws_entry_bytes(int wcap, int smem_kb) {
   const size_t budget = smem_kb > 0 ? (size_t)smem_kb * 1024 : kWsSmem;
-  const long per_slot = (long)((budget - ws_hdr_bytes() - ws_old_bytes<RT, VSet<RT, NO, TWO>::NC>()) / kWsSlots) - ws_r_bytes<RT>(NO);
+  const long per_slot = (long)((budget - ws_hdr_bytes() - ws_old_bytes<RT, VSet<RT, NO, P>::NC>()) / kWsSlots) - ws_r_bytes<RT>(NO);
   long e = std::max<long>(per_slot, (long)wcap * 128);
   return (int)(e & ~127L);
 }
 
-// Launch shape of a sweep over `slices` slices (layer: of a layer of a backward
-// pass, a launch per layer).
+// Launch shape of a sweep over `slices` slices, or of a layer of a backward pass (a
+// launch per layer).
 // A layer is as long as its longest warp, so the warp-per-slice kernel spreads
 // one over all the warps it can (a sweep gives a warp at least four slices, which
 // keeps its copies ahead of its sums).  Measured per layer, two chains: 200 slices
@@ -1546,8 +1554,9 @@ static int ws_entry_bytes(int wcap, int smem_kb) {
 // against 8.3 / 16.5, two chains 9.4 / 28.9 against 10.4 / 22.2).
 template <int NC>
 constexpr int kLayerSlices = NC <= 2 ? 7 : 3;
-template <typename RT, int NO, bool TWO = false>
-static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, bool layer, PipeRange *pr, size_t *smem, int *blocks) {
+template <typename RT, int NO, Pass P>
+static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, PipeRange *pr, size_t *smem, int *blocks) {
+  constexpr bool layer = P != kSweep;
   pr->zero_second = 0;
   // the warp-per-slice kernel's stages
   const int stage = stage_bytes_for(a.wcap);
@@ -1555,18 +1564,18 @@ static cudaError_t pipe_config(const SolveArgs &a, int64_t slices, bool layer, P
   const bool ws = a.spw == 1 && !a.small_ctas;   // one state per slice: the warp-specialized sweep, any width
   int per_sm = 0;
   if (warp_smem <= 227 * 1024 && (!ws || (layer && sizeof(RT) == 4))) {
-    cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO, TWO>);
+    cudaError_t e = allow_max_smem((const void *)bellman_kernel<RT, NO, P>);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO, TWO>, 32 * kWarps, warp_smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel<RT, NO, P>, 32 * kWarps, warp_smem);
     if (e != cudaSuccess) return e;
   }
-  if (ws && slices > (int64_t)num_sms() * per_sm * kWarps * kLayerSlices<VSet<RT, NO, TWO>::NC>) {
+  if (ws && slices > (int64_t)num_sms() * per_sm * kWarps * kLayerSlices<VSet<RT, NO, P>::NC>) {
     pr->grouped = 2;
-    pr->stage_bytes = ws_entry_bytes<RT, NO, TWO>(a.wcap, a.sweep_smem_kb);
-    *smem = ws_hdr_bytes() + ws_old_bytes<RT, VSet<RT, NO, TWO>::NC>() + (size_t)kWsSlots * (ws_r_bytes<RT>(NO) + pr->stage_bytes);
-    cudaError_t e = allow_max_smem((const void *)bellman_kernel_ws<RT, NO, TWO>);
+    pr->stage_bytes = ws_entry_bytes<RT, NO, P>(a.wcap, a.sweep_smem_kb);
+    *smem = ws_hdr_bytes() + ws_old_bytes<RT, VSet<RT, NO, P>::NC>() + (size_t)kWsSlots * (ws_r_bytes<RT>(NO) + pr->stage_bytes);
+    cudaError_t e = allow_max_smem((const void *)bellman_kernel_ws<RT, NO, P>);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel_ws<RT, NO, TWO>, 32 * (kWsCons + 1), *smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bellman_kernel_ws<RT, NO, P>, 32 * (kWsCons + 1), *smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t b = (int64_t)num_sms() * per_sm;
@@ -1631,8 +1640,8 @@ __global__ void finalize_multi_kernel(const double *stats_base, size_t blk, int 
 
 // pdl: the launch may start while the previous kernel of the stream finishes
 // (the layers of a layered pass).
-template <typename RT, int NO, bool TWO>
-static void launch_sweep(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, const PipeRange &pr, int blocks,
+template <typename RT, int NO, Pass P>
+static void launch_sweep(const SolveArgs &a, const VSet<RT, NO, P> &v, int k, const PipeRange &pr, int blocks,
                          size_t smem, cudaStream_t st, bool pdl = false) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)blocks);
@@ -1644,8 +1653,8 @@ static void launch_sweep(const SolveArgs &a, const VSet<RT, NO, TWO> &v, int k, 
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (pr.grouped == 2) cudaLaunchKernelEx(&cfg, bellman_kernel_ws<RT, NO, TWO>, a, v, k, pr);
-  else cudaLaunchKernelEx(&cfg, bellman_kernel<RT, NO, TWO>, a, v, k, pr);
+  if (pr.grouped == 2) cudaLaunchKernelEx(&cfg, bellman_kernel_ws<RT, NO, P>, a, v, k, pr);
+  else cudaLaunchKernelEx(&cfg, bellman_kernel<RT, NO, P>, a, v, k, pr);
 }
 
 // Objective o's status block: stats_d + o*(4 + max_sweeps) holds sweeps,
@@ -1681,7 +1690,7 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
   PipeRange pr;
   size_t smem = 0;
   int blocks = 1;
-  cudaError_t e = pipe_config<RT, NO>(a, a.n_slices, false, &pr, &smem, &blocks);
+  cudaError_t e = pipe_config<RT, NO, kSweep>(a, a.n_slices, &pr, &smem, &blocks);
   if (e != cudaSuccess) return e;
   pr.sl_lo = 0;
   pr.sl_hi = a.n_slices;
@@ -1742,9 +1751,9 @@ static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, doub
   size_t smem = 0;
   int blocks = 1;
   // every layer has the same number of slices (up to one straddling slice)
-  cudaError_t e = pipe_config<RT, NO>(a, (a.Nc + a.spw - 1) / a.spw + 1, true, &pr0, &smem, &blocks);
+  cudaError_t e = pipe_config<RT, NO, kLayer>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
   if (e != cudaSuccess) return e;
-  VSet<RT, NO> v;
+  VSet<RT, NO, kLayer> v;
   Pk *t = static_cast<Pk *>(NO == 1 ? io.V[0] : io.table[0]);
   v.in = t;
   v.out = t;
@@ -1822,9 +1831,9 @@ static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, u
   PipeRange pr0;
   size_t smem = 0;
   int blocks = 1;
-  cudaError_t e = pipe_config<float, NO, true>(a, (a.Nc + a.spw - 1) / a.spw + 1, true, &pr0, &smem, &blocks);
+  cudaError_t e = pipe_config<float, NO, kChains>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
   if (e != cudaSuccess) return e;
-  VSet<float, NO, true> v;
+  VSet<float, NO, kChains> v;
   auto *t = static_cast<VPack<float, 2 * NO> *>(io.table[0]);
   v.in = t;
   v.out = t;

@@ -304,7 +304,7 @@ struct BatchCta {
 // grouped: models with one state per slice whose width fits the grouped
 // sweep (bellman_grouped_fits); else the warp-per-slice sweep
 bool bellman_grouped_fits(int spw, int wcap);
-cudaError_t prepare_bellman_batch(int wcap, int grouped, int *stage_bytes, int *per_sm);
+cudaError_t prepare_bellman_batch(int wcap, int grouped, int layered, int *stage_bytes, int *per_sm);
 // sweep k: a plan launch spreads the models' recomputed slices over G + n
 // CTA entries (ctas_d), then the sweep launch; n <= 1023 models
 // layered: step k (1..max nt) is the in-place pass over layer nt - k of
