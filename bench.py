@@ -98,12 +98,12 @@ def bellman_bytes_per_sweep(info, nS, n_obj=1, chains=0):
 
 def solve_passes(st, env, jacobi=True):
     """(passes over P in full-sweep units, chains per pass, launches) of one
-    solve: a Jacobi run that ends in sweep nt + 1 comes from one backward pass
+    solve: a Jacobi run that ends in sweep nt or nt + 1 comes from one backward pass
     of two chains (two backups per state and action; one launch per layer and
     a finalize); others from sweeps over the layers that changed (nt + 1
     launches, those after convergence exiting at once, and a finalize)."""
     full = st.backups / (env.nS * env.A)
-    if jacobi and st.sweeps == env.nt + 1 and st.backups == 2 * env.nS * env.A:
+    if jacobi and st.sweeps >= env.nt and st.backups == 2 * env.nS * env.A:
         return 1.0, 2, env.nt + 1
     return full, 0 if jacobi else 1, env.nt + 2 if jacobi else env.nt
 

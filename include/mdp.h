@@ -187,10 +187,10 @@ typedef enum {
                                 * whose successor layer t+1 changed in the previous sweep; every
                                 * other state has V_{k+1}(s) = V_k(s) exactly, so iterates, policy,
                                 * residuals and sweep count equal MDP_SOLVE_JACOBI_FULL bit for bit.
-                                * A cold-started FP32 run that is certain to end in sweep nt + 1 (two
-                                * backward chains over the layers bound every earlier residual from
-                                * below) is returned from those chains, without sweeping: the same V,
-                                * policy, sweeps and residual bit for bit */
+                                * A cold-started FP32 run that is certain to end in sweep nt or nt + 1
+                                * (two backward chains over the layers bound every earlier residual
+                                * from below) is returned from those chains, without sweeping: the
+                                * same V, policy, sweeps and residual bit for bit */
   MDP_SOLVE_LAYERED = 1,      /* one backward pass over time layers t = nt-1..0 (same fixed point) */
   MDP_SOLVE_JACOBI_FULL = 2,  /* Jacobi sweeps over every state in every sweep */
   MDP_SOLVE_WARM = 16         /* flag, OR-ed into MDP_SOLVE_JACOBI or _JACOBI_FULL of mdp_solve

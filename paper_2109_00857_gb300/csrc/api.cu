@@ -212,11 +212,14 @@ mdp_status make_actions(const mdp_actions *ac, double lam, ActionTable *t, int *
   return MDP_OK;
 }
 
-struct Pinned {
+struct Pinned {   // p[0 .. CNT_N): a build's counters; p[CNT_N]: SolveStop::host
   unsigned long long *p = nullptr;
-  Pinned() { cudaMallocHost((void **)&p, sizeof(unsigned long long) * CNT_N * 2); }
+  unsigned int calls = 0;
+  Pinned() { cudaMallocHost((void **)&p, sizeof(unsigned long long) * (CNT_N + 1)); if (p) p[CNT_N] = 0; }
   ~Pinned() { if (p) cudaFreeHost(p); }
 };
+static thread_local Pinned pin;
+static SolveStop solve_stop() { return SolveStop{pin.p ? reinterpret_cast<unsigned int *>(pin.p + CNT_N) : nullptr, ++pin.calls}; }
 
 static void free_model_memory(mdp_model_t *m, cudaStream_t st) {
   dev_free(m->pool, st);
@@ -564,7 +567,6 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
     *out = m;
     return MDP_OK;
   }
-  static thread_local Pinned pin;
   if (!pin.p) return fail(cuda_fail(cudaErrorMemoryAllocation, "cudaMallocHost"));
   const unsigned long long *c = pin.p;
   for (int attempt = 0;; ++attempt) {
@@ -822,7 +824,7 @@ static mdp_status solve_sweeps(mdp_model m, int32_t n, const int32_t *objs, int3
   cudaEventCreate(&e1);
   cudaEventRecord(e0, st);
   if (ce == cudaSuccess) {
-    if (jac) ce = launch_jacobi_multi(a, m->precision, max_sweeps, io, sd, st);
+    if (jac) ce = launch_jacobi_multi(a, m->precision, max_sweeps, io, sd, solve_stop(), st);
     else ce = launch_layered_multi(a, m->precision, m->nt, io, sd, st);
   }
   cudaEventRecord(e1, st);
@@ -834,7 +836,8 @@ static mdp_status solve_sweeps(mdp_model m, int32_t n, const int32_t *objs, int3
     ce = cudaMemcpyAsync(work.data(), a.work, sizeof(unsigned long long) * max_sweeps, cudaMemcpyDeviceToHost, st);
   dev_free(sd, st);
   if (tables) dev_free(tables, st);
-  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+  const cudaError_t se = cudaStreamSynchronize(st);   // (launched sweeps may still store to the pinned word)
+  if (ce == cudaSuccess) ce = se;
   float ms = 0.f;
   if (ce == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
@@ -865,18 +868,17 @@ static mdp_status solve_sweeps(mdp_model m, int32_t n, const int32_t *objs, int3
 
 // A cold-started FP32 Jacobi run by two backward chains (bellman.cu): fills V,
 // policy and stats of every objective whose run is certain to end in sweep
-// nt + 1, sets done[o] for those and leaves the others to the sweeps.
+// nt or nt + 1, sets done[o] for those and leaves the others to the sweeps.
 static mdp_status solve_two_chains(mdp_model m, int32_t n, const int32_t *objs, double tol, void *const *V,
                                    int16_t *const *policy, void *stream, mdp_solve_stats *stats, bool *done,
                                    float *ms) {
   cudaStream_t st = (cudaStream_t)stream;
   const int nc = n == 1 ? 2 : (n == 2 ? 4 : 8);   // packed components per state
-  const size_t tbytes = sizeof(float) * (size_t)nc * (size_t)(m->nS + 1);
-  const size_t nd = (size_t)n * m->nt;   // residual bounds, then the error word
-  Scratch tab(st), dd(st);
+  const size_t state = sizeof(float) * (size_t)nc;
+  const size_t table = state * (size_t)(m->nS + 1), words = (table + 31) & ~(size_t)31;   // (then the words)
+  Scratch tab(st);
   EventPair ev;
-  MDP_CUDA_TRY(dev_alloc(&tab.p, tbytes, st));
-  MDP_CUDA_TRY(dev_alloc(&dd.p, sizeof(unsigned int) * (nd + 1), st));
+  MDP_CUDA_TRY(dev_alloc(&tab.p, words + chain_words_bytes(m->nt), st));
   SolveIO io{};
   io.n = n;
   for (int o = 0; o < n; ++o) {
@@ -885,33 +887,37 @@ static mdp_status solve_two_chains(mdp_model m, int32_t n, const int32_t *objs, 
     io.policy[o] = policy[o];
   }
   io.table[0] = tab.p;
-  MDP_CUDA_TRY(cudaMemsetAsync(tab.p, 0, tbytes, st));
-  MDP_CUDA_TRY(cudaMemsetAsync(dd.p, 0, sizeof(unsigned int) * (nd + 1), st));
+  // (a layer's values are written before they are read; rows without successors
+  // read the last entry)
+  char *base = static_cast<char *>(tab.p);
+  MDP_CUDA_TRY(cudaMemsetAsync(base + table - state, 0, words - table + state + chain_words_bytes(m->nt), st));
+  ChainWords *w = reinterpret_cast<ChainWords *>(base + words);
   SolveArgs a = solve_args(m, io, tol);
-  unsigned int *d = static_cast<unsigned int *>(dd.p);
-  a.err = reinterpret_cast<int *>(d + nd);
+  a.err = &w->err;
   take_test_injection(a);
   cudaEventRecord(ev.e[0], st);
-  MDP_CUDA_TRY(launch_two_chains(a, m->nt, io, d, st));
+  cudaError_t ce = launch_two_chains(a, m->nt, io, w, solve_stop(), st);
   cudaEventRecord(ev.e[1], st);
-  std::vector<unsigned int> hd(nd + 1);
-  MDP_CUDA_TRY(cudaMemcpyAsync(hd.data(), d, sizeof(unsigned int) * (nd + 1), cudaMemcpyDeviceToHost, st));
-  MDP_CUDA_TRY(cudaStreamSynchronize(st));
-  if (hd[nd]) {
+  std::vector<char> hw(chain_head_bytes(m->nt));
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(hw.data(), w, hw.size(), cudaMemcpyDeviceToHost, st);
+  const cudaError_t se = cudaStreamSynchronize(st);   // (launched layers may still store to the pinned word)
+  if (ce != cudaSuccess || se != cudaSuccess) return cuda_fail(ce != cudaSuccess ? ce : se, "launch_two_chains");
+  ChainWords *h = reinterpret_cast<ChainWords *>(hw.data());
+  if (h->err & kErrTimeout) {
     set_error("a bounded device wait expired in the Bellman pipeline");
     return MDP_ERR_TIMEOUT;
   }
   cudaEventElapsedTime(ms, ev.e[0], ev.e[1]);
+  const uint32_t *above = chain_above(h);
   for (int o = 0; o < n; ++o) {
-    done[o] = true;
-    for (int t = 0; t < m->nt && done[o]; ++t) {
-      float x;
-      memcpy(&x, &hd[(size_t)o * m->nt + t], sizeof(x));
-      done[o] = (double)x > tol;   // sweep nt - t does not stop the run
-    }
+    done[o] = (h->err & kErrNotProven) == 0;
+    for (int t = 1; t < m->nt && done[o]; ++t) done[o] = (above[t] >> o & 1u) != 0;   // sweep nt - t does not stop the run
     if (done[o] && stats) {
-      stats[o].sweeps = m->nt + 1;
-      stats[o].residual = 0.0;
+      const bool last = (above[0] >> o & 1u) != 0;   // nor does sweep nt
+      float d0;
+      memcpy(&d0, &h->first[o], sizeof(d0));
+      stats[o].sweeps = last ? m->nt + 1 : m->nt;
+      stats[o].residual = last ? 0.0 : (double)d0;
       stats[o].solve_ms = *ms;
       stats[o].backups = 2 * m->nS * m->A;   // one per chain
     }

@@ -18,6 +18,7 @@
 // exits at once, so a fixed launch sequence needs no host round trip between
 // sweeps.
 #include <algorithm>
+#include <cmath>
 #include <cfloat>
 
 #include "build_common.cuh"
@@ -211,6 +212,14 @@ struct PipeRange {
   int64_t s_lo, s_hi;     // states whose V this launch writes
   int stage_bytes;        // bytes per stage
   int zero_second;        // two-chain pass: the second chain's values of this layer are 0
+  // two-chain pass: this layer's slots, layer t + 1's (nullptr: there is none) and
+  // where their union goes; the largest float <= SolveArgs::tol
+  ChainSlot *slots;
+  const ChainSlot *next_slots;
+  uint32_t *next_above;
+  int first;              // layer 0: the slots take the largest differences themselves, too
+  float tol;
+  SolveStop stop;
   int grouped;            // 1: bellman_body_g (kGS states per warp step, batched sweeps); 2: bellman_kernel_ws
                           // (stage_bytes = entry bytes per slot)
 };
@@ -281,15 +290,16 @@ __device__ __forceinline__ void add_spill(const SolveArgs &a, int64_t sl, int la
   }
 }
 
-// Programmatic dependent launch (the layered passes): a layer's kernel may
-// start while the previous layer's finishes -- its prologue and first entry
-// copies touch nothing that kernel writes -- and waits here before it reads V.
+// Programmatic dependent launch: a layer's kernel may start while the previous
+// layer's finishes -- its prologue and first entry copies touch nothing that
+// kernel writes -- and waits here before it reads V.  A sweep waits at once (it
+// starts from the previous one's residuals): that hides a launch's latency alone.
 // Both return at once in kernels launched without the attribute.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// A CTA whose solve has timed out (its error word is set) gives up before it
-// waits on anything.  The word may be set while the CTA starts -- by the layer
+// A CTA whose solve has timed out or proven nothing (its error word is set) gives
+// up before it waits on anything.  The word may be set while the CTA starts -- by the layer
 // that a dependent launch overlaps, or by another CTA of the same launch -- so
 // one thread reads it for all: threads that disagreed would leave the others
 // with barriers nobody initialized.  A dependent launch still waits for the
@@ -300,6 +310,58 @@ __device__ __forceinline__ bool cta_gives_up(const SolveArgs &a) {
   if (!__syncthreads_or(threadIdx.x == 0 && *(volatile int *)a.err != 0)) return false;
   pdl_wait();
   return true;
+}
+
+// A two-chain pass ends as soon as it proves nothing for any objective.  Every CTA
+// says in a slot of its layer for which objectives it saw differences above tol
+// (the CTAs spread over the slots: 608 stores to one address took 6 us a layer,
+// more than the layer itself).  The first warp of the next layer's launch unites
+// the slots -- the loads are issued with the first gathers and used at the end,
+// so no layer waits for them -- and, where there is nothing, tells the layers
+// still to start, by the error word, and the host, which stops launching them.
+__device__ __forceinline__ uint32_t chains_look(const PipeRange &pr) {   // one warp
+  return pr.next_slots ? __ldcg(&pr.next_slots[threadIdx.x & 31].above) : 1u;
+}
+__device__ __forceinline__ void chains_tell(const SolveArgs &a, const PipeRange &pr, uint32_t above) {
+  if (!pr.next_slots) return;
+  above = __reduce_or_sync(0xffffffffu, above);
+  if ((threadIdx.x & 31) != 0) return;
+  *pr.next_above = above;
+  if (above != 0u) return;
+  atomicOr(a.err, kErrNotProven);
+  if (pr.stop.host) *(volatile unsigned int *)pr.stop.host = pr.stop.token;
+}
+// A sweep that finds nothing left to do: no more need be launched.
+__device__ __forceinline__ void tell_host(const PipeRange &pr) {
+  if (pr.stop.host && blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned int *)pr.stop.host = pr.stop.token;
+}
+// Publishes the largest differences m[o] of the chains over a CTA's states (wmax:
+// shared memory for a value per warp and objective; all threads call it).  In
+// floats and their bits: FP64 maxima like the sweeps' would cost 2 us a layer.
+// (It takes 0.3 us of a layer of 40,000 slices, 14.9 us before; told by each warp as
+// soon as it is seen, 0.9 us.)
+template <int NO, int WARPS>
+__device__ __forceinline__ void chains_publish(const PipeRange &pr, const float (&m)[NO], double *wmax) {
+  unsigned int *top = reinterpret_cast<unsigned int *>(wmax);
+  const int tid = threadIdx.x, warp = tid >> 5;
+#pragma unroll
+  for (int o = 0; o < NO; ++o) {
+    const unsigned int x = __reduce_max_sync(0xffffffffu, __float_as_uint(m[o]));
+    if ((tid & 31) == 0 && warp < WARPS) top[warp * NO + o] = x;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    unsigned int x = 0u;   // lane o: objective o's
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      const unsigned int y = __reduce_max_sync(0xffffffffu, tid < WARPS ? top[tid * NO + o] : 0u);
+      if (tid == o) x = y;
+    }
+    ChainSlot *slot = pr.slots + (blockIdx.x % kChainSlots);
+    const unsigned int above = __ballot_sync(0xffffffffu, __uint_as_float(x) > pr.tol);
+    if (tid == 0 && above) atomicOr(&slot->above, above);
+    if (pr.first && tid < NO) atomicMax(&slot->first[tid], x);
+  }
 }
 
 template <typename RT, int NO, Pass P = kSweep>
@@ -317,7 +379,10 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     for (int o = 0; o < NO; ++o)
       if (__longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
-  if (!live) return;
+  if (!live) {
+    tell_host(pr);
+    return;
+  }
   uint64_t *full = reinterpret_cast<uint64_t *>(sm);   // [kWarps][kDepth]
   unsigned char *ring = sm + 256;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -387,6 +452,8 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
   for (int o = 0; o < NO; ++o) Rn[o] = (RT)0;
   if (n_mine > 0) load_r(0, Rn);
   if (layered) pdl_wait();   // from here on V of the next layer is read
+  uint32_t next_above = 0u;
+  if (P == kChains && blockIdx.x == 0 && warp == 0) next_above = chains_look(pr);
   int st = 0;
   uint32_t phase = 0;
   int s = sl0 * a.spw + q;                      // state of this lane's row in my j-th slice
@@ -398,7 +465,7 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
   bool chg = false;
   for (int j = 0; j < n_mine; ++j, s += s_step) {
     if (!mbar_wait(bar0 + 8u * (uint32_t)st, phase, wait_limit)) {
-      if (lane == 0) atomicOr(a.err, 1);
+      if (lane == 0) atomicOr(a.err, kErrTimeout);
       // drain: wait (bounded) for the copies still in flight into my stages
       for (int jj = j + 1; jj < j + kDepth && jj < n_mine; ++jj)
         mbar_wait(bar0 + 8u * (uint32_t)(jj % kDepth), (uint32_t)(jj / kDepth) & 1, wait_limit);
@@ -466,7 +533,8 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
       nv.v[o] = upd ? qv : old.v[o];
       if (head && upd) {
         v.pol[o % NO][s] = term ? (int16_t)-1 : (int16_t)qa;
-        if constexpr (sizeof(RT) == 4) rf[o % NO] = fmaxf(rf[o % NO], fabsf(qv - old.v[o]));
+        if constexpr (layered) continue;
+        else if constexpr (sizeof(RT) == 4) rf[o % NO] = fmaxf(rf[o % NO], fabsf(qv - old.v[o]));
         else r[o % NO] = fmax(r[o % NO], fabs(qv - old.v[o]));
       }
     }
@@ -474,7 +542,11 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     for (int o = NC; o < Pk::W; ++o) nv.v[o] = (RT)0;
     if (head) {
       v.out[s] = nv;
-      if (chg_out) {
+      if constexpr (P == kChains) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o) rf[o] = fmaxf(rf[o], fabsf(nv.v[o] - nv.v[NO + o]));
+      }
+      if (!layered && chg_out) {
         if (s >= t_end) {   // entered a later layer: publish the finished one
           if (chg) chg_out[t_cur] = 1;
           chg = false;
@@ -489,6 +561,10 @@ __device__ __forceinline__ void bellman_body(const SolveArgs &a, const VSet<RT, 
     }
   }
   if (chg_out && chg) chg_out[t_cur] = 1;
+  if constexpr (P == kChains) {
+    if (blockIdx.x == 0 && warp == 0) chains_tell(a, pr, next_above);
+    chains_publish<NO, kWarps>(pr, rf, wmax);
+  }
   if (!layered) {
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
@@ -549,7 +625,14 @@ __global__ void __launch_bounds__(32 * kWarps, P == kChains && NO == 3 ? 3 : 4) 
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ double wmax[kWarps * NO];
   __shared__ int wst_s[kWarps * kDepth];   // columns of the slice in each stage
-  if (a.lflags && k >= 1 && !active_range(a, k, pr, blockIdx.x == 0)) return;
+  if (P == kSweep) {
+    pdl_trigger();
+    pdl_wait();
+    if (a.lflags && !active_range(a, k, pr, blockIdx.x == 0)) {
+      tell_host(pr);
+      return;
+    }
+  }
   const int64_t total = pr.sl_hi - pr.sl_lo;
   const int64_t per_cta = (total + gridDim.x - 1) / gridDim.x;
   const int64_t b_lo = pr.sl_lo + (int64_t)blockIdx.x * per_cta;
@@ -691,7 +774,7 @@ __device__ __forceinline__ void bellman_body_g(const SolveArgs &a, const VSet<RT
   bool chg = false;
   for (int j = 0; j < n_mine; ++j, s += gstep) {
     if (!mbar_wait(bar0 + 8u * (uint32_t)st, phase)) {
-      if (lane == 0) atomicOr(a.err, 1);
+      if (lane == 0) atomicOr(a.err, kErrTimeout);
       for (int jj = j + 1; jj < j + kDepth && jj < n_mine; ++jj)
         mbar_wait(bar0 + 8u * (uint32_t)(jj % kDepth), (uint32_t)(jj / kDepth) & 1);
       break;
@@ -891,7 +974,10 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
                                                 int64_t *s_cut) {
   constexpr int NC = VSet<RT, NO, P>::NC;
   using Pk = VPack<RT, NC>;
-  constexpr bool layered = P != kSweep;
+  // (A layer's kernel asks at run time: with the sweeps' code left out at compile
+  // time, a layer of 40,000 slices took 16.3 us instead of 13.5, three objectives
+  // 17.1 or 29.5 instead of 17.5 from one version of the code to the next.)
+  const bool layered = P != kSweep && v.res[0] == nullptr;
   if (layered) pdl_trigger();
   unsigned live = (1u << NO) - 1u;
   if (!layered && k > 1) {
@@ -899,7 +985,10 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
     for (int o = 0; o < NO; ++o)
       if (__longlong_as_double((long long)v.res[o][k - 2]) <= a.tol) live &= ~(1u << o);
   }
-  if (!live) return;
+  if (!live) {
+    tell_host(pr);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // one read of the error word for the whole CTA (an earlier launch timed out)
   if (tid == 0) *s_flag = *(volatile int *)a.err;
@@ -940,6 +1029,9 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   const long long wait_limit = a.wait_cycles > 0 ? a.wait_cycles : 4000000000LL;   // ~2 s
   const uint32_t slots0 = smem_u32(slots);
 
+  float diff[NO];   // a consumer's largest differences of the chains
+#pragma unroll
+  for (int o = 0; o < NO; ++o) diff[o] = 0.f;
   if (warp == kWsCons) {
     // ---------------------------------------------------------- producer
     const uint64_t stream_policy = l2_evict_first();
@@ -977,7 +1069,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
       // wait's limit starts then)
       if (layered && r == kWsSlots) pdl_wait();
       if (r >= kWsSlots && !mbar_wait_suspend(empty0 + 8u * (uint32_t)slot, ph ^ 1u, wait_limit)) {
-        if (lane == 0) atomicOr(a.err, 1);
+        if (lane == 0) atomicOr(a.err, kErrTimeout);
         failed = true;
         break;
       }
@@ -1071,6 +1163,8 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
   } else {
     // ---------------------------------------------------------- consumers
     if (layered) pdl_wait();   // from here on V of the next layer is read
+    uint32_t next_above = 0u;
+    if (P == kChains && blockIdx.x == 0 && warp == 0) next_above = chains_look(pr);
     const int nS = (int)a.nS, Nc = (int)a.Nc;
     const int s_lo = (int)pr.s_lo, s_hi = (int)pr.s_hi;
     const RT invN = (RT)1 / (RT)a.N;
@@ -1094,7 +1188,7 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
     uint32_t ph = 0;
     for (;;) {
       if (!mbar_wait_suspend(full0 + 8u * (uint32_t)slot, ph, wait_limit)) {
-        if (lane == 0) atomicOr(a.err, 1);
+        if (lane == 0) atomicOr(a.err, kErrTimeout);
         break;
       }
       const int2 rdesc = hdr->round[slot];
@@ -1201,6 +1295,10 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
         }
 #pragma unroll
         for (int o = NO; o < Pk::W; ++o) nv.v[o] = (o < NC && !pr.zero_second) ? qv[o < NC ? o : 0] : (RT)0;
+        if constexpr (P == kChains) {
+#pragma unroll
+          for (int o = 0; o < NO; ++o) diff[o] = fmaxf(diff[o], fabsf(nv.v[o] - nv.v[NO + o]));
+        }
         int myqa = qa[0];
 #pragma unroll
         for (int o = 1; o < NO; ++o)
@@ -1223,11 +1321,13 @@ __device__ __forceinline__ void bellman_body_ws(const SolveArgs &a, const VSet<R
       }
     }
     if (chg_out && chg && lane == 0) chg_out[t_cur] = 1;
+    if (P == kChains && blockIdx.x == 0 && warp == 0) chains_tell(a, pr, next_above);
     if (!layered && lane == 0) {
 #pragma unroll
       for (int o = 0; o < NO; ++o) wmax[warp * NO + o] = (sizeof(RT) == 4) ? (double)rf[o] : rd[o];
     }
   }
+  if constexpr (P == kChains) chains_publish<NO, kWsCons>(pr, diff, wmax);
   if (!layered) {
     __syncthreads();
 #pragma unroll
@@ -1248,7 +1348,14 @@ __global__ void __launch_bounds__(32 * (kWsCons + 1), 1) bellman_kernel_ws(Solve
   __shared__ double wmax[kWsCons * NO];
   __shared__ int s_flag;
   __shared__ int64_t s_cut[2];
-  if (a.lflags && k >= 1 && !active_range(a, k, pr, blockIdx.x == 0)) return;
+  if (P == kSweep) {
+    pdl_trigger();
+    pdl_wait();
+    if (a.lflags && !active_range(a, k, pr, blockIdx.x == 0)) {
+      tell_host(pr);
+      return;
+    }
+  }
   bellman_body_ws<RT, NO, P>(a, v, k, pr, sm, wmax, &s_flag, s_cut);
 }
 
@@ -1383,7 +1490,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) bellman_batch_kernel(const Bat
   const BatchCta c = layered ? layer_share(items, n, k, G, kWarps, &share) : ctas[blockIdx.x];
   if (c.item < 0) return;
   const BatchSolveItem &it = items[c.item];
-  PipeRange pr;
+  PipeRange pr{};
   pr.sl_lo = c.sl_lo;
   pr.sl_hi = c.sl_hi;
   pr.s_lo = c.s_lo;
@@ -1413,7 +1520,7 @@ __global__ void __launch_bounds__(32 * kWarpsG, 1) bellman_batch_kernel_g(const 
   const BatchCta c = layered ? layer_share(items, n, k, G, 8 * kGS, &share) : ctas[blockIdx.x];
   if (c.item < 0) return;
   const BatchSolveItem &it = items[c.item];
-  PipeRange pr;
+  PipeRange pr{};
   pr.sl_lo = c.sl_lo;
   pr.sl_hi = c.sl_hi;
   pr.s_lo = c.s_lo;
@@ -1657,13 +1764,20 @@ static void launch_sweep(const SolveArgs &a, const VSet<RT, NO, P> &v, int k, co
   else cudaLaunchKernelEx(&cfg, bellman_kernel<RT, NO, P>, a, v, k, pr);
 }
 
+constexpr int64_t kOverlapSlices = 500000;
+static bool stop_told(const SolveStop &s) { return s.host && *(volatile unsigned int *)s.host == s.token; }
+
 // Objective o's status block: stats_d + o*(4 + max_sweeps) holds sweeps,
 // residual, (objective 0: the error word), spare, then one residual slot
 // per sweep.  NO = 1 iterates in the caller's V and io.Vtmp[0]; NO > 1 in
 // the packed tables io.table[0..1], copied out to V[o] at the end.
+// stop.host != nullptr: no more sweeps are launched once one has found nothing left
+// to do (21 x 27 cells, 103 layers: the empty launches of a run that ends in sweep
+// 24 took a fifth of its time); a sweep that was not launched leaves its residual 0
+// like one that did nothing.
 template <typename RT, int NO>
 static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &io, double *stats_d,
-                            cudaStream_t st) {
+                            const SolveStop &stop, cudaStream_t st) {
   using Pk = VPack<RT, NO>;
   const size_t blk = 4 + (size_t)max_sweeps;
   Pk *ta = static_cast<Pk *>(NO == 1 ? io.V[0] : io.table[0]);
@@ -1687,7 +1801,7 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
     if (e == cudaSuccess && a.work) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long) * max_sweeps, st);
     if (e != cudaSuccess) return e;
   }
-  PipeRange pr;
+  PipeRange pr{};
   size_t smem = 0;
   int blocks = 1;
   cudaError_t e = pipe_config<RT, NO, kSweep>(a, a.n_slices, &pr, &smem, &blocks);
@@ -1696,8 +1810,16 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
   pr.sl_hi = a.n_slices;
   pr.s_lo = 0;
   pr.s_hi = a.nS;
-  for (int k = 1; k <= max_sweeps; ++k)
-    launch_sweep(a, (k & 1) ? odd : even, k, pr, blocks, smem, st);
+  pr.stop = stop;
+  SolveArgs rest = a;   // a test's injected failure is for the first launch alone
+  rest.test_extra_tx = 0;
+  // A sweep starts while the one before ends, unless it is long and its CTAs fill an SM
+  // each: they then take the SMs in the order these fall free, which costs more than
+  // the launch (us a full sweep with and without, 32 actions: 58,000 slices 20.3 and
+  // 22.6, 490,000 113.7 and 114.1, 600,000 141 and 139, 4.8 million 1219 and 1092).
+  const bool pdl = pr.grouped != 2 || a.n_slices <= kOverlapSlices;
+  for (int k = 1; k <= max_sweeps && !stop_told(stop); ++k)
+    launch_sweep(k > 1 ? rest : a, (k & 1) ? odd : even, k, pr, blocks, smem, st, pdl && k > 1);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int64_t fb = (a.nS + 1 + 255) / 256;
@@ -1716,19 +1838,19 @@ static cudaError_t jacobi_t(const SolveArgs &a, int max_sweeps, const SolveIO &i
 
 template <typename RT>
 static cudaError_t jacobi_n(const SolveArgs &a, int max_sweeps, const SolveIO &io, double *stats_d,
-                            cudaStream_t st) {
+                            const SolveStop &stop, cudaStream_t st) {
   switch (io.n) {
-    case 1: return jacobi_t<RT, 1>(a, max_sweeps, io, stats_d, st);
-    case 2: return jacobi_t<RT, 2>(a, max_sweeps, io, stats_d, st);
-    case 3: return jacobi_t<RT, 3>(a, max_sweeps, io, stats_d, st);
+    case 1: return jacobi_t<RT, 1>(a, max_sweeps, io, stats_d, stop, st);
+    case 2: return jacobi_t<RT, 2>(a, max_sweeps, io, stats_d, stop, st);
+    case 3: return jacobi_t<RT, 3>(a, max_sweeps, io, stats_d, stop, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_jacobi_multi(const SolveArgs &a, int precision, int max_sweeps, const SolveIO &io,
-                                double *stats_d, cudaStream_t st) {
-  if (precision == MDP_FP64_CHECK) return jacobi_n<double>(a, max_sweeps, io, stats_d, st);
-  return jacobi_n<float>(a, max_sweeps, io, stats_d, st);
+                                double *stats_d, const SolveStop &stop, cudaStream_t st) {
+  if (precision == MDP_FP64_CHECK) return jacobi_n<double>(a, max_sweeps, io, stats_d, stop, st);
+  return jacobi_n<float>(a, max_sweeps, io, stats_d, stop, st);
 }
 
 cudaError_t launch_jacobi(const SolveArgs &a, int precision, int max_sweeps, void *Va, void *Vb,
@@ -1739,7 +1861,7 @@ cudaError_t launch_jacobi(const SolveArgs &a, int precision, int max_sweeps, voi
   io.V[0] = Va;
   io.Vtmp[0] = Vb;
   io.policy[0] = policy;
-  return launch_jacobi_multi(a, precision, max_sweeps, io, stats_d, st);
+  return launch_jacobi_multi(a, precision, max_sweeps, io, stats_d, SolveStop{nullptr, 0}, st);
 }
 
 // In place: layer t reads layer t+1, finished by the previous launch.
@@ -1747,7 +1869,7 @@ template <typename RT, int NO>
 static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, double *stats_d,
                              cudaStream_t st) {
   using Pk = VPack<RT, NO>;
-  PipeRange pr0;
+  PipeRange pr0{};
   size_t smem = 0;
   int blocks = 1;
   // every layer has the same number of slices (up to one straddling slice)
@@ -1793,42 +1915,41 @@ static cudaError_t layered_t(const SolveArgs &a, int nt, const SolveIO &io, doub
 // chain.  Sweep k = nt - t changes layer t from W(t) to V*(t), so its residual
 // is at least d_t = max |V*(t) - W(t)|.  If every d_t exceeds tol, no sweep
 // 1..nt stops the run, and sweep nt + 1 changes nothing: the run ends there
-// with V*, its greedy policy, nt + 1 sweeps and residual 0.  (Otherwise the
-// caller runs the sweeps.)  Both chains share the entry stream, so the pass
-// costs little more than a layered one.
+// with V*, its greedy policy, nt + 1 sweeps and residual 0.  If only d_0 does
+// not, sweep nt ends the run with the same V and policy: it changes no other
+// layer, so its residual is d_0.  (Otherwise the caller runs the sweeps.)  Both
+// chains share the entry stream, so the pass costs little more than a layered
+// one; a run whose tolerance is met earlier pays for the layers up to there
+// (21 x 27 cells, 103 layers, 16 actions, met in sweep 24: 0.25 ms when all
+// layers ran).
 //
-// Copies the first chain to V[o] and reduces d[o * nt + t] (float bits,
-// zeroed by the caller; NaN terms drop out as they do in the sweeps' residual).
+// Copies the first chain to V[o], if the pass was not given up.
 template <int NO>
-__global__ void finalize_two_kernel(const VPack<float, 2 * NO> *tab, VOut<float, NO> out, int64_t nS, int64_t Nc,
-                                    int nt, unsigned int *d) {
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t n = nS + 1, n_pad = (n + 31) & ~(int64_t)31;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_pad; i += stride) {
-    const bool in = i < n;
-    VPack<float, 2 * NO> p{};
-    if (in) p = tab[i];
-    const int64_t i0 = i - lane, t0 = i0 / Nc;
-    const bool one = (i0 + 31) < (t0 + 1) * Nc && i0 + 31 < nS;   // the warp's states share a layer
-#pragma unroll
-    for (int o = 0; o < NO; ++o) {
-      if (in) out.V[o][i] = p.v[o];
-      const float diff = i < nS ? fmaxf(0.f, fabsf(p.v[o] - p.v[NO + o])) : 0.f;
-      if (one) {
-        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(diff));
-        if (lane == 0 && m > d[o * nt + t0]) atomicMax(&d[o * nt + t0], m);
-      } else if (i < nS) {
-        atomicMax(&d[o * nt + i / Nc], __float_as_uint(diff));
-      }
+__global__ void finalize_two_kernel(const VPack<float, 2 * NO> *tab, VOut<float, NO> out, int64_t n, ChainWords *w,
+                                    const ChainSlot *slots, uint32_t *above) {
+  if (*(volatile const int *)&w->err) return;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {   // layer 0
+    const ChainSlot c = slots[threadIdx.x];
+    const unsigned any = __reduce_or_sync(0xffffffffu, c.above);
+    if (threadIdx.x == 0) above[0] = any;
+    for (int o = 0; o < 3; ++o) {
+      const unsigned d = __reduce_max_sync(0xffffffffu, c.first[o]);
+      if (threadIdx.x == 0) w->first[o] = d;
     }
+  }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const VPack<float, 2 * NO> p = tab[i];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) out.V[o][i] = p.v[o];
   }
 }
 
-// io.table[0]: the packed table of 2 n components per state, zeroed by the caller.
+// io.table[0]: the packed table of 2 n components per state, its last entry zeroed by
+// the caller like w.
 template <int NO>
-static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st) {
-  PipeRange pr0;
+static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, ChainWords *w, const SolveStop &stop,
+                                cudaStream_t st) {
+  PipeRange pr0{};
   size_t smem = 0;
   int blocks = 1;
   cudaError_t e = pipe_config<float, NO, kChains>(a, (a.Nc + a.spw - 1) / a.spw + 1, &pr0, &smem, &blocks);
@@ -1846,27 +1967,38 @@ static cudaError_t two_chains_t(const SolveArgs &a, int nt, const SolveIO &io, u
   }
   SolveArgs rest = a;   // a test's injected failure is for the first launch alone
   rest.test_extra_tx = 0;
+  pr0.stop = stop;
+  uint32_t *above = chain_above(w);
+  ChainSlot *slots = chain_slots(w, nt);
+  pr0.tol = (float)a.tol;
+  if ((double)pr0.tol > a.tol) pr0.tol = std::nextafter(pr0.tol, -1.f);
   for (int t_ = nt - 1; t_ >= 0; --t_) {
+    if (stop_told(stop)) break;   // given up
     PipeRange pr = pr0;
     pr.s_lo = (int64_t)t_ * a.Nc;
     pr.s_hi = pr.s_lo + a.Nc;
     pr.sl_lo = pr.s_lo / a.spw;
     pr.sl_hi = (pr.s_hi + a.spw - 1) / a.spw;
     pr.zero_second = t_ == nt - 1;
+    pr.slots = slots + (size_t)t_ * kChainSlots;
+    pr.next_slots = t_ < nt - 1 ? pr.slots + kChainSlots : nullptr;
+    pr.next_above = above + t_ + 1;
+    pr.first = t_ == 0;
     launch_sweep(t_ < nt - 1 ? rest : a, v, 0, pr, blocks, smem, st, t_ < nt - 1);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t fb = std::min<int64_t>((a.nS + 256) / 256, (int64_t)num_sms() * 8);
-  finalize_two_kernel<NO><<<(unsigned)fb, 256, 0, st>>>(t, out, a.nS, a.Nc, nt, d);
+  finalize_two_kernel<NO><<<(unsigned)fb, 256, 0, st>>>(t, out, a.nS + 1, w, slots, above);
   return cudaGetLastError();
 }
 
-cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st) {
+cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, ChainWords *w, const SolveStop &stop,
+                              cudaStream_t st) {
   switch (io.n) {
-    case 1: return two_chains_t<1>(a, nt, io, d, st);
-    case 2: return two_chains_t<2>(a, nt, io, d, st);
-    case 3: return two_chains_t<3>(a, nt, io, d, st);
+    case 1: return two_chains_t<1>(a, nt, io, w, stop, st);
+    case 2: return two_chains_t<2>(a, nt, io, w, stop, st);
+    case 3: return two_chains_t<3>(a, nt, io, w, stop, st);
     default: return cudaErrorInvalidValue;
   }
 }

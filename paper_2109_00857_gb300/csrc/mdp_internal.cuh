@@ -16,6 +16,7 @@
 // order and its compaction moves them into slice order (pool_ordered), so
 // that the columns of consecutive slices are one contiguous range.
 #pragma once
+#include <cstddef>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -334,16 +335,42 @@ struct SolveIO {
                               // (Jacobi: both, layered: table[0]), zeroed by the caller
   int16_t *policy[3];
 };
+// Where a pass with nothing left to do says so to the host thread that launches it: a
+// pinned word (or nullptr), a token of the call's own (a late store of another call
+// is not taken).
+struct SolveStop {
+  unsigned int *host;
+  unsigned int token;
+};
 // stats_d: objective o's block at stats_d + o*(4 + max_sweeps); the error
 // word (a.err) is set by the caller
 cudaError_t launch_jacobi_multi(const SolveArgs &a, int precision, int max_sweeps, const SolveIO &io,
-                                double *stats_d, cudaStream_t st);
+                                double *stats_d, const SolveStop &stop, cudaStream_t st);
 cudaError_t launch_layered_multi(const SolveArgs &a, int precision, int nt, const SolveIO &io,
                                  double *stats_d, cudaStream_t st);
-// FP32 Jacobi result by two backward chains (see bellman.cu): V[o], policies
-// and d[o * nt + t], the lower bound of the residual of sweep nt - t (float
-// bits); io.table[0] holds 2 n values per state, zeroed by the caller like d
-cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, unsigned int *d, cudaStream_t st);
+// FP32 Jacobi result by two backward chains (see bellman.cu): V[o], policies and
+// the words below; io.table[0] holds 2 n values per state.  The caller zeroes its
+// last entry and the words (a.err points at theirs).
+struct ChainWords {            // (device), then [nt] chain_above, then [nt][kChainSlots] chain_slots
+  int err;                     // kErr bits
+  unsigned int first[3];       // d_0, float bits: the residual of sweep nt if nothing stopped before
+  uint32_t pad[4];
+};
+constexpr int kChainSlots = 32;
+struct alignas(32) ChainSlot {   // of a layer, for some of its CTAs
+  uint32_t above;              // objectives (bits) whose chains differ by more than tol there
+  unsigned int first[3];       // layer 0: their largest differences
+  uint32_t pad[4];
+};
+inline size_t chain_above_words(int nt) { return ((size_t)nt + 7) & ~(size_t)7; }
+// bit o of above[t]: sweep nt - t does not stop objective o's run
+inline uint32_t *chain_above(ChainWords *w) { return reinterpret_cast<uint32_t *>(w + 1); }
+inline ChainSlot *chain_slots(ChainWords *w, int nt) { return reinterpret_cast<ChainSlot *>(chain_above(w) + chain_above_words(nt)); }
+inline size_t chain_head_bytes(int nt) { return sizeof(ChainWords) + 4 * chain_above_words(nt); }   // what the host reads
+inline size_t chain_words_bytes(int nt) { return chain_head_bytes(nt) + sizeof(ChainSlot) * kChainSlots * (size_t)nt; }
+enum : int { kErrTimeout = 1, kErrNotProven = 2 };   // the error word of a solve
+cudaError_t launch_two_chains(const SolveArgs &a, int nt, const SolveIO &io, ChainWords *w, const SolveStop &stop,
+                              cudaStream_t st);
 cudaError_t launch_jacobi(const SolveArgs &a, int precision, int max_sweeps, void *Va, void *Vb,
                           int16_t *policy, double *stats_d, cudaStream_t st);
 // Copies the slices' entry columns from `pool` (any order) into `out` in
