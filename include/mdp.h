@@ -508,9 +508,11 @@ const char *mdp_version(void);
  *     round of the one-state-per-slice sweep expects `value` bytes (a multiple
  *     of 16, <= 1 MiB) that are never copied, so that wait runs out (one shot);
  *   MDP_TEST_WAIT_LIMIT_CYCLES: the limit of those waits (0 = the default,
- *     about 2 s).
+ *     about 2 s);
+ *   MDP_TEST_ALLOCATION_FAILS: the value-th device allocation from now fails for
+ *     want of memory (one shot; 0: none).
  * Returns MDP_ERR_ARG for other keys or values.  The paper has no counterpart. */
-enum { MDP_TEST_WAIT_NEVER_COMPLETES = 1, MDP_TEST_WAIT_LIMIT_CYCLES = 2 };
+enum { MDP_TEST_WAIT_NEVER_COMPLETES = 1, MDP_TEST_WAIT_LIMIT_CYCLES = 2, MDP_TEST_ALLOCATION_FAILS = 3 };
 mdp_status mdp_test_inject(int32_t what, int64_t value);
 
 #ifdef __cplusplus

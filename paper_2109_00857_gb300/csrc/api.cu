@@ -46,9 +46,12 @@ int ensure_device_init() {
   return dev;
 }
 
+static std::atomic<long long> g_test_alloc_fails{0};   // (mdp_test_inject) allocations up to the one that fails
 cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
   if (bytes == 0) bytes = 256;
+  if (g_test_alloc_fails.load(std::memory_order_relaxed) > 0 && g_test_alloc_fails.fetch_sub(1) == 1)
+    return cudaErrorMemoryAllocation;
   return cudaMallocAsync(p, bytes, st);
 }
 
@@ -276,6 +279,10 @@ extern "C" mdp_status mdp_test_inject(int32_t what, int64_t value) {
   }
   if (what == MDP_TEST_WAIT_LIMIT_CYCLES && value >= 0) {
     g_test_wait_cycles.store((long long)value);
+    return MDP_OK;
+  }
+  if (what == MDP_TEST_ALLOCATION_FAILS && value >= 0) {
+    g_test_alloc_fails.store((long long)value);
     return MDP_OK;
   }
   set_error("invalid argument: mdp_test_inject(what, value)");
@@ -868,7 +875,9 @@ static mdp_status solve_sweeps(mdp_model m, int32_t n, const int32_t *objs, int3
 
 // A cold-started FP32 Jacobi run by two backward chains (bellman.cu): fills V,
 // policy and stats of every objective whose run is certain to end in sweep
-// nt or nt + 1, sets done[o] for those and leaves the others to the sweeps.
+// nt or nt + 1, sets done[o] for those and leaves the others to the sweeps -- all
+// of them if there is no memory for the chains' table (8 bytes a state for one
+// objective, where the sweeps need 4).
 static mdp_status solve_two_chains(mdp_model m, int32_t n, const int32_t *objs, double tol, void *const *V,
                                    int16_t *const *policy, void *stream, mdp_solve_stats *stats, bool *done,
                                    float *ms) {
@@ -878,7 +887,13 @@ static mdp_status solve_two_chains(mdp_model m, int32_t n, const int32_t *objs, 
   const size_t table = state * (size_t)(m->nS + 1), words = (table + 31) & ~(size_t)31;   // (then the words)
   Scratch tab(st);
   EventPair ev;
-  MDP_CUDA_TRY(dev_alloc(&tab.p, words + chain_words_bytes(m->nt), st));
+  *ms = 0.f;
+  const cudaError_t ae = dev_alloc(&tab.p, words + chain_words_bytes(m->nt), st);
+  if (ae == cudaErrorMemoryAllocation) {
+    cudaGetLastError();   // (it is not the call's)
+    return MDP_OK;
+  }
+  MDP_CUDA_TRY(ae);
   SolveIO io{};
   io.n = n;
   for (int o = 0; o < n; ++o) {

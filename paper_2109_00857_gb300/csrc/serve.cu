@@ -160,10 +160,11 @@ ReqShape req_shape(const EnvEntry &e, const mdp_request &r) {
 // The most device memory a request can hold with an entry pool of pool_cols
 // columns: every allocation of its build (coefficients, pool, slice and row
 // arrays, R, cell classes, offsets, deferred-slice list, the compacted pool and
-// its scan while the first pool is still live), its solve (status words, the
-// Jacobi partner vector and layer flags) and the request's own V and policy,
-// each rounded up to 4 KiB, plus 1 MiB; with spill_words > 0 also a spill area
-// of that many words and its per-slice offsets.
+// its scan while the first pool is still live), its solve (the table of the two
+// chains, 8 bytes a state, and their words, or the Jacobi partner vector, status
+// words and layer flags) and the request's own V and policy, each rounded up to
+// 4 KiB, plus 1 MiB; with spill_words > 0 also a spill area of that many words and
+// its per-slice offsets.
 int64_t charge_bytes(const EnvEntry &e, const mdp_request &r, uint64_t pool_cols, uint64_t spill_words) {
   const ReqShape g = req_shape(e, r);
   auto al = [](int64_t x) { return (x + 4095) & ~(int64_t)4095; };
@@ -175,7 +176,8 @@ int64_t charge_bytes(const EnvEntry &e, const mdp_request &r, uint64_t pool_cols
   b += al(4 * g.n_slices) + al(g.n_slices) + al(g.rows_pad) + al(2 * g.rows_pad) + al(4 * g.rows_pad);
   b += al(g.nS) + al(4 * g.nbins) + al(4 * g.n_slices);                                        // classes, offsets, defer
   b += al(8 * (4 + 2 * max_sweeps + (3 * (g.nt + 1) + 7) / 8 + 1));                           // solve status
-  b += 3 * al(4 * (g.nS + 1)) + al(2 * g.nS);                                                  // V, partner, policy
+  b += al(4 * (g.nS + 1)) + al(2 * g.nS);                                                      // V, policy
+  b += al(8 * (g.nS + 1)) + al(chain_words_bytes(g.nt) + 32);                                  // chains' table (or the partner)
   b += al((int64_t)e.grid.nx * e.grid.ny);                                                     // target mask
   if (spill_words) b += al(4 * g.n_slices) + al(4 * (int64_t)spill_words);                     // spill area
   return b + (1 << 20);
