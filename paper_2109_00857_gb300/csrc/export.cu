@@ -9,11 +9,12 @@ namespace mdpgb {
 // ------------------------------------------------------ prefix sums ----
 // Exclusive sums over tiles of kTile values: x[i] holds the sum within the tile,
 // tile[i / kTile] the sum of the tiles before (after scan_offsets), so that the
-// consumer adds the two and no pass over x is spent on it.
+// consumer adds the two and no pass over x is spent on it.  x is a plain array or
+// scattered over another one (At: where value i lies).
 constexpr int kScanThreads = 512, kScanItems = 8, kTile = kScanThreads * kScanItems;
 
-template <class Load>
-__global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(Load load, int64_t n, int64_t *x, int64_t *tile) {
+template <class Load, class At>
+__global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(Load load, int64_t n, At x, int64_t *tile) {
   __shared__ int64_t wsum[kScanThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t base = (int64_t)blockIdx.x * kTile + warp * (32 * kScanItems);   // a warp's values are consecutive
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(Load load, int
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     const int64_t at = base + 32 * i + lane;
-    if (at < n) x[at] = v[i] + before;
+    if (at < n) *x(at) = v[i] + before;
   }
   if (threadIdx.x == 0) tile[blockIdx.x] = all;
 }
@@ -54,9 +55,14 @@ __global__ void scan_add_kernel(int64_t *x, int64_t n, const int64_t *tile) {
     x[i] += tile[i / kTile];
 }
 
+struct Words {
+  int64_t *x;
+  __device__ __forceinline__ int64_t *operator()(int64_t i) const { return x + i; }
+};
+template <class At>
 struct LoadWords {
-  const int64_t *x;
-  __device__ __forceinline__ int64_t operator()(int64_t i) const { return x[i]; }
+  At at;
+  __device__ __forceinline__ int64_t operator()(int64_t i) const { return *at(i); }
 };
 struct LoadBytes {
   const uint8_t *x;
@@ -74,15 +80,15 @@ static int64_t scan_words(int64_t n) {
 }
 
 // x and tile as above (load may read x itself: a thread reads its values before it writes them)
-template <class Load>
-static cudaError_t scan_offsets(Load load, int64_t n, int64_t *x, int64_t *tile, cudaStream_t st) {
+template <class Load, class At>
+static cudaError_t scan_offsets(Load load, int64_t n, At x, int64_t *tile, cudaStream_t st) {
   const int64_t tiles = (n + kTile - 1) / kTile;
   scan_tiles_kernel<<<(unsigned)tiles, kScanThreads, 0, st>>>(load, n, x, tile);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (tiles == 1) return cudaMemsetAsync(tile, 0, sizeof(int64_t), st);
   int64_t *up = tile + tiles;
-  e = scan_offsets(LoadWords{tile}, tiles, tile, up, st);
+  e = scan_offsets(LoadWords<Words>{{tile}}, tiles, Words{tile}, up, st);
   if (e != cudaSuccess || tiles <= kTile) return e;   // one tile of tiles: its offset is 0
   scan_add_kernel<<<(unsigned)std::min<int64_t>((tiles + 255) / 256, 8192), 256, 0, st>>>(tile, tiles, up);
   return cudaGetLastError();
@@ -118,7 +124,7 @@ cudaError_t launch_pool_reorder(const uint32_t *pool, uint32_t *out, uint32_t *s
   cudaError_t e = dev_alloc((void **)&x, sizeof(int64_t) * (size_t)(n_slices + scan_words(n_slices)), st);
   if (e != cudaSuccess) return e;
   int64_t *tile = x + n_slices;
-  e = scan_offsets(LoadBytes{slice_w}, n_slices, x, tile, st);
+  e = scan_offsets(LoadBytes{slice_w}, n_slices, Words{x}, tile, st);
   if (e == cudaSuccess) {
     const int64_t blocks = std::min<int64_t>(num_sms() * 16, (n_slices + 7) / 8);
     pool_reorder_kernel<<<(unsigned)blocks, 256, 0, st>>>(pool, out, slice_off, slice_w, x, tile, n_slices);
@@ -134,6 +140,9 @@ cudaError_t launch_pool_reorder(const uint32_t *pool, uint32_t *out, uint32_t *s
 // Bound by memory: the entries are read once (4 bytes) and written once (12).
 //   lengths   per (action, block) the sum of its rows' lengths; scanned over
 //             a nb + b, it is where the block's rows of action a begin.
+//             (Where there is no memory for the sums, they lie in the caller's
+//             rowptr, each where its block's first row ends up; always there,
+//             the exports below took 10 to 18 % longer.)
 //   fill      the block's slices are staged in shared memory, words of slice j
 //             rotated by j so that reading one action's row of every state
 //             meets every bank once; warp by action, lane by state, the row's
@@ -153,7 +162,8 @@ struct ExportArgs {
   const uint16_t *sinkc;
   int64_t nS, Nc, n_slices, blocks;
   int32_t A, A_pad, spw;
-  int64_t *sums;          // [A][blocks], then their scan
+  int64_t *sums;          // of (action, block) at act * sum_act + block * sum_block, then their scan
+  int64_t sum_act, sum_block;
   const int64_t *tile;
   int64_t *rowptr, *col;
   int32_t *count;
@@ -164,6 +174,16 @@ __device__ __forceinline__ int spill_len(const ExportArgs &a, int64_t sl, int la
   const uint32_t off = a.spill_off[sl];
   return off == kNoSlice ? 0 : (int)(a.spill[off + lane + 1] - a.spill[off + lane]);
 }
+
+// Sum i = a nb + b of the lengths (and its scan) in rowptr.
+struct RowptrSums {
+  int64_t *rowptr;
+  int64_t nS, blocks;
+  __device__ __forceinline__ int64_t *operator()(int64_t i) const {
+    const int64_t act = layer_of(i, blocks, nS);   // (i <= nS)
+    return rowptr + act * nS + (i - act * blocks) * kXState;
+  }
+};
 
 // warp per block: lane = row of a slice
 __global__ void __launch_bounds__(256) export_lengths_kernel(ExportArgs a) {
@@ -180,7 +200,7 @@ __global__ void __launch_bounds__(256) export_lengths_kernel(ExportArgs a) {
         len += (unsigned)(a.nnz[ir] + spill_len(a, sl, lane) + (a.sinkc[ir] ? 1 : 0));
     }
     for (int off = a.A_pad; off < 32; off <<= 1) len += __shfl_xor_sync(0xffffffffu, len, off);
-    if (q == 0 && act < a.A) a.sums[(int64_t)act * a.blocks + b] = (int64_t)len;
+    if (q == 0 && act < a.A) a.sums[(int64_t)act * a.sum_act + b * a.sum_block] = (int64_t)len;
   }
 }
 
@@ -238,6 +258,8 @@ __global__ void __launch_bounds__(32 * kXWarps) export_fill_kernel(const ExportA
     const int64_t s = s0 + lane;
     const int j = lane / spw, q = lane % spw;
     for (int act = warp; act < a.A; act += kXWarps) {
+      const int64_t begin = a.sums[(int64_t)act * a.sum_act + b * a.sum_block] + a.tile[((int64_t)act * a.blocks + b) / kTile];
+      __syncwarp();   // (the sum's place may be a row's of this block)
       const int l = q * a.A_pad + act, to = (l + j) & 31;
       const bool on = s < a.nS;
       const uint32_t rw = on ? sm.row[j * 32 + to] : 0u;
@@ -251,7 +273,6 @@ __global__ void __launch_bounds__(32 * kXWarps) export_fill_kernel(const ExportA
         if (lane >= d) incl += o;
       }
       const int total = __shfl_sync(0xffffffffu, incl, 31), mine = incl - len;
-      const int64_t at = (int64_t)act * a.blocks + b, begin = a.sums[at] + a.tile[at / kTile];
       const int64_t r = (int64_t)act * a.nS + s;
       if (on) {
         a.rowptr[r] = begin + mine;
@@ -320,13 +341,26 @@ cudaError_t launch_export(const mdp_model_t *m, int obj, int64_t *rowptr, int64_
   a.rowptr = rowptr; a.col = col; a.count = count;
   const int64_t n = a.A * a.blocks;
   int64_t *x = nullptr;
+  a.sum_act = a.blocks;
+  a.sum_block = 1;
   cudaError_t e = dev_alloc((void **)&x, sizeof(int64_t) * (size_t)(n + scan_words(n)), st);
+  const bool in_rowptr = e == cudaErrorMemoryAllocation;
+  if (in_rowptr) {
+    cudaGetLastError();   // (it is not the call's)
+    a.sum_act = m->nS;
+    a.sum_block = kXState;
+    e = dev_alloc((void **)&x, sizeof(int64_t) * (size_t)scan_words(n), st);
+  }
   if (e != cudaSuccess) return e;
-  a.sums = x;
-  a.tile = x + n;
+  a.sums = in_rowptr ? rowptr : x;
+  int64_t *tile = in_rowptr ? x : x + n;
+  a.tile = tile;
+  const RowptrSums scattered{rowptr, m->nS, a.blocks};
   export_lengths_kernel<<<(unsigned)std::min<int64_t>((a.blocks + 7) / 8, (int64_t)num_sms() * 8), 256, 0, st>>>(a);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = scan_offsets(LoadWords{x}, n, x, x + n, st);
+  if (e == cudaSuccess)
+    e = in_rowptr ? scan_offsets(LoadWords<RowptrSums>{scattered}, n, scattered, tile, st)
+                  : scan_offsets(LoadWords<Words>{{x}}, n, Words{x}, tile, st);
   if (e == cudaSuccess)
     e = m->precision == MDP_FP64_CHECK ? fill_t<double>(a, m, obj, R, st) : fill_t<float>(a, m, obj, R, st);
   dev_free(x, st);

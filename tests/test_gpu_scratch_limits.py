@@ -47,3 +47,20 @@ def test_allocations_that_are_needed_still_fail_the_call(mdp):
         finally:
             lib.mdp_test_inject(3, 0)
         call()
+
+
+@pytest.mark.parametrize("nx, ny, nt, headings, speeds", [(60, 50, 20, 16, 1), (60, 50, 20, 16, 2), (7, 5, 3, 3, 1),
+                                                          (1, 1, 1, 16, 1), (9, 7, 3, 31, 1), (40, 40, 300, 1, 1)])
+def test_an_export_without_memory_for_its_sums(mdp, nx, ny, nt, headings, speeds):
+    env = inputs.make_env(nx=nx, ny=max(ny, 2), nt=nt, K=2, N=30, L=11, sigma=(0.2, 0.1), seed=5, amplitude=1.0,
+                          n_headings=headings, n_speeds=speeds, with_gbar=True, objectives=(0, 2))
+    m = mdp.mdp_build(mdp.DeviceEnv(env), objs=env.objectives)
+    for entries in (True, False):
+        want = mdp.mdp_export_csr(m, 1, with_entries=entries)
+        assert mdp.load().mdp_test_inject(3, 1) == 0
+        try:
+            got = mdp.mdp_export_csr(m, 1, with_entries=entries)
+        finally:
+            mdp.load().mdp_test_inject(3, 0)
+        for x, y in zip(got, want):
+            assert (x is None and y is None) or np.array_equal(x.cpu().numpy(), y.cpu().numpy())
