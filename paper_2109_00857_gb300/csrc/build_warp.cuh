@@ -437,32 +437,47 @@ __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, i
   sm.st[q] = st;
 }
 
-// Counts state s again with the exact table g (the warp owning its slice;
-// tab: the state's table memory).  Rare: see the file comment.
+// Counts state s again with the exact table g (the warp owning its slice; st: the
+// state's set-up, tab: its table memory; care: some fraction lies below
+// act.rank_trap).  Rare where windows hold 5 standard deviations and more, but every
+// second state or so where a share is small for its states (few actions, wide
+// spreads): hence the counting loop's lookups and two rows in flight.
 template <int KT, int MODE>
-__device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables &rt, int64_t s, const FineGeo g,
-                                           uint32_t *tab, int words) {
-  const int lane = threadIdx.x & 31, K = KT > 0 ? KT : a.K, B = a.act.rank_buckets;
+__device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables &rt, const StateSetup &st, int64_t s,
+                                           const FineGeo g, uint32_t *tab, int words, bool care) {
+  const int lane = threadIdx.x & 31, K = KT > 0 ? KT : a.K, B = a.act.rank_buckets, N = a.N;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
-  const int64_t t = s / a.Nc, c = s % a.Nc;
-  const float *vbar = static_cast<const float *>(a.vbar), *modes = static_cast<const float *>(a.modes);
-  const float *Yt = static_cast<const float *>(a.Y) + (size_t)t * a.N * K;
-  const float vbx = vbar[2 * s], vby = vbar[2 * s + 1];
+  for (int i = lane; i < words; i += 32) tab[i] = 0u;
+  __syncwarp();
+  if (g.gx == 1 && g.gy == 1) {   // every realization in one cell
+    if (lane == 0) tab[g.pitch + 1] = (uint32_t)N;
+    __syncwarp();
+    return;
+  }
+  const int64_t t = st.layer;
+  const float *Yt = static_cast<const float *>(a.Y) + (size_t)t * N * K;
+  const float vbx = st.vbx, vby = st.vby, lam = a.lam, bk = int_float((uint32_t)B);
   float phx[kPhi<KT>], phy[kPhi<KT>];
 #pragma unroll
   for (int k = 0; k < kPhi<KT>; ++k) {
     phx[k] = phy[k] = 0.f;
     if (KT > 0 || k < K) {
-      const float2 ph = *reinterpret_cast<const float2 *>(modes + 2 * ((t * K + k) * a.Nc + c));
+      const float2 ph = __ldg(reinterpret_cast<const float2 *>(a.modes) + t * (K - 1) * a.Nc + s + k * a.Nc);
       phx[k] = ph.x;
       phy[k] = ph.y;
     }
   }
-  for (int i = lane; i < words; i += 32) tab[i] = 0u;
-  __syncwarp();
-  for (int w = lane; w < a.N; w += 32) {
-    float y[kPhi<KT>], wx = vbx, wy = vby;
-    load_row<KT>(Yt + (size_t)w * K, K, y);
+  // byte address of fine cell (n S + rank, ...), n as its floor's bits (modulo 2^32)
+  const uint32_t pitch = (uint32_t)g.pitch, aN = 4u * (uint32_t)Sx * pitch, bN = 4u * (uint32_t)Sy;
+  const uint32_t c0 = smem_u32(tab) + 4u * ((uint32_t)(1 - g.xmin) * pitch + (uint32_t)(1 - g.ymin)) - kFloorBits * (aN + bN);
+  auto rank4c = [&](float f, int axis) -> uint32_t {   // (rank4; the compiler may interleave it)
+    const uint32_t l = rt.L[axis][__float_as_uint(__fmul_rd(f, bk))];
+    const float *T = rt.T[axis] + (l >> 2);
+    if (MODE == 1) return f < T[0] ? l - 4u : l;
+    return l + (T[1] <= f ? 4u : 0u) + (T[2] <= f ? 4u : 0u);
+  };
+  auto cell = [&](const float (&y)[kPhi<KT>]) -> uint32_t {
+    float wx = vbx, wy = vby;
 #pragma unroll
     for (int k = 0; k < kPhi<KT>; ++k) {
       if (KT > 0 || k < K) {
@@ -470,9 +485,31 @@ __device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables 
         wy = fmaf(y[k], phy[k], wy);
       }
     }
-    const int X = fine_coord<MODE>(fmaf(wx, a.lam, 0.5f), Sx, rt, 0, B) - g.xmin;
-    const int Y = fine_coord<MODE>(fmaf(wy, a.lam, 0.5f), Sy, rt, 1, B) - g.ymin;
-    red_add_shared(smem_u32(tab) + 4u * (uint32_t)((X + 1) * g.pitch + Y + 1), 1u);
+    const float ux = fmaf(wx, lam, 0.5f), uy = fmaf(wy, lam, 0.5f);
+    if (MODE > 2 || care) {
+      const int X = fine_coord<MODE>(ux, Sx, rt, 0, B), Y = fine_coord<MODE>(uy, Sy, rt, 1, B);
+      return c0 + kFloorBits * (aN + bN) + 4u * ((uint32_t)X * pitch + (uint32_t)Y);
+    }
+    const float tx = __fadd_rd(ux, kFloorMagic), ty = __fadd_rd(uy, kFloorMagic);
+    const uint32_t rx = rank4c(__saturatef(ux - (tx - kFloorMagic)), 0), ry = rank4c(__saturatef(uy - (ty - kFloorMagic)), 1);
+    return c0 + __float_as_uint(tx) * aN + rx * pitch + __float_as_uint(ty) * bN + ry;
+  };
+  constexpr int kRows = KT == 0 ? 1 : 2;
+  int w = lane;
+  for (; w + 32 * (kRows - 1) < N; w += 32 * kRows) {
+    float y[kRows][kPhi<KT>];
+    uint32_t at[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) load_row<KT>(Yt + (size_t)(w + 32 * i) * K, K, y[i]);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) at[i] = cell(y[i]);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) red_add_shared(at[i], 1u);
+  }
+  for (; w < N; w += 32) {
+    float y[kPhi<KT>];
+    load_row<KT>(Yt + (size_t)w * K, K, y);
+    red_add_shared(cell(y), 1u);
   }
   __syncwarp();
 }
@@ -573,7 +610,8 @@ __device__ __noinline__ FineGeo pack_slice(const BuildArgs &a, const GroupSmem &
     FineGeo g = exact_table<MODE>(state_extreme(ext, warp * spw + q, NW, G), Sx, Sy, sm.rt, B);
     const int cells = (int)table_cells(g);
     g.base = base;
-    recount_state<KT, MODE>(a, sm.rt, sl * spw + q, g, grid + base, cells);
+    recount_state<KT, MODE>(a, sm.rt, sm.st[warp * spw + q], sl * spw + q, g, grid + base, cells,
+                            MODE <= 2 && (sm.trap >> (warp * spw + q) & 1u));
     if (SUM) prefix_table(grid + base, g);
     if (q == q_l) mine = g;
     base += cells;
@@ -1166,7 +1204,8 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
           pack = true;
           continue;
         }
-        if (!defer && !pack) recount_state<KT, MODE>(a, sm.rt, s, g, grid + g.base, share);
+        if (!defer && !pack)
+          recount_state<KT, MODE>(a, sm.rt, sm.st[qg], s, g, grid + g.base, share, MODE <= 2 && (sm.trap >> qg & 1u));
       }
       if (q == q_l) r.g = g;
       if (SPW != 1 && !defer && !pack) prefix_table(grid + g.base, g);
@@ -1191,8 +1230,9 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
     uint64_t blk;
     const BoxCells bc = box_cells<SPW>(a, sl, r, sr, blk);
     if (SPW == 1 && sm.st[warp].layer >= 0) prefix_table(grid + r.g.base, r.g);
-    if (sr.small) rc = count_small<SPW>(a, sm.rt, grid, r, bc, blk, stage, sr);
-    if (!sr.small) {
+    if (sr.small) {   // (right for rows longer than are staged, too)
+      rc = count_small<SPW>(a, sm.rt, grid, r, bc, blk, stage, sr);
+    } else {
       const uint32_t sink = r.kind == KIND_SINK ? (uint32_t)N : 0u;
       rc = count_general<HYB>(a, sl, grid, r);
       rc.sink += sink;
