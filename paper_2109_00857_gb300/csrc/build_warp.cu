@@ -120,6 +120,7 @@ static cudaError_t launch_g(const BuildArgs &a, int warps, int sms, cudaStream_t
 template <int SPW, int MODE>
 static cudaError_t launch_k(const BuildArgs &a, int warps, int sms, cudaStream_t st) {
   switch (a.K) {
+    case 0: return launch_g<kNoModes, 0, MODE>(a, warps, sms, st);
     case 1: return launch_g<1, SPW, MODE>(a, warps, sms, st);
     case 2: return launch_g<2, SPW, MODE>(a, warps, sms, st);
     case 3: return launch_g<3, SPW, MODE>(a, warps, sms, st);
@@ -134,7 +135,8 @@ static cudaError_t launch_k(const BuildArgs &a, int warps, int sms, cudaStream_t
 
 // Instantiations: 32 and 16 actions (one and two states per slice) with the
 // one- and the two-comparison lookup and up to eight modes; fewer actions with
-// the one-comparison lookup; everything else with runtime sizes.
+// the one-comparison lookup; no modes with either; everything else with runtime
+// sizes.
 cudaError_t launch_build_warp(const BuildArgs &a, int warps, int sms, cudaStream_t st) {
   const int mode = a.act.rank_mode;
   if (mode == 1) {
@@ -145,7 +147,7 @@ cudaError_t launch_build_warp(const BuildArgs &a, int warps, int sms, cudaStream
   if (mode == 2) {
     if (a.spw == 1) return launch_k<1, 2>(a, warps, sms, st);
     if (a.spw == 2) return launch_k<2, 2>(a, warps, sms, st);
-    return launch_g<0, 0, 2>(a, warps, sms, st);
+    return a.K == 0 ? launch_g<kNoModes, 0, 2>(a, warps, sms, st) : launch_g<0, 0, 2>(a, warps, sms, st);
   }
   return launch_g<0, 0, 3>(a, warps, sms, st);
 }

@@ -104,9 +104,17 @@ __device__ __forceinline__ f2 add2_down(f2 a, f2 b) {
   return r;
 }
 
-// Mode-count variants: KT > 0 exactly KT modes; KT == 0 up to kMaxModes (runtime).
+// Mode-count variants: KT > 0 exactly KT modes; KT == 0 up to kMaxModes (runtime);
+// KT == kNoModes: none, so that all realizations are the same -- a state is counted
+// once, by N (100 x 90 cells, 20 layers, 32 actions, N = 500: 1.55 ms as a run-time
+// mode count of 0).
+constexpr int kNoModes = -1;
 template <int KT>
-constexpr int kPhi = KT > 0 ? KT : kMaxModes;
+constexpr int kPhi = KT > 0 ? KT : (KT == kNoModes ? 1 : kMaxModes);
+template <int KT>
+__device__ __forceinline__ int mode_count(int K) {
+  return KT > 0 ? KT : (KT == kNoModes ? 0 : K);
+}
 
 // A realization's coefficient row, with the widest loads its alignment allows
 // (coeffs are 16-byte aligned).
@@ -445,7 +453,7 @@ __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, i
 template <int KT, int MODE>
 __device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables &rt, const StateSetup &st, int64_t s,
                                            const FineGeo g, uint32_t *tab, int words, bool care) {
-  const int lane = threadIdx.x & 31, K = KT > 0 ? KT : a.K, B = a.act.rank_buckets, N = a.N;
+  const int lane = threadIdx.x & 31, K = mode_count<KT>(a.K), B = a.act.rank_buckets, N = a.N;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
   for (int i = lane; i < words; i += 32) tab[i] = 0u;
   __syncwarp();
@@ -974,7 +982,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
                                              F &&next_first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int spw = SPW > 0 ? SPW : a.spw;
-  const int K = KT > 0 ? KT : a.K;
+  const int K = mode_count<KT>(a.K);
   // model scalars in registers: the loops below also store to memory, so
   // loads through `a` (shared memory in the batched kernel) would repeat
   const int N = a.N;
@@ -1039,7 +1047,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
       auto red = [&](uint32_t lin, uint32_t bytes, uint32_t base) {
         uint32_t addr;
         asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(addr) : "r"(lin), "r"(bytes), "r"(base));
-        red_add_shared(addr, 1u);
+        red_add_shared(addr, KT == kNoModes ? (uint32_t)N : 1u);
       };
       // u of a realization for both states (FMA chain over ascending k, then u =
       // fma(w, lam, 1/2): the CTA kernel's operations)
@@ -1102,9 +1110,10 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         mny1 = min_nan(mny1, uy.y, vy.y); mxy1 = max_nan(mxy1, uy.y, vy.y);
       };
       const float *yp = static_cast<const float *>(a.Y) + ((size_t)t * N + w0) * K;
-      int w = on0 || on1 ? w0 : N;
+      const int N_run = KT == kNoModes ? 1 : N;   // realizations to run through
+      int w = on0 || on1 ? w0 : N_run;
 #pragma unroll 1
-      for (; w + step < N; w += 2 * step, yp += (size_t)(2 * step) * K) {   // two realizations per trip
+      for (; w + step < N_run; w += 2 * step, yp += (size_t)(2 * step) * K) {   // two realizations per trip
         float y0[kPhi<KT>], y1[kPhi<KT>];
         load_row<KT>(yp, K, y0);
         load_row<KT>(yp + (size_t)step * K, K, y1);
@@ -1115,7 +1124,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
         count(ax, ay);
         count(bx, by);
       }
-      if (w < N) {   // the last of an odd number
+      if (w < N_run) {   // the last of an odd number
         float y0[kPhi<KT>];
         load_row<KT>(yp, K, y0);
         f2 ax, ay;

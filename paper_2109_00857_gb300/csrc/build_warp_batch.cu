@@ -102,6 +102,7 @@ template <int SPW, int MODE>
 static cudaError_t launch_gb_k(const BuildArgs *items_d, const int64_t *prefix_d, int n, unsigned long long *work_d,
                                int cap_bins, int K, int spw, cudaStream_t st) {
   switch (K) {
+    case 0: return launch_gb<kNoModes, 0, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
     case 1: return launch_gb<1, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
     case 2: return launch_gb<2, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
     case 3: return launch_gb<3, SPW, MODE>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
@@ -129,7 +130,8 @@ cudaError_t launch_build_warp_batch(const BuildArgs *items_d, const int64_t *pre
   if (rank_mode == 2) {
     if (spw == 1) return launch_gb_k<1, 2>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
     if (spw == 2) return launch_gb_k<2, 2>(items_d, prefix_d, n, work_d, cap_bins, K, spw, st);
-    return launch_gb<0, 0, 2>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
+    return K == 0 ? launch_gb<kNoModes, 0, 2>(items_d, prefix_d, n, work_d, cap_bins, spw, st)
+                  : launch_gb<0, 0, 2>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
   }
   return launch_gb<0, 0, 3>(items_d, prefix_d, n, work_d, cap_bins, spw, st);
 }

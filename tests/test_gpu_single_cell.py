@@ -55,3 +55,20 @@ def test_rows_longer_than_are_staged(mdp, headings, speeds, hist_cap):
                      sigma=np.full(K, 0.6), seed=4, actions=inputs.action_table(headings, speeds, 1.0), obstacle=obstacle,
                      target=target, gbar=rng.random((nt, ny, nx)), r_term=2.0, r_outbound=-5.0)
     assert same_model(mdp, env, hist_cap).max_row_nnz > 14
+
+
+def test_batched_models_without_modes(mdp):
+    rng = np.random.default_rng(3)
+    envs = []
+    for i, headings in enumerate((16, 16, 8, 1)):
+        nx, ny, nt = 9 + i, 8, 4
+        envs.append(custom_env(nx=nx, ny=ny, nt=nt, K=0, N=60 + i, L=9, vbar=rng.uniform(-1, 1, (nt, ny, nx, 2)),
+                               modes=np.zeros((nt, 0, ny, nx, 2)), sigma=np.zeros(0), gbar=rng.random((nt, ny, nx)),
+                               actions=inputs.action_table(headings, 1 + i % 2, 1.0), r_outbound=-5.0))
+    b = mdp.Batch([mdp.DeviceEnv(e) for e in envs])
+    b.run()
+    for e, V, pi in zip(envs, b.V, b.policy):
+        same_model(mdp, e)
+        m = mdp.mdp_build(mdp.DeviceEnv(e))
+        V1, p1, _ = mdp.mdp_solve(m, 0, method=mdp.MDP_SOLVE_LAYERED)
+        assert np.array_equal(V.cpu().numpy(), V1.cpu().numpy()) and np.array_equal(pi.cpu().numpy(), p1.cpu().numpy())
