@@ -361,10 +361,11 @@ mdp_status mdp_rollout(const mdp_env *env, const mdp_grid *grid, const mdp_actio
  * authors tuned threads per block by hand for each GPU, Sec. IV-D; here the
  * library does it).  A class is (actions padded to a power of two, modes, N
  * and cells rounded to powers of two, objectives, precision).  The shapes:
- * warps per CTA (4, 8: the kernel takes at most 4) and fine-table words per
- * slice (1536..4096, the power of two below) of the group build kernel, the CTA size of the full-window kernel when the
- * calibration defers slices to it, and the shared memory of the
- * one-state-per-slice Bellman sweep (132, 160, 190 KiB: its slot size).
+ * fine-table words per slice of the group build kernel (1536..4096; its groups
+ * are at most four slices: build_warps is recorded as 4, and 8 in a file is taken
+ * as 4), the CTA size of the full-window kernel when the calibration defers
+ * slices to it, and the shared memory of the one-state-per-slice Bellman sweep
+ * (132, 160, 190 KiB: its slot size).
  * No choice changes a count, entry, R, value or policy -- only the speed.
  * mdp_build, mdp_solve, mdp_solve_multi and the batch use the process-wide
  * table's entry for a model's class wherever the caller leaves an option 0.

@@ -4,10 +4,9 @@
 //
 // A workload class is (actions padded to a power of two, modes, N and cells
 // rounded to powers of two, objectives, precision).  The shapes tuned are the
-// warps per CTA (a group has at most four) and the fine-table capacity of the
-// group build kernel, the CTA size of the full-window build kernel (when the calibration
-// defers slices to it), and the shared memory of the one-state-per-slice
-// Bellman sweep (which sets its slot size).  None of them changes a count, an
+// fine-table capacity of the group build kernel, the CTA size of the full-window
+// build kernel (when the calibration defers slices to it), and the shared memory
+// of the one-state-per-slice Bellman sweep (which sets its slot size).  None of them changes a count, an
 // entry, an R value, a value or a policy: the table only picks the fastest
 // launch.  mdp_build, mdp_solve and the batch use the table's entry for a
 // model's class whenever the caller leaves the corresponding option at 0.
@@ -65,6 +64,8 @@ static void tuning_erase(const std::string &key) {
 // ------------------------------------------------------------------- JSON --
 // The file is one object of objects of integers:
 //   {"<class>": {"build_warps": 8, "hist_cap": 2048, ...}, ...}
+// (build_warps: files recorded with 8 stay loadable; a group has at most four slices)
+constexpr int kGroupSlices = 4;
 static const char *kFields[] = {"build_warps", "hist_cap", "threads", "chunk", "sweep_smem_kb"};
 
 static int32_t *field_of(Tuning &t, const std::string &name) {
@@ -239,29 +240,27 @@ extern "C" mdp_status mdp_autotune(const mdp_env *env, const mdp_grid *grid, con
   double best_build = 1e300;
   int timed = 0;
   int64_t deferred = 0;
-  for (int warps : {8, 4}) {
-    for (int cap : {2048, 1536, 3072, 4096}) {
-      Tuning t;
-      t.build_warps = warps;
-      t.hist_cap = cap;
-      double ms = 1e300;
-      for (int rep = 0; rep < 2; ++rep) {
-        mdp_model m = nullptr;
-        mdp_status s = build_with(t, &m);
-        if (s != MDP_OK) {
-          restore();
-          return s;
-        }
-        ms = std::min(ms, m->kernel_ms);
-        if (warps == 8 && cap == 2048) deferred = m->deferred;
-        mdp_model_free(m);
+  best.build_warps = kGroupSlices;
+  for (int cap : {2048, 1536, 2560, 3072, 3584, 4096}) {
+    Tuning t;
+    t.build_warps = kGroupSlices;
+    t.hist_cap = cap;
+    double ms = 1e300;
+    for (int rep = 0; rep < 2; ++rep) {
+      mdp_model m = nullptr;
+      mdp_status s = build_with(t, &m);
+      if (s != MDP_OK) {
+        restore();
+        return s;
       }
-      ++timed;
-      if (ms < best_build) {
-        best_build = ms;
-        best.build_warps = warps;
-        best.hist_cap = cap;
-      }
+      ms = std::min(ms, m->kernel_ms);
+      if (cap == 2048) deferred = m->deferred;
+      mdp_model_free(m);
+    }
+    ++timed;
+    if (ms < best_build) {
+      best_build = ms;
+      best.hist_cap = cap;
     }
   }
   if (deferred > 0) {   // the full-window kernel has work: tune its CTA size too
