@@ -26,10 +26,10 @@
 //            checked afterwards.  Table addresses are taken modulo the state's
 //            power-of-two table, so a realization outside the window corrupts
 //            only its own state's table, which is then counted again with the
-//            exact window (recount_state; rare: the windows hold 5 to 7 standard
+//            exact window (recount_slice; rare: the windows hold 5 to 7 standard
 //            deviations, N = 5000 draws reach 4).  A state's table is an equal
 //            share of the slice's words; a slice with a state that needs more has
-//            all its states' exact tables packed and counted again (pack_slice).
+//            all its states' exact tables packed and counted again (recount_slice).
 //            Bound by issue and the LSU: 46 warp instructions and 11 LSU
 //            wavefronts per 32 (state, realization) items -- 17 FMAs, 4 lookups,
 //            3 wavefronts of shared counts, 4 of coefficients (the earlier
@@ -257,7 +257,7 @@ struct FineGeo {
 // [NW][NW spw] float4, then NW slices of `words` table words each.  A state
 // counts into its share of them, a power of two; a slice with a state that needs
 // more than its share has its states' exact tables packed into the whole
-// (pack_slice).
+// (recount_slice).
 // Per-warp totals, added to the model's counters by warp_flush().
 struct WarpAcc {
   unsigned long long samples, nnz, dom, maxrow;
@@ -267,7 +267,10 @@ struct WarpAcc {
 // modulo the table by 32-bit overflow, lin = n_x aN + r4_x aR + n_y bN + r4_y bR +
 // c0 in units of 2^32 / words, its byte offset the high half of lin * bytes.
 struct StateSetup {
-  int4 win;              // the window's (xmin, ymin, gx, pitch << 8 | rotation); gy = pitch - 1
+  int4 win;              // the window's (xmin, ymin, gx, pitch); gy = pitch - 1
+  float4 u;              // extremes of u: (min x, min y, max x, max y)
+  int4 X;                // and their fine coordinates
+  int32_t off;           // the window's first word in the slice's table memory
   uint32_t base, bytes, aN, aR, c0;
   int32_t layer;         // time layer; -1: not sampled
   int32_t kind;          // state_kind
@@ -431,7 +434,8 @@ __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, i
   const int rot = room < table ? (q * 32 / G - centre) & 31 : 0;
   if (lane % per != 0) return;
   StateSetup st;
-  st.win = make_int4(xmin, ymin, gx, pitch << 8 | rot);
+  st.win = make_int4(xmin, ymin, gx, pitch);
+  st.off = lane / per * table + rot;
   st.layer = sample ? (int32_t)t : -1;
   st.kind = ld.kind;
   st.vbx = ld.vb.x;
@@ -445,21 +449,23 @@ __device__ __forceinline__ void setup_slice(const BuildArgs &a, GroupSmem &sm, i
   sm.st[q] = st;
 }
 
-// Counts state s again with the exact table g (the warp owning its slice; st: the
-// state's set-up, tab: its table memory; care: some fraction lies below
-// act.rank_trap).  Rare where windows hold 5 standard deviations and more, but every
+// Counts state s, the group's q-th, again with the exact table g (the warp owning its
+// slice), in the `words` words at g.base of the slice's memory.  Rare where windows hold 5 standard deviations and more, but every
 // second state or so where a share is small for its states (few actions, wide
 // spreads): hence the counting loop's lookups and two rows in flight.
 template <int KT, int MODE>
-__device__ __noinline__ void recount_state(const BuildArgs &a, const RankTables &rt, const StateSetup &st, int64_t s,
-                                           const FineGeo g, uint32_t *tab, int words, bool care) {
+__device__ __forceinline__ void recount_state(const BuildArgs &a, const GroupSmem &sm, int64_t s, int q, const FineGeo &g,
+                                              uint32_t *grid, int words) {
+  const RankTables &rt = sm.rt;
+  const StateSetup &st = sm.st[q];
+  uint32_t *tab = grid + g.base;
+  const bool care = MODE <= 2 && (sm.trap >> q & 1u);   // some fraction lies below act.rank_trap
   const int lane = threadIdx.x & 31, K = mode_count<KT>(a.K), B = a.act.rank_buckets, N = a.N;
   const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1;
   for (int i = lane; i < words; i += 32) tab[i] = 0u;
   __syncwarp();
   if (g.gx == 1 && g.gy == 1) {   // every realization in one cell
     if (lane == 0) tab[g.pitch + 1] = (uint32_t)N;
-    __syncwarp();
     return;
   }
   const int64_t t = st.layer;
@@ -577,54 +583,58 @@ __device__ __forceinline__ float state_extreme(const float4 *ext, int qg, int NW
   m = min_nan(m, __shfl_xor_sync(0xffffffffu, m, 16));
   return lane & 2 ? -m : m;
 }
-// The table of exactly a state's extremes (m of state_extreme), base unset.
-template <int MODE>
-__device__ __forceinline__ FineGeo exact_table(float m, int Sx, int Sy, const RankTables &rt, int buckets) {
-  const int lane = threadIdx.x & 31;
-  const int X = fine_coord<MODE>(m, lane & 1 ? Sy : Sx, rt, lane & 1, buckets);
+// The table of exactly a state's extremes, base unset.
+__device__ __forceinline__ FineGeo exact_table(const StateSetup &st) {
   FineGeo g;
-  g.xmin = __shfl_sync(0xffffffffu, X, 0);
-  g.ymin = __shfl_sync(0xffffffffu, X, 1);
-  g.gx = __shfl_sync(0xffffffffu, X, 2) - g.xmin + 1;
-  g.gy = __shfl_sync(0xffffffffu, X, 3) - g.ymin + 1;
+  g.xmin = st.X.x;
+  g.ymin = st.X.y;
+  g.gx = st.X.z - st.X.x + 1;
+  g.gy = st.X.w - st.X.y + 1;
   g.pitch = (g.gy + 1) | 1;
   g.base = 0;
   return g;
 }
 __device__ __forceinline__ long long table_cells(const FineGeo &g) { return (long long)(g.gx + 1) * g.pitch; }
 
-// A slice with a state that needs more than its share of the table memory: the
-// states' exact tables back to back in all `words` words, each counted again (and
-// summed, if SUM) -- what a state leaves is another's.  Returns the table of the
-// lane's row (base -1 in every lane: they do not fit together).  Whole warp; rare.
-template <int KT, int MODE, bool SUM>
-__device__ __noinline__ FineGeo pack_slice(const BuildArgs &a, const GroupSmem &sm, const float4 *ext, int64_t sl,
-                                           uint32_t *grid, int words, int spw) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5, G = NW * spw;
-  const int Sx = a.act.Dx + 1, Sy = a.act.Dy + 1, B = a.act.rank_buckets, q_l = lane / (32 / spw);
-  FineGeo mine{};
-  long long total = 0;
-  for (int q = 0; q < spw; ++q) {
-    if (sm.st[warp * spw + q].layer < 0) continue;
-    total += table_cells(exact_table<MODE>(state_extreme(ext, warp * spw + q, NW, G), Sx, Sy, sm.rt, B));
-  }
-  if (total > (long long)words) {
-    mine.base = -1;
-    return mine;
+// Counts again the states `missed` (bits q) of a slice, whose predicted windows did not
+// hold them, each with its exact table in its share of the slice's memory -- or, if
+// one of them needs more, every sampled state, the tables back to back in all `words`
+// words: what a state leaves is another's.  These tables become the states' windows
+// (false: they do not fit together).  Whole warp.
+template <int KT, int MODE>
+__device__ __noinline__ bool recount_slice(const BuildArgs &a, GroupSmem &sm, int64_t sl, uint32_t *grid, int words,
+                                           int share, int spw, uint32_t missed) {
+  const int lane = threadIdx.x & 31, first = (threadIdx.x >> 5) * spw;
+  StateSetup *st = sm.st + first;
+  bool pack = false;
+  for (uint32_t left = missed; left; left &= left - 1u)
+    pack |= table_cells(exact_table(st[__ffs(left) - 1])) > (long long)share;
+  if (pack) {
+    missed = 0u;
+    long long total = 0;
+    for (int q = 0; q < spw; ++q) {
+      if (st[q].layer < 0) continue;
+      missed |= 1u << q;
+      total += table_cells(exact_table(st[q]));
+    }
+    if (total > (long long)words) return false;
   }
   int base = 0;
-  for (int q = 0; q < spw; ++q) {
-    if (sm.st[warp * spw + q].layer < 0) continue;
-    FineGeo g = exact_table<MODE>(state_extreme(ext, warp * spw + q, NW, G), Sx, Sy, sm.rt, B);
+  for (uint32_t left = missed; left; left &= left - 1u) {
+    const int q = __ffs(left) - 1;
+    FineGeo g = exact_table(st[q]);
     const int cells = (int)table_cells(g);
-    g.base = base;
-    recount_state<KT, MODE>(a, sm.rt, sm.st[warp * spw + q], sl * spw + q, g, grid + base, cells,
-                            MODE <= 2 && (sm.trap >> (warp * spw + q) & 1u));
-    if (SUM) prefix_table(grid + base, g);
-    if (q == q_l) mine = g;
+    g.base = pack ? base : q * share;
     base += cells;
+    recount_state<KT, MODE>(a, sm, sl * spw + q, first + q, g, grid, pack ? cells : share);
+    __syncwarp();
+    if (lane == 0) {
+      st[q].win = make_int4(g.xmin, g.ymin, g.gx, g.pitch);
+      st[q].off = g.base;
+    }
   }
-  return mine;
+  __syncwarp();
+  return true;
 }
 
 // One row of a slice (lane l = row (q, a)) and its state's prefix table.
@@ -1172,56 +1182,55 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   uint32_t *stage = tabs - (size_t)(NW - warp) * (32 * kStage);   // the stages precede the tables
   RowGeo r{};
   r.hix = r.hiy = -1;
-  bool build = sl < a.slice_end, defer = false, pack = false;
+  bool build = sl < a.slice_end, defer = false;
   if (build) {
     const int q_l = lane / (32 / spw), a_l = lane % (32 / spw);
     r.kind = a_l < a.A ? sm.st[warp * spw + q_l].kind : (int)KIND_NONE;
     r.rows = r.kind == KIND_SAMPLE;
+    // the states' extremes and whether they lie in the predicted windows, lane & 3 =
+    // component of (min x, min y, max x, max y)
+    uint32_t missed = 0u;
     for (int q = 0; q < spw; ++q) {
-      const int qg = warp * spw + q;
-      const int64_t s = sl * spw + q;
-      const int layer = sm.st[qg].layer;
-      if (layer == -1) continue;   // not sampled
-      const float m = state_extreme(ext, qg, NW, G);
+      StateSetup &st = sm.st[warp * spw + q];
+      if (st.layer < 0) continue;   // not sampled
+      const float m = state_extreme(ext, warp * spw + q, NW, G);
       if (!__all_sync(0xffffffffu, m > -kTame && m < kTame)) {   // non-finite or far velocities: the CTA kernel's path
         defer = true;
-        continue;
+        break;
       }
-      const float mnx = __shfl_sync(0xffffffffu, m, 0), mny = __shfl_sync(0xffffffffu, m, 1);
-      const float mxx = __shfl_sync(0xffffffffu, m, 2), mxy = __shfl_sync(0xffffffffu, m, 3);
+      const bool y = lane & 1, top = lane & 2;
+      const int X = fine_coord<MODE>(m, y ? Sy : Sx, sm.rt, y, B);
+      const int4 win = st.win;
+      const int lo = y ? win.y : win.x, n = y ? win.w - 1 : win.z;
+      const bool out = top ? X >= lo + n : X < lo;
+      if (__any_sync(0xffffffffu, out) || (MODE <= 2 && ((sm.trap >> (warp * spw + q)) & 1u))) missed |= 1u << q;
+      if (lane < 4) {
+        (&st.u.x)[lane] = m;
+        (&st.X.x)[lane] = X;
+      }
+    }
+    __syncwarp();
+    if (missed && !defer) defer = !recount_slice<KT, MODE>(a, sm, sl, grid, words, share, spw, missed);
+    for (int q = 0; q < spw && !defer; ++q) {
+      const StateSetup &st = sm.st[warp * spw + q];
+      if (st.layer < 0) continue;
+      const float4 u = st.u;
       if (q == q_l && r.rows) {
         const int cxa = sm.rt.c[0][a_l], cya = sm.rt.c[1][a_l];
         const float thxa = sm.rt.th[0][a_l], thya = sm.rt.th[1][a_l];
-        r.lox = land_offset(mnx, cxa, thxa); r.hix = land_offset(mxx, cxa, thxa);
-        r.loy = land_offset(mny, cya, thya); r.hiy = land_offset(mxy, cya, thya);
+        r.lox = land_offset(u.x, cxa, thxa); r.hix = land_offset(u.z, cxa, thxa);
+        r.loy = land_offset(u.y, cya, thya); r.hiy = land_offset(u.w, cya, thya);
         if (r.lox < -a.h || r.hix > a.h || r.loy < -a.h || r.hiy > a.h) {   // sub-grid overflow
           r.rows = false;
           atomicAdd(&a.cnt[CNT_OVERFLOW], 1ULL);
         }
       }
       // the exact table inside the window (its pitch, its own origin)
-      FineGeo g = exact_table<MODE>(m, Sx, Sy, sm.rt, B);
-      const int4 win = sm.st[qg].win;
-      const int exact_pitch = g.pitch;
-      g.pitch = win.w >> 8;
-      g.base = q * share + (win.w & 255) + (g.xmin - win.x) * g.pitch + (g.ymin - win.y);
-      if ((MODE <= 2 && ((sm.trap >> qg) & 1u)) || g.xmin < win.x || g.ymin < win.y || g.xmin + g.gx > win.x + win.z || g.ymin + g.gy >= win.y + g.pitch) {
-        // outside the predicted window (or a trapped fraction): the exact table, if it fits
-        g.pitch = exact_pitch;
-        g.base = q * share;
-        if (table_cells(g) > (long long)share) {
-          pack = true;
-          continue;
-        }
-        if (!defer && !pack)
-          recount_state<KT, MODE>(a, sm.rt, sm.st[qg], s, g, grid + g.base, share, MODE <= 2 && (sm.trap >> qg & 1u));
-      }
+      FineGeo g = exact_table(st);
+      g.pitch = st.win.w;
+      g.base = st.off + (g.xmin - st.win.x) * g.pitch + (g.ymin - st.win.y);
       if (q == q_l) r.g = g;
-      if (SPW != 1 && !defer && !pack) prefix_table(grid + g.base, g);
-    }
-    if (pack && !defer) {   // a state needs more than its share
-      r.g = pack_slice<KT, MODE, SPW != 1>(a, sm, ext, sl, grid, words, spw);
-      defer = r.g.base < 0;
+      if (SPW != 1) prefix_table(grid + g.base, g);
     }
     if (defer) {   // too wide (or not finite): the CTA kernel builds the slice
       build = false;
@@ -1239,9 +1248,11 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
     uint64_t blk;
     const BoxCells bc = box_cells<SPW>(a, sl, r, sr, blk);
     if (SPW == 1 && sm.st[warp].layer >= 0) prefix_table(grid + r.g.base, r.g);
-    if (sr.small) {   // (right for rows longer than are staged, too)
-      rc = count_small<SPW>(a, sm.rt, grid, r, bc, blk, stage, sr);
-    } else {
+    // (the small scan's counts are right for rows longer than are staged, too; counted
+    // again all the same in the batched kernel, which is 1.3 % faster that way)
+    const bool boxed = HYB && sr.small;
+    if (sr.small) rc = count_small<SPW>(a, sm.rt, grid, r, bc, blk, stage, sr);
+    if (!boxed && !sr.small) {
       const uint32_t sink = r.kind == KIND_SINK ? (uint32_t)N : 0u;
       rc = count_general<HYB>(a, sl, grid, r);
       rc.sink += sink;
@@ -1289,8 +1300,7 @@ __device__ __forceinline__ void group_slices(const BuildArgs &a, int64_t sl0, Gr
   // the slice's tables are zero again
   __syncwarp();
   uint4 *p = reinterpret_cast<uint4 *>(grid);
-  const int used = (pack ? words : share * spw) / 4;
-  for (int i = lane; i < used; i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = lane; i < words / 4; i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
   if (next_first(g1) >= 0) setup_slice<SPW, MODE>(a, sm, next_first(g1), ld, tabs, words, share);
 }
 
