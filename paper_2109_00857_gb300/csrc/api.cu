@@ -509,7 +509,7 @@ mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_action
   ba.pool = m->pool; ba.pool_cap_cols = cap_cols; ba.slice_off = m->slice_off; ba.slice_w = m->slice_w; ba.nnz = m->nnz; ba.sinkc = m->sinkc;
   ba.R = m->R; ba.cnt = m->cnt;
   ba.slice_begin = 0; ba.slice_end = m->n_slices;
-  ba.slices_per_warp = lim ? lim->slices_per_warp : 0;
+  ba.groups_per_cta = lim ? lim->groups_per_cta : 0;
   // spill area: the caller's size when it fixes the pool (the server), else none yet
   uint64_t spill_cap = (lim && lim->pool_cols) ? lim->spill_words : 0;
   auto alloc_spill = [&](uint64_t words) -> cudaError_t {

@@ -48,7 +48,7 @@ cudaError_t launch_coeff_moments(const float *Y, int nt, int N, int K, float2 *m
 }
 
 // Single model: CTAs pull groups of slices from the model's work queue --
-// persistent CTAs, or at most a.slices_per_warp groups each (the grid then
+// persistent CTAs, or at most a.groups_per_cta groups each (the grid then
 // covers the model, so every group is taken).
 template <int KT, int SPW, int MODE>
 __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_kernel(const __grid_constant__ BuildArgs a, int words,
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, kMinCtas<KT>) build_group_ke
     const long long g = sm.next[par];
     if (g >= n_groups) break;
     long long next = n_groups;   // this CTA's share may end with this group
-    if (threadIdx.x == 0 && (a.slices_per_warp == 0 || n < a.slices_per_warp)) {
+    if (threadIdx.x == 0 && (a.groups_per_cta == 0 || n < a.groups_per_cta)) {
       if (left > 0) {
         next = g + 1;
         --left;
@@ -109,9 +109,9 @@ static cudaError_t launch_g(const BuildArgs &a, int warps, int sms, cudaStream_t
   // groups per queue grab: at least 32 grabs a CTA, at most 8 groups (the
   // queue's one address takes about 2 ns per grab)
   int chunk = (int)std::min<int64_t>(8, std::max<int64_t>(1, groups / (32 * blocks)));
-  if (a.slices_per_warp > 0) chunk = 1;
-  if (a.slices_per_warp > 0)   // bounded CTAs: a grid that covers every group
-    blocks = (groups + a.slices_per_warp - 1) / a.slices_per_warp;
+  if (a.groups_per_cta > 0) chunk = 1;
+  if (a.groups_per_cta > 0)   // bounded CTAs: a grid that covers every group
+    blocks = (groups + a.groups_per_cta - 1) / a.groups_per_cta;
   build_group_kernel<KT, SPW, MODE><<<(unsigned)std::max<int64_t>(blocks, 1), nw * 32, smem, st>>>(
       a, words, share_words(a.cap_bins, a.spw), chunk);
   return cudaGetLastError();

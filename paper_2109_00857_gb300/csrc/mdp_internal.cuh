@@ -148,7 +148,7 @@ struct alignas(16) BuildArgs {
   // group); q > 0 = each CTA builds at most q groups and the grid covers the
   // model, so CTAs retire all along the build and the block scheduler can
   // place higher-priority work (another request's launches) between them
-  int32_t slices_per_warp;
+  int32_t groups_per_cta;
   ActionTable act;           // last: see ActionTable
 };
 
@@ -408,7 +408,7 @@ struct BuildLimits {
   uint64_t pool_cols_needed = 0;   // out (MDP_ERR_BUDGET): the columns the slices need
   uint64_t spill_words = 0;        // in (with pool_cols): spill words to allocate (0: none)
   uint64_t spill_words_needed = 0; // out (MDP_ERR_BUDGET): the spill words the rows need
-  int32_t slices_per_warp = 0;     // in: BuildArgs::slices_per_warp of the group kernel
+  int32_t groups_per_cta = 0;     // in: BuildArgs::groups_per_cta of the group kernel
 };
 mdp_status build_impl(const mdp_env *env, const mdp_grid *grid, const mdp_actions *actions, int32_t N,
                       int32_t subgrid_L, const int32_t *objs_h, int32_t n_obj, const mdp_build_opts *opts,

@@ -33,8 +33,8 @@
 // oldest request in flight runs the persistent kernels (a build and sweeps
 // that occupy every SM); a younger request runs beside it only when its work
 // (states x N) is at most kServeShareFraction of the oldest one's, with
-// kernels that leave the SMs along their run (build warps that take
-// kServeSlicesPerWarp slices each, sweeps of small CTAs); a larger one waits
+// kernels that leave the SMs along their run (build CTAs that take
+// kServeGroupsPerCta groups of slices each, sweeps of small CTAs); a larger one waits
 // until it is the oldest, since two full-GPU builds would only slow the older
 // one down.  Idle workers wait on their own condition variables and a new
 // request wakes the most recently idle one, whose stream and buffers are warm.
@@ -203,8 +203,8 @@ __global__ void target_block_kernel(uint8_t *tgt, int nx, int ny, int i0, int j0
   }
 }
 
-// slices per build warp when requests share the GPU (BuildArgs::slices_per_warp)
-constexpr int kServeSlicesPerWarp = 8;
+// groups of slices per build CTA when requests share the GPU (BuildArgs::groups_per_cta)
+constexpr int kServeGroupsPerCta = 8;
 // a younger request runs beside the oldest one only when its work is at most
 // this fraction of the oldest one's
 constexpr double kServeShareFraction = 0.25;
@@ -262,7 +262,7 @@ bool run_job(mdp_server_t *S, Job &job, cudaStream_t st, uint8_t *tgt) {
     std::lock_guard<std::mutex> lk(S->mu);
     return !S->running.empty() && S->running.front().get() != &job;
   };
-  lim.slices_per_warp = younger() ? kServeSlicesPerWarp : 0;
+  lim.groups_per_cta = younger() ? kServeGroupsPerCta : 0;
   mdp_status s = build_impl(&env, &grid, &e.actions, r.N, e.L, &obj, 1, nullptr, st, &m, nullptr, &lim);
   if (s == MDP_ERR_BUDGET &&
       (lim.pool_cols_needed > job.pool_cols || lim.spill_words_needed > job.spill_words)) {
