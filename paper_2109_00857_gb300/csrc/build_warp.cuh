@@ -299,7 +299,10 @@ __host__ __device__ constexpr int group_warps(int warps, int spw) {
   const int most = 32 / spw < kGroupWarps ? 32 / spw : kGroupWarps;   // at most one state per lane
   return warps < most ? warps : most;
 }
-constexpr int kStage = 12;   // entries per row the emit stages (longest row measured: 12); 1.5 KB per warp
+// Entries per row that the emit stages, 1.5 KB per warp (the workloads' longest row: 12).
+// A slice with a longer row is written by a second scan; with more staged, a fifth CTA
+// would no longer fit an SM from 18 on.
+constexpr int kStage = 12;
 // Bytes before the table memory (the head, the extremes, the entry stages), and
 // of a CTA's dynamic shared memory.
 // `before`: bytes the kernel puts in front of GroupSmem (a multiple of 16).
